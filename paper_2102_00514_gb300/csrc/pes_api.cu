@@ -221,6 +221,7 @@ void fill_workspace(pes_handle* h, KParams<T>& p, const Shape& s)
     p.lin = static_cast<T*>(h->lin);
     p.aggF = static_cast<T*>(h->aggF);
     p.aggS = static_cast<T*>(h->aggS);
+    p.agg_blocks = h->nb_max;
     p.bar = h->bar;
     p.status = h->status;
     p.conv = h->conv;
@@ -228,7 +229,7 @@ void fill_workspace(pes_handle* h, KParams<T>& p, const Shape& s)
     p.traj_iters = nullptr;
     p.L = s.L;
     p.NL = s.nb * s.nt;
-    p.cs = p.lanes_layout ? (int64_t)s.L * p.NL : p.N;
+    p.cs = (int64_t)s.L * p.NL;
     p.timeout_ns = h->timeout_ns;
     p.ptime = h->ptime;
     h->ptime_blocks = s.nb;
@@ -283,31 +284,38 @@ pes_status run_persistent_shaped(pes_handle* h, KParams<T>& p, int lin, const Sh
     return PES_OK;
 }
 
-template <typename T>
-pes_status run_persistent(pes_handle* h, KParams<T>& p, int lin, pes_precision prec, cudaStream_t st)
-{
-    Shape s;
-    pes_status r = make_shape<T>(h, lin, prec, p.N, s);
-    if (r != PES_OK) return r;
-    return run_persistent_shaped(h, p, lin, s, st);
-}
-
 }  // namespace
 
+// The scans over given arrays stream lane-major copies of them, in the memory of
+// the run's stored linearisation (62 and 65 components in) and of its trajectory
+// (20 out): read in place, a lane's strided values cost every step the sectors of
+// the whole chunk (N = 128,128, FP32: 128 and 100 us per scan).
 template <typename T>
 static pes_status filter_scan_t(pes_handle* h, const void* F, const void* c, const void* Qp, const void* H,
                                 const void* d, const void* Rp, const void* y, const void* m0, const void* P0,
                                 const int64_t* offsets, int32_t B, int64_t N, void* xf, void* Pf, pes_precision prec,
                                 cudaStream_t st, double* loglik = nullptr)
 {
+    Shape s;
+    pes_status r = make_shape<T>(h, LIN_ARRAYS, prec, N, s);
+    if (r != PES_OK) return r;
+    const int NL = s.nb * s.nt;
+    const int64_t cs = (int64_t)s.L * NL;
+    T* in = static_cast<T*>(h->lin);
+    T* out = static_cast<T*>(h->lanes);
+    LaneArrays<T> ai, ao;
+    ai.add(F, 25).add(c, 5).add(Qp, 15).add(H, 10).add(d, 2).add(Rp, 3).add(y, 2);
+    ao.add(xf, 5).add(Pf, 15);
+    PES_CUDA(h, launch_lanes_move(ai, in, N, s.L, NL, MOVE_IN_BLOCKED, st));
     KParams<T> p{};
     p.N = N; p.offsets = offsets; p.B = B; p.mode = MODE_FILTER; p.iters = 1;
     if (loglik) PES_CUDA(h, cudaMemsetAsync(loglik, 0, sizeof(double) * B, st));
     p.loglik = loglik;
-    p.F = (const T*)F; p.c = (const T*)c; p.Qp = (const T*)Qp; p.H = (const T*)H; p.d = (const T*)d;
-    p.Rp = (const T*)Rp; p.y = (const T*)y; p.m0 = (const T*)m0; p.P0 = (const T*)P0;
-    p.xf = (T*)xf; p.Pf = (T*)Pf;
-    return run_persistent<T>(h, p, LIN_ARRAYS, prec, st);
+    p.m0 = (const T*)m0; p.P0 = (const T*)P0;
+    p.xf = out; p.Pf = out + 5 * cs;
+    if ((r = run_persistent_shaped(h, p, LIN_ARRAYS, s, st)) != PES_OK) return r;
+    PES_CUDA(h, launch_lanes_move(ao, out, N, s.L, NL, MOVE_OUT, st));
+    return PES_OK;
 }
 
 template <typename T>
@@ -315,11 +323,59 @@ static pes_status smooth_scan_t(pes_handle* h, const void* F, const void* c, con
                                 const void* Pf, const int64_t* offsets, int32_t B, int64_t N, void* xs, void* Ps,
                                 pes_precision prec, cudaStream_t st)
 {
+    Shape s;
+    pes_status r = make_shape<T>(h, LIN_ARRAYS, prec, N, s);
+    if (r != PES_OK) return r;
+    const int NL = s.nb * s.nt;
+    const int64_t cs = (int64_t)s.L * NL;
+    T* in = static_cast<T*>(h->lin);
+    T* out = static_cast<T*>(h->lanes);
+    LaneArrays<T> ai, ao;
+    ai.add(F, 25).add(c, 5).add(Qp, 15).add(xf, 5).add(Pf, 15);
+    ao.add(xs, 5).add(Ps, 15);
+    PES_CUDA(h, launch_lanes_move(ai, in, N, s.L, NL, MOVE_IN_BLOCKED, st));
     KParams<T> p{};
     p.N = N; p.offsets = offsets; p.B = B; p.mode = MODE_SMOOTH; p.iters = 1;
-    p.F = (const T*)F; p.c = (const T*)c; p.Qp = (const T*)Qp;
-    p.xf = (T*)xf; p.Pf = (T*)Pf; p.x = (T*)xs; p.P = (T*)Ps;
-    return run_persistent<T>(h, p, LIN_ARRAYS, prec, st);
+    p.x = out; p.P = out + 5 * cs;
+    if ((r = run_persistent_shaped(h, p, LIN_ARRAYS, s, st)) != PES_OK) return r;
+    PES_CUDA(h, launch_lanes_move(ao, out, N, s.L, NL, MOVE_OUT, st));
+    return PES_OK;
+}
+
+// A run's lane-major arrays in h->lanes, from lx on: the trajectory's means (5),
+// covariances (15) and the measurements (2). In: the measurements and the given
+// parts of the initial nominal; out: the smoothed moments.
+template <typename T>
+static pes_status move_in(pes_handle* h, T* lx, const void* y, const void* x_init, const void* P_init, int64_t N,
+                          const Shape& s, cudaStream_t st)
+{
+    const int NL = s.nb * s.nt;
+    const int64_t cs = (int64_t)s.L * NL;
+    LaneArrays<T> a;
+    if (x_init) a.add(x_init, 5);
+    if (x_init && P_init) a.add(P_init, 15);
+    // one launch for arrays that are neighbours on the lane-major side
+    if (a.n == 2) {
+        a.add(y, 2);
+        PES_CUDA(h, launch_lanes_move(a, lx, N, s.L, NL, MOVE_IN, st));
+        return PES_OK;
+    }
+    if (a.n) PES_CUDA(h, launch_lanes_move(a, lx, N, s.L, NL, MOVE_IN, st));
+    LaneArrays<T> b;
+    const bool P_only = !x_init && P_init;
+    if (P_only) b.add(P_init, 15);
+    b.add(y, 2);
+    PES_CUDA(h, launch_lanes_move(b, lx + (P_only ? 5 : 20) * cs, N, s.L, NL, MOVE_IN, st));
+    return PES_OK;
+}
+
+template <typename T>
+static pes_status move_out(pes_handle* h, T* lx, void* x_out, void* P_out, int64_t N, const Shape& s, cudaStream_t st)
+{
+    LaneArrays<T> a;
+    a.add(x_out, 5).add(P_out, 15);
+    PES_CUDA(h, launch_lanes_move(a, lx, N, s.L, s.nb * s.nt, MOVE_OUT, st));
+    return PES_OK;
 }
 
 template <typename T>
@@ -338,10 +394,8 @@ static pes_status ieks_run_t(pes_handle* h, const pes_model* model, pes_method m
     T* lx = static_cast<T*>(h->lanes);
     T* lP = lx + 5 * cs;
     T* ly = lP + 15 * cs;
-    PES_CUDA(h, launch_lanes_transpose<T>((const T*)y, ly, 2, N, s.L, NL, true, st));
     const bool cub = (method != PES_IEKS);
-    if (x_init) PES_CUDA(h, launch_lanes_transpose<T>((const T*)x_init, lx, 5, N, s.L, NL, true, st));
-    if (cub && P_init) PES_CUDA(h, launch_lanes_transpose<T>((const T*)P_init, lP, 15, N, s.L, NL, true, st));
+    if ((r = move_in<T>(h, lx, y, x_init, cub ? P_init : nullptr, N, s, st)) != PES_OK) return r;
     if (!x_init || (cub && !P_init))
         PES_CUDA(h, launch_init_nominal_lanes<T>(offsets, B, N, s.L, NL, (const T*)m0, (const T*)P0,
                                                  x_init ? nullptr : lx, (cub && !P_init) ? lP : nullptr, st));
@@ -352,11 +406,9 @@ static pes_status ieks_run_t(pes_handle* h, const pes_model* model, pes_method m
     if (rm != PES_OK) return rm;
     p.y = ly; p.m0 = (const T*)m0; p.P0 = (const T*)P0;
     p.x = lx; p.P = lP;
-    p.lanes_layout = 1;
     r = run_persistent_shaped<T>(h, p, lin, s, st);
     if (r != PES_OK) return r;
-    PES_CUDA(h, launch_lanes_transpose<T>(lx, (T*)x_out, 5, N, s.L, NL, false, st));
-    PES_CUDA(h, launch_lanes_transpose<T>(lP, (T*)P_out, 15, N, s.L, NL, false, st));
+    if ((r = move_out<T>(h, lx, x_out, P_out, N, s, st)) != PES_OK) return r;
     if (tol > 0.0 || iters_used) {
         int it = 0;
         r = read_status(h, st, &it);
@@ -367,7 +419,7 @@ static pes_status ieks_run_t(pes_handle* h, const pes_model* model, pes_method m
 }
 
 // The sequential counterpart: one thread per trajectory over the caller's
-// layout, the nominal held in x_out / P_out, smoothing elements in h->hand.
+// layout, the nominal held in x_out / P_out, smoothing elements in h->lin.
 template <typename T>
 static pes_status ieks_run_sequential_t(pes_handle* h, const pes_model* model, pes_method method, const void* y,
                                         const int64_t* offsets, int32_t B, int64_t N, const void* m0, const void* P0,
@@ -387,9 +439,8 @@ static pes_status ieks_run_sequential_t(pes_handle* h, const pes_model* model, p
     if (rm != PES_OK) return rm;
     p.y = (const T*)y; p.m0 = (const T*)m0; p.P0 = (const T*)P0;
     p.x = (T*)x_out; p.P = (T*)P_out;
-    p.lanes_layout = 0;
     p.cs = N;
-    p.hand = static_cast<T*>(h->hand);
+    p.lin = static_cast<T*>(h->lin);
     p.status = h->status;
     p.iters_done = h->iters_done;
     p.traj_iters = nullptr;
@@ -459,14 +510,14 @@ static pes_status ieks_run_mixed(pes_handle* h, const pes_model* model, pes_meth
     return r;
 }
 
-// The refinement workspace: nominal and filtered moments (20 + 20 floats per
-// slot), residual elements (RE), stored transitions (RT), the filter's
-// correction (RD), for every lane-major slot the handle can hold.
+// The refinement workspace: the nominal (20 floats per slot), residual elements
+// (RE), stored transitions (RT), the filter's correction (RD), for every
+// lane-major slot the handle can hold.
 static pes_status ensure_refine_workspace(pes_handle* h)
 {
     if (h->refw) return PES_OK;
     const size_t slots = (size_t)h->max_states + (size_t)h->nl_max;
-    PES_CUDA(h, cudaMalloc(&h->refw, sizeof(float) * (20 + 20 + RE + RT + RD) * slots));
+    PES_CUDA(h, cudaMalloc(&h->refw, sizeof(float) * (20 + RE + RT + RD) * slots));
     return PES_OK;
 }
 
@@ -474,7 +525,7 @@ static pes_status ensure_refine_workspace(pes_handle* h)
 // iteration in FP32 and its Newton refinement (pes_refine.cuh): float-float
 // residuals of the filter and RTS recursions about the FP32 solution, and the
 // corrections from two FP32 scans. Everything stays in the lane-major layout
-// of the smoother kernel; the refinement workspace (155 floats per slot) is
+// of the smoother kernel; the refinement workspace (135 floats per slot) is
 // allocated by the first call on the handle.
 static pes_status ieks_run_refined(pes_handle* h, const pes_model* model, pes_method method, const void* y,
                                    const int64_t* offsets, int32_t B, int64_t N, const void* m0, const void* P0,
@@ -504,14 +555,11 @@ static pes_status ieks_run_refined(pes_handle* h, const pes_model* model, pes_me
     float* lP = lx + 5 * cs;
     float* ly = lP + 15 * cs;
     float* nom = static_cast<float*>(h->refw);
-    float* filt = nom + 20 * cs;
-    float* elem = filt + 20 * cs;
+    float* elem = nom + 20 * cs;
     float* trans = elem + RE * cs;
     float* dlt = trans + RT * cs;
-    PES_CUDA(h, launch_lanes_transpose<float>((const float*)y, ly, 2, N, s.L, NL, true, st));
     const bool cub = (method != PES_IEKS);
-    if (x_init) PES_CUDA(h, launch_lanes_transpose<float>((const float*)x_init, lx, 5, N, s.L, NL, true, st));
-    if (cub && P_init) PES_CUDA(h, launch_lanes_transpose<float>((const float*)P_init, lP, 15, N, s.L, NL, true, st));
+    if ((r = move_in<float>(h, lx, y, x_init, cub ? P_init : nullptr, N, s, st)) != PES_OK) return r;
     if (!x_init || (cub && !P_init))
         PES_CUDA(h, launch_init_nominal_lanes<float>(offsets, B, N, s.L, NL, (const float*)m0, (const float*)P0,
                                                      x_init ? nullptr : lx, (cub && !P_init) ? lP : nullptr, st));
@@ -520,7 +568,6 @@ static pes_status ieks_run_refined(pes_handle* h, const pes_model* model, pes_me
     if ((r = device_model<float>(h, *model, B, st, p.model, method)) != PES_OK) return r;
     p.y = ly; p.m0 = (const float*)m0; p.P0 = (const float*)P0;
     p.x = lx; p.P = lP;
-    p.lanes_layout = 1;
     int32_t it32 = 0;
     pes_status r32 = PES_OK;
     if (max_iters > 1) {
@@ -536,12 +583,11 @@ static pes_status ieks_run_refined(pes_handle* h, const pes_model* model, pes_me
             it32 = max_iters - 1;
         }
     }
-    // the final iteration's nominal, then the iteration itself with its filtered moments kept
+    // the final iteration's nominal, then the iteration itself, which leaves its filtered moments in h->hand
     PES_CUDA(h, cudaMemcpyAsync(nom, lx, sizeof(float) * 20 * cs, cudaMemcpyDeviceToDevice, st));
     p.iters = 1;
     p.tol = 0.0;
     p.write_P_every_iter = 1;
-    p.fstore = filt;
     {
         pes::TraceRange trace_("final FP32 iteration");
         if ((r = run_persistent_shaped<float>(h, p, lin, s, st)) != PES_OK) return r;
@@ -552,7 +598,7 @@ static pes_status ieks_run_refined(pes_handle* h, const pes_model* model, pes_me
         rp.N = N; rp.offsets = offsets; rp.B = B; rp.L = s.L; rp.NL = NL; rp.cs = cs;
         rp.model = p.model;
         rp.y = ly; rp.m0 = (const float*)m0; rp.P0 = (const float*)P0;
-        rp.nom = nom; rp.filt = filt; rp.xs = lx;
+        rp.nom = nom; rp.filt = static_cast<const float*>(h->hand); rp.xs = lx;
         rp.elem = elem; rp.trans = trans; rp.dlt = dlt;
         rp.agg = static_cast<float*>(h->aggF);
         rp.bar = h->bar;
@@ -567,8 +613,7 @@ static pes_status ieks_run_refined(pes_handle* h, const pes_model* model, pes_me
         e = launch_refine_scan(rp, false, s.nt, s.nb, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "cooperative launch of the refinement scan");
     }
-    PES_CUDA(h, launch_lanes_transpose<float>(lx, (float*)x_out, 5, N, s.L, NL, false, st));
-    PES_CUDA(h, launch_lanes_transpose<float>(lP, (float*)P_out, 15, N, s.L, NL, false, st));
+    if ((r = move_out<float>(h, lx, x_out, P_out, N, s, st)) != PES_OK) return r;
     if (tol > 0.0 || iters_used) {
         r = read_status(h, st);
         if (iters_used) *iters_used = it32 + 1;
@@ -691,8 +736,7 @@ static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_preci
     for (int i = 0; i < 5; ++i) lp.c[i] = model->c[i];
     for (int i = 0; i < 10; ++i) lp.H[i] = model->H[i];
     for (int i = 0; i < 2; ++i) lp.d[i] = model->d[i];
-    PES_CUDA(h, launch_lanes_transpose<T>((const T*)y, ly, 2, N, s.L, NL, true, st));
-    if (x_init) PES_CUDA(h, launch_lanes_transpose<T>((const T*)x_init, lx, 5, N, s.L, NL, true, st));
+    if ((r = move_in<T>(h, lx, y, x_init, nullptr, N, s, st)) != PES_OK) return r;
     // covariances start at the prior's: a trajectory whose every step is
     // rejected returns them
     PES_CUDA(h, launch_init_nominal_lanes<T>(offsets, B, N, s.L, NL, (const T*)m0, (const T*)P0,
@@ -708,7 +752,6 @@ static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_preci
     p.model.lm_traj = lam;
     p.y = ly; p.m0 = (const T*)m0; p.P0 = (const T*)P0;
     p.x = lx; p.P = lP;
-    p.lanes_layout = 1;
     int it = 0;
     bool all = false;
     for (it = 1; it <= max_iters; ++it) {
@@ -730,8 +773,7 @@ static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_preci
         }
     }
     if (it > max_iters) it = max_iters;
-    PES_CUDA(h, launch_lanes_transpose<T>(lx, (T*)x_out, 5, N, s.L, NL, false, st));
-    PES_CUDA(h, launch_lanes_transpose<T>(lP, (T*)P_out, 15, N, s.L, NL, false, st));
+    if ((r = move_out<T>(h, lx, x_out, P_out, N, s, st)) != PES_OK) return r;
     if (lambda_out) {
         T* tmp = new (std::nothrow) T[B];
         if (!tmp) return fail(h, PES_ERR_CUDA, "out of host memory");
@@ -788,8 +830,8 @@ pes_status pes_create(pes_handle** out, int64_t max_states, int32_t max_batch)
     e = cudaMalloc(&h->hand, hand_elems * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->lanes, (size_t)22 * ((size_t)max_states + (size_t)h->nl_max) * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->lin, (size_t)LINS * ((size_t)max_states + (size_t)h->nl_max) * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&h->aggF, (size_t)h->nb_max * FE * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&h->aggS, (size_t)h->nb_max * SE * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&h->aggF, (size_t)h->nb_max * 2 * FE * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&h->aggS, (size_t)h->nb_max * 2 * SE * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->bar, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->status, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->conv, sizeof(double) * 4 * (size_t)max_batch);

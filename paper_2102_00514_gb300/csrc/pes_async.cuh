@@ -2,9 +2,9 @@
 // asynchronous copies (cp.async.bulk, completion counted on an mbarrier).
 //
 // The handoff buffers are laid out [warp][step][component][32 lanes], so the
-// data a warp needs at one step is one contiguous block. A stream keeps two
+// data a warp needs at one step is one contiguous block. A stream keeps a few
 // shared-memory stages per warp: while the warp consumes step s from one
-// stage, the copy of the next step lands in the other. One lane issues the
+// stage, the copies of the next steps land in the others. One lane issues the
 // copies; every lane reads its own column of the stage.
 //
 // Every wait is bounded: after about a second a wait gives up, sets
@@ -28,12 +28,17 @@ PES_DEV void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.clust
 // Order earlier generic-proxy shared-memory accesses before later bulk copies.
 PES_DEV void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// Bulk copy of `bytes` (multiple of 16, both addresses 16-byte aligned) from
-// global to shared memory, completing a transaction count on `bar`.
-PES_DEV void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
+// The one arrival of a phase of `bar`, which completes with `bytes` copied.
+PES_DEV void bulk_expect(uint64_t* bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
+}
+
+// Bulk copy of `bytes` (multiple of 16, both addresses 16-byte aligned) from
+// global to shared memory, counted on `bar`.
+PES_DEV void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
+{
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
             smem_u32(dst)),
@@ -75,35 +80,42 @@ PES_DEV void mbar_wait(uint64_t* bar, uint32_t parity, int* status)
     }
 }
 
-// Stream of one warp through blocks of NC * 32 scalars spaced SLOT * 32
-// scalars apart (step s of the warp's slot range at base + s * SLOT * 32).
-template <typename T, int NC, int SLOT>
+// Stream of one warp through blocks of NC * 32 scalars, ST stages deep.
+template <typename T, int NC, int ST>
 struct WarpStream {
-    static constexpr uint32_t kBytes = NC * 32 * sizeof(T);
-    static_assert(kBytes % 16 == 0, "bulk copies move multiples of 16 bytes");
-    const T* base;   // global: this warp's step 0
-    T* stage;        // shared: [2][NC * 32]
-    uint64_t* bar;   // shared: 2 barriers
+    static_assert((32 * sizeof(T)) % 16 == 0, "bulk copies move multiples of 16 bytes");
+    T* stage;        // shared: [ST][NC * 32]
+    uint64_t* bar;   // shared: a barrier per stage
     uint32_t parity; // expected parity per stage (bit i)
     int lane;
 
     // `par` is the warp's barrier parity state, carried across streams that
     // reuse the same barriers.
-    PES_DEV void init(const T* warp_base, T* stage_mem, uint64_t* bars, uint32_t par)
+    PES_DEV void init(T* stage_mem, uint64_t* bars, uint32_t par)
     {
-        base = warp_base;
         stage = stage_mem;
         bar = bars;
         parity = par;
         lane = threadIdx.x & 31;
     }
-    // Start the copy of step s into stage i (all lanes call; lane 0 issues).
+    // Start the copy of a block into stage i (all lanes call; lane 0 issues).
     // The stage must no longer be read (a __syncwarp since its last use).
-    PES_DEV void issue(int s, int i)
+    PES_DEV void issue(const T* src, int i)
     {
         if (lane == 0) {
             fence_proxy_async();
-            bulk_g2s(stage + i * NC * 32, base + (size_t)s * SLOT * 32, kBytes, bar + i);
+            bulk_expect(bar + i, NC * 32 * sizeof(T));
+            bulk_g2s(stage + i * NC * 32, src, NC * 32 * sizeof(T), bar + i);
+        }
+    }
+    // The same for a block in two parts of n1 and n2 components (n1 + n2 = NC).
+    PES_DEV void issue2(const T* src1, int n1, const T* src2, int n2, int i)
+    {
+        if (lane == 0) {
+            fence_proxy_async();
+            bulk_expect(bar + i, NC * 32 * sizeof(T));
+            bulk_g2s(stage + i * NC * 32, src1, n1 * 32 * sizeof(T), bar + i);
+            bulk_g2s(stage + i * NC * 32 + n1 * 32, src2, n2 * 32 * sizeof(T), bar + i);
         }
     }
     PES_DEV void wait(int i, int* status)

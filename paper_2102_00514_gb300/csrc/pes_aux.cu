@@ -78,54 +78,125 @@ template cudaError_t launch_convert<float>(const double*, float*, int, cudaStrea
 template cudaError_t launch_convert<double>(const double*, double*, int, cudaStream_t);
 
 // Caller layout [nc][N] <-> the kernel's lane-major layout [nc][L][NL], where
-// state k = lane * L + s sits at s * NL + lane. 32 x 32 tiles through shared
-// memory keep both sides coalesced.
-template <typename T, bool TO_LANES>
-__global__ void lanes_transpose_kernel(const T* src, T* dst, int64_t N, int L, int NL, int64_t cs)
+// state k = lane * L + s sits at s * NL + lane, for several arrays in one
+// launch (their components consecutive on the lane-major side).
+//
+// Bound by memory latency: what counts is bytes in flight. A block takes G lanes
+// of a few components: with L <= W steps a component's states are one
+// contiguous run of the caller's array, so both sides are read and written in
+// full lines whatever L is; longer chunks are cut into pieces of W steps, a warp
+// reading a lane's piece. Everything a block reads is in flight at once, copied
+// into the tile by cp.async, and its stores do not wait. The tile's rows are
+// steps, an odd number of words apart: no bank conflicts on either side. (32 x
+// 32 tiles of (lane, step) leave columns empty and start every row off a line's
+// boundary: the 20 components of 2^20 states, L = 27, took 62 us, here 40; the 7
+// components in 28, here 21.)
+constexpr int MV_W = 63, MV_THREADS = 256;
+template <typename T>
+constexpr int MV_G = sizeof(T) == 4 ? 128 : 64;
+
+template <typename T>
+PES_DEV void copy_async(T* dst, const T* src)
 {
-    __shared__ T tile[32][33];
-    const int c = blockIdx.z;
-    const int l0 = blockIdx.x * 32, s0 = blockIdx.y * 32;
-    const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-    for (int r = ty; r < 32; r += 8) {
-        if (TO_LANES) {
-            // read: for lane l0 + r, steps s0 + tx (contiguous in the caller layout)
-            const int l = l0 + r, s = s0 + tx;
-            const int64_t k = (int64_t)l * L + s;
-            if (l < NL && s < L && k < N) tile[r][tx] = src[(int64_t)c * N + k];
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(sizeof(T)) : "memory");
+}
+
+template <typename T, bool TO_LANES, bool BLOCKED>
+__global__ void __launch_bounds__(MV_THREADS) lanes_move_kernel(const LaneArrays<T> a, T* lanes, int64_t N, int L,
+                                                                int NL, int nc, int per_block)
+{
+    constexpr int G = MV_G<T>, RS = G + 1;
+    extern __shared__ __align__(16) unsigned char mv_raw[];
+    T* tiles = reinterpret_cast<T*>(mv_raw);
+    const int64_t cs = (int64_t)L * NL;
+    const int l0 = blockIdx.x * G, s0 = blockIdx.y * MV_W;
+    const int w = min(MV_W, L - s0), g = min(G, NL - l0);
+    const int64_t k0 = (int64_t)l0 * L + s0;
+    const int64_t left = N - k0;   // states from k0 on
+    const int t = threadIdx.x;
+    const int c0 = blockIdx.z * per_block, c1 = min(nc, c0 + per_block);
+    // f(word of the tile, place in the caller's array from k0 on)
+    auto caller_side = [&](auto f) {
+        if (w == L) {
+            const int n = (int)min((int64_t)g * w, left);
+            const int dl = MV_THREADS / w, dr = MV_THREADS - dl * w;
+            int l = t / w, r = t - l * w;
+            for (int q = t; q < n; q += MV_THREADS) {
+                f(r * RS + l, (int64_t)q);
+                l += dl;
+                r += dr;
+                if (r >= w) r -= w, ++l;
+            }
         } else {
-            // read: for step s0 + r, lanes l0 + tx (contiguous in the lane layout)
-            const int l = l0 + tx, s = s0 + r;
-            const int64_t k = (int64_t)l * L + s;
-            if (l < NL && s < L && k < N) tile[tx][r] = src[(int64_t)c * cs + (int64_t)s * NL + l];
+            for (int l = t >> 5; l < g; l += MV_THREADS / 32)
+                for (int r = t & 31; r < w; r += 32)
+                    if ((int64_t)l * L + r < left) f(r * RS + l, (int64_t)l * L + r);
+        }
+    };
+    // f(word of the tile, place among the component's lane-major values from (s0, l0) on)
+    auto lane_side = [&](auto f) {
+        const int l = t % G;
+        const int64_t most = left - (int64_t)l * L;   // steps from s0 on that the lane has
+        const int64_t row = BLOCKED ? nc * 32 : NL;
+        const int64_t at = BLOCKED ? (int64_t)(l >> 5) * L * row + (l & 31) : l;
+        if (l < g)
+            for (int r = t / G; r < w && r < most; r += MV_THREADS / G) f(r * RS + l, r * row + at);
+    };
+    auto lane_major = [&](int c) {
+        return lanes + (BLOCKED ? ((int64_t)(l0 >> 5) * L + s0) * (nc * 32) + c * 32 : c * cs + (int64_t)s0 * NL + l0);
+    };
+    auto caller_of = [&](int c) {
+        int arr = 0;
+        while (c >= a.nc[arr]) c -= a.nc[arr++];
+        return a.ptr[arr] + (int64_t)c * N + k0;
+    };
+    for (int c = c0; c < c1; ++c) {
+        T* tile = tiles + (c - c0) * w * RS;
+        if (TO_LANES) {
+            const T* src = caller_of(c);
+            caller_side([&](int i, int64_t k) { copy_async(tile + i, src + k); });
+        } else {
+            const T* src = lane_major(c);
+            lane_side([&](int i, int64_t ix) { copy_async(tile + i, src + ix); });
         }
     }
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
+    for (int c = c0; c < c1; ++c) {
+        const T* tile = tiles + (c - c0) * w * RS;
         if (TO_LANES) {
-            const int l = l0 + tx, s = s0 + r;
-            const int64_t k = (int64_t)l * L + s;
-            if (l < NL && s < L && k < N) dst[(int64_t)c * cs + (int64_t)s * NL + l] = tile[tx][r];
+            T* dst = lane_major(c);
+            lane_side([&](int i, int64_t ix) { dst[ix] = tile[i]; });
         } else {
-            const int l = l0 + r, s = s0 + tx;
-            const int64_t k = (int64_t)l * L + s;
-            if (l < NL && s < L && k < N) dst[(int64_t)c * N + k] = tile[r][tx];
+            T* dst = caller_of(c);
+            caller_side([&](int i, int64_t k) { dst[k] = tile[i]; });
         }
     }
 }
 
 template <typename T>
-cudaError_t launch_lanes_transpose(const T* src, T* dst, int nc, int64_t N, int L, int NL, bool to_lanes,
-                                   cudaStream_t st)
+cudaError_t launch_lanes_move(const LaneArrays<T>& a, T* lanes, int64_t N, int L, int NL, LanesMove how, cudaStream_t st)
 {
-    const dim3 grid((NL + 31) / 32, (L + 31) / 32, nc), block(32, 8);
-    if (to_lanes) lanes_transpose_kernel<T, true><<<grid, block, 0, st>>>(src, dst, N, L, NL, (int64_t)L * NL);
-    else lanes_transpose_kernel<T, false><<<grid, block, 0, st>>>(src, dst, N, L, NL, (int64_t)L * NL);
+    constexpr int G = MV_G<T>;
+    int nc = 0;
+    for (int i = 0; i < a.n; ++i) nc += a.nc[i];
+    // up to about 32 steps of components a block: 16 KB in flight, of which an
+    // SM holds eight; fewer where the grid would not fill the SMs
+    const int w = std::min(L, MV_W);
+    const int64_t pieces = (int64_t)((NL + G - 1) / G) * ((L + MV_W - 1) / MV_W);
+    const int per_block = (int)std::max<int64_t>(1, std::min<int64_t>({nc, 32 / w, nc * pieces / 608}));
+    const size_t smem = sizeof(T) * per_block * w * (G + 1);   // at most 33 KB
+    const dim3 grid((NL + G - 1) / G, (L + MV_W - 1) / MV_W, (nc + per_block - 1) / per_block);
+    auto kern = how == MOVE_OUT  ? lanes_move_kernel<T, false, false>
+                : how == MOVE_IN ? lanes_move_kernel<T, true, false>
+                                 : lanes_move_kernel<T, true, true>;
+    kern<<<grid, MV_THREADS, smem, st>>>(a, lanes, N, L, NL, nc, per_block);
     return cudaGetLastError();
 }
 
-template cudaError_t launch_lanes_transpose<float>(const float*, float*, int, int64_t, int, int, bool, cudaStream_t);
-template cudaError_t launch_lanes_transpose<double>(const double*, double*, int, int64_t, int, int, bool, cudaStream_t);
+template cudaError_t launch_lanes_move<float>(const LaneArrays<float>&, float*, int64_t, int, int, LanesMove, cudaStream_t);
+template cudaError_t launch_lanes_move<double>(const LaneArrays<double>&, double*, int64_t, int, int, LanesMove,
+                                               cudaStream_t);
 
 // Prior nominal in the lane-major layout: state k of trajectory b gets (m0_b, P0_b).
 template <typename T>
@@ -203,7 +274,7 @@ __global__ void linearize_kernel(const KParams<T> p, T* F, T* c, T* Qp, T* H, T*
         const bool has_obs = k > __ldg(p.offsets + b);
         if (has_next) {
             Trans<T> tr;
-            ok &= get_trans<T, LIN>(p, k, k, tr);
+            ok &= get_trans<T, LIN>(p, k, tr);
             T Fx[5];
             mv(tr.F, tr.xn, Fx);
 #pragma unroll
@@ -222,7 +293,7 @@ __global__ void linearize_kernel(const KParams<T> p, T* F, T* c, T* Qp, T* H, T*
         }
         if (has_obs) {
             Obs<T> ob;
-            ok &= get_obs<T, LIN>(p, k, k, b, ob);
+            ok &= get_obs<T, LIN>(p, k, b, ob);
             T y[2];
             load_y(p, k, y);
             // h(xn), the measurement y_used and d = zbar - H xn with zbar = y_used - r_offset

@@ -7,19 +7,22 @@ namespace pes {
 template <typename T, int NT>
 static cudaError_t launch_nt(const KParams<T>& p, int lin, int nb, cudaStream_t st)
 {
-    if (lin == LIN_ARRAYS) return launch_cfg<T, LIN_ARRAYS, NT>(p, nb, st);
-    if (lin == LIN_IEKS) return launch_cfg<T, LIN_IEKS, NT>(p, nb, st);
-    if (lin == LIN_GH) return launch_cfg<T, LIN_GH, NT>(p, nb, st);
-    return launch_cfg<T, LIN_CUBATURE, NT>(p, nb, st);
+    const bool ct = p.model.kind == MODEL_CT_BEARINGS;
+    if (lin == LIN_ARRAYS) return launch_cfg<T, KK_ARRAYS, NT>(p, nb, st);
+    if (lin == LIN_IEKS) return ct ? launch_cfg<T, KK_IEKS, NT>(p, nb, st) : launch_cfg<T, KK_IEKS_ANY, NT>(p, nb, st);
+    if (lin == LIN_GH) return launch_cfg<T, KK_GH, NT>(p, nb, st);
+    return ct ? launch_cfg<T, KK_CUBATURE, NT>(p, nb, st) : launch_cfg<T, KK_CUBATURE_ANY, NT>(p, nb, st);
 }
 
+// The model is not known here: the smaller capacity of the two forms.
 template <typename T, int NT>
 static int capacity_nt(int lin, int device)
 {
-    if (lin == LIN_ARRAYS) return capacity_cfg<T, LIN_ARRAYS, NT>(device);
-    if (lin == LIN_IEKS) return capacity_cfg<T, LIN_IEKS, NT>(device);
-    if (lin == LIN_GH) return capacity_cfg<T, LIN_GH, NT>(device);
-    return capacity_cfg<T, LIN_CUBATURE, NT>(device);
+    if (lin == LIN_ARRAYS) return capacity_cfg<T, KK_ARRAYS, NT>(device);
+    if (lin == LIN_GH) return capacity_cfg<T, KK_GH, NT>(device);
+    const int a = lin == LIN_IEKS ? capacity_cfg<T, KK_IEKS, NT>(device) : capacity_cfg<T, KK_CUBATURE, NT>(device);
+    const int b = lin == LIN_IEKS ? capacity_cfg<T, KK_IEKS_ANY, NT>(device) : capacity_cfg<T, KK_CUBATURE_ANY, NT>(device);
+    return a < b ? a : b;
 }
 
 cudaError_t launch_persistent(const KParams<float>& p, int lin, int nt, int nb, cudaStream_t st)

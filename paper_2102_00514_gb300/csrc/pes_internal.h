@@ -9,9 +9,9 @@ namespace pes {
 
 // One configuration of the persistent kernel (defined in pes_launch_impl.cuh,
 // instantiated by the pes_k_*.cu translation units).
-template <typename T, int LIN, int NT>
+template <typename T, int K, int NT>
 cudaError_t launch_cfg(const KParams<T>& p, int nb, cudaStream_t st);
-template <typename T, int LIN, int NT>
+template <typename T, int K, int NT>
 int capacity_cfg(int device);
 
 // Dispatch over the compiled configurations (pes_dispatch.cu). `lin` is one of
@@ -38,10 +38,26 @@ cudaError_t launch_convert_ff(const Ti* in, To* out, int64_t n, cudaStream_t st)
 // Element-wise double -> T copy (model sensors into the kernel precision).
 template <typename T>
 cudaError_t launch_convert(const double* in, T* out, int n, cudaStream_t st);
-// Caller layout [nc][N] <-> lane-major [nc][L][NL] (state k = lane * L + s).
+// Arrays of the caller, nc[i] components of N values each.
 template <typename T>
-cudaError_t launch_lanes_transpose(const T* src, T* dst, int nc, int64_t N, int L, int NL, bool to_lanes,
-                                   cudaStream_t st);
+struct LaneArrays {
+    static constexpr int kMax = 8;
+    T* ptr[kMax];
+    int nc[kMax];
+    int n = 0;
+    LaneArrays& add(const void* p, int components)
+    {
+        ptr[n] = static_cast<T*>(const_cast<void*>(p));
+        nc[n++] = components;
+        return *this;
+    }
+};
+// Caller layout [nc][N] <-> lane-major [nc][L][NL] (state k = lane * L + s), the
+// arrays' components one after another on the lane-major side; MOVE_IN_BLOCKED:
+// to [warp][L][nc][32 lanes], a step's values of a warp in one run.
+enum LanesMove { MOVE_IN, MOVE_IN_BLOCKED, MOVE_OUT };
+template <typename T>
+cudaError_t launch_lanes_move(const LaneArrays<T>& a, T* lanes, int64_t N, int L, int NL, LanesMove how, cudaStream_t st);
 template <typename T>
 cudaError_t launch_init_nominal_lanes(const int64_t* offsets, int B, int64_t N, int L, int NL, const T* m0,
                                       const T* P0, T* x, T* P, cudaStream_t st);

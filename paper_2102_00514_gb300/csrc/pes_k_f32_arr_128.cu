@@ -1,3 +1,3 @@
-// Persistent smoother kernel: float, LIN_ARRAYS, 128 threads per block.
+// Persistent smoother kernel: float, the given arrays, 128 threads per block.
 #include "pes_launch_impl.cuh"
-PES_INSTANTIATE(float, pes::LIN_ARRAYS, 128)
+PES_INSTANTIATE(float, pes::KK_ARRAYS, 128)

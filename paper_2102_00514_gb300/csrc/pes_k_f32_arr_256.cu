@@ -1,3 +1,3 @@
-// Persistent smoother kernel: float, LIN_ARRAYS, 256 threads per block.
+// Persistent smoother kernel: float, the given arrays, 256 threads per block.
 #include "pes_launch_impl.cuh"
-PES_INSTANTIATE(float, pes::LIN_ARRAYS, 256)
+PES_INSTANTIATE(float, pes::KK_ARRAYS, 256)

@@ -1,3 +1,3 @@
-// Persistent smoother kernel: float, LIN_CUBATURE, 128 threads per block.
+// Persistent smoother kernel: float, cubature / unscented, coordinated turn, 128 threads per block.
 #include "pes_launch_impl.cuh"
-PES_INSTANTIATE(float, pes::LIN_CUBATURE, 128)
+PES_INSTANTIATE(float, pes::KK_CUBATURE, 128)

@@ -1,3 +1,3 @@
-// Persistent smoother kernel: float, LIN_CUBATURE, 256 threads per block.
+// Persistent smoother kernel: float, cubature / unscented, coordinated turn, 256 threads per block.
 #include "pes_launch_impl.cuh"
-PES_INSTANTIATE(float, pes::LIN_CUBATURE, 256)
+PES_INSTANTIATE(float, pes::KK_CUBATURE, 256)

@@ -1,0 +1,3 @@
+// Persistent smoother kernel: float, cubature / unscented, any model, 256 threads per block.
+#include "pes_launch_impl.cuh"
+PES_INSTANTIATE(float, pes::KK_CUBATURE_ANY, 256)

@@ -1,3 +1,3 @@
-// Persistent smoother kernel: float, LIN_GH (Gauss-Hermite product rule), 256 threads per block.
+// Persistent smoother kernel: float, Gauss-Hermite, 256 threads per block.
 #include "pes_launch_impl.cuh"
-PES_INSTANTIATE(float, pes::LIN_GH, 256)
+PES_INSTANTIATE(float, pes::KK_GH, 256)

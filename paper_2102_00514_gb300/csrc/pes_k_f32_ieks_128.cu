@@ -1,3 +1,3 @@
-// Persistent smoother kernel: float, LIN_IEKS, 128 threads per block.
+// Persistent smoother kernel: float, Taylor, coordinated turn, 128 threads per block.
 #include "pes_launch_impl.cuh"
-PES_INSTANTIATE(float, pes::LIN_IEKS, 128)
+PES_INSTANTIATE(float, pes::KK_IEKS, 128)

@@ -1,3 +1,3 @@
-// Persistent smoother kernel: float, LIN_IEKS, 256 threads per block.
+// Persistent smoother kernel: float, Taylor, coordinated turn, 256 threads per block.
 #include "pes_launch_impl.cuh"
-PES_INSTANTIATE(float, pes::LIN_IEKS, 256)
+PES_INSTANTIATE(float, pes::KK_IEKS, 256)

@@ -1,3 +1,3 @@
-// Persistent smoother kernel: double, LIN_ARRAYS, 128 threads per block.
+// Persistent smoother kernel: double, the given arrays, 128 threads per block.
 #include "pes_launch_impl.cuh"
-PES_INSTANTIATE(double, pes::LIN_ARRAYS, 128)
+PES_INSTANTIATE(double, pes::KK_ARRAYS, 128)

@@ -1,3 +1,3 @@
-// Persistent smoother kernel: double, LIN_CUBATURE, 128 threads per block.
+// Persistent smoother kernel: double, cubature / unscented, coordinated turn, 128 threads per block.
 #include "pes_launch_impl.cuh"
-PES_INSTANTIATE(double, pes::LIN_CUBATURE, 128)
+PES_INSTANTIATE(double, pes::KK_CUBATURE, 128)

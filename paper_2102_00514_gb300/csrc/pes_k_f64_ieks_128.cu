@@ -1,3 +1,3 @@
-// Persistent smoother kernel: double, LIN_IEKS, 128 threads per block.
+// Persistent smoother kernel: double, Taylor, coordinated turn, 128 threads per block.
 #include "pes_launch_impl.cuh"
-PES_INSTANTIATE(double, pes::LIN_IEKS, 128)
+PES_INSTANTIATE(double, pes::KK_IEKS, 128)

@@ -5,38 +5,84 @@
 // and re-linearises about the smoothed means between iterations (Sec. 3).
 //
 // Scan layout. The N states are split into NB x NT contiguous chunks of L
-// steps, one per thread ("lane"). Each scan is a three-level reduce-then-scan:
-//   1. every lane folds its chunk into one element (sequentially, exact);
-//   2. a Blelloch up-sweep over the NT lane elements of a block in shared
-//      memory gives the block's element, published to global memory;
+// steps, one per thread ("lane"). A lane's filtering element maps the predicted
+// state at its chunk's start to the predicted state at the next chunk's start:
+// update and predict, step by step. Both scans are three-level
+// reduce-then-scans over the lanes:
+//   1. every lane folds its chunk into one filtering element;
+//   2. a tree over the NT lane elements of a block in shared memory gives the
+//      block's element, published to global memory (pes_tree.cuh);
 //   3. after a grid barrier every block reduces the elements of the blocks
-//      before it (filtering) or after it (smoothing) with a tree in shared
-//      memory; since the sequence starts with a prior element and ends with
-//      a last-state element, that reduction is a Gaussian;
-//   4. a Blelloch down-sweep pushes that Gaussian through the lane tree, so
-//      every lane gets the Gaussian of the state just before (filtering) or
-//      after (smoothing) its chunk, and
-//   5. each lane re-runs its chunk sequentially from it, which yields the
-//      filtered (smoothed) moments of every state in the chunk.
-// The filtering re-run also builds the smoothing elements of its chunk and
-// folds them, so the smoothing pass starts at level 2.
+//      before it; since the sequence starts with a prior, that is a Gaussian;
+//   4. the tree pushes that Gaussian down, so that every lane gets the
+//      predicted Gaussian at its chunk's start;
+//   5. each lane re-runs its chunk as a Kalman filter from it and keeps the
+//      filtered moments.
+// The smoothing element of a whole chunk (from the state after it to its first
+// state) follows from that Gaussian and the lane's filtering element: the chunk
+// is one step of Eq. 17 with the transition (A, b, C) from the state
+// conditioned on the chunk's measurements, D = (P^{-1} + J)^{-1}. So the
+// smoothing scan needs no fold of per-step elements (350 multiply-adds per
+// state), and its levels 2 and 3 do not depend on the filtering re-run: its
+// block elements are published before the re-run, which hides the wait for the
+// other blocks' (measured at T = 2^20, FP32: see pes_persistent_kernel). The RTS
+// pass then builds each step's element from the kept filtered moments.
+//
+// A chunk's passes read only its own states' nominal, so no barrier separates
+// iterations: the block aggregates are double-buffered, and a block can reach
+// the aggregates of iteration i + 2 only after every block has passed the first
+// barrier of iteration i + 1, that is, has read those of iteration i. Only the
+// tolerance mode waits for all blocks at an iteration's end.
 //
 // Grid barriers spin on a global counter with a wall-clock limit; on timeout
 // they set ST_TIMEOUT and return, so the kernel always terminates.
 #pragma once
 
 #include "pes_async.cuh"
-#include "pes_ops.cuh"
+#include "pes_tree.cuh"
 
 namespace pes {
 
 enum { MODE_FILTER = 0, MODE_SMOOTH = 1, MODE_RUN = 2 };
 
-constexpr int FE = sizeof(FElem<double>) / sizeof(double);   // 70
-constexpr int SE = sizeof(SElem<double>) / sizeof(double);   // 50
-constexpr int GE = sizeof(Gauss<double>) / sizeof(double);   // 20
-constexpr int HAND = 50;                                      // handoff scalars per state: one SElem
-constexpr int LINS = 65;                                      // stored linearisation scalars per state
+constexpr int HAND = 20;          // filtered moments kept per state
+constexpr int LINS = 65;          // stored linearisation scalars per state, at most
+
+// The compiled forms of the smoother: the linearisation, and whether the model
+// is known to be the coordinated turn (the structure of its slopes, and no code
+// for the linear model in the loops) or is looked up (_ANY).
+enum { KK_ARRAYS = 0, KK_IEKS = 1, KK_CUBATURE = 2, KK_GH = 3, KK_IEKS_ANY = 4, KK_CUBATURE_ANY = 5 };
+template <int K>
+constexpr int kLinOf = K == KK_IEKS_ANY ? LIN_IEKS : (K == KK_CUBATURE_ANY ? LIN_CUBATURE : K);
+template <int K>
+constexpr int kFS = K == KK_IEKS ? FS_CT : (K == KK_CUBATURE ? FS_SLR : FS_DENSE);
+
+// Whether the fold hands its linearisation of every state to the later passes
+// instead of their linearising again. The sigma-point linearisations cost far
+// more than the traffic; the Taylor one does not.
+template <int K>
+constexpr bool kStoreLin = kSigma<kLinOf<K>>;
+// Scalars stored per state; the transition's are kLinTrans of them, from
+// kLinTransAt. Compact form (the coordinated turn's cubature regression): F rows
+// 0-3 (20), fx (4), Q' (10), H (4), r (2), R' (3); the nominal is read from the
+// trajectory, the rest is constant. Dense form: H (10), r (2), R' (3), xn (5),
+// F (25), fx (5), Q' (15).
+template <int K>
+constexpr int kLinScalars = K == KK_CUBATURE ? 43 : LINS;
+template <int K>
+constexpr int kLinTransAt = K == KK_CUBATURE ? 0 : 15;
+template <int K>
+constexpr int kLinTrans = K == KK_CUBATURE ? 34 : 50;
+// Stream stages: of the re-run (beside the smoother's tree, which is live), and
+// of the RTS pass.
+template <int K>
+constexpr int kLinStages = K == KK_CUBATURE ? 2 : 1;
+template <int K>
+constexpr int kRtsStages = (kStoreLin<K> && K != KK_CUBATURE) ? 3 : 4;
+constexpr int kMaxStages = 4;
+// Whether the trees keep combine_filter's rounding (fold_filter_arrays).
+template <int K, typename T>
+constexpr bool kKeepRounding = K == KK_ARRAYS && sizeof(T) == 4;
 
 template <typename T>
 struct KParams {
@@ -48,30 +94,26 @@ struct KParams {
     double tol;               // RUN: relative update-norm tolerance (<= 0: fixed iterations)
     int write_P_every_iter;   // RUN: write smoothed covariances in every iteration
     DevModel<T> model;
-    const T* y;               // [2][N] (slot of each x_0 ignored)
+    // per-state arrays, component-major with stride cs. In the scans they are in
+    // the kernel's lane-major layout; the element-wise kernels and the sequential
+    // smoother use the caller's (cs = N).
+    const T* y;               // [2] (slot of each x_0 ignored)
     const T* m0;              // [B][5]
     const T* P0;              // [B][15]
-    // linearisation arrays (MODE_FILTER / MODE_SMOOTH), SoA [ncomp][N]
-    const T* F;
-    const T* c;
-    const T* Qp;
-    const T* H;
-    const T* d;
-    const T* Rp;
-    // filtered moments (MODE_FILTER output, MODE_SMOOTH input), SoA
+    // filtered moments (MODE_FILTER output)
     T* xf;
     T* Pf;
     // smoothed moments: MODE_SMOOTH output; MODE_RUN nominal (in place) and output
     T* x;
     T* P;
-    // MODE_RUN: the filtered moments of every state, [20][cs] in the layout of
-    // x and P (means then packed covariances), or NULL (not stored)
-    T* fstore;
     // workspace
-    T* hand;           // MODE_RUN handoff of smoothing elements: [warp][s][c][32 lanes]
-    T* lin;            // MODE_RUN cubature linearisation handed from the fold to the re-run: [warp][s][LINS][32]
-    T* aggF;           // [NB][FE]
-    T* aggS;           // [NB][SE]
+    T* hand;           // MODE_RUN: filtered moments, kept for the RTS pass: [warp][s][HAND][32 lanes]
+    // MODE_RUN: the sigma-point linearisation, handed from the fold to the later
+    // passes; MODE_FILTER / MODE_SMOOTH: the given arrays: [warp][s][component][32]
+    T* lin;
+    T* aggF;           // [2][agg_blocks][FE]: the blocks' filtering elements, by iteration parity
+    T* aggS;           // [2][agg_blocks][SE]: their smoothing elements
+    int agg_blocks;    // blocks the aggregates have room for
     unsigned* bar;     // grid barrier counter, zero at launch
     int* status;       // ST_* bits
     double* conv;      // [2][B][2] update-norm accumulators, zero at launch
@@ -80,8 +122,7 @@ struct KParams {
     double* loglik;    // FILTER: [B] log p(y_{1:T_b}) accumulated (zero at launch), or NULL
     int L;             // steps per lane
     int NL;            // lanes = NB * NT
-    int lanes_layout;  // x, P, y use the kernel's lane-major layout (MODE_RUN)
-    int64_t cs;        // component stride of x, P, y
+    int64_t cs;        // component stride of the per-state arrays
     long long timeout_ns;
     long long* ptime;  // optional per-block phase timestamps of the first iteration (NULL: off)
 };
@@ -111,16 +152,25 @@ PES_DEV unsigned ld_acquire(const unsigned* p)
     return v;
 }
 
-// Grid-wide barrier for a cooperative launch (all blocks co-resident).
+// Grid-wide barrier for a cooperative launch (all blocks co-resident), in two
+// halves: arrive publishes the block's earlier writes, wait returns once every
+// block has arrived.
 template <typename T>
-PES_DEV void grid_barrier(const KParams<T>& p, unsigned& gen)
+PES_DEV void grid_arrive(const KParams<T>& p, unsigned& gen)
 {
     __syncthreads();
+    ++gen;
     if (threadIdx.x == 0) {
-        ++gen;
-        const unsigned target = gen * gridDim.x;
         __threadfence();
         atomicAdd(p.bar, 1u);
+    }
+}
+
+template <typename T>
+PES_DEV void grid_wait(const KParams<T>& p, unsigned gen)
+{
+    if (threadIdx.x == 0) {
+        const unsigned target = gen * gridDim.x;
         const long long t0 = globaltimer_ns();
         unsigned polls = 0;
         while (ld_acquire(p.bar) < target) {
@@ -129,7 +179,7 @@ PES_DEV void grid_barrier(const KParams<T>& p, unsigned& gen)
                 atomicOr(p.status, ST_TIMEOUT);
                 break;
             }
-            __nanosleep(128);
+            __nanosleep(32);
         }
         __threadfence();
     }
@@ -209,22 +259,12 @@ PES_DEV void load_y(const KParams<T>& p, int64_t ix, T* y)
     y[1] = __ldg(p.y + p.cs + ix);
 }
 
-// Index of state k of the chunk [a, e) of `lane` in the per-state arrays the
-// kernel reads and writes (x, P, y): in MODE_RUN the kernel's lane-major
-// layout [component][step][lane], in which a warp's accesses at one step are
-// contiguous; otherwise the caller's [component][N] layout.
+// Place of step s of a lane in the per-state arrays: [component][step][lane], in
+// which a warp's accesses at one step are contiguous.
 template <typename T>
-PES_DEV int64_t state_ix(const KParams<T>& p, int64_t k, int64_t a, int lane)
+PES_DEV int64_t lane_ix(const KParams<T>& p, int64_t s, int lane)
 {
-    return p.lanes_layout ? (k - a) * p.NL + lane : k;
-}
-
-// Index of the state just before the chunk (k = a - 1): the last state of the
-// previous lane's chunk, which is full.
-template <typename T>
-PES_DEV int64_t prev_ix(const KParams<T>& p, int64_t a, int lane)
-{
-    return p.lanes_layout ? (int64_t)(p.L - 1) * p.NL + (lane - 1) : a - 1;
+    return s * p.NL + lane;
 }
 
 // ---- linearisation of one step ------------------------------------------------
@@ -241,7 +281,7 @@ struct StateIn {
 template <typename T, int LIN>
 PES_DEV void load_state(const KParams<T>& p, int64_t ix, StateIn<T, LIN>& s)
 {
-    if (LIN != LIN_ARRAYS) load_nominal(p, ix, s.x);
+    load_nominal(p, ix, s.x);
     if (kSigma<LIN>) load_nominal_cov(p, ix, s.P);
     load_y(p, ix, s.y);
 }
@@ -262,235 +302,271 @@ PES_DEV bool factor_state(const StateIn<T, LIN>& s, Factor<T, LIN>& f)
 
 // Transition k -> k+1 (Eq. 10 or Eq. 7).
 template <typename T, int LIN>
-PES_DEV void lin_trans(const KParams<T>& p, int64_t k, const StateIn<T, LIN>& s, const Factor<T, LIN>& f,
-                       Trans<T>& tr)
+PES_DEV void lin_trans(const KParams<T>& p, const StateIn<T, LIN>& s, const Factor<T, LIN>& f, Trans<T>& tr)
 {
-    if (LIN == LIN_ARRAYS) {
-#pragma unroll
-        for (int i = 0; i < 25; ++i) tr.F[i] = __ldg(p.F + i * p.N + k);
-#pragma unroll
-        for (int i = 0; i < 5; ++i) {
-            tr.fx[i] = __ldg(p.c + i * p.N + k);
-            tr.xn[i] = T(0);
-        }
-#pragma unroll
-        for (int i = 0; i < 15; ++i) tr.Q[i] = __ldg(p.Qp + i * p.N + k);
-    } else if (LIN == LIN_IEKS) {
-        lin_trans_taylor(p.model, s.x, tr);
-    } else if (LIN == LIN_GH) {
-        lin_trans_gh(p.model, s.x, f.L, f.rd, tr);
-    } else {
-        lin_trans_cubature(p.model, s.x, f.L, f.rd, tr);
-    }
+    if (LIN == LIN_IEKS) lin_trans_taylor(p.model, s.x, tr);
+    else if (LIN == LIN_GH) lin_trans_gh(p.model, s.x, f.L, f.rd, tr);
+    else lin_trans_cubature(p.model, s.x, f.L, f.rd, tr);
 }
 
 // Observation at k (Eq. 10 or Eq. 9).
 template <typename T, int LIN>
-PES_DEV void lin_obs(const KParams<T>& p, int64_t k, int b, const StateIn<T, LIN>& s, const Factor<T, LIN>& f,
-                     Obs<T>& ob)
+PES_DEV void lin_obs(const KParams<T>& p, int b, const StateIn<T, LIN>& s, const Factor<T, LIN>& f, Obs<T>& ob)
 {
-    if (LIN == LIN_ARRAYS) {
-#pragma unroll
-        for (int i = 0; i < 10; ++i) ob.H[i] = __ldg(p.H + i * p.N + k);
-        ob.r[0] = s.y[0] - __ldg(p.d + k);
-        ob.r[1] = s.y[1] - __ldg(p.d + p.N + k);
-#pragma unroll
-        for (int i = 0; i < 5; ++i) ob.xn[i] = T(0);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) ob.R[i] = __ldg(p.Rp + i * p.N + k);
-    } else if (LIN == LIN_IEKS) {
-        lin_obs_taylor(p.model, b, s.x, s.y, ob);
-    } else if (LIN == LIN_GH) {
-        lin_obs_gh(p.model, b, s.x, f.L, f.rd, s.y, ob);
-    } else {
-        lin_obs_cubature(p.model, b, s.x, f.L, f.rd, s.y, ob);
-    }
+    if (LIN == LIN_IEKS) lin_obs_taylor(p.model, b, s.x, s.y, ob);
+    else if (LIN == LIN_GH) lin_obs_gh(p.model, b, s.x, f.L, f.rd, s.y, ob);
+    else lin_obs_cubature(p.model, b, s.x, f.L, f.rd, s.y, ob);
 }
 
 // One-shot forms used by the stand-alone linearisation kernel.
 template <typename T, int LIN>
-PES_DEV bool get_trans(const KParams<T>& p, int64_t k, int64_t ix, Trans<T>& tr)
+PES_DEV bool get_trans(const KParams<T>& p, int64_t ix, Trans<T>& tr)
 {
     StateIn<T, LIN> s;
     load_state(p, ix, s);
     Factor<T, LIN> f;
     const bool ok = factor_state(s, f);
-    lin_trans(p, k, s, f, tr);
+    lin_trans(p, s, f, tr);
     return ok;
 }
 
 template <typename T, int LIN>
-PES_DEV bool get_obs(const KParams<T>& p, int64_t k, int64_t ix, int b, Obs<T>& ob)
+PES_DEV bool get_obs(const KParams<T>& p, int64_t ix, int b, Obs<T>& ob)
 {
     StateIn<T, LIN> s;
     load_state(p, ix, s);
     Factor<T, LIN> f;
     const bool ok = factor_state(s, f);
-    lin_obs(p, k, b, s, f, ob);
+    lin_obs(p, b, s, f, ob);
     return ok;
+}
+
+// The linearisation of a compiled form of the smoother.
+template <int K, typename T>
+PES_DEV void form_trans(const KParams<T>& p, const StateIn<T, kLinOf<K>>& s, const Factor<T, kLinOf<K>>& f,
+                        Trans<T>& tr)
+{
+    if constexpr (K == KK_IEKS) ct_trans_taylor(p.model, s.x, tr);
+    else if constexpr (K == KK_CUBATURE) ct_trans_cubature(p.model, s.x, f.L, f.rd, tr);
+    else lin_trans<T, kLinOf<K>>(p, s, f, tr);
+}
+
+template <int K, typename T>
+PES_DEV void form_obs(const KParams<T>& p, int b, const StateIn<T, kLinOf<K>>& s,
+                      const Factor<T, kLinOf<K>>& f, Obs<T>& ob)
+{
+    if constexpr (K == KK_IEKS) ct_obs_taylor(p.model, b, s.x, s.y, ob);
+    else if constexpr (K == KK_CUBATURE) ct_obs_cubature(p.model, b, s.x, f.L, f.rd, s.y, ob);
+    else lin_obs<T, kLinOf<K>>(p, b, s, f, ob);
 }
 
 // ---- lane-level passes -------------------------------------------------------------
 
-// Whether the fold hands its linearisation of every state to the filtering
-// re-run (65 scalars per state) instead of the re-run linearising again. The
-// cubature linearisation (2 n_x sigma points through f and h) costs far more
-// than the traffic; the Taylor one does not.
-template <int LIN>
-constexpr bool kStoreLin = kSigma<LIN>;
-
-// Layout [warp][s][LINS][32 lanes]; per state: H (10), r (2), R' (3), xn (5),
-// F (25), fx (5), Q' (15).
-template <typename T>
+// Stored linearisation, [warp][s][kLinScalars][32 lanes].
+template <int K, typename T>
 PES_DEV T* lin_slot(const KParams<T>& p, int s, int lane)
 {
-    return p.lin + ((size_t)(lane >> 5) * p.L + s) * (LINS * 32) + (lane & 31);
+    return p.lin + ((size_t)(lane >> 5) * p.L + s) * (kLinScalars<K> * 32) + (lane & 31);
 }
 
-template <typename T>
+template <int K, typename T>
 PES_DEV void store_lin_obs(const KParams<T>& p, int s, int lane, const Obs<T>& ob)
 {
-    T* h = lin_slot(p, s, lane);
+    T* h = lin_slot<K>(p, s, lane);
+    if constexpr (K == KK_CUBATURE) {
 #pragma unroll
-    for (int i = 0; i < 5; ++i) h[(15 + i) * 32] = ob.xn[i];
+        for (int r = 0; r < 2; ++r) {
+            h[(34 + 2 * r) * 32] = ob.H[r * 5];
+            h[(35 + 2 * r) * 32] = ob.H[r * 5 + 1];
+            h[(38 + r) * 32] = ob.r[r];
+        }
 #pragma unroll
-    for (int i = 0; i < 10; ++i) h[i * 32] = ob.H[i];
-    h[10 * 32] = ob.r[0];
-    h[11 * 32] = ob.r[1];
+        for (int i = 0; i < 3; ++i) h[(40 + i) * 32] = ob.R[i];
+    } else {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) h[(12 + i) * 32] = ob.R[i];
+        for (int i = 0; i < 5; ++i) h[(15 + i) * 32] = ob.xn[i];
+#pragma unroll
+        for (int i = 0; i < 10; ++i) h[i * 32] = ob.H[i];
+        h[10 * 32] = ob.r[0];
+        h[11 * 32] = ob.r[1];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) h[(12 + i) * 32] = ob.R[i];
+    }
 }
 
-template <typename T>
+// packed index of entry q of the leading 4x4 block of a symmetric 5x5 matrix
+__host__ __device__ constexpr int si4(int q) { return q < 4 ? q : (q < 7 ? q + 1 : (q < 9 ? q + 2 : q + 3)); }
+
+template <int K, typename T>
 PES_DEV void store_lin_trans(const KParams<T>& p, int s, int lane, const Trans<T>& tr)
 {
-    T* h = lin_slot(p, s, lane);
+    T* h = lin_slot<K>(p, s, lane);
+    if constexpr (K == KK_CUBATURE) {
 #pragma unroll
-    for (int i = 0; i < 5; ++i) h[(15 + i) * 32] = tr.xn[i];
+        for (int i = 0; i < 20; ++i) h[i * 32] = tr.F[i];
 #pragma unroll
-    for (int i = 0; i < 25; ++i) h[(20 + i) * 32] = tr.F[i];
+        for (int i = 0; i < 4; ++i) h[(20 + i) * 32] = tr.fx[i];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) h[(45 + i) * 32] = tr.fx[i];
+        for (int i = 0; i < 10; ++i) h[(24 + i) * 32] = tr.Q[si4(i)];
+    } else {
 #pragma unroll
-    for (int i = 0; i < 15; ++i) h[(50 + i) * 32] = tr.Q[i];
+        for (int i = 0; i < 5; ++i) h[(15 + i) * 32] = tr.xn[i];
+#pragma unroll
+        for (int i = 0; i < 25; ++i) h[(20 + i) * 32] = tr.F[i];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) h[(45 + i) * 32] = tr.fx[i];
+#pragma unroll
+        for (int i = 0; i < 15; ++i) h[(50 + i) * 32] = tr.Q[i];
+    }
 }
 
-template <typename T>
-PES_DEV void load_lin_obs(const KParams<T>& p, int s, int lane, Obs<T>& ob)
+// The slot range of a lane's warp at step s.
+template <int K, typename T>
+PES_DEV const T* lin_warp(const KParams<T>& p, int s, int lane)
 {
-    const T* h = lin_slot(p, s, lane);
-#pragma unroll
-    for (int i = 0; i < 10; ++i) ob.H[i] = h[i * 32];
-    ob.r[0] = h[10 * 32];
-    ob.r[1] = h[11 * 32];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) ob.R[i] = h[(12 + i) * 32];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) ob.xn[i] = h[(15 + i) * 32];
+    return p.lin + ((size_t)(lane >> 5) * p.L + s) * (kLinScalars<K> * 32);
 }
 
-template <typename T>
-PES_DEV void load_lin_trans(const KParams<T>& p, int s, int lane, Trans<T>& tr)
-{
-    const T* h = lin_slot(p, s, lane);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) tr.xn[i] = h[(15 + i) * 32];
-#pragma unroll
-    for (int i = 0; i < 25; ++i) tr.F[i] = h[(20 + i) * 32];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) tr.fx[i] = h[(45 + i) * 32];
-#pragma unroll
-    for (int i = 0; i < 15; ++i) tr.Q[i] = h[(50 + i) * 32];
-}
-
-// Per-thread asynchronous prefetch of the next state's inputs (nominal mean
-// and covariance, measurement: 22 scalars) into shared memory, for the
-// sigma-point folds, whose register pressure rules out a register prefetch.
-// Each thread copies its own scalars with cp.async (L1-allocating, like the
-// plain loads it replaces; every read of the nominal follows a grid barrier's
-// acquire) into one of two stages and reads only its own stage back after
-// cp.async.wait_group, so no block synchronisation is involved. Element c of
-// stage s sits at base[(s * NS + c) * stride] (thread-contiguous columns).
-template <typename T>
-struct StatePrefetch {
-    static constexpr int NS = 22;
+// Per-thread asynchronous prefetch of the next states' inputs into shared
+// memory: NS components of a state, consecutive rows of the per-state arrays from
+// `src` on. For the sigma-point folds, whose register pressure rules out a
+// register prefetch (nominal mean and covariance, measurement). Each thread
+// copies its own scalars with cp.async and reads only its own stages back, so no block synchronisation is involved. Element c of
+// stage i sits at base[(i * NS + c) * stride] (thread-contiguous columns).
+template <typename T, int NS>
+struct Prefetch {
     T* base;
     int stride;
-    PES_DEV void copy(T* dst, const T* src) const
+    const T* src;
+    int64_t cs;
+    PES_DEV void issue(int64_t ix, int i) const
     {
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(sizeof(T))
-                     : "memory");
-    }
-    PES_DEV void issue(const KParams<T>& p, int64_t ix, int s) const
-    {
-        T* d = base + (size_t)s * NS * stride;
+        T* d = base + (size_t)i * NS * stride;
+        const T* q = src + ix;
 #pragma unroll
-        for (int i = 0; i < 5; ++i) copy(d + i * stride, p.x + i * p.cs + ix);
-#pragma unroll
-        for (int i = 0; i < 15; ++i) copy(d + (5 + i) * stride, p.P + i * p.cs + ix);
-        copy(d + 20 * stride, p.y + ix);
-        copy(d + 21 * stride, p.y + p.cs + ix);
+        for (int c = 0; c < NS; ++c)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(d + c * stride)), "l"(q + c * cs),
+                         "n"(sizeof(T))
+                         : "memory");
     }
     PES_DEV static void commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
     // all but the most recent group complete
     PES_DEV static void wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-    template <int LIN>
-    PES_DEV void take(int s, StateIn<T, LIN>& st) const
-    {
-        const T* d = base + (size_t)s * NS * stride;
-#pragma unroll
-        for (int i = 0; i < 5; ++i) st.x[i] = d[i * stride];
-#pragma unroll
-        for (int i = 0; i < 15; ++i) st.P[i] = d[(5 + i) * stride];
-        st.y[0] = d[20 * stride];
-        st.y[1] = d[21 * stride];
-    }
+    PES_DEV static void wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+    PES_DEV T get(int i, int c) const { return base[((size_t)i * NS + c) * stride]; }
 };
-
-// Filtering, level 1: fold the lane's chunk [a, e) into one element. Step k
-// folds the update with its own observation and then the prediction through
-// its outgoing transition (k -> k+1), both linearised about the nominal of k,
-// so the state's sigma-point factor serves both and no earlier state's inputs
-// stay live. The transition into the chunk's first state is linearised once
-// before the loop; the outgoing transition of the chunk's last state is
-// linearised only to be stored for the re-run (the next lane folds it itself).
-// With a stored linearisation (MODE_RUN, cubature) both are kept for the
-// re-run, the transition at the slot of its source state.
-template <typename T, int LIN>
-PES_DEV bool fold_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, FElem<T>& acc,
-                               const StatePrefetch<T>* pf = nullptr)
+constexpr int kStateIn = 22;    // a run's inputs: x, P, y
+// The scans over given arrays stream a state's components: the filter's F, c, Q',
+// H, d, R', y (three stages in the re-run, where a step needs the one before it
+// too), the smoother's F, c, Q' and filtered mean and covariance.
+constexpr int kFilterIn = 62, kSmoothIn = 65;
+template <typename T>
+using FoldStream = WarpStream<T, kFilterIn, 2>;
+template <typename T>
+using FilterStream = WarpStream<T, kFilterIn, 3>;
+template <typename T>
+using SmoothStream = WarpStream<T, kSmoothIn, 2>;
+// The slot range of a lane's warp at step s, [warp][s][NC][32 lanes].
+template <int NC, typename T>
+PES_DEV const T* array_warp(const KParams<T>& p, int s, int lane)
 {
+    return p.lin + ((size_t)(lane >> 5) * p.L + s) * (NC * 32);
+}
+
+template <typename T, class S>
+PES_DEV void array_trans(const S& q, int i, Trans<T>& tr)
+{
+#pragma unroll
+    for (int c = 0; c < 25; ++c) tr.F[c] = q.get(i, c);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+        tr.fx[c] = q.get(i, 25 + c);
+        tr.xn[c] = T(0);
+    }
+#pragma unroll
+    for (int c = 0; c < 15; ++c) tr.Q[c] = q.get(i, 30 + c);
+}
+
+template <typename T, class S>
+PES_DEV void array_obs(const S& q, int i, Obs<T>& ob)
+{
+#pragma unroll
+    for (int c = 0; c < 10; ++c) ob.H[c] = q.get(i, 45 + c);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) ob.r[r] = q.get(i, 60 + r) - q.get(i, 55 + r);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ob.R[c] = q.get(i, 57 + c);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) ob.xn[c] = T(0);
+}
+
+// The transition out of the last state of the lane before `lane`.
+template <typename T>
+PES_DEV void load_array_trans(const KParams<T>& p, int lane, Trans<T>& tr)
+{
+    const T* h = array_warp<kFilterIn>(p, p.L - 1, lane - 1) + ((lane - 1) & 31);
+#pragma unroll
+    for (int i = 0; i < 25; ++i) tr.F[i] = __ldg(h + i * 32);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        tr.fx[i] = __ldg(h + (25 + i) * 32);
+        tr.xn[i] = T(0);
+    }
+#pragma unroll
+    for (int i = 0; i < 15; ++i) tr.Q[i] = __ldg(h + (30 + i) * 32);
+}
+
+// acc <- acc (x) the Levenberg-Marquardt pseudo-measurement of a state's nominal
+// xb. Out of line: a damped run pays for the call, the others keep the
+// operator's code and registers out of their loops.
+template <typename T>
+__device__ __noinline__ void damp_element(FElem<T>& acc, const T* xb, T lambda)
+{
+    FElem<T> dmp;
+    felem_damping(dmp, xb, lambda);
+    combine_filter(acc, dmp, acc);
+}
+
+template <typename T>
+__device__ __noinline__ void damp_gauss(Gauss<T>& g, const T* xb, T lambda)
+{
+    FElem<T> dmp;
+    felem_damping(dmp, xb, lambda);
+    apply_filter(g, dmp, g);
+}
+
+// Filtering, level 1: fold the lane's chunk [a, e) into one element, from the
+// predicted state at a to the predicted state at e. Step k folds the update
+// with its own observation and then the prediction through its outgoing
+// transition (k -> k+1), both linearised about the nominal of k, so the state's
+// sigma-point factor serves both. With a stored linearisation (MODE_RUN,
+// sigma-point rules) both are kept for the re-run and the RTS pass.
+template <int K, typename T>
+PES_DEV bool fold_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, FElem<T>& acc,
+                               const Prefetch<T, kStateIn>& pf)
+{
+    constexpr int LIN = kLinOf<K>, FS = kFS<K>;
     bool ok = true;
     T zero[5] = {T(0), T(0), T(0), T(0), T(0)};
     felem_identity(acc, zero);
     if (a >= e) return ok;
-    const bool store_lin = kStoreLin<LIN> && p.mode == MODE_RUN;
+    const bool store_lin = kStoreLin<K> && p.mode == MODE_RUN;
     SegCursor cur;
     cur.init(p.offsets, p.B, a);
-    const int64_t dix = p.lanes_layout ? p.NL : 1;
-    int64_t ix = state_ix(p, a, a, lane);
+    const int64_t dix = p.NL;
+    int64_t ix = lane;
     StateIn<T, LIN> sc, sn;   // inputs of states k, k+1
-    if (!cur.is_head(a)) {
-        StateIn<T, LIN> sp;
-        load_state(p, prev_ix(p, a, lane), sp);
-        Trans<T> tr;
-        Factor<T, LIN> fp;
-        ok &= factor_state(sp, fp);
-        lin_trans(p, a - 1, sp, fp, tr);
-        felem_identity(acc, tr.xn);
-        fold_predict(acc, tr);
-    }
     // the next state's inputs are loaded a step ahead: into registers for
     // the Taylor linearisation; for the sigma-point ones, whose register
-    // pressure makes a register prefetch cost more in spills than it hides
-    // (measured: fold 202 -> 194 us per iteration at T = 2^20 without it),
-    // into shared memory by cp.async when the caller provides the stages
+    // pressure makes a register prefetch cost more in spills than it hides,
+    // into shared memory
     constexpr bool prefetch = !kSigma<LIN>;
-    const bool async_pf = kSigma<LIN> && pf != nullptr;
-    if (prefetch) load_state(p, ix, sc);
-    if (async_pf) {
-        pf->issue(p, ix, 0);
-        StatePrefetch<T>::commit();
+    if (prefetch) {
+        load_state(p, ix, sc);
+        felem_identity(acc, sc.x);
+    } else {
+        pf.issue(ix, 0);
+        pf.commit();
     }
 #pragma unroll 1
     for (int64_t k = a; k < e; ++k, ix += dix) {
@@ -498,13 +574,17 @@ PES_DEV bool fold_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int la
         const int s = (int)(k - a);
         if (prefetch) {
             if (k + 1 < e) load_state(p, ix + dix, sn);
-        } else if (async_pf) {
-            if (k + 1 < e) pf->issue(p, ix + dix, (s + 1) & 1);
-            StatePrefetch<T>::commit();
-            StatePrefetch<T>::wait_prev();
-            pf->take(s & 1, sc);
         } else {
-            load_state(p, ix, sc);
+            if (k + 1 < e) pf.issue(ix + dix, (s + 1) & 1);
+            pf.commit();
+            pf.wait_prev();
+#pragma unroll
+            for (int i = 0; i < 5; ++i) sc.x[i] = pf.get(s & 1, i);
+#pragma unroll
+            for (int i = 0; i < 15; ++i) sc.P[i] = pf.get(s & 1, 5 + i);
+            sc.y[0] = pf.get(s & 1, 20);
+            sc.y[1] = pf.get(s & 1, 21);
+            if (s == 0) felem_identity(acc, sc.x);   // the input is measured from the nominal of a
         }
         Factor<T, LIN> fc;
         ok &= factor_state(sc, fc);
@@ -514,152 +594,178 @@ PES_DEV bool fold_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int la
             felem_apply_prior(acc, m0, P0);
         } else {
             Obs<T> ob;
-            lin_obs(p, k, cur.b, sc, fc, ob);
-            if (store_lin) store_lin_obs(p, s, lane, ob);
-            ok &= fold_update(acc, ob);
+            form_obs<K>(p, cur.b, sc, fc, ob);
+            if (store_lin) store_lin_obs<K>(p, s, lane, ob);
+            ok &= fold_update<FS>(acc, ob);
         }
-        if (LIN != LIN_ARRAYS && lm_of(p.model, cur.b) > T(0)) {
-            // Levenberg-Marquardt pseudo-measurement of this state's nominal
-            FElem<T> dmp;
-            felem_damping(dmp, sc.x, lm_of(p.model, cur.b));
-            combine_filter(acc, dmp, acc);
+        if (lm_of(p.model, cur.b) > T(0)) {
+            FElem<T> tmp = acc;
+            T xb[5];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) xb[i] = sc.x[i];
+            damp_element(tmp, xb, lm_of(p.model, cur.b));
+            acc = tmp;
         }
-        if (!cur.is_tail(k) && (k + 1 < e || store_lin)) {
+        if (!cur.is_tail(k)) {
             Trans<T> tr;
-            lin_trans(p, k, sc, fc, tr);
-            if (store_lin) store_lin_trans(p, s, lane, tr);
-            if (k + 1 < e) fold_predict(acc, tr);
+            form_trans<K>(p, sc, fc, tr);
+            if (store_lin) store_lin_trans<K>(p, s, lane, tr);
+            fold_predict<FS>(acc, tr);
         }
         if (prefetch) sc = sn;
     }
+    if (!prefetch) pf.wait_all();
     return ok;
 }
 
-// Filtered moments in the caller's arrays (MODE_FILTER output, MODE_SMOOTH input).
+// The same over given arrays (the filter scan). Its chunks' boundaries are the
+// filtered states, each step predicting from the previous state and then
+// updating: its results keep the rounding that they always had, which the FP64
+// log-likelihoods of FP32 runs show.
 template <typename T>
-PES_DEV void store_filtered(const KParams<T>& p, int64_t k, const T* m, const T* P)
+PES_DEV bool fold_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, FElem<T>& acc, T* wstage,
+                                uint64_t* wbar, uint32_t& wpar)
 {
+    bool ok = true;
+    T zero[5] = {T(0), T(0), T(0), T(0), T(0)};
+    felem_identity(acc, zero);
+    FoldStream<T> ws;
+    ws.init(wstage, wbar, wpar);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) p.xf[i * p.N + k] = m[i];
-#pragma unroll
-    for (int i = 0; i < 15; ++i) p.Pf[i * p.N + k] = P[i];
+    for (int i = 0; i < 2; ++i)
+        if (i < p.L) ws.issue(array_warp<kFilterIn>(p, i, lane), i);
+    SegCursor cur;
+    if (a < e) {
+        cur.init(p.offsets, p.B, a);
+        if (!cur.is_head(a)) {   // the transition out of the previous lane's last state
+            Trans<T> tr;
+            load_array_trans(p, lane, tr);
+            fold_predict(acc, tr);
+        }
+    }
+#pragma unroll 1
+    for (int s = 0; s < p.L; ++s) {
+        const int64_t k = a + s;
+        const int st = s & 1;
+        ws.wait(st, p.status);
+        if (k < e) {
+            cur.forward(k);
+            if (cur.is_head(k)) {
+                T m0[5], P0[15];
+                load_prior(p, cur.b, m0, P0);
+                felem_apply_prior(acc, m0, P0);
+            } else {
+                Obs<T> ob;
+                array_obs(ws, st, ob);
+                ok &= fold_update(acc, ob);
+            }
+            if (!cur.is_tail(k) && k + 1 < e) {
+                Trans<T> tr;
+                array_trans(ws, st, tr);
+                fold_predict(acc, tr);
+            }
+        }
+        __syncwarp();
+        if (s + 2 < p.L) ws.issue(array_warp<kFilterIn>(p, s + 2, lane), st);
+    }
+    wpar = ws.parity;
+    return ok;
 }
 
+// Filtered moments in the given arrays (MODE_FILTER output).
 template <typename T>
-PES_DEV void load_filtered(const KParams<T>& p, int64_t k, T* m, T* P)
+PES_DEV void store_filtered(const KParams<T>& p, int64_t ix, const T* m, const T* P)
 {
 #pragma unroll
-    for (int i = 0; i < 5; ++i) m[i] = __ldg(p.xf + i * p.N + k);
+    for (int i = 0; i < 5; ++i) p.xf[i * p.cs + ix] = m[i];
 #pragma unroll
-    for (int i = 0; i < 15; ++i) P[i] = __ldg(p.Pf + i * p.N + k);
+    for (int i = 0; i < 15; ++i) p.Pf[i * p.cs + ix] = P[i];
 }
 
-// MODE_RUN: the smoothing element of state a + s of a lane, kept between the
-// filtering re-run that builds it and the RTS pass that applies it. Layout
-// [warp][s][component][32 lanes]: a warp's accesses for one step are one
-// contiguous, coalesced run, and its consecutive steps are adjacent.
-template <typename T>
-PES_DEV T* selem_slot(const KParams<T>& p, int s, int lane)
-{
-    return p.hand + ((size_t)(lane >> 5) * p.L + s) * (HAND * 32) + (lane & 31);
-}
-
-template <typename T>
-PES_DEV void store_selem(const KParams<T>& p, int s, int lane, const SElem<T>& el)
-{
-    T* h = selem_slot(p, s, lane);
-    const T* src = reinterpret_cast<const T*>(&el);
-#pragma unroll
-    for (int i = 0; i < HAND; ++i) h[i * 32] = src[i];
-}
-
-template <typename T>
-PES_DEV void load_selem(const KParams<T>& p, int s, int lane, SElem<T>& el)
-{
-    const T* h = selem_slot(p, s, lane);
-    T* dst = reinterpret_cast<T*>(&el);
-#pragma unroll
-    for (int i = 0; i < HAND; ++i) dst[i] = h[i * 32];
-}
-
-// MODE_RUN handoff alternative: the filtered moments (x*, P*) of state a + s,
-// from which the RTS pass rebuilds the smoothing element (same slot layout).
+// MODE_RUN: the filtered moments (x*, P*) of state a + s of a lane, kept
+// between the filtering re-run and the RTS pass, which builds the smoothing
+// element from them (20 scalars per state; handing over finished elements, 50
+// scalars, cost more in traffic than the element's prediction does in
+// arithmetic). Layout [warp][s][component][32 lanes]: a warp's accesses for one
+// step are one contiguous, coalesced run.
 template <typename T>
 PES_DEV void store_xP(const KParams<T>& p, int s, int lane, const T* m, const T* P)
 {
-    T* h = selem_slot(p, s, lane);
+    T* h = p.hand + ((size_t)(lane >> 5) * p.L + s) * (HAND * 32) + (lane & 31);
 #pragma unroll
     for (int i = 0; i < 5; ++i) h[i * 32] = m[i];
 #pragma unroll
     for (int i = 0; i < 15; ++i) h[(5 + i) * 32] = P[i];
 }
 
-template <typename T>
-PES_DEV void load_xP(const KParams<T>& p, int s, int lane, T* m, T* P)
+// The linearisation of stage `i` of a stream (layout of store_lin_*; `off` is
+// what precedes slot component 0 in the stage); xn the state's nominal (read
+// where it is not stored).
+template <int K, typename T, class S>
+PES_DEV void obs_from_stage(const S& ws, int i, const T* xn, Obs<T>& ob)
 {
-    const T* h = selem_slot(p, s, lane);
+    if constexpr (K == KK_CUBATURE) {
 #pragma unroll
-    for (int i = 0; i < 5; ++i) m[i] = h[i * 32];
+        for (int r = 0; r < 2; ++r) {
+            ob.H[r * 5] = ws.get(i, 34 + 2 * r);
+            ob.H[r * 5 + 1] = ws.get(i, 35 + 2 * r);
+            ob.r[r] = ws.get(i, 38 + r);
+        }
 #pragma unroll
-    for (int i = 0; i < 15; ++i) P[i] = h[(5 + i) * 32];
+        for (int c = 0; c < 3; ++c) ob.R[c] = ws.get(i, 40 + c);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) ob.xn[c] = xn[c];
+    } else {
+#pragma unroll
+        for (int c = 0; c < 10; ++c) ob.H[c] = ws.get(i, c);
+        ob.r[0] = ws.get(i, 10);
+        ob.r[1] = ws.get(i, 11);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) ob.R[c] = ws.get(i, 12 + c);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) ob.xn[c] = ws.get(i, 15 + c);
+    }
 }
 
-// Whether the filtering re-run hands the RTS pass finished smoothing elements
-// (50 scalars per state) or the filtered moments (20 scalars per state) from
-// which the RTS pass would rebuild them. The re-run builds every element
-// anyway (it folds them for the smoother's tree), so handing them over saves
-// the RTS pass a transition linearisation, a prediction and a Cholesky per
-// step for 120 more bytes of traffic per state (measured: IEKS 326 -> 304 us
-// per iteration at T = 2^20).
-template <int LIN>
-constexpr bool kStoreElements = (LIN != LIN_ARRAYS);
-
-// Stored linearisation of step stage `i` of a lane-stream (layout of store_lin_*).
-template <typename T, class S>
-PES_DEV void obs_from_stage(const S& ws, int i, Obs<T>& ob)
+template <int K, typename T, class S>
+PES_DEV void trans_from_stage(const KParams<T>& p, const S& ws, int i, int off, const T* xn, Trans<T>& tr)
 {
+    if constexpr (K == KK_CUBATURE) {
 #pragma unroll
-    for (int c = 0; c < 10; ++c) ob.H[c] = ws.get(i, c);
-    ob.r[0] = ws.get(i, 10);
-    ob.r[1] = ws.get(i, 11);
+        for (int c = 0; c < 20; ++c) tr.F[c] = ws.get(i, off + c);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) ob.R[c] = ws.get(i, 12 + c);
+        for (int c = 0; c < 4; ++c) tr.fx[c] = ws.get(i, off + 20 + c);
+        tr.fx[4] = xn[4];
 #pragma unroll
-    for (int c = 0; c < 5; ++c) ob.xn[c] = ws.get(i, 15 + c);
+        for (int c = 0; c < 15; ++c) tr.Q[c] = p.model.Q[c];
+#pragma unroll
+        for (int c = 0; c < 10; ++c) tr.Q[si4(c)] = ws.get(i, off + 24 + c);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) tr.xn[c] = xn[c];
+    } else {
+#pragma unroll
+        for (int c = 0; c < 5; ++c) tr.xn[c] = ws.get(i, off + 15 + c);
+#pragma unroll
+        for (int c = 0; c < 25; ++c) tr.F[c] = ws.get(i, off + 20 + c);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) tr.fx[c] = ws.get(i, off + 45 + c);
+#pragma unroll
+        for (int c = 0; c < 15; ++c) tr.Q[c] = ws.get(i, off + 50 + c);
+    }
 }
 
-template <typename T, class S>
-PES_DEV void trans_from_stage(const S& ws, int i, Trans<T>& tr)
+// Filtering, level 5: re-run the chunk from the predicted Gaussian at its start,
+// keeping the filtered moments. The loop runs over the L steps of the chunk in
+// every lane of the warp (lanes whose chunk is shorter idle), so that a warp
+// stream can feed it the stored linearisation.
+template <int K, typename T>
+PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, const Gauss<T>& G, T* wstage,
+                                uint64_t* wbar, uint32_t& wpar)
 {
-#pragma unroll
-    for (int c = 0; c < 5; ++c) tr.xn[c] = ws.get(i, 15 + c);
-#pragma unroll
-    for (int c = 0; c < 25; ++c) tr.F[c] = ws.get(i, 20 + c);
-#pragma unroll
-    for (int c = 0; c < 5; ++c) tr.fx[c] = ws.get(i, 45 + c);
-#pragma unroll
-    for (int c = 0; c < 15; ++c) tr.Q[c] = ws.get(i, 50 + c);
-}
-
-// Filtering, level 5: re-run the chunk from the Gaussian of the state before it,
-// storing filtered moments; in MODE_RUN also build and fold the chunk's
-// smoothing elements (Eqs. 17-18) into accS. The loop runs over the L steps
-// of the chunk in every lane of the warp (lanes whose chunk is shorter idle),
-// so that a warp stream can feed it the stored linearisation: step s reads
-// the transition into state s from the previous step's stage, then releases
-// that stage for the copy of step s + 1, then reads its observation.
-template <typename T, int LIN>
-PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, const Gauss<T>& G,
-                                SElem<T>& accS, T* wstage, uint64_t* wbar, uint32_t& wpar)
-{
+    constexpr int LIN = kLinOf<K>, FS = kFS<K>, ST = kLinStages<K>;
     bool ok = true;
-    selem_identity(accS);
-    const bool smooth = (p.mode == MODE_RUN);
-    double ll = 0.0;   // log-likelihood terms of trajectory llb (filter scan with given arrays only)
-    int llb = -1;
     const bool any = a < e;
-    constexpr bool stored_lin = kStoreLin<LIN>;
-    const bool use_lin = stored_lin && smooth;
+    constexpr bool use_lin = kStoreLin<K>;
     SegCursor cur;
     if (any) cur.init(p.offsets, p.B, a);
     T m[5], P[15];
@@ -667,253 +773,356 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
     for (int i = 0; i < 5; ++i) m[i] = G.m[i];
 #pragma unroll
     for (int i = 0; i < 15; ++i) P[i] = G.P[i];
-    const int64_t dix = p.lanes_layout ? p.NL : 1;
-    int64_t ix = state_ix(p, a, a, lane);
-    StateIn<T, LIN> sp, sc, sn;   // inputs of states k-1, k, k+1 (when linearising here)
-    if (!use_lin && any) {
-        if (!cur.is_head(a)) load_state(p, prev_ix(p, a, lane), sp);
-        load_state(p, ix, sc);
-    }
-    WarpStream<T, LINS, LINS> ws;
+    const int64_t dix = p.NL;
+    int64_t ix = lane;
+    StateIn<T, LIN> sc, sn;   // inputs of states k, k+1 (when linearising here)
+    constexpr bool want_x = K == KK_CUBATURE;   // the stored form leaves the nominal out
+    T xc[5], xn[5];
+    if (!use_lin && any) load_state(p, ix, sc);
+    if (want_x && any) load_nominal(p, ix, xc);
+    WarpStream<T, kLinScalars<K>, ST> ws;
     if (use_lin) {
-        ws.init(p.lin + (size_t)(lane >> 5) * p.L * (LINS * 32), wstage, wbar, wpar);
-        ws.issue(0, 0);
+        ws.init(wstage, wbar, wpar);
+#pragma unroll
+        for (int i = 0; i < ST; ++i)
+            if (i < p.L) ws.issue(lin_warp<K>(p, i, lane), i);
     }
 #pragma unroll 1
     for (int s = 0; s < p.L; ++s, ix += dix) {
         const int64_t k = a + s;
-        const bool act = k < e;
-        if (use_lin) ws.wait(s & 1, p.status);
-        T mp[5], Pp[15];
-        bool head = false;
-        if (act) {
+        const int st = s % ST;
+        if (use_lin) ws.wait(st, p.status);
+        if (k < e) {
             cur.forward(k);
             if (!use_lin && k + 1 < e) load_state(p, ix + dix, sn);
-            head = cur.is_head(k);
-            if (head) {
-                if (smooth && k > a) {
-                    SElem<T> el;
-                    selem_last(el, m, P);
-                    combine_smoother(accS, el, accS);
-                    if (kStoreElements<LIN>) store_selem(p, s - 1, lane, el);
-                }
-            } else {
-                Trans<T> tr;
-                if (use_lin) {
-                    if (s == 0) load_lin_trans(p, p.L - 1, lane - 1, tr);
-                    else trans_from_stage<T>(ws, (s - 1) & 1, tr);
-                } else {
-                    Factor<T, LIN> fp;
-                    ok &= factor_state(sp, fp);
-                    lin_trans(p, k - 1, sp, fp, tr);
-                }
-                T FP[25];
-                predict(tr, m, P, mp, FP, Pp);
-                if (smooth && k > a) {
-                    SElem<T> el;
-                    ok &= selem_from_prediction(m, P, FP, Pp, mp, el);
-                    combine_smoother(accS, el, accS);
-                    if (kStoreElements<LIN>) store_selem(p, s - 1, lane, el);
-                }
-            }
-        }
-        if (use_lin) {
-            // every lane is done with the previous step's stage: refill it
-            __syncwarp();
-            if (s + 1 < p.L) ws.issue(s + 1, (s + 1) & 1);
-        }
-        if (act) {
-            if (head) {
+            if (want_x && k + 1 < e) load_nominal(p, ix + dix, xn);
+            Factor<T, LIN> fc;
+            if (!use_lin) ok &= factor_state(sc, fc);
+            if (cur.is_head(k)) {
                 load_prior(p, cur.b, m, P);
             } else {
                 Obs<T> ob;
-                if (use_lin) {
-                    obs_from_stage<T>(ws, s & 1, ob);
-                } else {
-                    Factor<T, LIN> fc;
-                    ok &= factor_state(sc, fc);
-                    lin_obs(p, k, cur.b, sc, fc, ob);
-                }
-                if constexpr (LIN == LIN_ARRAYS) {
-                    if (p.loglik) {
-                        double term;
-                        ok &= kf_update(ob, mp, Pp, m, P, &term);
-                        if (cur.b != llb) {
-                            if (llb >= 0) atomicAdd(p.loglik + llb, ll);
-                            ll = 0.0;
-                            llb = cur.b;
-                        }
-                        ll += term;
-                    } else {
-                        ok &= kf_update(ob, mp, Pp, m, P);
-                    }
-                } else {
-                    ok &= kf_update(ob, mp, Pp, m, P);
-                }
+                if constexpr (use_lin) obs_from_stage<K>(ws, st, xc, ob);
+                else form_obs<K>(p, cur.b, sc, fc, ob);
+                T mn[5], Pn[15];
+                ok &= kf_update<FS>(ob, m, P, mn, Pn);
+#pragma unroll
+                for (int i = 0; i < 5; ++i) m[i] = mn[i];
+#pragma unroll
+                for (int i = 0; i < 15; ++i) P[i] = Pn[i];
             }
-            if (LIN != LIN_ARRAYS && lm_of(p.model, cur.b) > T(0)) {
-                // Levenberg-Marquardt pseudo-measurement of this state's nominal
+            if (lm_of(p.model, cur.b) > T(0)) {
                 T xb[5];
                 load_nominal(p, ix, xb);
-                FElem<T> dmp;
-                felem_damping(dmp, xb, lm_of(p.model, cur.b));
-                Gauss<T> g, gd;
+                Gauss<T> g;
 #pragma unroll
                 for (int i = 0; i < 5; ++i) g.m[i] = m[i];
 #pragma unroll
                 for (int i = 0; i < 15; ++i) g.P[i] = P[i];
-                apply_filter(g, dmp, gd);
+                damp_gauss(g, xb, lm_of(p.model, cur.b));
 #pragma unroll
-                for (int i = 0; i < 5; ++i) m[i] = gd.m[i];
+                for (int i = 0; i < 5; ++i) m[i] = g.m[i];
 #pragma unroll
-                for (int i = 0; i < 15; ++i) P[i] = gd.P[i];
+                for (int i = 0; i < 15; ++i) P[i] = g.P[i];
             }
-            if (!smooth) store_filtered(p, k, m, P);
-            else if (!kStoreElements<LIN>) store_xP(p, s, lane, m, P);
-            if (p.fstore) {
+            store_xP(p, s, lane, m, P);
+            if (k + 1 < e && !cur.is_tail(k)) {
+                Trans<T> tr;
+                if constexpr (use_lin) trans_from_stage<K>(p, ws, st, 0, xc, tr);
+                else form_trans<K>(p, sc, fc, tr);
+                T mp[5], FP[25], Pp[15];
+                predict<FS>(tr, m, P, mp, FP, Pp);
 #pragma unroll
-                for (int i = 0; i < 5; ++i) p.fstore[i * p.cs + ix] = m[i];
+                for (int i = 0; i < 5; ++i) m[i] = mp[i];
 #pragma unroll
-                for (int i = 0; i < 15; ++i) p.fstore[(5 + i) * p.cs + ix] = P[i];
+                for (int i = 0; i < 15; ++i) P[i] = Pp[i];
             }
-            if (!use_lin) {
-                sp = sc;
-                sc = sn;
-            }
+            if (!use_lin) sc = sn;
+            if (want_x)
+#pragma unroll
+                for (int i = 0; i < 5; ++i) xc[i] = xn[i];
+        }
+        if (use_lin) {
+            __syncwarp();   // every lane is done with the stage: refill it
+            if (s + ST < p.L) ws.issue(lin_warp<K>(p, s + ST, lane), st);
         }
     }
     if (use_lin) wpar = ws.parity;
-    if (llb >= 0) atomicAdd(p.loglik + llb, ll);
-    if (smooth && any) {
-        // smoothing element of the chunk's last state: the transition out of the
-        // chunk is linearised about the last state's nominal
-        SElem<T> el;
-        if (cur.is_tail(e - 1)) {
-            selem_last(el, m, P);
-        } else {
-            Trans<T> tr;
-            if (use_lin) {
-                trans_from_stage<T>(ws, (p.L - 1) & 1, tr);
-            } else {
-                Factor<T, LIN> fp;
-                ok &= factor_state(sp, fp);
-                lin_trans(p, e - 1, sp, fp, tr);
-            }
-            T mp[5], FP[25], Pp[15];
-            predict(tr, m, P, mp, FP, Pp);
-            ok &= selem_from_prediction(m, P, FP, Pp, mp, el);
-        }
-        combine_smoother(accS, el, accS);
-        if (kStoreElements<LIN>) store_selem(p, (int)(e - 1 - a), lane, el);
-    }
     return ok;
+}
+
+// The same over given arrays, with the log-likelihoods if they are wanted.
+template <typename T>
+PES_DEV bool rerun_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, const Gauss<T>& G, T* wstage,
+                                 uint64_t* wbar, uint32_t& wpar)
+{
+    bool ok = true;
+    LogLik<T> ll;   // of the measurements of trajectory llb in the chunk
+    int llb = -1;
+    SegCursor cur;
+    if (a < e) cur.init(p.offsets, p.B, a);
+    T m[5], P[15];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) m[i] = G.m[i];
+#pragma unroll
+    for (int i = 0; i < 15; ++i) P[i] = G.P[i];
+    FilterStream<T> ws;
+    ws.init(wstage, wbar, wpar);
+    ws.issue(array_warp<kFilterIn>(p, 0, lane), 0);
+    if (p.L > 1) ws.issue(array_warp<kFilterIn>(p, 1, lane), 1);
+    int st = 0;
+#pragma unroll 1
+    for (int s = 0; s < p.L; ++s) {
+        const int64_t k = a + s;
+        const int other = st == 0 ? 2 : st - 1;   // the stage of steps s - 1 and s + 2
+        ws.wait(st, p.status);
+        const bool head = k < e && (cur.forward(k), cur.is_head(k));
+        T mp[5], Pp[15];
+        if (k < e && !head) {
+            Trans<T> tr;
+            if (s > 0) array_trans(ws, other, tr);
+            else load_array_trans(p, lane, tr);
+            T FP[25];
+            predict(tr, m, P, mp, FP, Pp);
+        }
+        __syncwarp();   // every lane is done with step s - 1
+        if (s + 2 < p.L) ws.issue(array_warp<kFilterIn>(p, s + 2, lane), other);
+        if (k < e) {
+            if (head) {
+                load_prior(p, cur.b, m, P);
+            } else {
+                Obs<T> ob;
+                array_obs(ws, st, ob);
+                if (p.loglik) {
+                    if (cur.b != llb) {
+                        if (llb >= 0) atomicAdd(p.loglik + llb, ll.value());
+                        ll = LogLik<T>();
+                        llb = cur.b;
+                    }
+                    ok &= kf_update(ob, mp, Pp, m, P, &ll);
+                } else {
+                    ok &= kf_update(ob, mp, Pp, m, P);
+                }
+            }
+            store_filtered(p, lane_ix(p, s, lane), m, P);
+        }
+        st = st == 2 ? 0 : st + 1;
+    }
+    __syncwarp();
+    wpar = ws.parity;
+    if (llb >= 0) atomicAdd(p.loglik + llb, ll.value());
+    return ok;
+}
+
+// The smoothing element of a lane's whole chunk [a, e), from the state at e to
+// the state at a: Eq. 17 for the chunk as one transition. G is the predicted
+// Gaussian at a, f the chunk's filtering element. Conditioned on the chunk's
+// measurements, x_a ~ N(m + D (eta - J (m - xr)), D) with D = (P^{-1} + J)^{-1},
+// and x_e given x_a is (A, b, C). A trajectory that ends within the chunk cuts
+// the element (E = 0); the state before a trajectory's first one ignores it.
+template <typename T>
+PES_DEV bool chunk_selem(const KParams<T>& p, int64_t a, int64_t e, const FElem<T>& f, const Gauss<T>& G,
+                         SElem<T>& el)
+{
+    selem_identity(el);
+    if (a >= e) return true;
+    SegCursor cur;
+    cur.init(p.offsets, p.B, a);
+    if (cur.is_head(a)) {
+        T z[15];
+#pragma unroll
+        for (int i = 0; i < 15; ++i) z[i] = T(0);
+        selem_last(el, z, z);
+        return true;
+    }
+    T D[15], dm[5], u[5], Du[5], md[5];
+    info_update_cov(G.P, f.J, D);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) dm[i] = G.m[i] - f.xr[i];
+    sv(f.J, dm, u);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) u[i] = f.eta[i] - u[i];
+    sv(D, u, Du);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) md[i] = G.m[i] + Du[i];
+    if (cur.next <= e) {
+        selem_last(el, md, D);
+        return true;
+    }
+    T mp[5], AD[25], Pp[15];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) dm[i] += Du[i];
+    mv(f.A, dm, mp);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) mp[i] += f.b[i];
+    m_s(f.A, D, AD);
+    abt_sym_add(AD, f.A, f.C, Pp);
+    return selem_from_prediction(md, D, AD, Pp, mp, el);
+}
+
+// The smoothing element of a state from stage i of the given arrays' stream.
+template <typename T>
+PES_DEV bool array_selem(const SmoothStream<T>& ws, int i, bool tail, SElem<T>& el)
+{
+    T m[5], P[15];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) m[c] = ws.get(i, 45 + c);
+#pragma unroll
+    for (int c = 0; c < 15; ++c) P[c] = ws.get(i, 50 + c);
+    if (tail) {
+        selem_last(el, m, P);
+        return true;
+    }
+    Trans<T> tr;
+    array_trans(ws, i, tr);
+    T mp[5], FP[25], Pp[15];
+    predict(tr, m, P, mp, FP, Pp);
+    return selem_from_prediction(m, P, FP, Pp, mp, el);
 }
 
 // Smoothing, level 1 in MODE_SMOOTH: fold the chunk's smoothing elements from
 // the given filtered moments and transitions.
-template <typename T, int LIN>
-PES_DEV bool fold_smoother_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, SElem<T>& accS)
+template <typename T>
+PES_DEV bool fold_smoother_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, SElem<T>& accS, T* wstage,
+                                  uint64_t* wbar, uint32_t& wpar)
 {
     bool ok = true;
     selem_identity(accS);
-    if (a >= e) return ok;
     SegCursor cur;
-    cur.init(p.offsets, p.B, a);
+    if (a < e) cur.init(p.offsets, p.B, a);
+    SmoothStream<T> ws;
+    ws.init(wstage, wbar, wpar);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+        if (i < p.L) ws.issue(array_warp<kSmoothIn>(p, i, lane), i);
 #pragma unroll 1
-    for (int64_t k = a; k < e; ++k) {
-        cur.forward(k);
-        T m[5], P[15];
-        load_filtered(p, k, m, P);
-        SElem<T> el;
-        if (cur.is_tail(k)) {
-            selem_last(el, m, P);
-        } else {
-            Trans<T> tr;
-            ok &= get_trans<T, LIN>(p, k, k, tr);
-            T mp[5], FP[25], Pp[15];
-            predict(tr, m, P, mp, FP, Pp);
-            ok &= selem_from_prediction(m, P, FP, Pp, mp, el);
+    for (int s = 0; s < p.L; ++s) {
+        ws.wait(s & 1, p.status);
+        if (a + s < e) {
+            cur.forward(a + s);
+            SElem<T> el;
+            ok &= array_selem(ws, s & 1, cur.is_tail(a + s), el);
+            combine_smoother(accS, el, accS);
         }
-        combine_smoother(accS, el, accS);
+        __syncwarp();
+        if (s + 2 < p.L) ws.issue(array_warp<kSmoothIn>(p, s + 2, lane), s & 1);
     }
+    wpar = ws.parity;
+    return ok;
+}
+
+// Smoothing, level 5 in MODE_SMOOTH.
+template <typename T>
+PES_DEV bool rts_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, const Gauss<T>& G, T* wstage,
+                        uint64_t* wbar, uint32_t& wpar)
+{
+    bool ok = true;
+    SegCursor cur;
+    if (a < e) cur.init(p.offsets, p.B, e - 1);
+    Gauss<T> s = G;
+    SmoothStream<T> ws;
+    ws.init(wstage, wbar, wpar);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+        if (i < p.L) ws.issue(array_warp<kSmoothIn>(p, p.L - 1 - i, lane), i);
+    int st = 0;
+#pragma unroll 1
+    for (int sidx = p.L - 1; sidx >= 0; --sidx, st ^= 1) {
+        const int64_t k = a + sidx;
+        ws.wait(st, p.status);
+        if (k < e) {
+            cur.backward(k);
+            const int64_t ix = lane_ix(p, sidx, lane);
+            SElem<T> el;
+            ok &= array_selem(ws, st, cur.is_tail(k), el);
+            apply_smoother(el, s, s);
+            bool finite = true;
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                finite = finite && isfinite(s.m[i]);
+                p.x[i * p.cs + ix] = s.m[i];
+            }
+            if (!finite) atomicOr(p.status, ST_NONFINITE);
+#pragma unroll
+            for (int i = 0; i < 15; ++i) p.P[i * p.cs + ix] = s.P[i];
+        }
+        __syncwarp();
+        if (sidx >= 2) ws.issue(array_warp<kSmoothIn>(p, sidx - 2, lane), st);
+    }
+    wpar = ws.parity;
     return ok;
 }
 
 // Smoothing, level 5: Rauch-Tung-Striebel re-run backwards from the Gaussian of
 // the state after the chunk: x_k ~ E_k (x_{k+1} - xr_k) + g_k with covariance
-// E P E^T + L (a last state has E = 0). In MODE_RUN the stored elements (or
-// the stored filtered moments, from which the elements are rebuilt) arrive
-// through a warp stream and the smoothed moments replace the nominal in
-// place; in MODE_SMOOTH the elements are rebuilt from the given arrays.
-template <typename T, int LIN>
+// E P E^T + L (a last state has E = 0), each element built from the state's
+// filtered moments and its outgoing transition. The filtered moments (and the
+// stored linearisation, if any) arrive through a warp stream and the smoothed
+// moments replace the nominal in place.
+template <int K, typename T>
 PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, const Gauss<T>& G, bool write_P,
                        bool want_norm, double* conv, int& nb, double& num, double& den, T* wstage, uint64_t* wbar,
                        uint32_t& wpar)
 {
+    constexpr int LIN = kLinOf<K>, FS = kFS<K>;
     bool ok = true;
     const bool any = a < e;
     SegCursor cur;
     if (any) cur.init(p.offsets, p.B, e - 1);
     Gauss<T> s = G;
-    const bool run = (p.mode == MODE_RUN);
-    const bool stored = run && kStoreElements<LIN>;
-    const T* wbase = p.hand + (size_t)(lane >> 5) * p.L * (HAND * 32);
-    WarpStream<T, HAND, HAND> we;   // stored smoothing elements
-    WarpStream<T, 20, HAND> wx;     // stored filtered moments
-    if (run) {
-        if (stored) {
-            we.init(wbase, wstage, wbar, wpar);
-            we.issue(p.L - 1, 0);
-        } else {
-            wx.init(wbase, wstage, wbar, wpar);
-            wx.issue(p.L - 1, 0);
-        }
-    }
+    constexpr bool use_lin = kStoreLin<K>;
+    constexpr int ST = kRtsStages<K>;
+    WarpStream<T, HAND + (use_lin ? kLinTrans<K> : 0), ST> ws;
+    const T* hand = p.hand + (size_t)(lane >> 5) * p.L * (HAND * 32);
+    auto issue = [&](int sidx, int st) {
+        if (use_lin) ws.issue2(hand + (size_t)sidx * (HAND * 32), HAND, lin_warp<K>(p, sidx, lane) + kLinTransAt<K> * 32,
+                               kLinTrans<K>, st);
+        else ws.issue(hand + (size_t)sidx * (HAND * 32), st);
+    };
+    ws.init(wstage, wbar, wpar);
+#pragma unroll
+    for (int i = 0; i < ST; ++i)
+        if (i < p.L) issue(p.L - 1 - i, i);
+    // the nominal (to linearise about, and for the update norm) a step ahead
+    const bool want_x = !use_lin || K == KK_CUBATURE || want_norm;
+    T xc[5], xn[5];
+    if (want_x && any) load_nominal(p, lane_ix(p, e - 1 - a, lane), xc);
+    int st = 0;
 #pragma unroll 1
-    for (int it = 0; it < p.L; ++it) {
-        const int sidx = p.L - 1 - it;
+    for (int sidx = p.L - 1; sidx >= 0; --sidx) {
         const int64_t k = a + sidx;
-        const int st = it & 1;
-        if (run) {
-            if (stored) {
-                if (it + 1 < p.L) we.issue(sidx - 1, st ^ 1);
-                we.wait(st, p.status);
-            } else {
-                if (it + 1 < p.L) wx.issue(sidx - 1, st ^ 1);
-                wx.wait(st, p.status);
-            }
-        }
+        ws.wait(st, p.status);
         if (k < e) {
             cur.backward(k);
-            SElem<T> ec;
-            if (stored) {
-                T* dst = reinterpret_cast<T*>(&ec);
+            const int64_t ix = lane_ix(p, sidx, lane);
+            if (want_x && k > a) load_nominal(p, ix - p.NL, xn);
+            T m[5], P[15];
 #pragma unroll
-                for (int c = 0; c < HAND; ++c) dst[c] = we.get(st, c);
+            for (int c = 0; c < 5; ++c) m[c] = ws.get(st, c);
+#pragma unroll
+            for (int c = 0; c < 15; ++c) P[c] = ws.get(st, 5 + c);
+            if (cur.is_tail(k)) {
+#pragma unroll
+                for (int c = 0; c < 5; ++c) s.m[c] = m[c];
+#pragma unroll
+                for (int c = 0; c < 15; ++c) s.P[c] = P[c];
             } else {
-                T m[5], P[15];
-                if (run) {
-#pragma unroll
-                    for (int c = 0; c < 5; ++c) m[c] = wx.get(st, c);
-#pragma unroll
-                    for (int c = 0; c < 15; ++c) P[c] = wx.get(st, 5 + c);
+                Trans<T> tr;
+                if constexpr (use_lin) {
+                    trans_from_stage<K>(p, ws, st, HAND - kLinTransAt<K>, xc, tr);
                 } else {
-                    load_filtered(p, k, m, P);
+                    StateIn<T, LIN> in;
+                    Factor<T, LIN> fc;
+#pragma unroll
+                    for (int c = 0; c < 5; ++c) in.x[c] = xc[c];
+                    form_trans<K>(p, in, fc, tr);
                 }
-                if (cur.is_tail(k)) {
-                    selem_last(ec, m, P);
-                } else {
-                    Trans<T> tr;
-                    ok &= get_trans<T, LIN>(p, k, state_ix(p, k, a, lane), tr);
-                    T mp[5], FP[25], Pp[15];
-                    predict(tr, m, P, mp, FP, Pp);
-                    ok &= selem_from_prediction(m, P, FP, Pp, mp, ec);
-                }
+                T mp[5], FP[25], Pp[15];
+                predict<FS>(tr, m, P, mp, FP, Pp);
+                SElem<T> ec;
+                ok &= selem_from_prediction(m, P, FP, Pp, mp, ec);
+                apply_smoother(ec, s, s);
             }
-            apply_smoother(ec, s, s);
-            const int64_t ix = state_ix(p, k, a, lane);
-            T xold[5];
-            if (want_norm) load_nominal(p, ix, xold);
             bool finite = true;
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
@@ -937,224 +1146,66 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
                 }
 #pragma unroll
                 for (int i = 0; i < 5; ++i) {
-                    const double dv = double(s.m[i]) - double(xold[i]);
+                    const double dv = double(s.m[i]) - double(xc[i]);
                     num += dv * dv;
                     den += double(s.m[i]) * double(s.m[i]);
                 }
             }
+#pragma unroll
+            for (int c = 0; c < 5; ++c) xc[c] = xn[c];
         }
-        if (run) __syncwarp();
+        __syncwarp();   // every lane is done with the stage: refill it
+        if (sidx >= ST) issue(sidx - ST, st);
+        st = st + 1 == ST ? 0 : st + 1;
     }
-    if (run) wpar = stored ? we.parity : wx.parity;
+    wpar = ws.parity;
     return ok;
 }
 
 // ---- block and grid levels -------------------------------------------------------------
 
-// The filtering operator of the tree levels as one out-of-line function: the
-// lane and top-level trees then run the same copy of its ~2,000 instructions,
-// which stays in the instruction cache from level to level, where two inlined
-// copies were each fetched afresh (the smaller operators stay inline).
-template <typename T>
-__device__ __noinline__ void tree_combine_filter(const FElem<T>& a, const FElem<T>& b, FElem<T>& o)
+// Lane t's element into the tree's leaves, and the tree's up-sweep; the block's
+// element goes to slot `agg`.
+template <typename T, int NT, class Ops, typename Elem>
+PES_DEV void publish_block(const Elem& el, int nl, T* agg)
 {
-    combine_filter(a, b, o);
-}
-
-template <typename T, int NE>
-PES_DEV void copy_elem_to_global(const T* src, T* dst)
-{
-    for (int i = threadIdx.x; i < NE; i += blockDim.x) dst[i] = src[i];
-}
-
-// n blocks' aggregates (NE scalars each) from global into shared memory, eight
-// loads in flight per thread before their stores (one L2 round trip per eight
-// scalars instead of one per scalar).
-template <typename T, int NT, int NE>
-PES_DEV void load_aggregates(const T* src, T* dst, int n)
-{
-    constexpr int U = 8;
-    const int total = n * NE;
-#pragma unroll 1
-    for (int i0 = threadIdx.x; i0 < total; i0 += U * NT) {
-        T v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * NT;
-            v[u] = i < total ? src[i] : T(0);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * NT;
-            if (i < total) dst[i] = v[u];
-        }
-    }
-}
-
-// Filtering levels 2-4. elem[t] holds lane t's folded element on entry; returns
-// the Gaussian of the state before lane t's chunk.
-//
-// The operators of a tree level are issue-bound, one thread's instruction
-// stream each: a level costs one operator's time only while no SM
-// sub-partition runs two warps of it. So the operator at element 2t + 1 (or
-// 2t) runs on thread t < NT / 2: a level's active threads then sit in at most
-// NT / 64 warps, one per sub-partition, where the element's own thread would
-// spread them over all NT / 32 warps.
-template <typename T, int NT>
-PES_DEV void filter_block_scan(const KParams<T>& p, FElem<T>* elem, FElem<T>* top, Gauss<T>* gs,
-                               Gauss<T>* gblock, unsigned& gen, Gauss<T>& out, int it)
-{
+    constexpr int NC = Ops::NC;
+    static_assert(sizeof(Elem) == NC * sizeof(T), "the element's scalars");
     const int t = threadIdx.x;
-    const bool half = t < NT / 2;
-    const int to = 2 * t + 1, te = 2 * t;   // the odd and the even element of thread t
+    T* s = smem_as<T>();
+    if (t < nl) reinterpret_cast<Elem*>(s)[tree_place(t, nl)] = el;
     __syncthreads();
-    PES_PHASE(p, it, 1);
-#pragma unroll 1
-    for (int s = 1; s < NT; s <<= 1) {
-        if (half && ((to + 1) & (2 * s - 1)) == 0) tree_combine_filter(elem[to - s], elem[to], elem[to]);
-        __syncthreads();
-    }
-    copy_elem_to_global<T, FE>(reinterpret_cast<const T*>(&elem[NT - 1]), p.aggF + (size_t)blockIdx.x * FE);
-    PES_PHASE(p, it, 2);
-    grid_barrier(p, gen);
-    PES_PHASE(p, it, 3);
-    // level 3: Gaussian of the state before this block = product of blocks [0, blockIdx)
-    if (t == 0) {
-#pragma unroll
-        for (int i = 0; i < 5; ++i) gblock->m[i] = T(0);
-#pragma unroll
-        for (int i = 0; i < 15; ++i) gblock->P[i] = T(0);
-    }
-    const int j = blockIdx.x;
-#pragma unroll 1
-    for (int c0 = 0; c0 < j; c0 += NT) {
-        const int n = min(NT, j - c0);
-        __syncthreads();
-        load_aggregates<T, NT, FE>(p.aggF + (size_t)c0 * FE, reinterpret_cast<T*>(top), n);
-        __syncthreads();
-#pragma unroll 1
-        for (int s = 1; s < n; s <<= 1) {
-            if (half && (te & (2 * s - 1)) == 0 && te + s < n) tree_combine_filter(top[te], top[te + s], top[te]);
-            __syncthreads();
-        }
-        if (t == 0) apply_filter(*gblock, top[0], *gblock);
-    }
-    __syncthreads();
-    PES_PHASE(p, it, 4);
-    // level 4: down-sweep
-    if (t == NT - 1) gs[NT - 1] = *gblock;
-    __syncthreads();
-#pragma unroll 1
-    for (int s = NT / 2; s >= 1; s >>= 1) {
-        if (half && ((to + 1) & (2 * s - 1)) == 0) {
-            const Gauss<T> gin = gs[to];
-            Gauss<T> gr;
-            apply_filter(gin, elem[to - s], gr);
-            gs[to - s] = gin;
-            gs[to] = gr;
-        }
-        __syncthreads();
-    }
-    out = gs[t];
-    __syncthreads();
-    PES_PHASE(p, it, 5);
+    const int root = tree_reduce<T, NT, Ops>(0, -1, nl);
+    for (int c = t; c < NC; c += NT) agg[c] = s[root + c];
 }
 
-// Smoothing levels 2-4 (mirrored: subtrees accumulate at their left end).
-// Returns the Gaussian of the state after lane t's chunk.
-template <typename T, int NT>
-PES_DEV void smoother_block_scan(const KParams<T>& p, SElem<T>* elem, SElem<T>* top, Gauss<T>* gs,
-                                 Gauss<T>* gblock, unsigned& gen, Gauss<T>& out, int it)
+template <typename T, int K, int NT>
+constexpr size_t smem_bytes_for()
 {
-    const int t = threadIdx.x;
-    const bool half = t < NT / 2;
-    const int te = 2 * t;   // the operators run as in filter_block_scan
-    __syncthreads();
-    PES_PHASE(p, it, 7);
-#pragma unroll 1
-    for (int s = 1; s < NT; s <<= 1) {
-        if (half && (te & (2 * s - 1)) == 0) combine_smoother(elem[te], elem[te + s], elem[te]);
-        __syncthreads();
-    }
-    copy_elem_to_global<T, SE>(reinterpret_cast<const T*>(&elem[0]), p.aggS + (size_t)blockIdx.x * SE);
-    PES_PHASE(p, it, 8);
-    grid_barrier(p, gen);
-    PES_PHASE(p, it, 9);
-    if (t == 0) {
-#pragma unroll
-        for (int i = 0; i < 5; ++i) gblock->m[i] = T(0);
-#pragma unroll
-        for (int i = 0; i < 15; ++i) gblock->P[i] = T(0);
-    }
-    const int j = blockIdx.x;
-    const int nb = gridDim.x;
-#pragma unroll 1
-    for (int c1 = nb; c1 > j + 1;) {
-        const int n = min(NT, c1 - (j + 1));
-        const int c0 = c1 - n;
-        __syncthreads();
-        load_aggregates<T, NT, SE>(p.aggS + (size_t)c0 * SE, reinterpret_cast<T*>(top), n);
-        __syncthreads();
-#pragma unroll 1
-        for (int s = 1; s < n; s <<= 1) {
-            if (half && (te & (2 * s - 1)) == 0 && te + s < n) combine_smoother(top[te], top[te + s], top[te]);
-            __syncthreads();
-        }
-        if (t == 0) apply_smoother(top[0], *gblock, *gblock);
-        c1 = c0;
-    }
-    __syncthreads();
-    PES_PHASE(p, it, 10);
-    if (t == 0) gs[0] = *gblock;
-    __syncthreads();
-#pragma unroll 1
-    for (int s = NT / 2; s >= 1; s >>= 1) {
-        if (half && (te & (2 * s - 1)) == 0) {
-            const Gauss<T> gin = gs[te];
-            Gauss<T> gl;
-            apply_smoother(elem[te + s], gin, gl);
-            gs[te + s] = gin;
-            gs[te] = gl;
-        }
-        __syncthreads();
-    }
-    out = gs[t];
-    __syncthreads();
-    PES_PHASE(p, it, 11);
+    using M = TreeMem<T, NT>;
+    static_assert(M::kEnd - FE * NT >= NT * 2 * kStateIn, "the sigma-point folds' prefetch fits beside the leaves");
+    static_assert(K != KK_ARRAYS || (M::kEnd - FE * NT >= NT * 2 * kFilterIn && M::kEnd >= NT * 3 * kFilterIn &&
+                                     M::kEnd - SE * NT >= NT * 2 * kSmoothIn),
+                  "the streams of the scans over given arrays fit");
+    static_assert(M::kBlock - M::kAfterSmootherTree >= NT * kLinStages<K> * kLinScalars<K>, "the re-run's stages fit");
+    static_assert(M::kEnd >= NT * kRtsStages<K> * (HAND + (kStoreLin<K> ? kLinTrans<K> : 0)), "the RTS stages fit");
+    static_assert(M::kEnd >= 2 * NT * int(sizeof(double) / sizeof(T)), "the norm reduction fits");
+    return sizeof(T) * M::kEnd;
 }
 
-template <int NT>
-constexpr size_t smem_bytes_for(size_t scalar)
-{
-    // lane tree (filtering elements; smoothing elements alias it), top-level
-    // buffer, down-sweep Gaussians, one block Gaussian; the per-warp stream
-    // stages (2 x LINS x 32 scalars per warp) reuse this memory
-    static_assert(size_t(NT) * FE * 2 + size_t(NT) * GE + GE >= size_t(NT) * 2 * LINS, "stream stages must fit");
-    static_assert(FE >= 2 * StatePrefetch<double>::NS, "the fold's prefetch stages fit the top-level buffer");
-    return scalar * (size_t(NT) * FE * 2 + size_t(NT) * GE + GE);
-}
-
-template <typename T, int LIN, int NT>
+template <typename T, int K, int NT>
 __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> p)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    FElem<T>* elemF = reinterpret_cast<FElem<T>*>(smem_raw);
-    SElem<T>* elemS = reinterpret_cast<SElem<T>*>(smem_raw);
-    FElem<T>* topF = elemF + NT;
-    SElem<T>* topS = reinterpret_cast<SElem<T>*>(topF);
-    Gauss<T>* gs = reinterpret_cast<Gauss<T>*>(topF + NT);
-    Gauss<T>* gblock = gs + NT;
+    using M = TreeMem<T, NT>;
+    T* smem = smem_as<T>();
     __shared__ int s_flag;
-    __shared__ double s_red[NT];
     // per-warp stream stages reuse the tree memory during the sequential passes
-    __shared__ __align__(8) uint64_t s_bar[2 * (NT / 32)];
-    T* wstage = reinterpret_cast<T*>(smem_raw) + (size_t)(threadIdx.x >> 5) * 2 * LINS * 32;
-    uint64_t* wbar = s_bar + 2 * (threadIdx.x >> 5);
+    __shared__ __align__(8) uint64_t s_bar[kMaxStages * (NT / 32)];
+    const int warp = threadIdx.x >> 5;
+    uint64_t* wbar = s_bar + kMaxStages * warp;
     uint32_t wpar = 0;
-    if ((threadIdx.x & 31) == 0) {
-        mbar_init(wbar, 1);
-        mbar_init(wbar + 1, 1);
-    }
+    if ((threadIdx.x & 31) == 0)
+        for (int i = 0; i < kMaxStages; ++i) mbar_init(wbar + i, 1);
     mbar_init_fence();
     __syncthreads();
 
@@ -1162,6 +1213,8 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
     const int lane = blockIdx.x * NT + t;
     const int64_t a = min((int64_t)lane * p.L, p.N);
     const int64_t e = min(a + (int64_t)p.L, p.N);
+    // lanes of this block with a chunk (its first ones); one identity if none
+    const int nl = (int)max((int64_t)1, min((int64_t)NT, (p.N + p.L - 1) / p.L - (int64_t)blockIdx.x * NT));
     unsigned gen = 0;
     bool ok = true;
 
@@ -1175,52 +1228,86 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
     for (it = 0; it < p.iters; ++it) {
         if (*(volatile int*)p.status & (ST_TIMEOUT | ST_BADARG)) break;
         const bool last = (it == p.iters - 1);
-        SElem<T> accS;
+        T* aggF = p.aggF + (size_t)(it & 1) * p.agg_blocks * FE;
+        T* aggS = p.aggS + (size_t)(it & 1) * p.agg_blocks * SE;
         PES_PHASE(p, it, 0);
+        SElem<T> accS;
+        Gauss<T> G;
         if (do_filter) {
             FElem<T> acc;
-            // the sigma-point folds prefetch each next state into the
-            // top-level tree's memory, idle until after the block up-sweep
-            StatePrefetch<T> pf;
-            pf.base = reinterpret_cast<T*>(topF) + t;
-            pf.stride = NT;
-            ok &= fold_filter_chunk<T, LIN>(p, a, e, lane, acc, &pf);
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            elemF[t] = acc;
-            Gauss<T> G;
-            filter_block_scan<T, NT>(p, elemF, topF, gs, gblock, gen, G, it);
-            ok &= rerun_filter_chunk<T, LIN>(p, a, e, lane, G, accS, wstage, wbar, wpar);
-            __syncthreads();   // the stream stages overlap the smoothing lane tree
-            PES_PHASE(p, it, 6);
+            // the fold's prefetch goes to memory beside the leaves
+            if constexpr (K == KK_ARRAYS)
+                ok &= fold_filter_arrays(p, a, e, lane, acc, smem + FE * NT + (size_t)warp * 2 * kFilterIn * 32, wbar, wpar);
+            else
+                ok &= fold_filter_chunk<K>(p, a, e, lane, acc, Prefetch<T, kStateIn>{smem + FE * NT + t, NT, p.x, p.cs});
+            PES_PHASE(p, it, 1);
+            publish_block<T, NT, FilterOps<T, kKeepRounding<K, T>>>(acc, nl, aggF + (size_t)blockIdx.x * FE);
+            PES_PHASE(p, it, 2);
+            grid_arrive(p, gen);
+            grid_wait(p, gen);
+            PES_PHASE(p, it, 3);
+            tree_top<T, NT, FilterOps<T, kKeepRounding<K, T>>>(aggF, 0, blockIdx.x);
+            PES_PHASE(p, it, 4);
+            tree_down<T, NT, FilterOps<T, kKeepRounding<K, T>>>(nl);
+            G = reinterpret_cast<const Gauss<T>*>(smem + M::kGauss)[min(t, nl - 1)];
+            PES_PHASE(p, it, 5);
+            if (do_smooth) ok &= chunk_selem(p, a, e, reinterpret_cast<const FElem<T>*>(smem)[tree_place(min(t, nl - 1), nl)], G, accS);
+        } else {
+            if constexpr (K == KK_ARRAYS)
+                ok &= fold_smoother_arrays(p, a, e, lane, accS, smem + SE * NT + (size_t)warp * 2 * kSmoothIn * 32, wbar, wpar);
+        }
+        __syncthreads();   // the smoother's tree and the stream stages overlap the filter's
+        if (do_smooth) {
+            publish_block<T, NT, SmootherOps<T>>(accS, nl, aggS + (size_t)blockIdx.x * SE);
+            grid_arrive(p, gen);
+        }
+        PES_PHASE(p, it, 6);
+        if (do_filter) {
+            if constexpr (K == KK_ARRAYS) {
+                ok &= rerun_filter_arrays(p, a, e, lane, G, smem + (size_t)warp * 3 * kFilterIn * 32, wbar, wpar);
+            } else {
+                constexpr int kStage = kLinStages<K> * kLinScalars<K> * 32;
+                ok &= rerun_filter_chunk<K>(p, a, e, lane, G, smem + M::kAfterSmootherTree + (size_t)warp * kStage, wbar, wpar);
+            }
             if (track && blockIdx.x == 0) {
                 // the accumulators of the next iteration were last read before
                 // this iteration's first barrier; clear them for reuse
                 double* nxt = p.conv + (size_t)((it + 1) & 1) * 2 * p.B;
                 for (int i = t; i < 2 * p.B; i += NT) nxt[i] = 0.0;
             }
-        } else {
-            ok &= fold_smoother_chunk<T, LIN>(p, a, e, lane, accS);
         }
+        PES_PHASE(p, it, 7);
         if (do_smooth) {
-            elemS[t] = accS;
-            Gauss<T> Gs;
-            smoother_block_scan<T, NT>(p, elemS, topS, gs, gblock, gen, Gs, it);
-            const bool write_P = (p.mode != MODE_RUN) || kSigma<LIN> || last || p.write_P_every_iter;
+            grid_wait(p, gen);
+            PES_PHASE(p, it, 8);
+            tree_top<T, NT, SmootherOps<T>>(aggS, blockIdx.x + 1, gridDim.x);
+            PES_PHASE(p, it, 9);
+            tree_down<T, NT, SmootherOps<T>>(nl);
+            const Gauss<T> Gs = reinterpret_cast<const Gauss<T>*>(smem + M::kGauss)[min(t, nl - 1)];
+            __syncthreads();   // the stream stages overlap the tree
+            PES_PHASE(p, it, 10);
+            const bool write_P = kSigma<kLinOf<K>> || last || p.write_P_every_iter;
             int nb = -1;
             double num = 0.0, den = 0.0;
             double* conv = p.conv + (size_t)(it & 1) * 2 * p.B;
-            ok &= rts_chunk<T, LIN>(p, a, e, lane, Gs, write_P, track, conv, nb, num, den, wstage, wbar, wpar);
+            if constexpr (K == KK_ARRAYS) {
+                ok &= rts_arrays(p, a, e, lane, Gs, smem + (size_t)warp * 2 * kSmoothIn * 32, wbar, wpar);
+            } else {
+                constexpr int kStage = kRtsStages<K> * (HAND + (kStoreLin<K> ? kLinTrans<K> : 0)) * 32;
+                ok &= rts_chunk<K>(p, a, e, lane, Gs, write_P, track, conv, nb, num, den, smem + (size_t)warp * kStage, wbar, wpar);
+            }
             __syncthreads();
-            PES_PHASE(p, it, 12);
+            PES_PHASE(p, it, 11);
             if (track && nb >= 0) {
                 atomicAdd(conv + 2 * nb, num);
                 atomicAdd(conv + 2 * nb + 1, den);
             }
         }
-        if (p.mode == MODE_RUN && (!last || track)) {
-            grid_barrier(p, gen);
-            PES_PHASE(p, it, 13);
-            if (track) {
+        if (track) {
+            grid_arrive(p, gen);
+            grid_wait(p, gen);
+            PES_PHASE(p, it, 12);
+            {
                 // worst relative update norm over trajectories, identical in every block
                 const double* conv = p.conv + (size_t)(it & 1) * 2 * p.B;
                 double worst = 0.0;
@@ -1230,6 +1317,7 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
                     worst = fmax(worst, r);
                     if (p.traj_iters && blockIdx.x == 0 && r <= p.tol && p.traj_iters[b] == 0) p.traj_iters[b] = it + 1;
                 }
+                double* s_red = reinterpret_cast<double*>(smem);   // the sequential passes are over
                 s_red[t] = worst;
                 __syncthreads();
                 for (int s = NT / 2; s > 0; s >>= 1) {

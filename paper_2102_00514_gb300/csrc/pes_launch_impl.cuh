@@ -7,11 +7,11 @@
 
 namespace pes {
 
-template <typename T, int LIN, int NT>
+template <typename T, int K, int NT>
 cudaError_t launch_cfg(const KParams<T>& p, int nb, cudaStream_t st)
 {
-    auto kern = pes_persistent_kernel<T, LIN, NT>;
-    const size_t smem = smem_bytes_for<NT>(sizeof(T));
+    auto kern = pes_persistent_kernel<T, K, NT>;
+    const size_t smem = smem_bytes_for<T, K, NT>();
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     KParams<T> pc = p;
@@ -19,12 +19,12 @@ cudaError_t launch_cfg(const KParams<T>& p, int nb, cudaStream_t st)
     return cudaLaunchCooperativeKernel((const void*)kern, dim3(nb), dim3(NT), args, smem, st);
 }
 
-template <typename T, int LIN, int NT>
+template <typename T, int K, int NT>
 int capacity_cfg(int device)
 {
     // a failing call returns its negated error code (the caller reports it)
-    auto kern = pes_persistent_kernel<T, LIN, NT>;
-    const size_t smem = smem_bytes_for<NT>(sizeof(T));
+    auto kern = pes_persistent_kernel<T, K, NT>;
+    const size_t smem = smem_bytes_for<T, K, NT>();
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return -(int)e;
     int per_sm = 0, sms = 0;
@@ -35,8 +35,8 @@ int capacity_cfg(int device)
 
 }  // namespace pes
 
-#define PES_INSTANTIATE(T, LIN, NT)                                                              \
+#define PES_INSTANTIATE(T, K, NT)                                                              \
     namespace pes {                                                                              \
-    template cudaError_t launch_cfg<T, LIN, NT>(const KParams<T>&, int, cudaStream_t);           \
-    template int capacity_cfg<T, LIN, NT>(int);                                                  \
+    template cudaError_t launch_cfg<T, K, NT>(const KParams<T>&, int, cudaStream_t);           \
+    template int capacity_cfg<T, K, NT>(int);                                                  \
     }

@@ -24,6 +24,27 @@ template <int LIN>
 constexpr bool kSigma = (LIN == LIN_CUBATURE || LIN == LIN_GH);
 enum { ST_NOT_PD = 1, ST_NONFINITE = 2, ST_TIMEOUT = 4, ST_NOT_CONVERGED = 8, ST_BADARG = 16 };
 
+// Structure of the transition slope F and the observation slope H of a
+// linearisation, known at compile time: nothing (FS_DENSE); the coordinated
+// turn's Taylor slope (FS_CT); its regression slope (FS_SLR), whose last row is
+// e_4 (the turn rate is carried over, and the regression of a coordinate on the
+// state is that coordinate). Both have bearings, which see only the position.
+enum { FS_DENSE = 0, FS_CT = 1, FS_SLR = 2 };
+
+// Entry (i, j) of F: 0 zero, 1 one, 2 general.
+template <int FS>
+__host__ __device__ constexpr int f_entry(int i, int j)
+{
+    return FS == FS_DENSE ? 2
+           : i == 4       ? (j == 4 ? 1 : 0)
+           : FS == FS_SLR ? 2
+           : j >= 2       ? 2
+                          : (i == j ? 1 : 0);
+}
+// Columns of H from which on it is zero.
+template <int FS>
+constexpr int kHCols = FS == FS_DENSE ? 5 : 2;
+
 // Model parameters as passed to the kernels, already in the kernel's
 // precision (no conversions on the device). Q and R are packed (upper).
 template <typename T>
@@ -510,6 +531,232 @@ PES_DEV void lin_obs_cubature(const DevModel<T>& m, int b, const T* xbar, const 
         ob.r[0] = wrap_angle(y[0] - h_ref[0]) - zdev[0];
         ob.r[1] = wrap_angle(y[1] - h_ref[1]) - zdev[1];
     }
+#pragma unroll
+    for (int i = 0; i < 5; ++i) ob.xn[i] = xbar[i];
+}
+
+// ---- the coordinated turn, model known at compile time -------------------------
+
+// lin_trans_taylor of the coordinated turn; only F's general entries are written.
+template <typename T>
+PES_DEV void ct_trans_taylor(const DevModel<T>& m, const T* xn, Trans<T>& tr)
+{
+    const T dt = m.dt;
+    const CTCoef<T> k = ct_coef(xn[4], dt);
+    ct_jacobian(xn, k, dt, tr.F);
+    T inc[5];
+    ct_increment(xn, k, inc);
+    tr.fx[0] = xn[0] + inc[0];
+    tr.fx[1] = xn[1] + inc[1];
+    tr.fx[2] = inc[2];
+    tr.fx[3] = inc[3];
+    tr.fx[4] = inc[4];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) tr.xn[i] = xn[i];
+#pragma unroll
+    for (int i = 0; i < 15; ++i) tr.Q[i] = m.Q[i];
+}
+
+template <typename T>
+PES_DEV void ct_obs_taylor(const DevModel<T>& m, int b, const T* xn, const T* y, Obs<T>& ob)
+{
+#pragma unroll
+    for (int i = 0; i < 5; ++i) ob.xn[i] = xn[i];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) ob.R[i] = m.R[i];
+    T s[4];
+    load_sensors(m, b, s);
+    bearings_jacobian(xn, s, ob.H);
+    T hx[2];
+    bearings(xn, s, hx);
+    ob.r[0] = wrap_angle(y[0] - hx[0]);
+    ob.r[1] = wrap_angle(y[1] - hx[1]);
+}
+
+// lin_trans_cubature of the coordinated turn. For the pair xbar +- S (S column i
+// of scale chol(Pbar), zero above row i) the regression needs the odd part
+// D / 2 = (f+ - f-) / 2 and the even part U = (f+ + f-) / 2 - f(xbar). With the
+// turn angles a +- d (a = w dt, d = S_4 dt), the rotated (Rx, Ry) =
+// rot(a) (S_2, S_3) and the increment f(xbar) = (.., vx', vy', ..):
+//   velocities: D/2 = cos d R + sin d (-vy', vx'),
+//               U = -(1 - cos d) (vx', vy') + sin d (-Ry, Rx);
+//   positions, with A1(w +- S_4) = A1e +- A1o, A2 alike:
+//               D/2 = S + [A1e -A2e; A2e A1e] (S_2, S_3) + [A1o -A2o; A2o A1o] (vx, vy),
+//               U = [A1e - A1, -(A2e - A2); ..] (vx, vy) + [A1o -A2o; A2o A1o] (S_2, S_3).
+// For small angles A1, A2 and their odd and second-order even parts are Taylor
+// polynomials in a and d, so U is formed without cancellation. About 45
+// instructions per column against 110 for two evaluations of f: the fold's loop
+// body then fits the instruction cache (about 2,000 instructions; beyond that
+// one warp issues every 2.6 cycles and two share that, measured).
+template <typename T>
+PES_DEV void ct_trans_cubature(const DevModel<T>& m, const T* xbar, const T* L, const T* rdiag, Trans<T>& tr)
+{
+    const T dt = m.dt;
+    const T thr = sizeof(T) == 4 ? T(0.05) : T(0.01);
+    const CTCoef<T> kr = ct_coef(xbar[4], dt);
+    T inc[5];
+    ct_increment(xbar, kr, inc);
+    const T a = xbar[4] * dt, a2 = a * a;
+    const T vx = xbar[2], vy = xbar[3];
+    T Dm[20], U[20];   // rows 0..3 by columns: D / (2 scale), U
+    T zdev[4] = {T(0), T(0), T(0), T(0)};
+    const T isc = trcp(m.sp_scale);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const T Sx = i <= 2 ? m.sp_scale * L[2 * 5 + i] : T(0);
+        const T Sy = i <= 3 ? m.sp_scale * L[3 * 5 + i] : T(0);
+        const T Sw = m.sp_scale * L[4 * 5 + i];
+        const T d = Sw * dt, d2 = d * d;
+        T sd, omcd;
+        T A1e, A1o, A2e, A2o, dA1, dA2;   // dA: even part less the reference
+        if (fabs(a) + fabs(d) < thr) {
+            sd = d * (T(1) - d2 * (T(1) / T(6)) * (T(1) - d2 * (T(1) / T(20)) * (T(1) - d2 * (T(1) / T(42)))));
+            omcd = d2 * T(0.5) * (T(1) - d2 * (T(1) / T(12)) * (T(1) - d2 * (T(1) / T(30)) * (T(1) - d2 * (T(1) / T(56)))));
+            // A1 = dt (1 - a^2/6 + a^4/120), A2 = dt (a/2 - a^3/24 + a^5/720)
+            dA1 = dt * d2 * (T(-1) / T(6) + (T(6) * a2 + d2) * (T(1) / T(120)));
+            A1o = dt * a * d * (T(-1) / T(3) + (a2 + d2) * (T(1) / T(30)));
+            dA2 = dt * a * d2 * (T(-0.125) + (T(2) * a2 + d2) * (T(1) / T(144)));
+            A2o = dt * d * (T(0.5) - (T(3) * a2 + d2) * (T(1) / T(24)) +
+                            (T(5) * a2 * a2 + T(10) * a2 * d2 + d2 * d2) * (T(1) / T(720)));
+            A1e = kr.A1 + dA1;
+            A2e = kr.A2 + dA2;
+        } else {
+            T cd;
+            if (fabs(d) < T(0.05)) {
+                sd = d * (T(1) - d2 * (T(1) / T(6)) * (T(1) - d2 * (T(1) / T(20)) * (T(1) - d2 * (T(1) / T(42)))));
+                omcd = d2 * T(0.5) * (T(1) - d2 * (T(1) / T(12)) * (T(1) - d2 * (T(1) / T(30)) * (T(1) - d2 * (T(1) / T(56)))));
+            } else {
+                tsincos(d, &sd, &cd);
+                omcd = (cd > T(0)) ? sd * sd * trcp(T(1) + cd) : T(1) - cd;
+            }
+            cd = T(1) - omcd;
+            const T omcr = (kr.c > T(0)) ? kr.s * kr.s * trcp(T(1) + kr.c) : T(1) - kr.c;
+            T A1[2], A2[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const T sg = q == 0 ? T(1) : T(-1);
+                const T w = xbar[4] + sg * Sw, ap = w * dt;
+                if (fabs(ap) < thr) {
+                    const T p2 = ap * ap;
+                    A1[q] = dt * (T(1) - p2 * (T(1) / T(6)) + p2 * p2 * (T(1) / T(120)));
+                    A2[q] = dt * ap * (T(0.5) - p2 * (T(1) / T(24)) + p2 * p2 * (T(1) / T(720)));
+                } else {
+                    const T iw = trcp(w);
+                    A1[q] = (kr.s * cd + sg * kr.c * sd) * iw;
+                    A2[q] = (omcr + kr.c * omcd + sg * kr.s * sd) * iw;
+                }
+            }
+            A1e = T(0.5) * (A1[0] + A1[1]);
+            A1o = T(0.5) * (A1[0] - A1[1]);
+            A2e = T(0.5) * (A2[0] + A2[1]);
+            A2o = T(0.5) * (A2[0] - A2[1]);
+            dA1 = A1e - kr.A1;
+            dA2 = A2e - kr.A2;
+        }
+        // D / 2 (odd part)
+        T D0 = A1o * vx - A2o * vy, D1 = A2o * vx + A1o * vy;
+        T D2 = -sd * inc[3], D3 = sd * inc[2];
+        T U0 = dA1 * vx - dA2 * vy, U1 = dA2 * vx + dA1 * vy;
+        T U2 = -omcd * inc[2], U3 = -omcd * inc[3];
+        if (i <= 3) {
+            const T Rx = i <= 2 ? kr.c * Sx - kr.s * Sy : -kr.s * Sy;
+            const T Ry = i <= 2 ? kr.s * Sx + kr.c * Sy : kr.c * Sy;
+            if (i <= 2) {
+                D0 = fma(A1e, Sx, D0);
+                D1 = fma(A2e, Sx, D1);
+                U0 = fma(A1o, Sx, U0);
+                U1 = fma(A2o, Sx, U1);
+            }
+            D0 = fma(-A2e, Sy, D0);
+            D1 = fma(A1e, Sy, D1);
+            U0 = fma(-A2o, Sy, U0);
+            U1 = fma(A1o, Sy, U1);
+            const T cd = T(1) - omcd;
+            D2 = fma(cd, Rx, D2);
+            D3 = fma(cd, Ry, D3);
+            U2 = fma(-sd, Ry, U2);
+            U3 = fma(sd, Rx, U3);
+        }
+        // D / (2 scale); the positions' own offsets are exactly L's entries
+        Dm[0 * 5 + i] = i == 0 ? fma(D0, isc, L[0]) : D0 * isc;
+        Dm[1 * 5 + i] = i <= 1 ? fma(D1, isc, L[5 + i]) : D1 * isc;
+        Dm[2 * 5 + i] = D2 * isc;
+        Dm[3 * 5 + i] = D3 * isc;
+        U[0 * 5 + i] = U0;
+        U[1 * 5 + i] = U1;
+        U[2 * 5 + i] = U2;
+        U[3 * 5 + i] = U3;
+        zdev[0] += U0;
+        zdev[1] += U1;
+        zdev[2] += U2;
+        zdev[3] += U3;
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) zdev[r] *= m.sp_w;
+    solve_rows_lower_t<T, 4>(L, rdiag, Dm, tr.F);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int i = 0; i < 5; ++i) U[r * 5 + i] -= zdev[r];
+#pragma unroll
+    for (int i = 0; i < 15; ++i) tr.Q[i] = m.Q[i];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = r; q < 4; ++q) {
+            T s = U[r * 5] * U[q * 5];
+#pragma unroll
+            for (int i = 1; i < 5; ++i) s = fma(U[r * 5 + i], U[q * 5 + i], s);
+            tr.Q[si(r, q)] = fma(s, m.sp_w, fma(m.sp_w0c * zdev[r], zdev[q], m.Q[si(r, q)]));
+        }
+    tr.fx[0] = xbar[0] + inc[0] + zdev[0];
+    tr.fx[1] = xbar[1] + inc[1] + zdev[1];
+    tr.fx[2] = inc[2] + zdev[2];
+    tr.fx[3] = inc[3] + zdev[3];
+    tr.fx[4] = xbar[4];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) tr.xn[i] = xbar[i];
+}
+
+// lin_obs_cubature of the bearings: only the sigma directions 0 and 1 move the
+// position, so H has two columns and the other three points sit at the centre.
+template <typename T>
+PES_DEV void ct_obs_cubature(const DevModel<T>& m, int b, const T* xbar, const T* L, const T* rdiag, const T* y,
+                             Obs<T>& ob)
+{
+    T s[4], h_ref[2];
+    load_sensors(m, b, s);
+    bearings(xbar, s, h_ref);
+    const T sc = T(0.5) * trcp(m.sp_scale);
+    T U[2][2], zdev[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const T rx = xbar[0] - s[2 * r], ry = xbar[1] - s[2 * r + 1];
+        const T rr = rx * rx + ry * ry;
+        T D[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const T Sx = i == 0 ? m.sp_scale * L[0] : T(0), Sy = m.sp_scale * L[5 + i];
+            const T cross = i == 0 ? rx * Sy - ry * Sx : rx * Sy;
+            const T rs = i == 0 ? rx * Sx + ry * Sy : ry * Sy;
+            const T zp = tatan2(cross, rr + rs), zm = tatan2(-cross, rr - rs);
+            D[i] = (zp - zm) * sc;
+            U[r][i] = T(0.5) * (zp + zm);
+        }
+        zdev[r] = (U[r][0] + U[r][1]) * m.sp_w;
+        ob.H[r * 5 + 1] = D[1] * rdiag[1];
+        ob.H[r * 5] = fma(-ob.H[r * 5 + 1], L[5], D[0]) * rdiag[0];
+        ob.r[r] = wrap_angle(y[r] - h_ref[r]) - zdev[r];
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int q = r; q < 2; ++q) {
+            T v = T(3) * zdev[r] * zdev[q];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) v = fma(U[r][i] - zdev[r], U[q][i] - zdev[q], v);
+            ob.R[si2(r, q)] = fma(v, m.sp_w, fma(m.sp_w0c * zdev[r], zdev[q], m.R[si2(r, q)]));
+        }
 #pragma unroll
     for (int i = 0; i < 5; ++i) ob.xn[i] = xbar[i];
 }

@@ -34,8 +34,8 @@ constexpr int64_t kLaneCap = kMaxStates + (int64_t)kMaxBlocks * kMaxThreads;
 constexpr size_t kHand = (size_t)pes::HAND * kLaneCap;
 constexpr size_t kLanes = (size_t)22 * kLaneCap;
 constexpr size_t kLin = (size_t)pes::LINS * kLaneCap;
-constexpr size_t kAggF = (size_t)kMaxBlocks * pes::FE;
-constexpr size_t kAggS = (size_t)kMaxBlocks * pes::SE;
+constexpr size_t kAggF = (size_t)kMaxBlocks * 2 * pes::FE;
+constexpr size_t kAggS = (size_t)kMaxBlocks * 2 * pes::SE;
 constexpr size_t kConv = (size_t)4 * kMaxBatch;
 constexpr size_t kSens = (size_t)4 * kMaxBatch;
 constexpr size_t kWords = 4;                   // barrier counter, status, iteration count (one double each)

@@ -15,33 +15,166 @@
 // (I + J_j C_i)^{-1} = I - J_j D.
 #pragma once
 
+#include "pes_ff.cuh"
 #include "pes_model.cuh"
 
 namespace pes {
 
+// Padded so that the fields that are loaded together start on 16 bytes, and
+// to sizes at which consecutive elements' 16-byte words fall in different
+// shared-memory banks (76 and 60 words).
 template <typename T>
-struct FElem {
+struct alignas(16) FElem {
     T A[25];
     T b[5];
+    T pad0[2];
     T C[15];
-    T eta[5];
+    T pad1;
     T J[15];
+    T pad2;
+    T eta[5];
     T xr[5];
+    T pad3[2];
 };
 
 template <typename T>
-struct SElem {
+struct alignas(16) SElem {
     T E[25];
     T g[5];
+    T pad0[2];
     T L[15];
+    T pad1;
     T xr[5];
+    T pad2[7];
 };
 
 template <typename T>
-struct Gauss {
+struct alignas(16) Gauss {
     T m[5];
     T P[15];
 };
+
+// ---- products with a structured slope ------------------------------------------
+//
+// The coordinated turn's slopes have entries that are 0 or 1 whatever the state
+// (f adds its increments to the positions and keeps the turn rate; bearings see
+// only the position). With the model known at compile time those terms are left
+// out: about 170 instead of 350 multiply-adds for a folded prediction, 230
+// instead of 305 for the update. In finite arithmetic the results are the same
+// to the bit, as a term 0 x or 1 x adds no rounding.
+
+// C = F B
+template <int FS, typename T>
+PES_DEV void f_mm(const T* F, const T* B, T* C)
+{
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            T s = T(0);
+            bool first = true;
+#pragma unroll
+            for (int l = 0; l < 5; ++l) {
+                const int k = f_entry<FS>(i, l);
+                if (k == 0) continue;
+                if (first) s = k == 1 ? B[l * 5 + j] : F[i * 5 + l] * B[l * 5 + j];
+                else s = k == 1 ? s + B[l * 5 + j] : fma(F[i * 5 + l], B[l * 5 + j], s);
+                first = false;
+            }
+            C[i * 5 + j] = s;
+        }
+}
+
+// C = F S, S symmetric packed
+template <int FS, typename T>
+PES_DEV void f_ms(const T* F, const T* S, T* C)
+{
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            T s = T(0);
+            bool first = true;
+#pragma unroll
+            for (int l = 0; l < 5; ++l) {
+                const int k = f_entry<FS>(i, l);
+                if (k == 0) continue;
+                if (first) s = k == 1 ? S[si(l, j)] : F[i * 5 + l] * S[si(l, j)];
+                else s = k == 1 ? s + S[si(l, j)] : fma(F[i * 5 + l], S[si(l, j)], s);
+                first = false;
+            }
+            C[i * 5 + j] = s;
+        }
+}
+
+// Out (sym) = A F^T + Add (sym), product known to be symmetric
+template <int FS, typename T>
+PES_DEV void f_abt_sym_add(const T* A, const T* F, const T* Add, T* Out)
+{
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = i; j < 5; ++j) {
+            T s = Add[si(i, j)];
+#pragma unroll
+            for (int l = 0; l < 5; ++l) {
+                const int k = f_entry<FS>(j, l);
+                if (k == 0) continue;
+                s = k == 1 ? s + A[i * 5 + l] : fma(A[i * 5 + l], F[j * 5 + l], s);
+            }
+            Out[si(i, j)] = s;
+        }
+}
+
+// y = F x
+template <int FS, typename T>
+PES_DEV void f_mv(const T* F, const T* x, T* y)
+{
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        T s = T(0);
+        bool first = true;
+#pragma unroll
+        for (int l = 0; l < 5; ++l) {
+            const int k = f_entry<FS>(i, l);
+            if (k == 0) continue;
+            if (first) s = k == 1 ? x[l] : F[i * 5 + l] * x[l];
+            else s = k == 1 ? s + x[l] : fma(F[i * 5 + l], x[l], s);
+            first = false;
+        }
+        y[i] = s;
+    }
+}
+
+// out (2x5) = H S, S symmetric packed, H zero from column HC on
+template <int HC, typename T>
+PES_DEV void h_ms(const T* H, const T* S, T* out)
+{
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            T s = H[r * 5] * S[si(0, j)];
+#pragma unroll
+            for (int l = 1; l < HC; ++l) s = fma(H[r * 5 + l], S[si(l, j)], s);
+            out[r * 5 + j] = s;
+        }
+}
+
+// out (2x2 sym) = A H^T + Add
+template <int HC, typename T>
+PES_DEV void h_abt_sym_add(const T* A, const T* H, const T* Add, T* out)
+{
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int q = r; q < 2; ++q) {
+            T s = Add[si2(r, q)];
+#pragma unroll
+            for (int l = 0; l < HC; ++l) s = fma(A[r * 5 + l], H[q * 5 + l], s);
+            out[si2(r, q)] = s;
+        }
+}
 
 // Identity of Eq. 15 with input reference xr: (A = I, b = xr, C = 0, eta = 0, J = 0).
 template <typename T>
@@ -108,24 +241,24 @@ PES_DEV void felem_apply_prior(FElem<T>& a, const T* m0, const T* P0)
 //   A = A- - K G,  b = b- + K v,  C = C- - K H C-,
 // and the likelihood of y_k given the input accumulates
 //   J += G^T S^{-1} G,  eta += G^T S^{-1} v.
-// The two halves of fold_filter_step: the prediction through the transition,
-// after which a describes x_k given the input, then the update with the
-// observation at k. Folding them separately keeps the transition and the
-// observation from being live together.
-template <typename T>
+// The two halves are folded separately, which keeps the transition and the
+// observation from being live together: the prediction through the transition,
+// after which a describes x_k given the input, and the update with the
+// observation at k.
+template <int FS = FS_DENSE, typename T>
 PES_DEV void fold_predict(FElem<T>& a, const Trans<T>& tr)
 {
     T Am[25];
-    mm(tr.F, a.A, Am);
+    f_mm<FS>(tr.F, a.A, Am);
     T dv[5], bm[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) dv[i] = a.b[i] - tr.xn[i];
-    mv(tr.F, dv, bm);
+    f_mv<FS>(tr.F, dv, bm);
 #pragma unroll
     for (int i = 0; i < 5; ++i) bm[i] += tr.fx[i];
     T FC[25], Cm[15];
-    m_s(tr.F, a.C, FC);
-    abt_sym_add(FC, tr.F, tr.Q, Cm);
+    f_ms<FS>(tr.F, a.C, FC);
+    f_abt_sym_add<FS>(FC, tr.F, tr.Q, Cm);
 #pragma unroll
     for (int i = 0; i < 25; ++i) a.A[i] = Am[i];
 #pragma unroll
@@ -134,33 +267,18 @@ PES_DEV void fold_predict(FElem<T>& a, const Trans<T>& tr)
     for (int i = 0; i < 15; ++i) a.C[i] = Cm[i];
 }
 
-template <typename T>
+template <int FS = FS_DENSE, typename T>
 PES_DEV bool fold_update(FElem<T>& a, const Obs<T>& ob)
 {
+    constexpr int HC = kHCols<FS>;
     const T* Am = a.A;
     const T* bm = a.b;
     const T* Cm = a.C;
     // H C-
-    T HC[10];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            T s = ob.H[r * 5] * Cm[si(0, j)];
-#pragma unroll
-            for (int l = 1; l < 5; ++l) s = fma(ob.H[r * 5 + l], Cm[si(l, j)], s);
-            HC[r * 5 + j] = s;
-        }
+    T HCm[10];
+    h_ms<HC>(ob.H, Cm, HCm);
     T S[3];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int q = r; q < 2; ++q) {
-            T s = ob.R[si2(r, q)];
-#pragma unroll
-            for (int l = 0; l < 5; ++l) s = fma(HC[r * 5 + l], ob.H[q * 5 + l], s);
-            S[si2(r, q)] = s;
-        }
+    h_abt_sym_add<HC>(HCm, ob.H, ob.R, S);
     T Si[3];
     const bool ok = inv2_spd(S, Si);
     // K^T = S^{-1} H C-,  G = H A-,  v
@@ -169,15 +287,15 @@ PES_DEV bool fold_update(FElem<T>& a, const Obs<T>& ob)
     for (int r = 0; r < 2; ++r) {
 #pragma unroll
         for (int j = 0; j < 5; ++j) {
-            KT[r * 5 + j] = Si[si2(r, 0)] * HC[j] + Si[si2(r, 1)] * HC[5 + j];
+            KT[r * 5 + j] = Si[si2(r, 0)] * HCm[j] + Si[si2(r, 1)] * HCm[5 + j];
             T s = ob.H[r * 5] * Am[j];
 #pragma unroll
-            for (int l = 1; l < 5; ++l) s = fma(ob.H[r * 5 + l], Am[l * 5 + j], s);
+            for (int l = 1; l < HC; ++l) s = fma(ob.H[r * 5 + l], Am[l * 5 + j], s);
             G[r * 5 + j] = s;
         }
         T hv = ob.r[r];
 #pragma unroll
-        for (int l = 0; l < 5; ++l) hv = fma(-ob.H[r * 5 + l], bm[l] - ob.xn[l], hv);
+        for (int l = 0; l < HC; ++l) hv = fma(-ob.H[r * 5 + l], bm[l] - ob.xn[l], hv);
         v[r] = hv;
     }
     T Anew[25], bnew[5], Cnew[15];
@@ -192,7 +310,7 @@ PES_DEV bool fold_update(FElem<T>& a, const Obs<T>& ob)
     for (int i = 0; i < 5; ++i)
 #pragma unroll
         for (int j = i; j < 5; ++j)
-            Cnew[si(i, j)] = fma(-KT[5 + i], HC[5 + j], fma(-KT[i], HC[j], Cm[si(i, j)]));
+            Cnew[si(i, j)] = fma(-KT[5 + i], HCm[5 + j], fma(-KT[i], HCm[j], Cm[si(i, j)]));
 #pragma unroll
     for (int i = 0; i < 25; ++i) a.A[i] = Anew[i];
 #pragma unroll
@@ -215,13 +333,6 @@ PES_DEV bool fold_update(FElem<T>& a, const Obs<T>& ob)
         a.eta[i] = fma(G[5 + i], Siv[1], fma(G[i], Siv[0], a.eta[i]));
     }
     return ok;
-}
-
-template <typename T>
-PES_DEV bool fold_filter_step(FElem<T>& a, const Trans<T>& tr, const Obs<T>& ob)
-{
-    fold_predict(a, tr);
-    return fold_update(a, ob);
 }
 
 // out = ai (x) aj, Eq. 15 (ai earlier in time). aj's input reference is the
@@ -402,43 +513,81 @@ PES_DEV bool selem_from_prediction(const T* xf, const T* Pf, const T* FP, const 
 }
 
 // Predicted moments of the transition tr applied to (m, P): mp, FP = F P, Pp.
-template <typename T>
+template <int FS = FS_DENSE, typename T>
 PES_DEV void predict(const Trans<T>& tr, const T* m, const T* P, T* mp, T* FP, T* Pp)
 {
     T dx[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) dx[i] = m[i] - tr.xn[i];
-    mv(tr.F, dx, mp);
+    f_mv<FS>(tr.F, dx, mp);
 #pragma unroll
     for (int i = 0; i < 5; ++i) mp[i] += tr.fx[i];
-    m_s(tr.F, P, FP);
-    abt_sym_add(FP, tr.F, tr.Q, Pp);
+    f_ms<FS>(tr.F, P, FP);
+    f_abt_sym_add<FS>(FP, tr.F, tr.Q, Pp);
 }
 
-// Kalman update of (mp, Pp) with the observation ob: (m, P).
+// Running log-likelihood of a trajectory's measurements: the sum over steps of
+// log N(v; 0, S) = -1/2 (v^T S^{-1} v + log det S) - log 2 pi, to FP64's accuracy
+// of the given S and v (1e-12 relative). The determinants are multiplied up with
+// the exponent kept apart, and one logarithm is taken at the end. FP32 runs form
+// the terms in float-float where the values allow it (neither near the ends of
+// the range nor a cancelling determinant): the FP64 pipe issues an instruction
+// per warp every 64 cycles, and with a logarithm and a quotient per step it was
+// more than half of the filter scan's re-run (41 us at N = 128,128).
 template <typename T>
-PES_DEV bool kf_update(const Obs<T>& ob, const T* mp, const T* Pp, T* m, T* P, double* loglik_term = nullptr)
+struct LogLik {
+    double q = 0.0, det = 1.0;
+    ff qf = {0.0f, 0.0f}, df = {1.0f, 0.0f};
+    int exponent = 0, steps = 0;
+    PES_DEV void add(T s00, T s01, T s11, T v0, T v1)
+    {
+        ++steps;
+        if constexpr (sizeof(T) == 4) {
+            const float a = s00, b = s11, top = fmaxf(fabsf(v0), fabsf(v1));
+            const ff p = two_prod(a, b), r = two_prod(s01, s01);
+            // both products exact; their difference to 2^-48 of them
+            const ff h = two_sum(p.hi, -r.hi);
+            const ff d = fast_two_sum(h.hi, __fadd_rn(h.lo, __fsub_rn(p.lo, r.lo)));
+            if (fminf(a, b) > 1e-7f && fmaxf(a, b) < 1e7f && top < 1e5f && d.hi > 1e-3f * p.hi) {
+                const ff n0 = ff_mul_f(two_prod(b, v0), v0), n1 = ff_mul_f(two_prod(a, v1), v1);
+                const ff n2 = ff_mul_f(two_prod(-2.0f * s01, v0), v1);
+                qf = ff_add(qf, ff_div(ff_add(ff_add(n0, n2), n1), d));
+                df = ff_mul(df, d);
+                const int e = (__float_as_int(df.hi) >> 23) - 127;   // df.hi > 0, normal
+                const float scale = __int_as_float((127 - e) << 23);
+                df.hi *= scale;
+                df.lo *= scale;
+                exponent += e;
+                return;
+            }
+        }
+        const double c00 = s00, c01 = s01, c11 = s11, w0 = v0, w1 = v1;
+        const double d = c00 * c11 - c01 * c01;
+        q += (c11 * w0 * w0 - 2.0 * c01 * w0 * w1 + c00 * w1 * w1) / d;
+        det *= d;
+        const int hi = __double2hiint(det), e = (hi >> 20) & 0x7ff;
+        if (e > 0 && e < 0x7ff) {   // to [1, 2); zeros, subnormals, infinities and NaN stay
+            exponent += e - 1023;
+            det = __hiloint2double((hi & 0x800fffff) | 0x3ff00000, __double2loint(det));
+        }
+    }
+    PES_DEV double value() const
+    {
+        const double ln2 = 0.69314718055994530942, log_2pi = 1.8378770664093454836;
+        const double quad = q + ((double)qf.hi + (double)qf.lo);
+        return -0.5 * (quad + (log(det * ((double)df.hi + (double)df.lo)) + exponent * ln2)) - steps * log_2pi;
+    }
+};
+
+// Kalman update of (mp, Pp) with the observation ob: (m, P).
+template <int FS = FS_DENSE, typename T>
+PES_DEV bool kf_update(const Obs<T>& ob, const T* mp, const T* Pp, T* m, T* P, LogLik<T>* loglik = nullptr)
 {
+    constexpr int HC = kHCols<FS>;
     T HP[10];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            T s = ob.H[r * 5] * Pp[si(0, j)];
-#pragma unroll
-            for (int l = 1; l < 5; ++l) s = fma(ob.H[r * 5 + l], Pp[si(l, j)], s);
-            HP[r * 5 + j] = s;
-        }
+    h_ms<HC>(ob.H, Pp, HP);
     T S[3];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int q = r; q < 2; ++q) {
-            T s = ob.R[si2(r, q)];
-#pragma unroll
-            for (int l = 0; l < 5; ++l) s = fma(HP[r * 5 + l], ob.H[q * 5 + l], s);
-            S[si2(r, q)] = s;
-        }
+    h_abt_sym_add<HC>(HP, ob.H, ob.R, S);
     T Si[3];
     const bool ok = inv2_spd(S, Si);
     T KT[10], v[2];
@@ -448,17 +597,10 @@ PES_DEV bool kf_update(const Obs<T>& ob, const T* mp, const T* Pp, T* m, T* P, d
         for (int j = 0; j < 5; ++j) KT[r * 5 + j] = Si[si2(r, 0)] * HP[j] + Si[si2(r, 1)] * HP[5 + j];
         T hv = ob.r[r];
 #pragma unroll
-        for (int l = 0; l < 5; ++l) hv = fma(-ob.H[r * 5 + l], mp[l] - ob.xn[l], hv);
+        for (int l = 0; l < HC; ++l) hv = fma(-ob.H[r * 5 + l], mp[l] - ob.xn[l], hv);
         v[r] = hv;
     }
-    if (loglik_term) {
-        // log N(v; 0, S): the term of step k in log p(y_{1:T}) = sum_k log p(y_k | y_{1:k-1})
-        const double s00 = S[si2(0, 0)], s01 = S[si2(0, 1)], s11 = S[si2(1, 1)];
-        const double det = s00 * s11 - s01 * s01;
-        const double v0 = v[0], v1 = v[1];
-        const double q = (s11 * v0 * v0 - 2.0 * s01 * v0 * v1 + s00 * v1 * v1) / det;
-        *loglik_term = -0.5 * (q + log(det)) - 1.8378770664093454836;   // log(2 pi)
-    }
+    if (loglik) loglik->add(S[si2(0, 0)], S[si2(0, 1)], S[si2(1, 1)], v[0], v[1]);
 #pragma unroll
     for (int i = 0; i < 5; ++i) m[i] = fma(KT[5 + i], v[1], fma(KT[i], v[0], mp[i]));
 #pragma unroll

@@ -16,6 +16,21 @@ PES_DEV void load20(const float* base, int64_t cs, int64_t ix, float* m, float* 
     for (int c = 0; c < 15; ++c) P[c] = base[(5 + c) * cs + ix];
 }
 
+// The filtered moments of step s of a lane, component c at [c * 32] (the
+// smoother kernel's handoff layout).
+PES_DEV const float* filt_slot(const RefineParams& p, int s, int lane)
+{
+    return p.filt + ((size_t)(lane >> 5) * p.L + s) * (HAND * 32) + (lane & 31);
+}
+
+PES_DEV void load_filt(const float* f, float* m, float* P)
+{
+#pragma unroll
+    for (int c = 0; c < 5; ++c) m[c] = f[c * 32];
+#pragma unroll
+    for (int c = 0; c < 15; ++c) P[c] = f[(5 + c) * 32];
+}
+
 PES_DEV void store_elem(const RefineParams& p, int64_t ix, const float* A, const float* w, const float* s,
                         const float* r)
 {
@@ -77,7 +92,7 @@ __global__ void __launch_bounds__(RT_THREADS) refine_fwd_kernel(const RefinePara
     const int b = traj_of(p.offsets, p.B, k);
     const int64_t head = __ldg(p.offsets + b), next = __ldg(p.offsets + b + 1);
     float xf[5], Pf[15];
-    load20(p.filt, p.cs, ix, xf, Pf);
+    load_filt(filt_slot(p, s, lane), xf, Pf);
     if (k == head) {
         float A[25], w[5], sres[5], r[15];
 #pragma unroll
@@ -139,7 +154,7 @@ __global__ void __launch_bounds__(RT_THREADS) refine_fwd_kernel(const RefinePara
     float A[25], w[5];
     ok &= ff_kalman_step(tr, ob, xf, Pf, mf, Pff, A, w, sc);
     float x1[5], P1[15], sres[5], r[15];
-    load20(p.filt, p.cs, ix1, x1, P1);
+    load_filt(s + 1 < p.L ? filt_slot(p, s + 1, lane) : filt_slot(p, 0, lane + 1), x1, P1);
 #pragma unroll
     for (int c = 0; c < 5; ++c) sres[c] = ff_to_f(ff_add_f(mf[c], -x1[c]));
 #pragma unroll
@@ -161,7 +176,8 @@ __global__ void __launch_bounds__(RT_THREADS) refine_bwd_kernel(const RefinePara
     const int b = traj_of(p.offsets, p.B, k);
     const int64_t next = __ldg(p.offsets + b + 1);
     // the refined filtered moments as float-float pairs
-    auto filt_ff = [&](int c) { return two_sum(p.filt[c * p.cs + ix], p.dlt[c * p.cs + ix]); };
+    const float* filt = filt_slot(p, s, lane);
+    auto filt_ff = [&](int c) { return two_sum(filt[c * 32], p.dlt[c * p.cs + ix]); };
     float* el = p.elem + ix;
 #pragma unroll
     for (int c = 0; c < 5; ++c) el[(25 + c) * p.cs] = 0.0f;

@@ -56,7 +56,7 @@ struct RefineParams {
     const float* m0;          // [B][5]
     const float* P0;          // [B][15]
     const float* nom;         // [20][cs]: the final iteration's nominal, means then covariances
-    const float* filt;        // [20][cs]: the FP32 filtered moments of the final iteration
+    const float* filt;        // the FP32 filtered moments of the final iteration, as the smoother kernel keeps them
     float* xs;                // [20][cs]: the FP32 smoothed moments; refined in place
     float* elem;              // [RE][cs]
     float* trans;             // [RT][cs]

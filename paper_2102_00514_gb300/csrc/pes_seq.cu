@@ -17,21 +17,36 @@ namespace pes {
 
 namespace {
 
-// Smoothing element of state k in the per-state scratch, component-major.
+// Smoothing element of state k in the per-state scratch, component-major (50
+// scalars, in the memory of the parallel path's stored linearisation).
+static_assert(LINS >= 50, "the scratch holds an element per state");
+
 template <typename T>
 PES_DEV void seq_store_el(const KParams<T>& p, int64_t k, const SElem<T>& el)
 {
-    const T* src = reinterpret_cast<const T*>(&el);
+    T* h = p.lin + k;
 #pragma unroll
-    for (int i = 0; i < HAND; ++i) p.hand[(size_t)i * p.N + k] = src[i];
+    for (int i = 0; i < 25; ++i) h[(size_t)i * p.N] = el.E[i];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) h[(size_t)(25 + i) * p.N] = el.g[i];
+#pragma unroll
+    for (int i = 0; i < 15; ++i) h[(size_t)(30 + i) * p.N] = el.L[i];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) h[(size_t)(45 + i) * p.N] = el.xr[i];
 }
 
 template <typename T>
 PES_DEV void seq_load_el(const KParams<T>& p, int64_t k, SElem<T>& el)
 {
-    T* dst = reinterpret_cast<T*>(&el);
+    const T* h = p.lin + k;
 #pragma unroll
-    for (int i = 0; i < HAND; ++i) dst[i] = p.hand[(size_t)i * p.N + k];
+    for (int i = 0; i < 25; ++i) el.E[i] = h[(size_t)i * p.N];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) el.g[i] = h[(size_t)(25 + i) * p.N];
+#pragma unroll
+    for (int i = 0; i < 15; ++i) el.L[i] = h[(size_t)(30 + i) * p.N];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) el.xr[i] = h[(size_t)(45 + i) * p.N];
 }
 
 // Write the smoothed moments of state k as the next nominal, accumulating the
@@ -91,14 +106,14 @@ __global__ void __launch_bounds__(64) sequential_smoother_kernel(const KParams<T
         seq_damp(p, a, m, P);
         for (int64_t k = a + 1; k < e; ++k) {
             Trans<T> tr;
-            ok &= get_trans<T, LIN>(p, k - 1, k - 1, tr);
+            ok &= get_trans<T, LIN>(p, k - 1, tr);
             T mp[5], FP[25], Pp[15];
             predict(tr, m, P, mp, FP, Pp);
             SElem<T> el;
             ok &= selem_from_prediction(m, P, FP, Pp, mp, el);
             seq_store_el(p, k - 1, el);
             Obs<T> ob;
-            ok &= get_obs<T, LIN>(p, k, k, b, ob);
+            ok &= get_obs<T, LIN>(p, k, b, ob);
             ok &= kf_update(ob, mp, Pp, m, P);
             seq_damp(p, k, m, P);
         }

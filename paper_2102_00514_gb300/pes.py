@@ -238,8 +238,8 @@ class Smoother:
     def sync(self, stream=None):
         return self._check(self.lib.pes_sync(self.h, _stream(stream)))
 
-    PHASES = ["fold", "filter up-sweep", "filter barrier", "filter top level", "filter down-sweep", "filter re-run",
-              "between passes", "smoother up-sweep", "smoother barrier", "smoother top level", "smoother down-sweep",
+    PHASES = ["fold", "filter up-sweep", "filter barrier", "filter top level", "filter down-sweep",
+              "smoother up-sweep", "filter re-run", "smoother barrier", "smoother top level", "smoother down-sweep",
               "RTS re-run", "end barrier"]
 
     def phase_times(self):
