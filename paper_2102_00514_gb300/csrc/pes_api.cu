@@ -608,7 +608,7 @@ static pes_status ieks_run_refined(pes_handle* h, const pes_model* model, pes_me
         PES_CUDA(h, cudaMemsetAsync(h->bar, 0, sizeof(unsigned), st));
         cudaError_t e = launch_refine_scan(rp, true, s.nt, s.nb, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "cooperative launch of the refinement scan");
-        PES_CUDA(h, launch_refine_bwd(rp, st));
+        PES_CUDA(h, launch_refine_bwd(rp, lin, st));
         PES_CUDA(h, cudaMemsetAsync(h->bar, 0, sizeof(unsigned), st));
         e = launch_refine_scan(rp, false, s.nt, s.nb, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "cooperative launch of the refinement scan");

@@ -71,7 +71,7 @@ cudaError_t launch_validate_offsets(const int64_t* offsets, int B, int64_t N, in
 // the correction scan (cooperative: nb blocks of nt threads, nt 128 or 256).
 struct RefineParams;
 cudaError_t launch_refine_fwd(const RefineParams& p, int lin, cudaStream_t st);
-cudaError_t launch_refine_bwd(const RefineParams& p, cudaStream_t st);
+cudaError_t launch_refine_bwd(const RefineParams& p, int lin, cudaStream_t st);
 cudaError_t launch_refine_scan(const RefineParams& p, bool fwd, int nt, int nb, cudaStream_t st);
 // Largest cooperative grid of the correction scan at nt threads (negated CUDA
 // error code on failure).

@@ -38,22 +38,25 @@ PES_DEV void store_elem(const RefineParams& p, int64_t ix, const float* A, const
 #pragma unroll
     for (int c = 0; c < 25; ++c) e[c * p.cs] = A[c];
 #pragma unroll
-    for (int c = 0; c < 5; ++c) e[(25 + c) * p.cs] = w[c];
+    for (int c = 0; c < 5; ++c) e[(25 + c) * p.cs] = s[c];
 #pragma unroll
-    for (int c = 0; c < 5; ++c) e[(30 + c) * p.cs] = s[c];
+    for (int c = 0; c < 15; ++c) e[(30 + c) * p.cs] = r[c];
 #pragma unroll
-    for (int c = 0; c < 15; ++c) e[(35 + c) * p.cs] = r[c];
+    for (int c = 0; c < 5; ++c) e[(45 + c) * p.cs] = w[c];
 }
 
 // The elements are read-only while the correction scan runs: loads through
 // the non-coherent path, which the compiler may move ahead of the scan's
 // stores.
+template <bool W>
 PES_DEV void load_elem(const RefineParams& p, int64_t ix, RElem& el)
 {
     const float* e = p.elem + ix;
     float* d = reinterpret_cast<float*>(&el);
 #pragma unroll
-    for (int c = 0; c < RE; ++c) d[c] = __ldg(e + c * p.cs);
+    for (int c = 0; c < 45; ++c) d[c] = __ldg(e + c * p.cs);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) el.w[c] = W ? __ldg(e + (45 + c) * p.cs) : 0.0f;
 }
 
 // (state, lane) of the thread's slot in the lane-major arrays; false past N.
@@ -80,7 +83,7 @@ constexpr size_t RT_SMEM = sizeof(float) * SCR_N * RT_THREADS;
 // state k + 1 (the Kalman step k -> k+1 from the FP32 filtered moments of k)
 // and, for a trajectory's first state, its own (the prior: A = 0); it also
 // stores the transition out of k for the RTS residuals.
-template <int LIN>
+template <int K>
 __global__ void __launch_bounds__(RT_THREADS) refine_fwd_kernel(const RefineParams p)
 {
     extern __shared__ float scr_raw[];
@@ -114,18 +117,20 @@ __global__ void __launch_bounds__(RT_THREADS) refine_fwd_kernel(const RefinePara
     {
         float xn[5], Pn[15];
         load20(p.nom, p.cs, ix, xn, Pn);
-        if (LIN == LIN_IEKS) {
-            lin_trans_taylor(m, xn, tr);
+        if constexpr (K == KK_IEKS || K == KK_IEKS_ANY) {
+            if constexpr (K == KK_IEKS) ct_trans_taylor(m, xn, tr);
+            else lin_trans_taylor(m, xn, tr);
 #pragma unroll
             for (int c = 0; c < 25; ++c) sc[SCR_F + c] = tr.F[c];
         } else {
             float Lc[25], rdc[5];
             ok &= cub_factor(Pn, Lc, rdc);
-            lin_trans_cubature(m, xn, Lc, rdc, tr);
+            if constexpr (K == KK_CUBATURE) ct_trans_cubature(m, xn, Lc, rdc, tr);
+            else lin_trans_cubature(m, xn, Lc, rdc, tr);
             cub_trans_slope_ff(m, xn, Lc, sc);
         }
     }
-    {
+    if constexpr (K != KK_IEKS) {   // the Taylor slope is formed again instead
         float* t = p.trans + ix;
 #pragma unroll 5
         for (int c = 0; c < 25; ++c) t[c * p.cs] = sc[SCR_F + c];
@@ -142,17 +147,20 @@ __global__ void __launch_bounds__(RT_THREADS) refine_fwd_kernel(const RefinePara
         load20(p.nom, p.cs, ix1, xn, Pn);
         y[0] = __ldg(p.y + ix1);
         y[1] = __ldg(p.y + p.cs + ix1);
-        if (LIN == LIN_IEKS) {
+        if constexpr (K == KK_IEKS) {
+            ct_obs_taylor(m, b, xn, y, ob);
+        } else if constexpr (K == KK_IEKS_ANY) {
             lin_obs_taylor(m, b, xn, y, ob);
         } else {
             float Lc[25], rdc[5];
             ok &= cub_factor(Pn, Lc, rdc);
-            lin_obs_cubature(m, b, xn, Lc, rdc, y, ob);
+            if constexpr (K == KK_CUBATURE) ct_obs_cubature(m, b, xn, Lc, rdc, y, ob);
+            else lin_obs_cubature(m, b, xn, Lc, rdc, y, ob);
         }
     }
     ff mf[5], Pff[15];
     float A[25], w[5];
-    ok &= ff_kalman_step(tr, ob, xf, Pf, mf, Pff, A, w, sc);
+    ok &= ff_kalman_step<kFS<K>>(tr, ob, xf, Pf, mf, Pff, A, w, sc);
     float x1[5], P1[15], sres[5], r[15];
     load_filt(s + 1 < p.L ? filt_slot(p, s + 1, lane) : filt_slot(p, 0, lane + 1), x1, P1);
 #pragma unroll
@@ -165,6 +173,7 @@ __global__ void __launch_bounds__(RT_THREADS) refine_fwd_kernel(const RefinePara
 
 // RTS residual elements, one per state, from the refined filtered moments
 // (FP32 value + the filter's correction) and the FP32 smoothed moments.
+template <int K>
 __global__ void __launch_bounds__(RT_THREADS) refine_bwd_kernel(const RefineParams p)
 {
     extern __shared__ float scr_raw[];
@@ -179,18 +188,23 @@ __global__ void __launch_bounds__(RT_THREADS) refine_bwd_kernel(const RefinePara
     const float* filt = filt_slot(p, s, lane);
     auto filt_ff = [&](int c) { return two_sum(filt[c * 32], p.dlt[c * p.cs + ix]); };
     float* el = p.elem + ix;
-#pragma unroll
-    for (int c = 0; c < 5; ++c) el[(25 + c) * p.cs] = 0.0f;
     if (k + 1 >= next) {
         // last state: smoothed = filtered
 #pragma unroll 5
         for (int c = 0; c < 25; ++c) el[c * p.cs] = 0.0f;
 #pragma unroll
-        for (int c = 0; c < 20; ++c) el[(30 + c) * p.cs] = ff_to_f(ff_add_f(filt_ff(c), -p.xs[c * p.cs + ix]));
+        for (int c = 0; c < 20; ++c) el[(25 + c) * p.cs] = ff_to_f(ff_add_f(filt_ff(c), -p.xs[c * p.cs + ix]));
         return;
     }
     Trans<float> tr;
-    {
+    if constexpr (K == KK_IEKS) {
+        float xn[5];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) xn[c] = p.nom[c * p.cs + ix];
+        ct_trans_taylor(p.model, xn, tr);
+#pragma unroll
+        for (int c = 0; c < 25; ++c) sc[SCR_F + c] = tr.F[c];
+    } else {
         const float* t = p.trans + ix;
 #pragma unroll 5
         for (int c = 0; c < 25; ++c) sc[SCR_F + c] = t[c * p.cs];
@@ -212,17 +226,17 @@ __global__ void __launch_bounds__(RT_THREADS) refine_bwd_kernel(const RefinePara
         for (int c = 0; c < 15; ++c) Pf[c] = filt_ff(5 + c);
         float xs1[5], Ps1[15];
         load20(p.xs, p.cs, ix1, xs1, Ps1);
-        ok = ff_rts_gain(tr, mf, Pf, xs1, Ps1, ms, dP, sc);
+        ok = ff_rts_gain<kFS<K>>(tr, mf, Pf, xs1, Ps1, ms, dP, sc);
     }
 #pragma unroll
-    for (int c = 0; c < 5; ++c) el[(30 + c) * p.cs] = ff_to_f(ff_add_f(ms[c], -p.xs[c * p.cs + ix]));
+    for (int c = 0; c < 5; ++c) el[(25 + c) * p.cs] = ff_to_f(ff_add_f(ms[c], -p.xs[c * p.cs + ix]));
     // covariance residuals, row by row: Pf + G dP G^T - Ps
 #pragma unroll 1
     for (int i = 0; i < 5; ++i) {
         rts_cov_row(i, dP, sc, [&](int j, ff v) {
             const int e = si_rt(i, j);
             const ff Ps = ff_add(filt_ff(5 + e), v);
-            el[(35 + e) * p.cs] = ff_to_f(ff_add_f(Ps, -p.xs[(5 + e) * p.cs + ix]));
+            el[(30 + e) * p.cs] = ff_to_f(ff_add_f(Ps, -p.xs[(5 + e) * p.cs + ix]));
         });
     }
     // G_ij = (G^T)_ji
@@ -301,20 +315,21 @@ __global__ void __launch_bounds__(NT, 1) refine_scan_kernel(const RefineParams p
     const int lane = blockIdx.x * NT + t;
     const int64_t a = min((int64_t)lane * p.L, p.N);
     const int64_t e = min(a + (int64_t)p.L, p.N);
-    // level 1: the chunk's composition (each new element applies after the
-    // ones already composed: forward from the chunk's first state, backward
-    // from its last)
+    // level 1: the chunk's composition, from the state that the re-run comes to
+    // last: what was read last, the first states of the re-run, is then still in
+    // the L2 cache when it starts (the elements, 200 bytes per state, pass it once
+    // per pass otherwise)
     {
         RElem acc, ek, en;
         relem_identity(acc);
         const int n = (int)(e - a);
-        if (n > 0) load_elem(p, (FWD ? 0 : n - 1) * (int64_t)p.NL + lane, en);
+        if (n > 0) load_elem<FWD>(p, (FWD ? n - 1 : 0) * (int64_t)p.NL + lane, en);
 #pragma unroll 1
         for (int q = 0; q < n; ++q) {
             ek = en;
-            const int sn = FWD ? q + 1 : n - 2 - q;   // the next state's step within the chunk
-            if (q + 1 < n) load_elem(p, sn * (int64_t)p.NL + lane, en);
-            relem_compose<W>(ek, acc, acc);
+            const int sn = FWD ? n - 2 - q : q + 1;   // the next state's step within the chunk
+            if (q + 1 < n) load_elem<FWD>(p, sn * (int64_t)p.NL + lane, en);
+            relem_compose<W>(acc, ek, acc);
         }
         el[t] = acc;
     }
@@ -410,7 +425,7 @@ __global__ void __launch_bounds__(NT, 1) refine_scan_kernel(const RefineParams p
         float xn[20], xc[20];
         auto slot = [&](int q) { return (int64_t)(FWD ? q : n - 1 - q) * p.NL + lane; };
         if (n > 0) {
-            load_elem(p, slot(0), en);
+            load_elem<FWD>(p, slot(0), en);
             if (!FWD)
 #pragma unroll
                 for (int c = 0; c < 20; ++c) xn[c] = p.xs[c * p.cs + slot(0)];
@@ -424,7 +439,7 @@ __global__ void __launch_bounds__(NT, 1) refine_scan_kernel(const RefineParams p
 #pragma unroll
                 for (int c = 0; c < 20; ++c) xc[c] = xn[c];
             if (q + 1 < n) {
-                load_elem(p, slot(q + 1), en);
+                load_elem<FWD>(p, slot(q + 1), en);
                 if (!FWD)
 #pragma unroll
                     for (int c = 0; c < 20; ++c) xn[c] = p.xs[c * p.cs + slot(q + 1)];
@@ -452,23 +467,29 @@ __global__ void __launch_bounds__(NT, 1) refine_scan_kernel(const RefineParams p
 
 // ---- launchers -----------------------------------------------------------------
 
-cudaError_t launch_refine_fwd(const RefineParams& p, int lin, cudaStream_t st)
+namespace {
+cudaError_t launch_residuals(void (*kern)(RefineParams), const RefineParams& p, cudaStream_t st)
 {
     const unsigned blocks = (unsigned)((p.cs + RT_THREADS - 1) / RT_THREADS);
-    auto kern = lin == LIN_IEKS ? refine_fwd_kernel<LIN_IEKS> : refine_fwd_kernel<LIN_CUBATURE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RT_SMEM);
     if (e != cudaSuccess) return e;
     kern<<<blocks, RT_THREADS, RT_SMEM, st>>>(p);
     return cudaGetLastError();
 }
+}  // namespace
 
-cudaError_t launch_refine_bwd(const RefineParams& p, cudaStream_t st)
+cudaError_t launch_refine_fwd(const RefineParams& p, int lin, cudaStream_t st)
 {
-    const unsigned blocks = (unsigned)((p.cs + RT_THREADS - 1) / RT_THREADS);
-    cudaError_t e = cudaFuncSetAttribute(refine_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RT_SMEM);
-    if (e != cudaSuccess) return e;
-    refine_bwd_kernel<<<blocks, RT_THREADS, RT_SMEM, st>>>(p);
-    return cudaGetLastError();
+    const bool ct = p.model.kind == MODEL_CT_BEARINGS;
+    if (lin == LIN_IEKS) return launch_residuals(ct ? refine_fwd_kernel<KK_IEKS> : refine_fwd_kernel<KK_IEKS_ANY>, p, st);
+    return launch_residuals(ct ? refine_fwd_kernel<KK_CUBATURE> : refine_fwd_kernel<KK_CUBATURE_ANY>, p, st);
+}
+
+cudaError_t launch_refine_bwd(const RefineParams& p, int lin, cudaStream_t st)
+{
+    const bool ct = p.model.kind == MODEL_CT_BEARINGS;
+    if (lin == LIN_IEKS) return launch_residuals(ct ? refine_bwd_kernel<KK_IEKS> : refine_bwd_kernel<KK_IEKS_ANY>, p, st);
+    return launch_residuals(ct ? refine_bwd_kernel<KK_CUBATURE> : refine_bwd_kernel<KK_CUBATURE_ANY>, p, st);
 }
 
 namespace {

@@ -41,8 +41,8 @@
 
 namespace pes {
 
-constexpr int RE = 50;   // correction element: Abar (or G) 25, w 5, s 5, r 15
-constexpr int RT = 45;   // stored transition: F 25, fx 5, Q' 15
+constexpr int RE = 50;   // correction element: Abar (or G) 25, s 5, r 15, w 5 (forward only)
+constexpr int RT = 45;   // stored transition (a linearisation that is not repeated): F 25, fx 5, Q' 15
 constexpr int RD = 20;   // correction of one state: means 5, covariance 15
 
 struct RefineParams {
@@ -69,9 +69,9 @@ struct RefineParams {
 
 struct RElem {
     float A[25];
-    float w[5];
     float s[5];
     float r[15];
+    float w[5];
 };
 
 struct RState {
@@ -210,31 +210,49 @@ PES_DEV void cub_trans_slope_ff(const DevModel<float>& m, const float* xbar, con
 }
 
 // ---- residuals ---------------------------------------------------------------------
+//
+// FS is the structure of F (pes_model.cuh): with the model known, the entries
+// that are 0 or 1 are left out, which is 1,900 of the forward step's 4,300 FP32
+// instructions per state and 1,500 of the RTS step's 7,700 (Taylor slope). The
+// loops over rows stay rolled (below).
 
-// One Kalman step in float-float from the FP32 filtered moments (m, P) of
-// state k, through the transition (k -> k+1: F in the scratch at SCR_F, fx,
-// Q', xn of tr) and the observation ob of state k+1: the step's
-// exact-arithmetic image (mf, Pf), to about 1e-14 relative of the operands,
-// and its derivatives Abar = (I - K H) F, w = F^T H^T S^{-1} v in FP32.
-// Returns false if S is not positive definite.
-template <int NT>
-PES_DEV bool ff_kalman_step(const Trans<float>& tr, const Obs<float>& ob, const float* m, const float* P, ff* mf,
-                            ff* Pf, float* Abar, float* w, Scratch<NT> sc)
+// a += x for a value that needs no product: float or float-float
+PES_DEV void acc_plus(ffacc& a, float x)
 {
+    const ff t = two_sum(a.s, x);
+    a.s = t.hi;
+    a.c = __fadd_rn(a.c, t.lo);
+}
+PES_DEV void acc_plus(ffacc& a, ff x) { acc_add(a, x); }
+PES_DEV ff ff_of(float x) { return ff_make(x); }
+PES_DEV ff ff_of(ff x) { return x; }
+
+// F P into the scratch (SCR_M), and F P F^T (upper triangle) into SCR_S, for a
+// symmetric packed P of floats or float-floats.
+template <int FS, int NT, typename V>
+PES_DEV void ff_predict_cov(const V* P, Scratch<NT> sc)
+{
+    constexpr int ROWS = FS == FS_DENSE ? 5 : 4, L0 = FS == FS_CT ? 2 : 0;
     // F P by rows
 #pragma unroll 1
-    for (int i = 0; i < 5; ++i) {
+    for (int i = 0; i < ROWS; ++i) {
         float Fi[5];
 #pragma unroll
-        for (int l = 0; l < 5; ++l) Fi[l] = sc[SCR_F + i * 5 + l];
+        for (int l = L0; l < 5; ++l) Fi[l] = sc[SCR_F + i * 5 + l];
 #pragma unroll
         for (int j = 0; j < 5; ++j) {
-            ffacc acc = acc_of(two_prod(Fi[0], P[si(0, j)]));
+            ffacc acc{0.0f, 0.0f};
+            if (FS == FS_CT) {   // rows 0 and 1 add P's own
+                if (i < 2) acc = acc_of(ff_of(i == 0 ? P[si(0, j)] : P[si(1, j)]));
+            }
 #pragma unroll
-            for (int l = 1; l < 5; ++l) acc_add(acc, Fi[l], P[si(l, j)]);
+            for (int l = L0; l < 5; ++l) acc_add(acc, P[si(l, j)], Fi[l]);
             sc.st(SCR_M + 2 * (i * 5 + j), acc_done(acc));
         }
     }
+    if (ROWS == 4)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) sc.st(SCR_M + 2 * (20 + j), ff_of(P[si(4, j)]));
     // (F P) F^T, upper triangle by rows
 #pragma unroll 1
     for (int i = 0; i < 5; ++i) {
@@ -242,25 +260,57 @@ PES_DEV bool ff_kalman_step(const Trans<float>& tr, const Obs<float>& ob, const 
 #pragma unroll
         for (int l = 0; l < 5; ++l) FPi[l] = sc.ld(SCR_M + 2 * (i * 5 + l));
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
+        for (int j = 0; j < ROWS; ++j) {
             if (j < i) continue;
-            ffacc acc = acc_of(ff_mul_f(FPi[0], sc[SCR_F + j * 5]));
+            ffacc acc{0.0f, 0.0f};
+            if (FS == FS_CT && j < 2) acc = acc_of(FPi[j]);
 #pragma unroll
-            for (int l = 1; l < 5; ++l) acc_add(acc, FPi[l], sc[SCR_F + j * 5 + l]);
+            for (int l = L0; l < 5; ++l) acc_add(acc, FPi[l], sc[SCR_F + j * 5 + l]);
             sc.st(SCR_S + 2 * si_rt(i, j), acc_done(acc));
         }
+        if (ROWS == 4) sc.st(SCR_S + 2 * si_rt(i, 4), FPi[4]);
     }
+}
+
+// fx + F d for a float-float d, row i by row.
+template <int FS, int NT>
+PES_DEV void ff_predict_mean(const float* fx, const ff* d, Scratch<NT> sc, ff* mp)
+{
+    constexpr int ROWS = FS == FS_DENSE ? 5 : 4, L0 = FS == FS_CT ? 2 : 0;
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        ffacc acc = acc_of_f(fx[i]);
+        if (FS == FS_CT && i < 2) acc_add(acc, d[i]);
+#pragma unroll
+        for (int l = L0; l < 5; ++l) acc_add(acc, d[l], sc[SCR_F + i * 5 + l]);
+        mp[i] = acc_done(acc);
+    }
+    if (ROWS == 4) {
+        ffacc acc = acc_of_f(fx[4]);
+        acc_add(acc, d[4]);
+        mp[4] = acc_done(acc);
+    }
+}
+
+// One Kalman step in float-float from the FP32 filtered moments (m, P) of
+// state k, through the transition (k -> k+1: F in the scratch at SCR_F, fx,
+// Q', xn of tr) and the observation ob of state k+1: the step's
+// exact-arithmetic image (mf, Pf), to about 1e-14 relative of the operands,
+// and its derivatives Abar = (I - K H) F, w = F^T H^T S^{-1} v in FP32.
+// Returns false if S is not positive definite.
+template <int FS, int NT>
+PES_DEV bool ff_kalman_step(const Trans<float>& tr, const Obs<float>& ob, const float* m, const float* P, ff* mf,
+                            ff* Pf, float* Abar, float* w, Scratch<NT> sc)
+{
+    constexpr int HC = kHCols<FS>;
+    ff_predict_cov<FS>(P, sc);
     ff Pp[15];
 #pragma unroll
     for (int i = 0; i < 15; ++i) Pp[i] = ff_add_f(sc.ld(SCR_S + 2 * i), tr.Q[i]);
-    ff mp[5];
+    ff d[5], mp[5];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        ffacc acc = acc_of_f(tr.fx[i]);
-#pragma unroll
-        for (int l = 0; l < 5; ++l) acc_add(acc, ff_diff_f(m[l], tr.xn[l]), sc[SCR_F + i * 5 + l]);
-        mp[i] = acc_done(acc);
-    }
+    for (int l = 0; l < 5; ++l) d[l] = ff_diff_f(m[l], tr.xn[l]);
+    ff_predict_mean<FS>(tr.fx, d, sc, mp);
     ff HP[10];
 #pragma unroll
     for (int r = 0; r < 2; ++r)
@@ -268,7 +318,7 @@ PES_DEV bool ff_kalman_step(const Trans<float>& tr, const Obs<float>& ob, const 
         for (int j = 0; j < 5; ++j) {
             ffacc acc = acc_of(ff_mul_f(Pp[si(0, j)], ob.H[r * 5]));
 #pragma unroll
-            for (int l = 1; l < 5; ++l) acc_add(acc, Pp[si(l, j)], ob.H[r * 5 + l]);
+            for (int l = 1; l < HC; ++l) acc_add(acc, Pp[si(l, j)], ob.H[r * 5 + l]);
             HP[r * 5 + j] = acc_done(acc);
         }
     ff S[3];
@@ -278,7 +328,7 @@ PES_DEV bool ff_kalman_step(const Trans<float>& tr, const Obs<float>& ob, const 
         for (int q = r; q < 2; ++q) {
             ffacc acc = acc_of_f(ob.R[si2(r, q)]);
 #pragma unroll
-            for (int l = 0; l < 5; ++l) acc_add(acc, HP[r * 5 + l], ob.H[q * 5 + l]);
+            for (int l = 0; l < HC; ++l) acc_add(acc, HP[r * 5 + l], ob.H[q * 5 + l]);
             S[si2(r, q)] = acc_done(acc);
         }
     const ff det = ff_sub(ff_mul(S[0], S[2]), ff_mul(S[1], S[1]));
@@ -296,7 +346,7 @@ PES_DEV bool ff_kalman_step(const Trans<float>& tr, const Obs<float>& ob, const 
     for (int r = 0; r < 2; ++r) {
         ffacc acc = acc_of_f(ob.r[r]);
 #pragma unroll
-        for (int l = 0; l < 5; ++l) acc_add(acc, ff_add_f(mp[l], -ob.xn[l]), -ob.H[r * 5 + l]);
+        for (int l = 0; l < HC; ++l) acc_add(acc, ff_add_f(mp[l], -ob.xn[l]), -ob.H[r * 5 + l]);
         v[r] = acc_done(acc);
     }
 #pragma unroll
@@ -315,28 +365,28 @@ PES_DEV bool ff_kalman_step(const Trans<float>& tr, const Obs<float>& ob, const 
             acc_add(acc, ff_neg(KT[5 + i]), HP[5 + j]);
             Pf[si(i, j)] = acc_done(acc);
         }
-    // derivatives, FP32
+    // derivatives, FP32: Abar = F - K (H F), w = (H F)^T S^{-1} v
+    float F[25], HF[10];
+#pragma unroll
+    for (int i = 0; i < 25; ++i) F[i] = f_entry<FS>(i / 5, i % 5) == 2 ? sc[SCR_F + i] : (f_entry<FS>(i / 5, i % 5) ? 1.0f : 0.0f);
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            float t = ob.H[r * 5] * F[j];
+#pragma unroll
+            for (int l = 1; l < HC; ++l) t = fmaf(ob.H[r * 5 + l], F[l * 5 + j], t);
+            HF[r * 5 + j] = t;
+        }
 #pragma unroll
     for (int i = 0; i < 5; ++i)
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            float t = 0.0f;
-#pragma unroll
-            for (int l = 0; l < 5; ++l) {
-                const float ikh = (i == l ? 1.0f : 0.0f) - KT[i].hi * ob.H[l] - KT[5 + i].hi * ob.H[5 + l];
-                t = fmaf(ikh, sc[SCR_F + l * 5 + j], t);
-            }
-            Abar[i * 5 + j] = t;
-        }
+        for (int j = 0; j < 5; ++j)
+            Abar[i * 5 + j] = fmaf(-KT[5 + i].hi, HF[5 + j], fmaf(-KT[i].hi, HF[j], F[i * 5 + j]));
     const float Siv0 = Si[0].hi * v[0].hi + Si[1].hi * v[1].hi;
     const float Siv1 = Si[1].hi * v[0].hi + Si[2].hi * v[1].hi;
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        float t = 0.0f;
-#pragma unroll
-        for (int l = 0; l < 5; ++l) t = fmaf(sc[SCR_F + l * 5 + i], ob.H[l] * Siv0 + ob.H[5 + l] * Siv1, t);
-        w[i] = t;
-    }
+    for (int i = 0; i < 5; ++i) w[i] = fmaf(HF[i], Siv0, HF[5 + i] * Siv1);
     return ok;
 }
 
@@ -347,39 +397,11 @@ PES_DEV bool ff_kalman_step(const Trans<float>& tr, const Obs<float>& ob, const 
 // returns the smoothed mean ms and dP = Ps1 - (F Pf F^T + Q'); the covariance
 // rows Pf + G dP G^T are formed by rts_cov_row.
 // Returns false if the predicted covariance is not positive definite.
-template <int NT>
+template <int FS, int NT>
 PES_DEV bool ff_rts_gain(const Trans<float>& tr, const ff* mf, const ff* Pf, const float* xs1, const float* Ps1,
                          ff* ms, ff* dP, Scratch<NT> sc)
 {
-    // F Pf by rows
-#pragma unroll 1
-    for (int i = 0; i < 5; ++i) {
-        float Fi[5];
-#pragma unroll
-        for (int l = 0; l < 5; ++l) Fi[l] = sc[SCR_F + i * 5 + l];
-#pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            ffacc acc = acc_of(ff_mul_f(Pf[si(0, j)], Fi[0]));
-#pragma unroll
-            for (int l = 1; l < 5; ++l) acc_add(acc, Pf[si(l, j)], Fi[l]);
-            sc.st(SCR_M + 2 * (i * 5 + j), acc_done(acc));
-        }
-    }
-    // (F Pf) F^T, upper triangle by rows
-#pragma unroll 1
-    for (int i = 0; i < 5; ++i) {
-        ff FPi[5];
-#pragma unroll
-        for (int l = 0; l < 5; ++l) FPi[l] = sc.ld(SCR_M + 2 * (i * 5 + l));
-#pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            if (j < i) continue;
-            ffacc acc = acc_of(ff_mul_f(FPi[0], sc[SCR_F + j * 5]));
-#pragma unroll
-            for (int l = 1; l < 5; ++l) acc_add(acc, FPi[l], sc[SCR_F + j * 5 + l]);
-            sc.st(SCR_S + 2 * si_rt(i, j), acc_done(acc));
-        }
-    }
+    ff_predict_cov<FS>(Pf, sc);
     ff Pp[15];
 #pragma unroll
     for (int i = 0; i < 15; ++i) Pp[i] = ff_add_f(sc.ld(SCR_S + 2 * i), tr.Q[i]);
@@ -426,14 +448,12 @@ PES_DEV bool ff_rts_gain(const Trans<float>& tr, const ff* mf, const ff* Pf, con
         for (int i = 0; i < 5; ++i) sc.st(SCR_M + 2 * (i * 5 + c), x[i]);
     }
     // ms = mf + G (xs1 - mp), mp = fx + F (mf - xn)
-    ff e[5];
+    ff e[5], d[5];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        ffacc acc = acc_of_f(tr.fx[i]);
+    for (int l = 0; l < 5; ++l) d[l] = ff_add_f(mf[l], -tr.xn[l]);
+    ff_predict_mean<FS>(tr.fx, d, sc, e);
 #pragma unroll
-        for (int l = 0; l < 5; ++l) acc_add(acc, ff_add_f(mf[l], -tr.xn[l]), sc[SCR_F + i * 5 + l]);
-        e[i] = ff_add_f(ff_neg(acc_done(acc)), xs1[i]);
-    }
+    for (int i = 0; i < 5; ++i) e[i] = ff_add_f(ff_neg(e[i]), xs1[i]);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
         ffacc acc = acc_of(mf[i]);
