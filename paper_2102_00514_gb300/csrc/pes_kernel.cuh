@@ -28,6 +28,14 @@
 // other blocks' (measured at T = 2^20, FP32: see pes_persistent_kernel). The RTS
 // pass then builds each step's element from the kept filtered moments.
 //
+// Within a chunk means are kept as deviations from the nominal (the filter's, the
+// fold's and the smoother's), re-referenced from state to state by the difference
+// of their nominals, and the trees' elements carry reference points: positions of
+// tens to thousands of units would otherwise be rounded at every step and level,
+// and the rounding of the means is what the next iteration's linearisation
+// amplifies (batch of 1,024 trajectories after three FP32 iterations, against 64
+// bits: means 6.0e-7 -> 1.5e-7, covariances 7e-6 -> 2.5e-6).
+//
 // A chunk's passes read only its own states' nominal, so no barrier separates
 // iterations: the block aggregates are double-buffered, and a block can reach
 // the aggregates of iteration i + 2 only after every block has passed the first
@@ -64,7 +72,7 @@ template <int K>
 constexpr bool kStoreLin = kSigma<kLinOf<K>>;
 // Scalars stored per state; the transition's are kLinTrans of them, from
 // kLinTransAt. Compact form (the coordinated turn's cubature regression): F rows
-// 0-3 (20), fx (4), Q' (10), H (4), r (2), R' (3); the nominal is read from the
+// 0-3 (20), fx (4; less xn), Q' (10), H (4), r (2), R' (3); the nominal is read from the
 // trajectory, the rest is constant. Dense form: H (10), r (2), R' (3), xn (5),
 // F (25), fx (5), Q' (15).
 template <int K>
@@ -341,14 +349,18 @@ PES_DEV bool get_obs(const KParams<T>& p, int64_t ix, int b, Obs<T>& ob)
     return ok;
 }
 
-// The linearisation of a compiled form of the smoother.
+// The linearisation of a compiled form of the smoother; fx is f(xn) - xn.
 template <int K, typename T>
 PES_DEV void form_trans(const KParams<T>& p, const StateIn<T, kLinOf<K>>& s, const Factor<T, kLinOf<K>>& f,
                         Trans<T>& tr)
 {
     if constexpr (K == KK_IEKS) ct_trans_taylor(p.model, s.x, tr);
     else if constexpr (K == KK_CUBATURE) ct_trans_cubature(p.model, s.x, f.L, f.rd, tr);
-    else lin_trans<T, kLinOf<K>>(p, s, f, tr);
+    else {
+        lin_trans<T, kLinOf<K>>(p, s, f, tr);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) tr.fx[i] -= tr.xn[i];
+    }
 }
 
 template <int K, typename T>
@@ -431,8 +443,8 @@ PES_DEV const T* lin_warp(const KParams<T>& p, int s, int lane)
 // memory: NS components of a state, consecutive rows of the per-state arrays from
 // `src` on. For the sigma-point folds, whose register pressure rules out a
 // register prefetch (nominal mean and covariance, measurement). Each thread
-// copies its own scalars with cp.async and reads only its own stages back, so no block synchronisation is involved. Element c of
-// stage i sits at base[(i * NS + c) * stride] (thread-contiguous columns).
+// copies its own scalars with cp.async and reads only its own stages back, so no
+// block synchronisation is involved. Element c of stage i sits at base[(i * NS + c) * stride] (thread-contiguous columns).
 template <typename T, int NS>
 struct Prefetch {
     T* base;
@@ -517,20 +529,22 @@ PES_DEV void load_array_trans(const KParams<T>& p, int lane, Trans<T>& tr)
 }
 
 // acc <- acc (x) the Levenberg-Marquardt pseudo-measurement of a state's nominal
-// xb. Out of line: a damped run pays for the call, the others keep the
+// (the zero deviation). Out of line: a damped run pays for the call, the others keep the
 // operator's code and registers out of their loops.
 template <typename T>
-__device__ __noinline__ void damp_element(FElem<T>& acc, const T* xb, T lambda)
+__device__ __noinline__ void damp_element(FElem<T>& acc, T lambda)
 {
     FElem<T> dmp;
+    const T xb[5] = {T(0), T(0), T(0), T(0), T(0)};
     felem_damping(dmp, xb, lambda);
     combine_filter(acc, dmp, acc);
 }
 
 template <typename T>
-__device__ __noinline__ void damp_gauss(Gauss<T>& g, const T* xb, T lambda)
+__device__ __noinline__ void damp_gauss(Gauss<T>& g, T lambda)
 {
     FElem<T> dmp;
+    const T xb[5] = {T(0), T(0), T(0), T(0), T(0)};
     felem_damping(dmp, xb, lambda);
     apply_filter(g, dmp, g);
 }
@@ -559,61 +573,74 @@ PES_DEV bool fold_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int la
     // the next state's inputs are loaded a step ahead: into registers for
     // the Taylor linearisation; for the sigma-point ones, whose register
     // pressure makes a register prefetch cost more in spills than it hides,
-    // into shared memory
+    // into shared memory, three stages: the state before is still needed
+    int st = 0;
     constexpr bool prefetch = !kSigma<LIN>;
     if (prefetch) {
         load_state(p, ix, sc);
-        felem_identity(acc, sc.x);
     } else {
         pf.issue(ix, 0);
         pf.commit();
     }
 #pragma unroll 1
-    for (int64_t k = a; k < e; ++k, ix += dix) {
+    for (int64_t k = a;; ++k, ix += dix) {
         cur.forward(k);
         const int s = (int)(k - a);
         if (prefetch) {
             if (k + 1 < e) load_state(p, ix + dix, sn);
         } else {
-            if (k + 1 < e) pf.issue(ix + dix, (s + 1) & 1);
+            if (k + 1 < e) pf.issue(ix + dix, st == 2 ? 0 : st + 1);
             pf.commit();
             pf.wait_prev();
 #pragma unroll
-            for (int i = 0; i < 5; ++i) sc.x[i] = pf.get(s & 1, i);
+            for (int i = 0; i < 5; ++i) sc.x[i] = pf.get(st, i);
 #pragma unroll
-            for (int i = 0; i < 15; ++i) sc.P[i] = pf.get(s & 1, 5 + i);
-            sc.y[0] = pf.get(s & 1, 20);
-            sc.y[1] = pf.get(s & 1, 21);
-            if (s == 0) felem_identity(acc, sc.x);   // the input is measured from the nominal of a
+            for (int i = 0; i < 15; ++i) sc.P[i] = pf.get(st, 5 + i);
+            sc.y[0] = pf.get(st, 20);
+            sc.y[1] = pf.get(st, 21);
+        }
+        if (!prefetch && s > 0) {
+#pragma unroll
+            for (int i = 0; i < 5; ++i) acc.b[i] += pf.get(st == 0 ? 2 : st - 1, i) - sc.x[i];
         }
         Factor<T, LIN> fc;
         ok &= factor_state(sc, fc);
         if (cur.is_head(k)) {
             T m0[5], P0[15];
             load_prior(p, cur.b, m0, P0);
+#pragma unroll
+            for (int i = 0; i < 5; ++i) m0[i] -= sc.x[i];
             felem_apply_prior(acc, m0, P0);
         } else {
             Obs<T> ob;
             form_obs<K>(p, cur.b, sc, fc, ob);
             if (store_lin) store_lin_obs<K>(p, s, lane, ob);
-            ok &= fold_update<FS>(acc, ob);
+            ok &= fold_update<FS, true>(acc, ob);
         }
         if (lm_of(p.model, cur.b) > T(0)) {
             FElem<T> tmp = acc;
-            T xb[5];
-#pragma unroll
-            for (int i = 0; i < 5; ++i) xb[i] = sc.x[i];
-            damp_element(tmp, xb, lm_of(p.model, cur.b));
+            damp_element(tmp, lm_of(p.model, cur.b));
             acc = tmp;
         }
         if (!cur.is_tail(k)) {
             Trans<T> tr;
             form_trans<K>(p, sc, fc, tr);
             if (store_lin) store_lin_trans<K>(p, s, lane, tr);
-            fold_predict<FS>(acc, tr);
+            fold_predict<FS, true>(acc, tr);
         }
-        if (prefetch) sc = sn;
+        if (k + 1 == e) break;
+        // from the next state's nominal on
+        if (prefetch) {
+#pragma unroll
+            for (int i = 0; i < 5; ++i) acc.b[i] += sc.x[i] - sn.x[i];
+            sc = sn;
+        }
+        st = st == 2 ? 0 : st + 1;
     }
+    // the reference points: of the output the last nominal, of the input the first
+    // (read again, which takes the loop fewer registers than keeping it)
+    felem_set_ref(acc, sc.x);
+    load_nominal(p, lane, acc.xr);
     if (!prefetch) pf.wait_all();
     return ok;
 }
@@ -682,7 +709,7 @@ PES_DEV void store_filtered(const KParams<T>& p, int64_t ix, const T* m, const T
     for (int i = 0; i < 15; ++i) p.Pf[i * p.cs + ix] = P[i];
 }
 
-// MODE_RUN: the filtered moments (x*, P*) of state a + s of a lane, kept
+// MODE_RUN: the filtered moments (x* less the nominal, P*) of state a + s of a lane, kept
 // between the filtering re-run and the RTS pass, which builds the smoothing
 // element from them (20 scalars per state; handing over finished elements, 50
 // scalars, cost more in traffic than the element's prediction does in
@@ -735,7 +762,7 @@ PES_DEV void trans_from_stage(const KParams<T>& p, const S& ws, int i, int off, 
         for (int c = 0; c < 20; ++c) tr.F[c] = ws.get(i, off + c);
 #pragma unroll
         for (int c = 0; c < 4; ++c) tr.fx[c] = ws.get(i, off + 20 + c);
-        tr.fx[4] = xn[4];
+        tr.fx[4] = T(0);
 #pragma unroll
         for (int c = 0; c < 15; ++c) tr.Q[c] = p.model.Q[c];
 #pragma unroll
@@ -776,10 +803,11 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
     const int64_t dix = p.NL;
     int64_t ix = lane;
     StateIn<T, LIN> sc, sn;   // inputs of states k, k+1 (when linearising here)
-    constexpr bool want_x = K == KK_CUBATURE;   // the stored form leaves the nominal out
-    T xc[5], xn[5];
-    if (!use_lin && any) load_state(p, ix, sc);
-    if (want_x && any) load_nominal(p, ix, xc);
+    T xc[5], xn[5];   // nominals of states k, k+1
+    if (any) {
+        if (use_lin) load_nominal(p, ix, xc);
+        else load_state(p, ix, sc);
+    }
     WarpStream<T, kLinScalars<K>, ST> ws;
     if (use_lin) {
         ws.init(wstage, wbar, wpar);
@@ -795,31 +823,40 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
         if (k < e) {
             cur.forward(k);
             if (!use_lin && k + 1 < e) load_state(p, ix + dix, sn);
-            if (want_x && k + 1 < e) load_nominal(p, ix + dix, xn);
+            if (use_lin && k + 1 < e) load_nominal(p, ix + dix, xn);
             Factor<T, LIN> fc;
             if (!use_lin) ok &= factor_state(sc, fc);
+            if (!use_lin)
+#pragma unroll
+                for (int i = 0; i < 5; ++i) {
+                    xc[i] = sc.x[i];
+                    xn[i] = sn.x[i];
+                }
+            if (s == 0)
+#pragma unroll
+                for (int i = 0; i < 5; ++i) m[i] += G.r[i] - xc[i];
             if (cur.is_head(k)) {
                 load_prior(p, cur.b, m, P);
+#pragma unroll
+                for (int i = 0; i < 5; ++i) m[i] -= xc[i];
             } else {
                 Obs<T> ob;
                 if constexpr (use_lin) obs_from_stage<K>(ws, st, xc, ob);
                 else form_obs<K>(p, cur.b, sc, fc, ob);
                 T mn[5], Pn[15];
-                ok &= kf_update<FS>(ob, m, P, mn, Pn);
+                ok &= kf_update<FS, true>(ob, m, P, mn, Pn);
 #pragma unroll
                 for (int i = 0; i < 5; ++i) m[i] = mn[i];
 #pragma unroll
                 for (int i = 0; i < 15; ++i) P[i] = Pn[i];
             }
             if (lm_of(p.model, cur.b) > T(0)) {
-                T xb[5];
-                load_nominal(p, ix, xb);
                 Gauss<T> g;
 #pragma unroll
                 for (int i = 0; i < 5; ++i) g.m[i] = m[i];
 #pragma unroll
                 for (int i = 0; i < 15; ++i) g.P[i] = P[i];
-                damp_gauss(g, xb, lm_of(p.model, cur.b));
+                damp_gauss(g, lm_of(p.model, cur.b));
 #pragma unroll
                 for (int i = 0; i < 5; ++i) m[i] = g.m[i];
 #pragma unroll
@@ -831,16 +868,15 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
                 if constexpr (use_lin) trans_from_stage<K>(p, ws, st, 0, xc, tr);
                 else form_trans<K>(p, sc, fc, tr);
                 T mp[5], FP[25], Pp[15];
-                predict<FS>(tr, m, P, mp, FP, Pp);
+                predict<FS, true>(tr, m, P, mp, FP, Pp);
 #pragma unroll
-                for (int i = 0; i < 5; ++i) m[i] = mp[i];
+                for (int i = 0; i < 5; ++i) m[i] = mp[i] + (xc[i] - xn[i]);   // from the next nominal on
 #pragma unroll
                 for (int i = 0; i < 15; ++i) P[i] = Pp[i];
             }
             if (!use_lin) sc = sn;
-            if (want_x)
 #pragma unroll
-                for (int i = 0; i < 5; ++i) xc[i] = xn[i];
+            for (int i = 0; i < 5; ++i) xc[i] = xn[i];
         }
         if (use_lin) {
             __syncwarp();   // every lane is done with the stage: refill it
@@ -863,7 +899,7 @@ PES_DEV bool rerun_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int 
     if (a < e) cur.init(p.offsets, p.B, a);
     T m[5], P[15];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) m[i] = G.m[i];
+    for (int i = 0; i < 5; ++i) m[i] = G.m[i] + G.r[i];
 #pragma unroll
     for (int i = 0; i < 15; ++i) P[i] = G.P[i];
     FilterStream<T> ws;
@@ -917,9 +953,10 @@ PES_DEV bool rerun_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int 
 // The smoothing element of a lane's whole chunk [a, e), from the state at e to
 // the state at a: Eq. 17 for the chunk as one transition. G is the predicted
 // Gaussian at a, f the chunk's filtering element. Conditioned on the chunk's
-// measurements, x_a ~ N(m + D (eta - J (m - xr)), D) with D = (P^{-1} + J)^{-1},
-// and x_e given x_a is (A, b, C). A trajectory that ends within the chunk cuts
-// the element (E = 0); the state before a trajectory's first one ignores it.
+// measurements, x_a - xr ~ N(d + D (eta - J d), D) with D = (P^{-1} + J)^{-1} and d
+// the Gaussian's mean less xr, and x_e given x_a is (A, b, C). A trajectory that
+// ends within the chunk cuts the element (E = 0); the state before a trajectory's
+// first one ignores it.
 template <typename T>
 PES_DEV bool chunk_selem(const KParams<T>& p, int64_t a, int64_t e, const FElem<T>& f, const Gauss<T>& G,
                          SElem<T>& el)
@@ -935,24 +972,24 @@ PES_DEV bool chunk_selem(const KParams<T>& p, int64_t a, int64_t e, const FElem<
         selem_last(el, z, z);
         return true;
     }
-    T D[15], dm[5], u[5], Du[5], md[5];
+    T D[15], dm[5], u[5], Du[5], md[5], ref[5];
     info_update_cov(G.P, f.J, D);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) dm[i] = G.m[i] - f.xr[i];
+    for (int i = 0; i < 5; ++i) dm[i] = G.m[i] + (G.r[i] - f.xr[i]);
     sv(f.J, dm, u);
 #pragma unroll
     for (int i = 0; i < 5; ++i) u[i] = f.eta[i] - u[i];
     sv(D, u, Du);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) md[i] = G.m[i] + Du[i];
+    for (int i = 0; i < 5; ++i) md[i] = dm[i] + Du[i];
+    felem_ref(f, ref);
+    selem_set_refs(el, ref, f.xr);
     if (cur.next <= e) {
         selem_last(el, md, D);
         return true;
     }
     T mp[5], AD[25], Pp[15];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) dm[i] += Du[i];
-    mv(f.A, dm, mp);
+    mv(f.A, md, mp);
 #pragma unroll
     for (int i = 0; i < 5; ++i) mp[i] += f.b[i];
     m_s(f.A, D, AD);
@@ -1020,6 +1057,8 @@ PES_DEV bool rts_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, con
     SegCursor cur;
     if (a < e) cur.init(p.offsets, p.B, e - 1);
     Gauss<T> s = G;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) s.m[i] += G.r[i];
     SmoothStream<T> ws;
     ws.init(wstage, wbar, wpar);
 #pragma unroll
@@ -1083,10 +1122,13 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
 #pragma unroll
     for (int i = 0; i < ST; ++i)
         if (i < p.L) issue(p.L - 1 - i, i);
-    // the nominal (to linearise about, and for the update norm) a step ahead
-    const bool want_x = !use_lin || K == KK_CUBATURE || want_norm;
-    T xc[5], xn[5];
-    if (want_x && any) load_nominal(p, lane_ix(p, e - 1 - a, lane), xc);
+    // the nominal a step ahead
+    T xc[5], xn[5];   // nominals of states k, k-1
+    if (any) {
+        load_nominal(p, lane_ix(p, e - 1 - a, lane), xc);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) s.m[c] += G.r[c] - xc[c];
+    }
     int st = 0;
 #pragma unroll 1
     for (int sidx = p.L - 1; sidx >= 0; --sidx) {
@@ -1095,7 +1137,7 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
         if (k < e) {
             cur.backward(k);
             const int64_t ix = lane_ix(p, sidx, lane);
-            if (want_x && k > a) load_nominal(p, ix - p.NL, xn);
+            if (k > a) load_nominal(p, ix - p.NL, xn);
             T m[5], P[15];
 #pragma unroll
             for (int c = 0; c < 5; ++c) m[c] = ws.get(st, c);
@@ -1118,7 +1160,7 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
                     form_trans<K>(p, in, fc, tr);
                 }
                 T mp[5], FP[25], Pp[15];
-                predict<FS>(tr, m, P, mp, FP, Pp);
+                predict<FS, true>(tr, m, P, mp, FP, Pp);
                 SElem<T> ec;
                 ok &= selem_from_prediction(m, P, FP, Pp, mp, ec);
                 apply_smoother(ec, s, s);
@@ -1127,7 +1169,7 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
                 finite = finite && isfinite(s.m[i]);
-                p.x[i * p.cs + ix] = s.m[i];
+                p.x[i * p.cs + ix] = xc[i] + s.m[i];
             }
             if (!finite) atomicOr(p.status, ST_NONFINITE);
             if (write_P) {
@@ -1146,13 +1188,17 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
                 }
 #pragma unroll
                 for (int i = 0; i < 5; ++i) {
-                    const double dv = double(s.m[i]) - double(xc[i]);
+                    const T x = xc[i] + s.m[i];
+                    const double dv = double(x) - double(xc[i]);
                     num += dv * dv;
-                    den += double(s.m[i]) * double(s.m[i]);
+                    den += double(x) * double(x);
                 }
             }
 #pragma unroll
-            for (int c = 0; c < 5; ++c) xc[c] = xn[c];
+            for (int c = 0; c < 5; ++c) {   // from the nominal of k - 1 on
+                s.m[c] += xc[c] - xn[c];
+                xc[c] = xn[c];
+            }
         }
         __syncwarp();   // every lane is done with the stage: refill it
         if (sidx >= ST) issue(sidx - ST, st);
@@ -1183,7 +1229,7 @@ template <typename T, int K, int NT>
 constexpr size_t smem_bytes_for()
 {
     using M = TreeMem<T, NT>;
-    static_assert(M::kEnd - FE * NT >= NT * 2 * kStateIn, "the sigma-point folds' prefetch fits beside the leaves");
+    static_assert(M::kEnd - FE * NT >= NT * 3 * kStateIn, "the sigma-point folds' prefetch fits beside the leaves");
     static_assert(K != KK_ARRAYS || (M::kEnd - FE * NT >= NT * 2 * kFilterIn && M::kEnd >= NT * 3 * kFilterIn &&
                                      M::kEnd - SE * NT >= NT * 2 * kSmoothIn),
                   "the streams of the scans over given arrays fit");

@@ -22,36 +22,77 @@ namespace pes {
 
 // Padded so that the fields that are loaded together start on 16 bytes, and
 // to sizes at which consecutive elements' 16-byte words fall in different
-// shared-memory banks (76 and 60 words).
+// shared-memory banks (76, 60 and 28 words). The padding holds reference points:
+// means are kept as small deviations from them, so that combining elements does
+// not round positions of tens to thousands of units over and over. The filtering
+// element's output mean is br + b (and its input is measured from xr); the
+// smoothing element maps x_next to E (x_next - (sr + xr)) + gr + g.
 template <typename T>
 struct alignas(16) FElem {
     T A[25];
     T b[5];
-    T pad0[2];
+    T br0[2];
     T C[15];
-    T pad1;
+    T br2;
     T J[15];
-    T pad2;
+    T br3;
     T eta[5];
     T xr[5];
-    T pad3[2];
+    T br4;
+    T pad;
 };
+
+template <typename T>
+PES_DEV void felem_set_ref(FElem<T>& f, const T* r)
+{
+    f.br0[0] = r[0];
+    f.br0[1] = r[1];
+    f.br2 = r[2];
+    f.br3 = r[3];
+    f.br4 = r[4];
+    f.pad = T(0);
+}
+template <typename T>
+PES_DEV void felem_ref(const FElem<T>& f, T* r)
+{
+    r[0] = f.br0[0];
+    r[1] = f.br0[1];
+    r[2] = f.br2;
+    r[3] = f.br3;
+    r[4] = f.br4;
+}
 
 template <typename T>
 struct alignas(16) SElem {
     T E[25];
     T g[5];
-    T pad0[2];
+    T sr0[2];
     T L[15];
-    T pad1;
+    T sr2;
     T xr[5];
-    T pad2[7];
+    T gr[5];
+    T sr3[2];
 };
+
+// References of the input (sr) and of g (gr).
+template <typename T>
+PES_DEV void selem_set_refs(SElem<T>& e, const T* sr, const T* gr)
+{
+    e.sr0[0] = sr[0];
+    e.sr0[1] = sr[1];
+    e.sr2 = sr[2];
+    e.sr3[0] = sr[3];
+    e.sr3[1] = sr[4];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) e.gr[i] = gr[i];
+}
 
 template <typename T>
 struct alignas(16) Gauss {
-    T m[5];
+    T m[5];   // mean less r
     T P[15];
+    T r[5];
+    T pad[3];
 };
 
 // ---- products with a structured slope ------------------------------------------
@@ -192,6 +233,8 @@ PES_DEV void felem_identity(FElem<T>& a, const T* xr)
         a.C[i] = T(0);
         a.J[i] = T(0);
     }
+    const T zero[5] = {T(0), T(0), T(0), T(0), T(0)};
+    felem_set_ref(a, zero);
 }
 
 // The Levenberg-Marquardt damping of state k as a filtering element: the
@@ -241,18 +284,22 @@ PES_DEV void felem_apply_prior(FElem<T>& a, const T* m0, const T* P0)
 //   A = A- - K G,  b = b- + K v,  C = C- - K H C-,
 // and the likelihood of y_k given the input accumulates
 //   J += G^T S^{-1} G,  eta += G^T S^{-1} v.
+// REL: means are measured from the nominal of the state that the linearisation
+// is about, and tr.fx is f(xn) - xn (the smoother kernel; the caller re-references
+// them from state to state). Otherwise means and tr.fx are absolute.
+//
 // The two halves are folded separately, which keeps the transition and the
 // observation from being live together: the prediction through the transition,
 // after which a describes x_k given the input, and the update with the
 // observation at k.
-template <int FS = FS_DENSE, typename T>
+template <int FS = FS_DENSE, bool REL = false, typename T>
 PES_DEV void fold_predict(FElem<T>& a, const Trans<T>& tr)
 {
     T Am[25];
     f_mm<FS>(tr.F, a.A, Am);
     T dv[5], bm[5];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) dv[i] = a.b[i] - tr.xn[i];
+    for (int i = 0; i < 5; ++i) dv[i] = REL ? a.b[i] : a.b[i] - tr.xn[i];
     f_mv<FS>(tr.F, dv, bm);
 #pragma unroll
     for (int i = 0; i < 5; ++i) bm[i] += tr.fx[i];
@@ -267,7 +314,7 @@ PES_DEV void fold_predict(FElem<T>& a, const Trans<T>& tr)
     for (int i = 0; i < 15; ++i) a.C[i] = Cm[i];
 }
 
-template <int FS = FS_DENSE, typename T>
+template <int FS = FS_DENSE, bool REL = false, typename T>
 PES_DEV bool fold_update(FElem<T>& a, const Obs<T>& ob)
 {
     constexpr int HC = kHCols<FS>;
@@ -295,7 +342,7 @@ PES_DEV bool fold_update(FElem<T>& a, const Obs<T>& ob)
         }
         T hv = ob.r[r];
 #pragma unroll
-        for (int l = 0; l < HC; ++l) hv = fma(-ob.H[r * 5 + l], bm[l] - ob.xn[l], hv);
+        for (int l = 0; l < HC; ++l) hv = fma(-ob.H[r * 5 + l], REL ? bm[l] : bm[l] - ob.xn[l], hv);
         v[r] = hv;
     }
     T Anew[25], bnew[5], Cnew[15];
@@ -336,7 +383,8 @@ PES_DEV bool fold_update(FElem<T>& a, const Obs<T>& ob)
 }
 
 // out = ai (x) aj, Eq. 15 (ai earlier in time). aj's input reference is the
-// point where ai's output is measured from.
+// point where ai's output is measured from. The elements' reference points are
+// not looked at: b and xr count as they are (so do g and xr below).
 template <typename T>
 PES_DEV void combine_filter(const FElem<T>& ai, const FElem<T>& aj, FElem<T>& out)
 {
@@ -460,6 +508,8 @@ PES_DEV void selem_identity(SElem<T>& a)
     }
 #pragma unroll
     for (int i = 0; i < 15; ++i) a.L[i] = T(0);
+    const T zero[5] = {T(0), T(0), T(0), T(0), T(0)};
+    selem_set_refs(a, zero, zero);
 }
 
 // Eq. 18: the last state of a trajectory, E = 0, g = x*, L = P*.
@@ -513,12 +563,12 @@ PES_DEV bool selem_from_prediction(const T* xf, const T* Pf, const T* FP, const 
 }
 
 // Predicted moments of the transition tr applied to (m, P): mp, FP = F P, Pp.
-template <int FS = FS_DENSE, typename T>
+template <int FS = FS_DENSE, bool REL = false, typename T>
 PES_DEV void predict(const Trans<T>& tr, const T* m, const T* P, T* mp, T* FP, T* Pp)
 {
     T dx[5];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) dx[i] = m[i] - tr.xn[i];
+    for (int i = 0; i < 5; ++i) dx[i] = REL ? m[i] : m[i] - tr.xn[i];
     f_mv<FS>(tr.F, dx, mp);
 #pragma unroll
     for (int i = 0; i < 5; ++i) mp[i] += tr.fx[i];
@@ -580,7 +630,7 @@ struct LogLik {
 };
 
 // Kalman update of (mp, Pp) with the observation ob: (m, P).
-template <int FS = FS_DENSE, typename T>
+template <int FS = FS_DENSE, bool REL = false, typename T>
 PES_DEV bool kf_update(const Obs<T>& ob, const T* mp, const T* Pp, T* m, T* P, LogLik<T>* loglik = nullptr)
 {
     constexpr int HC = kHCols<FS>;
@@ -597,7 +647,7 @@ PES_DEV bool kf_update(const Obs<T>& ob, const T* mp, const T* Pp, T* m, T* P, L
         for (int j = 0; j < 5; ++j) KT[r * 5 + j] = Si[si2(r, 0)] * HP[j] + Si[si2(r, 1)] * HP[5 + j];
         T hv = ob.r[r];
 #pragma unroll
-        for (int l = 0; l < HC; ++l) hv = fma(-ob.H[r * 5 + l], mp[l] - ob.xn[l], hv);
+        for (int l = 0; l < HC; ++l) hv = fma(-ob.H[r * 5 + l], REL ? mp[l] : mp[l] - ob.xn[l], hv);
         v[r] = hv;
     }
     if (loglik) loglik->add(S[si2(0, 0)], S[si2(0, 1)], S[si2(1, 1)], v[0], v[1]);

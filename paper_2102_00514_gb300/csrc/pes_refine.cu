@@ -17,18 +17,29 @@ PES_DEV void load20(const float* base, int64_t cs, int64_t ix, float* m, float* 
 }
 
 // The filtered moments of step s of a lane, component c at [c * 32] (the
-// smoother kernel's handoff layout).
+// smoother kernel's handoff layout; the means are less the nominal).
 PES_DEV const float* filt_slot(const RefineParams& p, int s, int lane)
 {
     return p.filt + ((size_t)(lane >> 5) * p.L + s) * (HAND * 32) + (lane & 31);
 }
 
-PES_DEV void load_filt(const float* f, float* m, float* P)
+PES_DEV float filt_mean(const RefineParams& p, const float* f, int c, int64_t ix)
+{
+    return __fadd_rn(p.nom[c * p.cs + ix], f[c * 32]);
+}
+
+PES_DEV void load_filt(const RefineParams& p, const float* f, int64_t ix, float* m, float* P)
 {
 #pragma unroll
-    for (int c = 0; c < 5; ++c) m[c] = f[c * 32];
+    for (int c = 0; c < 5; ++c) m[c] = filt_mean(p, f, c, ix);
 #pragma unroll
     for (int c = 0; c < 15; ++c) P[c] = f[(5 + c) * 32];
+}
+
+PES_DEV void less_nominal(Trans<float>& tr)
+{
+#pragma unroll
+    for (int i = 0; i < 5; ++i) tr.fx[i] -= tr.xn[i];
 }
 
 PES_DEV void store_elem(const RefineParams& p, int64_t ix, const float* A, const float* w, const float* s,
@@ -95,7 +106,7 @@ __global__ void __launch_bounds__(RT_THREADS) refine_fwd_kernel(const RefinePara
     const int b = traj_of(p.offsets, p.B, k);
     const int64_t head = __ldg(p.offsets + b), next = __ldg(p.offsets + b + 1);
     float xf[5], Pf[15];
-    load_filt(filt_slot(p, s, lane), xf, Pf);
+    load_filt(p, filt_slot(p, s, lane), ix, xf, Pf);
     if (k == head) {
         float A[25], w[5], sres[5], r[15];
 #pragma unroll
@@ -119,14 +130,14 @@ __global__ void __launch_bounds__(RT_THREADS) refine_fwd_kernel(const RefinePara
         load20(p.nom, p.cs, ix, xn, Pn);
         if constexpr (K == KK_IEKS || K == KK_IEKS_ANY) {
             if constexpr (K == KK_IEKS) ct_trans_taylor(m, xn, tr);
-            else lin_trans_taylor(m, xn, tr);
+            else lin_trans_taylor(m, xn, tr), less_nominal(tr);
 #pragma unroll
             for (int c = 0; c < 25; ++c) sc[SCR_F + c] = tr.F[c];
         } else {
             float Lc[25], rdc[5];
             ok &= cub_factor(Pn, Lc, rdc);
             if constexpr (K == KK_CUBATURE) ct_trans_cubature(m, xn, Lc, rdc, tr);
-            else lin_trans_cubature(m, xn, Lc, rdc, tr);
+            else lin_trans_cubature(m, xn, Lc, rdc, tr), less_nominal(tr);
             cub_trans_slope_ff(m, xn, Lc, sc);
         }
     }
@@ -162,7 +173,7 @@ __global__ void __launch_bounds__(RT_THREADS) refine_fwd_kernel(const RefinePara
     float A[25], w[5];
     ok &= ff_kalman_step<kFS<K>>(tr, ob, xf, Pf, mf, Pff, A, w, sc);
     float x1[5], P1[15], sres[5], r[15];
-    load_filt(s + 1 < p.L ? filt_slot(p, s + 1, lane) : filt_slot(p, 0, lane + 1), x1, P1);
+    load_filt(p, s + 1 < p.L ? filt_slot(p, s + 1, lane) : filt_slot(p, 0, lane + 1), ix1, x1, P1);
 #pragma unroll
     for (int c = 0; c < 5; ++c) sres[c] = ff_to_f(ff_add_f(mf[c], -x1[c]));
 #pragma unroll
@@ -186,7 +197,7 @@ __global__ void __launch_bounds__(RT_THREADS) refine_bwd_kernel(const RefinePara
     const int64_t next = __ldg(p.offsets + b + 1);
     // the refined filtered moments as float-float pairs
     const float* filt = filt_slot(p, s, lane);
-    auto filt_ff = [&](int c) { return two_sum(filt[c * 32], p.dlt[c * p.cs + ix]); };
+    auto filt_ff = [&](int c) { return two_sum(c < 5 ? filt_mean(p, filt, c, ix) : filt[c * 32], p.dlt[c * p.cs + ix]); };
     float* el = p.elem + ix;
     if (k + 1 >= next) {
         // last state: smoothed = filtered

@@ -42,7 +42,7 @@
 namespace pes {
 
 constexpr int RE = 50;   // correction element: Abar (or G) 25, s 5, r 15, w 5 (forward only)
-constexpr int RT = 45;   // stored transition (a linearisation that is not repeated): F 25, fx 5, Q' 15
+constexpr int RT = 45;   // stored transition (a linearisation that is not repeated): F 25, fx (less xn) 5, Q' 15
 constexpr int RD = 20;   // correction of one state: means 5, covariance 15
 
 struct RefineParams {
@@ -272,21 +272,21 @@ PES_DEV void ff_predict_cov(const V* P, Scratch<NT> sc)
     }
 }
 
-// fx + F d for a float-float d, row i by row.
+// xn + fx + F d for a float-float d, row i by row.
 template <int FS, int NT>
-PES_DEV void ff_predict_mean(const float* fx, const ff* d, Scratch<NT> sc, ff* mp)
+PES_DEV void ff_predict_mean(const float* xn, const float* fx, const ff* d, Scratch<NT> sc, ff* mp)
 {
     constexpr int ROWS = FS == FS_DENSE ? 5 : 4, L0 = FS == FS_CT ? 2 : 0;
 #pragma unroll
     for (int i = 0; i < ROWS; ++i) {
-        ffacc acc = acc_of_f(fx[i]);
+        ffacc acc = acc_of(two_sum(xn[i], fx[i]));
         if (FS == FS_CT && i < 2) acc_add(acc, d[i]);
 #pragma unroll
         for (int l = L0; l < 5; ++l) acc_add(acc, d[l], sc[SCR_F + i * 5 + l]);
         mp[i] = acc_done(acc);
     }
     if (ROWS == 4) {
-        ffacc acc = acc_of_f(fx[4]);
+        ffacc acc = acc_of(two_sum(xn[4], fx[4]));
         acc_add(acc, d[4]);
         mp[4] = acc_done(acc);
     }
@@ -310,7 +310,7 @@ PES_DEV bool ff_kalman_step(const Trans<float>& tr, const Obs<float>& ob, const 
     ff d[5], mp[5];
 #pragma unroll
     for (int l = 0; l < 5; ++l) d[l] = ff_diff_f(m[l], tr.xn[l]);
-    ff_predict_mean<FS>(tr.fx, d, sc, mp);
+    ff_predict_mean<FS>(tr.xn, tr.fx, d, sc, mp);
     ff HP[10];
 #pragma unroll
     for (int r = 0; r < 2; ++r)
@@ -447,11 +447,11 @@ PES_DEV bool ff_rts_gain(const Trans<float>& tr, const ff* mf, const ff* Pf, con
 #pragma unroll
         for (int i = 0; i < 5; ++i) sc.st(SCR_M + 2 * (i * 5 + c), x[i]);
     }
-    // ms = mf + G (xs1 - mp), mp = fx + F (mf - xn)
+    // ms = mf + G (xs1 - mp), mp = xn + fx + F (mf - xn)
     ff e[5], d[5];
 #pragma unroll
     for (int l = 0; l < 5; ++l) d[l] = ff_add_f(mf[l], -tr.xn[l]);
-    ff_predict_mean<FS>(tr.fx, d, sc, e);
+    ff_predict_mean<FS>(tr.xn, tr.fx, d, sc, e);
 #pragma unroll
     for (int i = 0; i < 5; ++i) e[i] = ff_add_f(ff_neg(e[i]), xs1[i]);
 #pragma unroll

@@ -30,10 +30,15 @@ namespace pes {
 
 constexpr int FE = sizeof(FElem<double>) / sizeof(double);   // 76
 constexpr int SE = sizeof(SElem<double>) / sizeof(double);   // 60
-constexpr int GE = sizeof(Gauss<double>) / sizeof(double);   // 20
+constexpr int GE = sizeof(Gauss<double>) / sizeof(double);   // 28
 // offsets of an element's fields
 constexpr int FA = 0, FB = 25, FC = 32, FJ = 48, FETA = 64, FXR = 69;
-constexpr int EE = 0, EG = 25, EL = 32, EXR = 48;
+constexpr int EE = 0, EG = 25, EL = 32, EXR = 48, EGR = 53;
+constexpr int GR = 20;
+// where entry q of a filtering element's output reference is, and of a smoothing
+// element's input reference
+PES_DEV int f_ref(int q) { return q < 2 ? 30 + q : (q == 2 ? 47 : (q == 3 ? 63 : 74)); }
+PES_DEV int s_ref(int q) { return q < 2 ? 30 + q : (q == 2 ? 47 : 55 + q); }
 
 // dynamic shared memory of the calling kernel, as scalars
 template <typename T>
@@ -103,7 +108,7 @@ PES_DEV void coop_combine_filter(int a, int b, int o, int part, int parts)
     const T* pa = s + a;
     const T* pb = s + b;
     T* po = s + o;
-    T J[16], D[15], C[16], xr[5], eta[5], z[5], add[5];
+    T J[16], D[15], C[16], off[5], eta[5], z[5], add[5];
     ld_vec<16>(pb + FJ, J);
     ld_vec<16>(pa + FC, C);
     int r, base;        // the packed row (column) of C (J) that the task writes, and its place
@@ -125,7 +130,7 @@ PES_DEV void coop_combine_filter(int a, int b, int o, int part, int parts)
     load_task(part);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        xr[i] = pb[FXR + i];
+        off[i] = pa[f_ref(i)] - pb[FXR + i];   // where a's output is measured from, to b's input
         eta[i] = pb[FETA + i];
     }
     info_update_cov(C, J, D);
@@ -154,7 +159,7 @@ PES_DEV void coop_combine_filter(int a, int b, int o, int part, int parts)
     for (int task = part;;) {
         T t[5], p[5], w[5];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) z[i] = vec ? z[i] - xr[i] : z[i];
+        for (int i = 0; i < 5; ++i) z[i] = vec ? z[i] + off[i] : z[i];
         sv(J, z, t);
 #pragma unroll
         for (int i = 0; i < 5; ++i) t[i] = row ? z[i] : (vec ? eta[i] - t[i] : t[i]);
@@ -196,6 +201,7 @@ PES_DEV void coop_combine_filter(int a, int b, int o, int part, int parts)
                 if (c <= r) po[base + si(c, c) - c] = v;
             }
             po[FXR + r] = pa[FXR + r];
+            po[f_ref(r)] = pb[f_ref(r)];
         }
         task += parts;
         if (task >= 11) break;
@@ -211,8 +217,8 @@ PES_DEV void coop_apply_filter(int g, int e, int o, int part, int parts)
     T* s = smem_as<T>();
     const T* pe = s + e;
     T* po = s + o;
-    T G[20], J[16], D[15], w[5], xr[5], eta[5], row[5], add[5], br;
-    ld_vec<20>(s + g, G);
+    T G[28], J[16], D[15], w[5], xr[5], eta[5], row[5], add[5], br, ref;
+    ld_vec<28>(s + g, G);
     ld_vec<16>(pe + FJ, J);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
@@ -228,6 +234,7 @@ PES_DEV void coop_apply_filter(int g, int e, int o, int part, int parts)
             add[i] = pe[FC + base + i];
         }
         br = pe[FB + r];
+        ref = pe[f_ref(r)];
     };
     load_row(part);
     T A[28];
@@ -236,7 +243,7 @@ PES_DEV void coop_apply_filter(int g, int e, int o, int part, int parts)
     {
         T dm[5], u[5], Du[5];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) dm[i] = G[i] - xr[i];
+        for (int i = 0; i < 5; ++i) dm[i] = G[i] + (G[GR + i] - xr[i]);
         sv(J, dm, u);
 #pragma unroll
         for (int i = 0; i < 5; ++i) u[i] = eta[i] - u[i];
@@ -252,6 +259,7 @@ PES_DEV void coop_apply_filter(int g, int e, int o, int part, int parts)
 #pragma unroll
         for (int i = 1; i < 5; ++i) m = fma(row[i], w[i], m);
         po[r] = m + br;
+        po[GR + r] = ref;
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
             T v = add[c];
@@ -279,7 +287,7 @@ PES_DEV void coop_combine_smoother(int a, int b, int o, int part, int parts)
     ld_vec<32>(pb + EE, Ej);
     ld_vec<16>(pb + EL, Lj);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) dg[i] = Ej[EG + i] - pa[EXR + i];
+    for (int i = 0; i < 5; ++i) dg[i] = (Ej[EG + i] - pa[EXR + i]) + (pb[EGR + i] - pa[s_ref(i)]);
 #pragma unroll 1
     for (int r = part; r < 5; r += parts) {
         T e[5], add[5], le[5], en[5];
@@ -289,7 +297,7 @@ PES_DEV void coop_combine_smoother(int a, int b, int o, int part, int parts)
             e[i] = pa[EE + 5 * r + i];
             add[i] = pa[base + i];
         }
-        const T gr = pa[EG + r], xr = pb[EXR + r];
+        const T gr = pa[EG + r], xr = pb[EXR + r], gref = pa[EGR + r], sref = pb[s_ref(r)];
         sv(Lj, e, le);
         mtv(Ej, e, en);
         T g = e[0] * dg[0];
@@ -297,6 +305,8 @@ PES_DEV void coop_combine_smoother(int a, int b, int o, int part, int parts)
         for (int i = 1; i < 5; ++i) g = fma(e[i], dg[i], g);
         po[EG + r] = g + gr;
         po[EXR + r] = xr;
+        po[EGR + r] = gref;
+        po[s_ref(r)] = sref;
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
             T v = add[c];
@@ -316,11 +326,11 @@ PES_DEV void coop_apply_smoother(int g, int e, int o, int part, int parts)
     T* s = smem_as<T>();
     const T* pe = s + e;
     T* po = s + o;
-    T E[28], G[20], dm[5];
+    T E[28], G[28], dm[5];
     ld_vec<28>(pe + EE, E);
-    ld_vec<20>(s + g, G);
+    ld_vec<28>(s + g, G);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) dm[i] = G[i] - pe[EXR + i];
+    for (int i = 0; i < 5; ++i) dm[i] = (G[i] - pe[EXR + i]) + (G[GR + i] - pe[s_ref(i)]);
 #pragma unroll 1
     for (int r = part; r < 5; r += parts) {
         T row[5], add[5], p[5];
@@ -330,12 +340,13 @@ PES_DEV void coop_apply_smoother(int g, int e, int o, int part, int parts)
             row[i] = pe[EE + 5 * r + i];
             add[i] = pe[EL + base + i];
         }
-        const T gr = pe[EG + r];
+        const T gr = pe[EG + r], gref = pe[EGR + r];
         sv(G + 5, row, p);
         T m = row[0] * dm[0];
 #pragma unroll
         for (int i = 1; i < 5; ++i) m = fma(row[i], dm[i], m);
         po[r] = m + gr;
+        po[GR + r] = gref;
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
             T v = add[c];
@@ -353,27 +364,31 @@ PES_DEV void combine_smoother1(int a, int b, int o)
     T* s = smem_as<T>();
     const T* pa = s + a;
     const T* pb = s + b;
-    T Ei[32], Ej[32], M[16], dg[5], xi[8], xj[8], Eo[32], Lo[16];   // E then g
+    // E then g and two of the input's reference; L and one more; xr, gr and the last two
+    T Ei[32], Ej[32], Li[16], Lj[16], xi[12], xj[12], dg[5], out[32], EL_[25];
     ld_vec<32>(pa + EE, Ei);
     ld_vec<32>(pb + EE, Ej);
-    ld_vec<8>(pa + EXR, xi);
+    ld_vec<16>(pa + EL, Li);
+    ld_vec<16>(pb + EL, Lj);
+    ld_vec<12>(pa + EXR, xi);
+    ld_vec<12>(pb + EXR, xj);
+    const T ri[5] = {Ei[30], Ei[31], Li[15], xi[10], xi[11]};
 #pragma unroll
-    for (int i = 0; i < 5; ++i) dg[i] = Ej[EG + i] - xi[i];
-    mv(Ei, dg, Eo + EG);
+    for (int i = 0; i < 5; ++i) dg[i] = (Ej[EG + i] - xi[i]) + (xj[5 + i] - ri[i]);
+    mv(Ei, dg, out + EG);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) Eo[EG + i] += Ei[EG + i];
-    Eo[30] = Eo[31] = T(0);
-    mm(Ei, Ej, Eo);
-    st_vec<32>(s + o + EE, Eo);
-    T EL_[25];
-    ld_vec<16>(pb + EL, M);
-    m_s(Ei, M, EL_);
-    ld_vec<16>(pa + EL, M);
-    abt_sym_add(EL_, Ei, M, Lo);
-    Lo[15] = T(0);
-    st_vec<16>(s + o + EL, Lo);
-    ld_vec<8>(pb + EXR, xj);
-    st_vec<8>(s + o + EXR, xj);
+    for (int i = 0; i < 5; ++i) out[EG + i] += Ei[EG + i];
+    out[30] = Ej[30];
+    out[31] = Ej[31];
+    mm(Ei, Ej, out);
+    st_vec<32>(s + o + EE, out);
+    m_s(Ei, Lj, EL_);
+    abt_sym_add(EL_, Ei, Li, out);
+    out[15] = Lj[15];
+    st_vec<16>(s + o + EL, out);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) xj[5 + i] = xi[5 + i];
+    st_vec<12>(s + o + EXR, xj);
 }
 
 template <typename T>
@@ -381,19 +396,24 @@ PES_DEV void apply_smoother1(int g, int e, int o)
 {
     T* s = smem_as<T>();
     const T* pe = s + e;
-    T E[32], G[20], L[16], x[8], dm[5], EP[25], out[20];
+    T E[32], G[28], L[16], x[12], dm[5], EP[25], out[28];
     ld_vec<32>(pe + EE, E);
-    ld_vec<20>(s + g, G);
-    ld_vec<8>(pe + EXR, x);
+    ld_vec<28>(s + g, G);
+    ld_vec<12>(pe + EXR, x);
     ld_vec<16>(pe + EL, L);
+    const T ri[5] = {E[30], E[31], L[15], x[10], x[11]};
 #pragma unroll
-    for (int i = 0; i < 5; ++i) dm[i] = G[i] - x[i];
+    for (int i = 0; i < 5; ++i) dm[i] = (G[i] - x[i]) + (G[GR + i] - ri[i]);
     mv(E, dm, out);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) out[i] += E[EG + i];
+    for (int i = 0; i < 5; ++i) {
+        out[i] += E[EG + i];
+        out[GR + i] = x[5 + i];
+    }
+    out[25] = out[26] = out[27] = T(0);
     m_s(E, G + 5, EP);
     abt_sym_add(EP, E, L, out + 5);
-    st_vec<20>(s + o, out);
+    st_vec<28>(s + o, out);
 }
 
 // The operators of the two scans, for the tree code below. `wide`: more than 32
@@ -404,6 +424,7 @@ PES_DEV void apply_smoother1(int g, int e, int o)
 template <typename T, bool KEEP = false>
 struct FilterOps {
     static constexpr int NC = FE, kMean = FB, kCov = FC;
+    PES_DEV static int ref(int q) { return f_ref(q); }
     static constexpr bool kSuffix = false;   // the Gaussian enters at the left
     PES_DEV static void combine(int a, int b, int o, int part, int parts, bool)
     {
@@ -415,6 +436,7 @@ struct FilterOps {
 template <typename T>
 struct SmootherOps {
     static constexpr int NC = SE, kMean = EG, kCov = EL;
+    PES_DEV static int ref(int q) { return EGR + q; }
     static constexpr bool kSuffix = true;    // the Gaussian enters at the right
     PES_DEV static void combine(int a, int b, int o, int part, int parts, bool wide)
     {
@@ -538,7 +560,7 @@ PES_DEV void level_copy_in(T* dst, const T* src, int n, int shift, int nodes)
 // Level 3: the Gaussian entering the block into kBlock, from the aggregates of
 // blocks [b0, b1): their product starts with a prior (ends with a last state),
 // so it is a Gaussian whatever precedes it: A = 0 and (b, C), or E = 0 and (g,
-// L). Zero if there are none.
+// L), with the references. Zero if there are none.
 template <typename T, int NT, class Ops>
 PES_DEV void tree_top(const T* agg, int b0, int b1)
 {
@@ -564,7 +586,8 @@ PES_DEV void tree_top(const T* agg, int b0, int b1)
         __syncthreads();
         root = tree_reduce<T, NT, Ops>(M::kTop, M::kTop2, n + had);
     }
-    if (t < GE) s[M::kBlock + t] = root >= 0 ? s[root + (t < 5 ? at + t : at2 + t - 5)] : T(0);
+    if (t < GE)
+        s[M::kBlock + t] = root < 0 || t >= 25 ? T(0) : s[root + (t < 5 ? at + t : (t < GR ? at2 + t - 5 : Ops::ref(t - GR)))];
     __syncthreads();
 }
 
