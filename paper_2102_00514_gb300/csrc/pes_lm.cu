@@ -168,9 +168,10 @@ __global__ void lm_cost_kernel(const LMParams p, double* cost_out, const T* x, c
 // Per trajectory: keep the step if it lowered the objective (damping / nu),
 // else keep the nominal (damping * nu); record convergence (the step's
 // relative size <= tol) and count the trajectories still unconverged. A step
-// within the tolerance changes the objective by about tol^2 of it, below the
-// rounding of its evaluation: such a step is also kept when the objective does
-// not tell the two apart, so that the result does not hang on that rounding.
+// within the tolerance, or of a relative size up to 1e-7, changes the objective by
+// about 1e-14 of it or less, which the rounding of its evaluation hides: such a
+// step is also kept when the objective does not tell the two apart, so that the
+// result and the iterations it takes do not hang on that rounding.
 template <typename T>
 __global__ void lm_decide_kernel(const LMParams p, T* lam, int it, double tol, double nu)
 {
@@ -178,7 +179,7 @@ __global__ void lm_decide_kernel(const LMParams p, T* lam, int it, double tol, d
     if (b >= p.B) return;
     const double num = p.num[b], den = p.den[b];
     const double rel = den > 0.0 ? sqrt(num / den) : sqrt(num);
-    const double tie = (tol > 0.0 && rel <= tol) ? 1e-13 * fabs(p.cost[b]) : 0.0;
+    const double tie = (tol > 0.0 && rel <= fmax(tol, 1e-7)) ? 1e-13 * fabs(p.cost[b]) : 0.0;
     const bool acc = p.cost_new[b] < p.cost[b] + tie;
     if (acc) {
         p.cost[b] = p.cost_new[b];
