@@ -393,7 +393,8 @@ pes_status pes_graph_destroy(pes_graph* g);
  * the shape is this library's choice): times pes_ieks_run of the given
  * workload with `iters` iterations for every distinct launch the candidates
  * give (threads per block 128 or 256 for FP32, 128 for FP64; at least
- * 4 .. 128 steps per lane, which sets the number of blocks when N is small)
+ * 4 .. 128 steps per lane, which sets the number of blocks when N is small;
+ * up to 8, the library chooses, and a small N gets fewer)
  * and keeps the fastest for this handle, method and precision: later calls
  * of any size use it (pes_launch_shape reports it). x_scratch [5][N] and
  * P_scratch [15][N] (DEVICE, the precision's type) receive the runs' outputs.
@@ -410,14 +411,17 @@ pes_status pes_autotune(pes_handle* h, const pes_model* model, pes_method method
  * without timing anything: a choice recorded by an earlier pes_autotune (for
  * example one cached on disk for this GPU). threads: a compiled block size
  * (128 or 256 for PES_FP32, 128 for PES_FP64), or 0 with min_steps 0 for the
- * defaults; min_steps: at least 1, the minimum steps per lane. prec PES_FP32
+ * defaults; min_steps: at least 1, the minimum steps per lane (up to 8: the
+ * library's choice, as by default). prec PES_FP32
  * also sets the shape of PES_MIXED's and PES_REFINED's FP32 iterations.
  * PES_ERR_INVALID_ARG for anything else; the previous choice then stays. */
 pes_status pes_set_launch_shape(pes_handle* h, pes_method method, pes_precision prec, int32_t threads,
                                 int32_t min_steps);
 
 /* Launch shape the next call of the given kind would use (for tests and the
- * benchmark): blocks, threads per block, steps per thread. */
+ * benchmark): blocks, threads per block, steps per thread of those that own
+ * states (a multiple of 32 threads of every block; the rest only help with the
+ * block's scans). */
 pes_status pes_launch_shape(pes_handle* h, pes_method method, pes_precision prec, int64_t N,
                             int32_t* blocks, int32_t* threads, int32_t* steps_per_thread);
 

@@ -175,7 +175,8 @@ pes_status check_model(pes_handle* h, const pes_model* m)
 // choice, for tuning.
 // Threads per block and minimum steps per lane: the autotuned values of the
 // handle if pes_autotune set them, else the defaults (256 threads for FP32,
-// the 128 that the FP64 kernel is compiled for).
+// the 128 that the FP64 kernel is compiled for). Up to kMinStepsPerThread, the
+// steps per lane of a run are make_shape's choice.
 static_assert(std::extent<decltype(pes_handle::tune)>::value > LIN_GH, "one tuning slot per linearisation");
 
 int choose_nt(const pes_handle* h, int lin, pes_precision prec)
@@ -192,8 +193,29 @@ int choose_min_steps(const pes_handle* h, int lin, pes_precision prec)
 }
 
 struct Shape {
-    int nb, nt, L;
+    int nb, nt, lpb, L;   // blocks, their threads, and of these lanes; steps per lane
 };
+
+// Time of one iteration by its launch shape, in microseconds: a step of every
+// lane (fold, re-run and RTS), a level of a block's trees and one of the grid
+// level's, each with at least 8, 4 or 2 threads to an operator (both scans, up and
+// down). Measured at T = 500 to 262,147 with 32 to 256 lanes per block.
+struct ShapeCost {
+    double step[2];    // Taylor, sigma points
+    double level[3];
+    double top[3];
+    int top_nodes;     // of a grid level at a time (TreeMem::TOPN)
+};
+constexpr ShapeCost kCost32{{4.2, 6.0}, {3.4, 6.9, 9.6}, {1.9, 4.9, 6.0}, 80};
+constexpr ShapeCost kCost64{{61.0, 100.0}, {54.0, 71.0, 100.0}, {28.0, 42.0, 60.0}, 76};
+
+// The tree over n elements.
+double tree_cost(const double (&c)[3], int nt, int n)
+{
+    double t = 0.0;
+    for (; n > 1; n = (n + 1) >> 1) t += n <= nt / 4 ? c[0] : (n <= nt / 2 ? c[1] : c[2]);
+    return t;
+}
 
 template <typename T>
 pes_status make_shape(pes_handle* h, int lin, pes_precision prec, int64_t N, Shape& s)
@@ -207,10 +229,47 @@ pes_status make_shape(pes_handle* h, int lin, pes_precision prec, int64_t N, Sha
                     cudaGetErrorString((cudaError_t)(-cap)));
     }
     if (cap == 0) return fail(h, PES_ERR_CUDA, "the smoother kernel cannot be made co-resident on this device");
-    const int64_t want = (N + (int64_t)s.nt * min_steps - 1) / ((int64_t)s.nt * min_steps);
-    s.nb = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)cap, want, (int64_t)h->nb_max}));
-    const int64_t lanes = (int64_t)s.nb * s.nt;
-    s.L = (int)((N + lanes - 1) / lanes);
+    const int64_t blocks = std::min(cap, h->nb_max);
+    if (lin == LIN_ARRAYS || min_steps > kMinStepsPerThread || N >= blocks * s.nt * kMinStepsPerThread) {
+        // A tuned shape; sizes at which all lanes have steps enough; and the scans
+        // over given arrays, which keep one partition for a size, and with it the
+        // rounding that their FP64 log-likelihoods of FP32 filters show.
+        const int64_t want = (N + (int64_t)s.nt * min_steps - 1) / ((int64_t)s.nt * min_steps);
+        s.nb = (int)std::max<int64_t>(1, std::min(blocks, want));
+        s.lpb = s.nt;
+        s.L = (int)((N + (int64_t)s.nb * s.nt - 1) / ((int64_t)s.nb * s.nt));
+        return PES_OK;
+    }
+    // A run: few steps per lane and few lanes per block, which the device's other
+    // multiprocessors make up for, against the levels of the grid's trees. A block of
+    // 32 lanes spares the first levels, whose operators have few threads each. With
+    // all the threads as lanes and at least 8 steps each: T = 500, FP64, 10
+    // iterations, 1 x 128 x 4: 7,570 us; 16 x 32 x 1: 4,750 us; T = 10,000 cubature,
+    // FP64, 5 iterations, 10 x 128 x 8: 7,250 us; 79 x 64 x 2: 4,250 us; 64
+    // trajectories of 1 to 400 states, cubature, FP32, 3 iterations, 6 x 256 x 8:
+    // 371 us; 117 x 96 x 1: 245 us. Full-size runs take all lanes either way.
+    const ShapeCost& c = sizeof(T) == 8 ? kCost64 : kCost32;
+    const int top_nodes = sizeof(T) == 4 && s.nt == 256 ? 152 : c.top_nodes;
+    double best = 1e300;
+    for (int lpb = 32; lpb <= s.nt; lpb += 32) {
+        const int64_t L0 = std::max<int64_t>((N + blocks * lpb - 1) / (blocks * lpb), sizeof(T) == 4 ? 2 : 1);
+        for (int64_t L = L0; L < L0 + 8; ++L) {
+            const int64_t lanes = (N + L - 1) / L, nb = (lanes + lpb - 1) / lpb;
+            if (L > L0 && L * nb * lpb > N + h->nl_max) break;   // the workspace
+            double t = L * c.step[lin != LIN_IEKS];
+            if (t >= best) break;
+            t += tree_cost(c.level, s.nt, (int)std::min<int64_t>(lanes, lpb));
+            for (int64_t left = nb; left > 1; left -= top_nodes - 1)
+                t += tree_cost(c.top, s.nt, (int)std::min<int64_t>(left, top_nodes));
+            if (t < best) {
+                best = t;
+                s.nb = (int)nb;
+                s.lpb = lpb;
+                s.L = (int)L;
+            }
+            if (nb == 1) break;
+        }
+    }
     return PES_OK;
 }
 
@@ -228,7 +287,8 @@ void fill_workspace(pes_handle* h, KParams<T>& p, const Shape& s)
     p.iters_done = h->iters_done;
     p.traj_iters = nullptr;
     p.L = s.L;
-    p.NL = s.nb * s.nt;
+    p.lpb = s.lpb;
+    p.NL = s.nb * s.lpb;
     p.cs = (int64_t)s.L * p.NL;
     p.timeout_ns = h->timeout_ns;
     p.ptime = h->ptime;
@@ -299,7 +359,7 @@ static pes_status filter_scan_t(pes_handle* h, const void* F, const void* c, con
     Shape s;
     pes_status r = make_shape<T>(h, LIN_ARRAYS, prec, N, s);
     if (r != PES_OK) return r;
-    const int NL = s.nb * s.nt;
+    const int NL = s.nb * s.lpb;
     const int64_t cs = (int64_t)s.L * NL;
     T* in = static_cast<T*>(h->lin);
     T* out = static_cast<T*>(h->lanes);
@@ -326,7 +386,7 @@ static pes_status smooth_scan_t(pes_handle* h, const void* F, const void* c, con
     Shape s;
     pes_status r = make_shape<T>(h, LIN_ARRAYS, prec, N, s);
     if (r != PES_OK) return r;
-    const int NL = s.nb * s.nt;
+    const int NL = s.nb * s.lpb;
     const int64_t cs = (int64_t)s.L * NL;
     T* in = static_cast<T*>(h->lin);
     T* out = static_cast<T*>(h->lanes);
@@ -349,7 +409,7 @@ template <typename T>
 static pes_status move_in(pes_handle* h, T* lx, const void* y, const void* x_init, const void* P_init, int64_t N,
                           const Shape& s, cudaStream_t st)
 {
-    const int NL = s.nb * s.nt;
+    const int NL = s.nb * s.lpb;
     const int64_t cs = (int64_t)s.L * NL;
     LaneArrays<T> a;
     if (x_init) a.add(x_init, 5);
@@ -374,7 +434,7 @@ static pes_status move_out(pes_handle* h, T* lx, void* x_out, void* P_out, int64
 {
     LaneArrays<T> a;
     a.add(x_out, 5).add(P_out, 15);
-    PES_CUDA(h, launch_lanes_move(a, lx, N, s.L, s.nb * s.nt, MOVE_OUT, st));
+    PES_CUDA(h, launch_lanes_move(a, lx, N, s.L, s.nb * s.lpb, MOVE_OUT, st));
     return PES_OK;
 }
 
@@ -389,7 +449,7 @@ static pes_status ieks_run_t(pes_handle* h, const pes_model* model, pes_method m
     pes_status r = make_shape<T>(h, lin, prec, N, s);
     if (r != PES_OK) return r;
     // the kernel's lane-major copies of x, P and y (state k = lane * L + s)
-    const int NL = s.nb * s.nt;
+    const int NL = s.nb * s.lpb;
     const int64_t cs = (int64_t)s.L * NL;
     T* lx = static_cast<T*>(h->lanes);
     T* lP = lx + 5 * cs;
@@ -549,7 +609,7 @@ static pes_status ieks_run_refined(pes_handle* h, const pes_model* model, pes_me
     if (cap < s.nb)
         return fail(h, PES_ERR_CUDA, "the refinement scan cannot be made co-resident (%d of %d blocks)", cap, s.nb);
     if ((r = ensure_refine_workspace(h)) != PES_OK) return r;
-    const int NL = s.nb * s.nt;
+    const int NL = s.nb * s.lpb;
     const int64_t cs = (int64_t)s.L * NL;
     float* lx = static_cast<float*>(h->lanes);
     float* lP = lx + 5 * cs;
@@ -595,7 +655,7 @@ static pes_status ieks_run_refined(pes_handle* h, const pes_model* model, pes_me
     {
         pes::TraceRange trace_refine_("refinement");
         RefineParams rp{};
-        rp.N = N; rp.offsets = offsets; rp.B = B; rp.L = s.L; rp.NL = NL; rp.cs = cs;
+        rp.N = N; rp.offsets = offsets; rp.B = B; rp.L = s.L; rp.lpb = s.lpb; rp.NL = NL; rp.cs = cs;
         rp.model = p.model;
         rp.y = ly; rp.m0 = (const float*)m0; rp.P0 = (const float*)P0;
         rp.nom = nom; rp.filt = static_cast<const float*>(h->hand); rp.xs = lx;
@@ -708,7 +768,7 @@ static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_preci
         const size_t per = 5 * sizeof(double) + 3 * sizeof(int);
         PES_CUDA(h, cudaMalloc(&h->lmw, per * (size_t)h->max_batch + 16));
     }
-    const int NL = s.nb * s.nt;
+    const int NL = s.nb * s.lpb;
     const int64_t cs = (int64_t)s.L * NL;
     T* lx = static_cast<T*>(h->lanes);
     T* lP = lx + 5 * cs;
@@ -1022,7 +1082,7 @@ pes_status pes_autotune(pes_handle* h, const pes_model* model, pes_method method
     PES_CUDA(h, cudaEventCreate(&e1));
     float best = 1e30f;
     pes_tune best_t;
-    int seen_nb[16], seen_nt[16], n_seen = 0;
+    int seen_nb[16], seen_nt[16], seen_L[16], n_seen = 0;
     pes_status r = PES_OK;
     for (int a = 0; a < n_nt && r == PES_OK; ++a) {
         for (int b = 0; b < 6 && r == PES_OK; ++b) {
@@ -1032,9 +1092,10 @@ pes_status pes_autotune(pes_handle* h, const pes_model* model, pes_method method
             r = (prec == PES_FP64) ? make_shape<double>(h, lin, prec, N, s) : make_shape<float>(h, lin, prec, N, s);
             if (r != PES_OK) break;
             bool dup = false;   // candidates that give the same launch are timed once
-            for (int q = 0; q < n_seen; ++q) dup |= (seen_nb[q] == s.nb && seen_nt[q] == s.nt);
+            for (int q = 0; q < n_seen; ++q) dup |= (seen_nb[q] == s.nb && seen_nt[q] == s.nt && seen_L[q] == s.L);
             if (dup) continue;
             seen_nb[n_seen] = s.nb;
+            seen_L[n_seen] = s.L;
             seen_nt[n_seen++] = s.nt;
             float ms = 1e30f;
             for (int rep = 0; rep < 2 && r == PES_OK; ++rep) {   // the first run warms up

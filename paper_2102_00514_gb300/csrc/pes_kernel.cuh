@@ -28,7 +28,7 @@
 // other blocks' (measured at T = 2^20, FP32: see pes_persistent_kernel). The RTS
 // pass then builds each step's element from the kept filtered moments.
 //
-// Within a chunk means are kept as deviations from the nominal (the filter's, the
+// In FP32, within a chunk means are kept as deviations from the nominal (the filter's, the
 // fold's and the smoother's), re-referenced from state to state by the difference
 // of their nominals, and the trees' elements carry reference points: positions of
 // tens to thousands of units would otherwise be rounded at every step and level,
@@ -72,7 +72,7 @@ template <int K>
 constexpr bool kStoreLin = kSigma<kLinOf<K>>;
 // Scalars stored per state; the transition's are kLinTrans of them, from
 // kLinTransAt. Compact form (the coordinated turn's cubature regression): F rows
-// 0-3 (20), fx (4; less xn), Q' (10), H (4), r (2), R' (3); the nominal is read from the
+// 0-3 (20), fx (4; less xn in FP32), Q' (10), H (4), r (2), R' (3); the nominal is read from the
 // trajectory, the rest is constant. Dense form: H (10), r (2), R' (3), xn (5),
 // F (25), fx (5), Q' (15).
 template <int K>
@@ -129,7 +129,8 @@ struct KParams {
     int* traj_iters;   // RUN with tol > 0: [B], the first iteration whose update met tol (0: none); or NULL
     double* loglik;    // FILTER: [B] log p(y_{1:T_b}) accumulated (zero at launch), or NULL
     int L;             // steps per lane
-    int NL;            // lanes = NB * NT
+    int lpb;           // lanes per block: a multiple of 32, at most NT
+    int NL;            // lanes = NB * lpb
     int64_t cs;        // component stride of the per-state arrays
     long long timeout_ns;
     long long* ptime;  // optional per-block phase timestamps of the first iteration (NULL: off)
@@ -349,7 +350,7 @@ PES_DEV bool get_obs(const KParams<T>& p, int64_t ix, int b, Obs<T>& ob)
     return ok;
 }
 
-// The linearisation of a compiled form of the smoother; fx is f(xn) - xn.
+// The linearisation of a compiled form of the smoother; fx is f(xn) - xn where kRel.
 template <int K, typename T>
 PES_DEV void form_trans(const KParams<T>& p, const StateIn<T, kLinOf<K>>& s, const Factor<T, kLinOf<K>>& f,
                         Trans<T>& tr)
@@ -359,7 +360,7 @@ PES_DEV void form_trans(const KParams<T>& p, const StateIn<T, kLinOf<K>>& s, con
     else {
         lin_trans<T, kLinOf<K>>(p, s, f, tr);
 #pragma unroll
-        for (int i = 0; i < 5; ++i) tr.fx[i] -= tr.xn[i];
+        for (int i = 0; i < 5 && kRel<T>; ++i) tr.fx[i] -= tr.xn[i];
     }
 }
 
@@ -529,22 +530,20 @@ PES_DEV void load_array_trans(const KParams<T>& p, int lane, Trans<T>& tr)
 }
 
 // acc <- acc (x) the Levenberg-Marquardt pseudo-measurement of a state's nominal
-// (the zero deviation). Out of line: a damped run pays for the call, the others keep the
-// operator's code and registers out of their loops.
+// xb (the zero deviation where kRel). Out of line: a damped run pays for the call,
+// the others keep the operator's code and registers out of their loops.
 template <typename T>
-__device__ __noinline__ void damp_element(FElem<T>& acc, T lambda)
+__device__ __noinline__ void damp_element(FElem<T>& acc, const T* xb, T lambda)
 {
     FElem<T> dmp;
-    const T xb[5] = {T(0), T(0), T(0), T(0), T(0)};
     felem_damping(dmp, xb, lambda);
     combine_filter(acc, dmp, acc);
 }
 
 template <typename T>
-__device__ __noinline__ void damp_gauss(Gauss<T>& g, T lambda)
+__device__ __noinline__ void damp_gauss(Gauss<T>& g, const T* xb, T lambda)
 {
     FElem<T> dmp;
-    const T xb[5] = {T(0), T(0), T(0), T(0), T(0)};
     felem_damping(dmp, xb, lambda);
     apply_filter(g, dmp, g);
 }
@@ -599,7 +598,9 @@ PES_DEV bool fold_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int la
             sc.y[0] = pf.get(st, 20);
             sc.y[1] = pf.get(st, 21);
         }
-        if (!prefetch && s > 0) {
+        if (!kRel<T> && s == 0) {   // the input is measured from the nominal of a
+            felem_identity(acc, sc.x);
+        } else if (kRel<T> && !prefetch && s > 0) {
 #pragma unroll
             for (int i = 0; i < 5; ++i) acc.b[i] += pf.get(st == 0 ? 2 : st - 1, i) - sc.x[i];
         }
@@ -609,38 +610,43 @@ PES_DEV bool fold_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int la
             T m0[5], P0[15];
             load_prior(p, cur.b, m0, P0);
 #pragma unroll
-            for (int i = 0; i < 5; ++i) m0[i] -= sc.x[i];
+            for (int i = 0; i < 5 && kRel<T>; ++i) m0[i] -= sc.x[i];
             felem_apply_prior(acc, m0, P0);
         } else {
             Obs<T> ob;
             form_obs<K>(p, cur.b, sc, fc, ob);
             if (store_lin) store_lin_obs<K>(p, s, lane, ob);
-            ok &= fold_update<FS, true>(acc, ob);
+            ok &= fold_update<FS, kRel<T>>(acc, ob);
         }
         if (lm_of(p.model, cur.b) > T(0)) {
             FElem<T> tmp = acc;
-            damp_element(tmp, lm_of(p.model, cur.b));
+            T xb[5];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) xb[i] = kRel<T> ? T(0) : sc.x[i];
+            damp_element(tmp, xb, lm_of(p.model, cur.b));
             acc = tmp;
         }
         if (!cur.is_tail(k)) {
             Trans<T> tr;
             form_trans<K>(p, sc, fc, tr);
             if (store_lin) store_lin_trans<K>(p, s, lane, tr);
-            fold_predict<FS, true>(acc, tr);
+            fold_predict<FS, kRel<T>>(acc, tr);
         }
         if (k + 1 == e) break;
         // from the next state's nominal on
         if (prefetch) {
 #pragma unroll
-            for (int i = 0; i < 5; ++i) acc.b[i] += sc.x[i] - sn.x[i];
+            for (int i = 0; i < 5 && kRel<T>; ++i) acc.b[i] += sc.x[i] - sn.x[i];
             sc = sn;
         }
         st = st == 2 ? 0 : st + 1;
     }
     // the reference points: of the output the last nominal, of the input the first
     // (read again, which takes the loop fewer registers than keeping it)
-    felem_set_ref(acc, sc.x);
-    load_nominal(p, lane, acc.xr);
+    if (kRel<T>) {
+        felem_set_ref(acc, sc.x);
+        load_nominal(p, lane, acc.xr);
+    }
     if (!prefetch) pf.wait_all();
     return ok;
 }
@@ -650,7 +656,7 @@ PES_DEV bool fold_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int la
 // updating: its results keep the rounding that they always had, which the FP64
 // log-likelihoods of FP32 runs show.
 template <typename T>
-PES_DEV bool fold_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, FElem<T>& acc, T* wstage,
+PES_DEV bool fold_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, int steps, FElem<T>& acc, T* wstage,
                                 uint64_t* wbar, uint32_t& wpar)
 {
     bool ok = true;
@@ -660,7 +666,7 @@ PES_DEV bool fold_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int l
     ws.init(wstage, wbar, wpar);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-        if (i < p.L) ws.issue(array_warp<kFilterIn>(p, i, lane), i);
+        if (i < steps) ws.issue(array_warp<kFilterIn>(p, i, lane), i);
     SegCursor cur;
     if (a < e) {
         cur.init(p.offsets, p.B, a);
@@ -671,7 +677,7 @@ PES_DEV bool fold_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int l
         }
     }
 #pragma unroll 1
-    for (int s = 0; s < p.L; ++s) {
+    for (int s = 0; s < steps; ++s) {
         const int64_t k = a + s;
         const int st = s & 1;
         ws.wait(st, p.status);
@@ -693,7 +699,7 @@ PES_DEV bool fold_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int l
             }
         }
         __syncwarp();
-        if (s + 2 < p.L) ws.issue(array_warp<kFilterIn>(p, s + 2, lane), st);
+        if (s + 2 < steps) ws.issue(array_warp<kFilterIn>(p, s + 2, lane), st);
     }
     wpar = ws.parity;
     return ok;
@@ -709,7 +715,7 @@ PES_DEV void store_filtered(const KParams<T>& p, int64_t ix, const T* m, const T
     for (int i = 0; i < 15; ++i) p.Pf[i * p.cs + ix] = P[i];
 }
 
-// MODE_RUN: the filtered moments (x* less the nominal, P*) of state a + s of a lane, kept
+// MODE_RUN: the filtered moments (x*, in FP32 less the nominal, P*) of state a + s of a lane, kept
 // between the filtering re-run and the RTS pass, which builds the smoothing
 // element from them (20 scalars per state; handing over finished elements, 50
 // scalars, cost more in traffic than the element's prediction does in
@@ -762,7 +768,7 @@ PES_DEV void trans_from_stage(const KParams<T>& p, const S& ws, int i, int off, 
         for (int c = 0; c < 20; ++c) tr.F[c] = ws.get(i, off + c);
 #pragma unroll
         for (int c = 0; c < 4; ++c) tr.fx[c] = ws.get(i, off + 20 + c);
-        tr.fx[4] = T(0);
+        tr.fx[4] = kRel<T> ? T(0) : xn[4];
 #pragma unroll
         for (int c = 0; c < 15; ++c) tr.Q[c] = p.model.Q[c];
 #pragma unroll
@@ -786,7 +792,7 @@ PES_DEV void trans_from_stage(const KParams<T>& p, const S& ws, int i, int off, 
 // every lane of the warp (lanes whose chunk is shorter idle), so that a warp
 // stream can feed it the stored linearisation.
 template <int K, typename T>
-PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, const Gauss<T>& G, T* wstage,
+PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, int steps, const Gauss<T>& G, T* wstage,
                                 uint64_t* wbar, uint32_t& wpar)
 {
     constexpr int LIN = kLinOf<K>, FS = kFS<K>, ST = kLinStages<K>;
@@ -813,10 +819,10 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
         ws.init(wstage, wbar, wpar);
 #pragma unroll
         for (int i = 0; i < ST; ++i)
-            if (i < p.L) ws.issue(lin_warp<K>(p, i, lane), i);
+            if (i < steps) ws.issue(lin_warp<K>(p, i, lane), i);
     }
 #pragma unroll 1
-    for (int s = 0; s < p.L; ++s, ix += dix) {
+    for (int s = 0; s < steps; ++s, ix += dix) {
         const int64_t k = a + s;
         const int st = s % ST;
         if (use_lin) ws.wait(st, p.status);
@@ -832,19 +838,19 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
                     xc[i] = sc.x[i];
                     xn[i] = sn.x[i];
                 }
-            if (s == 0)
+            if (kRel<T> && s == 0)
 #pragma unroll
                 for (int i = 0; i < 5; ++i) m[i] += G.r[i] - xc[i];
             if (cur.is_head(k)) {
                 load_prior(p, cur.b, m, P);
 #pragma unroll
-                for (int i = 0; i < 5; ++i) m[i] -= xc[i];
+                for (int i = 0; i < 5 && kRel<T>; ++i) m[i] -= xc[i];
             } else {
                 Obs<T> ob;
                 if constexpr (use_lin) obs_from_stage<K>(ws, st, xc, ob);
                 else form_obs<K>(p, cur.b, sc, fc, ob);
                 T mn[5], Pn[15];
-                ok &= kf_update<FS, true>(ob, m, P, mn, Pn);
+                ok &= kf_update<FS, kRel<T>>(ob, m, P, mn, Pn);
 #pragma unroll
                 for (int i = 0; i < 5; ++i) m[i] = mn[i];
 #pragma unroll
@@ -856,7 +862,10 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
                 for (int i = 0; i < 5; ++i) g.m[i] = m[i];
 #pragma unroll
                 for (int i = 0; i < 15; ++i) g.P[i] = P[i];
-                damp_gauss(g, lm_of(p.model, cur.b));
+                T xb[5];
+#pragma unroll
+                for (int i = 0; i < 5; ++i) xb[i] = kRel<T> ? T(0) : xc[i];
+                damp_gauss(g, xb, lm_of(p.model, cur.b));
 #pragma unroll
                 for (int i = 0; i < 5; ++i) m[i] = g.m[i];
 #pragma unroll
@@ -868,9 +877,9 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
                 if constexpr (use_lin) trans_from_stage<K>(p, ws, st, 0, xc, tr);
                 else form_trans<K>(p, sc, fc, tr);
                 T mp[5], FP[25], Pp[15];
-                predict<FS, true>(tr, m, P, mp, FP, Pp);
+                predict<FS, kRel<T>>(tr, m, P, mp, FP, Pp);
 #pragma unroll
-                for (int i = 0; i < 5; ++i) m[i] = mp[i] + (xc[i] - xn[i]);   // from the next nominal on
+                for (int i = 0; i < 5; ++i) m[i] = kRel<T> ? mp[i] + (xc[i] - xn[i]) : mp[i];   // from the next nominal on
 #pragma unroll
                 for (int i = 0; i < 15; ++i) P[i] = Pp[i];
             }
@@ -880,7 +889,7 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
         }
         if (use_lin) {
             __syncwarp();   // every lane is done with the stage: refill it
-            if (s + ST < p.L) ws.issue(lin_warp<K>(p, s + ST, lane), st);
+            if (s + ST < steps) ws.issue(lin_warp<K>(p, s + ST, lane), st);
         }
     }
     if (use_lin) wpar = ws.parity;
@@ -889,7 +898,7 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
 
 // The same over given arrays, with the log-likelihoods if they are wanted.
 template <typename T>
-PES_DEV bool rerun_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, const Gauss<T>& G, T* wstage,
+PES_DEV bool rerun_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, int steps, const Gauss<T>& G, T* wstage,
                                  uint64_t* wbar, uint32_t& wpar)
 {
     bool ok = true;
@@ -905,10 +914,10 @@ PES_DEV bool rerun_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int 
     FilterStream<T> ws;
     ws.init(wstage, wbar, wpar);
     ws.issue(array_warp<kFilterIn>(p, 0, lane), 0);
-    if (p.L > 1) ws.issue(array_warp<kFilterIn>(p, 1, lane), 1);
+    if (steps > 1) ws.issue(array_warp<kFilterIn>(p, 1, lane), 1);
     int st = 0;
 #pragma unroll 1
-    for (int s = 0; s < p.L; ++s) {
+    for (int s = 0; s < steps; ++s) {
         const int64_t k = a + s;
         const int other = st == 0 ? 2 : st - 1;   // the stage of steps s - 1 and s + 2
         ws.wait(st, p.status);
@@ -922,7 +931,7 @@ PES_DEV bool rerun_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int 
             predict(tr, m, P, mp, FP, Pp);
         }
         __syncwarp();   // every lane is done with step s - 1
-        if (s + 2 < p.L) ws.issue(array_warp<kFilterIn>(p, s + 2, lane), other);
+        if (s + 2 < steps) ws.issue(array_warp<kFilterIn>(p, s + 2, lane), other);
         if (k < e) {
             if (head) {
                 load_prior(p, cur.b, m, P);
@@ -981,15 +990,20 @@ PES_DEV bool chunk_selem(const KParams<T>& p, int64_t a, int64_t e, const FElem<
     for (int i = 0; i < 5; ++i) u[i] = f.eta[i] - u[i];
     sv(D, u, Du);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) md[i] = dm[i] + Du[i];
-    felem_ref(f, ref);
-    selem_set_refs(el, ref, f.xr);
+    for (int i = 0; i < 5; ++i) {
+        dm[i] += Du[i];
+        md[i] = kRel<T> ? dm[i] : G.m[i] + Du[i];   // from xr, or absolute
+    }
+    if (kRel<T>) {
+        felem_ref(f, ref);
+        selem_set_refs(el, ref, f.xr);
+    }
     if (cur.next <= e) {
         selem_last(el, md, D);
         return true;
     }
     T mp[5], AD[25], Pp[15];
-    mv(f.A, md, mp);
+    mv(f.A, dm, mp);
 #pragma unroll
     for (int i = 0; i < 5; ++i) mp[i] += f.b[i];
     m_s(f.A, D, AD);
@@ -1020,7 +1034,7 @@ PES_DEV bool array_selem(const SmoothStream<T>& ws, int i, bool tail, SElem<T>& 
 // Smoothing, level 1 in MODE_SMOOTH: fold the chunk's smoothing elements from
 // the given filtered moments and transitions.
 template <typename T>
-PES_DEV bool fold_smoother_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, SElem<T>& accS, T* wstage,
+PES_DEV bool fold_smoother_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, int steps, SElem<T>& accS, T* wstage,
                                   uint64_t* wbar, uint32_t& wpar)
 {
     bool ok = true;
@@ -1031,9 +1045,9 @@ PES_DEV bool fold_smoother_arrays(const KParams<T>& p, int64_t a, int64_t e, int
     ws.init(wstage, wbar, wpar);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-        if (i < p.L) ws.issue(array_warp<kSmoothIn>(p, i, lane), i);
+        if (i < steps) ws.issue(array_warp<kSmoothIn>(p, i, lane), i);
 #pragma unroll 1
-    for (int s = 0; s < p.L; ++s) {
+    for (int s = 0; s < steps; ++s) {
         ws.wait(s & 1, p.status);
         if (a + s < e) {
             cur.forward(a + s);
@@ -1042,7 +1056,7 @@ PES_DEV bool fold_smoother_arrays(const KParams<T>& p, int64_t a, int64_t e, int
             combine_smoother(accS, el, accS);
         }
         __syncwarp();
-        if (s + 2 < p.L) ws.issue(array_warp<kSmoothIn>(p, s + 2, lane), s & 1);
+        if (s + 2 < steps) ws.issue(array_warp<kSmoothIn>(p, s + 2, lane), s & 1);
     }
     wpar = ws.parity;
     return ok;
@@ -1050,7 +1064,7 @@ PES_DEV bool fold_smoother_arrays(const KParams<T>& p, int64_t a, int64_t e, int
 
 // Smoothing, level 5 in MODE_SMOOTH.
 template <typename T>
-PES_DEV bool rts_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, const Gauss<T>& G, T* wstage,
+PES_DEV bool rts_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, int steps, const Gauss<T>& G, T* wstage,
                         uint64_t* wbar, uint32_t& wpar)
 {
     bool ok = true;
@@ -1063,10 +1077,10 @@ PES_DEV bool rts_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, con
     ws.init(wstage, wbar, wpar);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-        if (i < p.L) ws.issue(array_warp<kSmoothIn>(p, p.L - 1 - i, lane), i);
+        if (i < steps) ws.issue(array_warp<kSmoothIn>(p, steps - 1 - i, lane), i);
     int st = 0;
 #pragma unroll 1
-    for (int sidx = p.L - 1; sidx >= 0; --sidx, st ^= 1) {
+    for (int sidx = steps - 1; sidx >= 0; --sidx, st ^= 1) {
         const int64_t k = a + sidx;
         ws.wait(st, p.status);
         if (k < e) {
@@ -1099,7 +1113,7 @@ PES_DEV bool rts_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, con
 // stored linearisation, if any) arrive through a warp stream and the smoothed
 // moments replace the nominal in place.
 template <int K, typename T>
-PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, const Gauss<T>& G, bool write_P,
+PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, int steps, const Gauss<T>& G, bool write_P,
                        bool want_norm, double* conv, int& nb, double& num, double& den, T* wstage, uint64_t* wbar,
                        uint32_t& wpar)
 {
@@ -1121,17 +1135,17 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
     ws.init(wstage, wbar, wpar);
 #pragma unroll
     for (int i = 0; i < ST; ++i)
-        if (i < p.L) issue(p.L - 1 - i, i);
+        if (i < steps) issue(steps - 1 - i, i);
     // the nominal a step ahead
     T xc[5], xn[5];   // nominals of states k, k-1
     if (any) {
         load_nominal(p, lane_ix(p, e - 1 - a, lane), xc);
 #pragma unroll
-        for (int c = 0; c < 5; ++c) s.m[c] += G.r[c] - xc[c];
+        for (int c = 0; c < 5 && kRel<T>; ++c) s.m[c] += G.r[c] - xc[c];
     }
     int st = 0;
 #pragma unroll 1
-    for (int sidx = p.L - 1; sidx >= 0; --sidx) {
+    for (int sidx = steps - 1; sidx >= 0; --sidx) {
         const int64_t k = a + sidx;
         ws.wait(st, p.status);
         if (k < e) {
@@ -1160,7 +1174,7 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
                     form_trans<K>(p, in, fc, tr);
                 }
                 T mp[5], FP[25], Pp[15];
-                predict<FS, true>(tr, m, P, mp, FP, Pp);
+                predict<FS, kRel<T>>(tr, m, P, mp, FP, Pp);
                 SElem<T> ec;
                 ok &= selem_from_prediction(m, P, FP, Pp, mp, ec);
                 apply_smoother(ec, s, s);
@@ -1169,7 +1183,7 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
                 finite = finite && isfinite(s.m[i]);
-                p.x[i * p.cs + ix] = xc[i] + s.m[i];
+                p.x[i * p.cs + ix] = kRel<T> ? xc[i] + s.m[i] : s.m[i];
             }
             if (!finite) atomicOr(p.status, ST_NONFINITE);
             if (write_P) {
@@ -1188,7 +1202,7 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
                 }
 #pragma unroll
                 for (int i = 0; i < 5; ++i) {
-                    const T x = xc[i] + s.m[i];
+                    const T x = kRel<T> ? xc[i] + s.m[i] : s.m[i];
                     const double dv = double(x) - double(xc[i]);
                     num += dv * dv;
                     den += double(x) * double(x);
@@ -1196,7 +1210,7 @@ PES_DEV bool rts_chunk(const KParams<T>& p, int64_t a, int64_t e, int lane, cons
             }
 #pragma unroll
             for (int c = 0; c < 5; ++c) {   // from the nominal of k - 1 on
-                s.m[c] += xc[c] - xn[c];
+                if (kRel<T>) s.m[c] += xc[c] - xn[c];
                 xc[c] = xn[c];
             }
         }
@@ -1256,11 +1270,14 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
     __syncthreads();
 
     const int t = threadIdx.x;
-    const int lane = blockIdx.x * NT + t;
-    const int64_t a = min((int64_t)lane * p.L, p.N);
+    // the block's first lpb threads, whole warps, are lanes; the others help with
+    // the trees only
+    const int lane = blockIdx.x * p.lpb + t;
+    const int steps = t < p.lpb ? p.L : 0;
+    const int64_t a = steps ? min((int64_t)lane * p.L, p.N) : p.N;
     const int64_t e = min(a + (int64_t)p.L, p.N);
     // lanes of this block with a chunk (its first ones); one identity if none
-    const int nl = (int)max((int64_t)1, min((int64_t)NT, (p.N + p.L - 1) / p.L - (int64_t)blockIdx.x * NT));
+    const int nl = (int)max((int64_t)1, min((int64_t)p.lpb, (p.N + p.L - 1) / p.L - (int64_t)blockIdx.x * p.lpb));
     unsigned gen = 0;
     bool ok = true;
 
@@ -1283,7 +1300,7 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
             FElem<T> acc;
             // the fold's prefetch goes to memory beside the leaves
             if constexpr (K == KK_ARRAYS)
-                ok &= fold_filter_arrays(p, a, e, lane, acc, smem + FE * NT + (size_t)warp * 2 * kFilterIn * 32, wbar, wpar);
+                ok &= fold_filter_arrays(p, a, e, lane, steps, acc, smem + FE * NT + (size_t)warp * 2 * kFilterIn * 32, wbar, wpar);
             else
                 ok &= fold_filter_chunk<K>(p, a, e, lane, acc, Prefetch<T, kStateIn>{smem + FE * NT + t, NT, p.x, p.cs});
             PES_PHASE(p, it, 1);
@@ -1300,7 +1317,7 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
             if (do_smooth) ok &= chunk_selem(p, a, e, reinterpret_cast<const FElem<T>*>(smem)[tree_place(min(t, nl - 1), nl)], G, accS);
         } else {
             if constexpr (K == KK_ARRAYS)
-                ok &= fold_smoother_arrays(p, a, e, lane, accS, smem + SE * NT + (size_t)warp * 2 * kSmoothIn * 32, wbar, wpar);
+                ok &= fold_smoother_arrays(p, a, e, lane, steps, accS, smem + SE * NT + (size_t)warp * 2 * kSmoothIn * 32, wbar, wpar);
         }
         __syncthreads();   // the smoother's tree and the stream stages overlap the filter's
         if (do_smooth) {
@@ -1310,10 +1327,10 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
         PES_PHASE(p, it, 6);
         if (do_filter) {
             if constexpr (K == KK_ARRAYS) {
-                ok &= rerun_filter_arrays(p, a, e, lane, G, smem + (size_t)warp * 3 * kFilterIn * 32, wbar, wpar);
+                ok &= rerun_filter_arrays(p, a, e, lane, steps, G, smem + (size_t)warp * 3 * kFilterIn * 32, wbar, wpar);
             } else {
                 constexpr int kStage = kLinStages<K> * kLinScalars<K> * 32;
-                ok &= rerun_filter_chunk<K>(p, a, e, lane, G, smem + M::kAfterSmootherTree + (size_t)warp * kStage, wbar, wpar);
+                ok &= rerun_filter_chunk<K>(p, a, e, lane, steps, G, smem + M::kAfterSmootherTree + (size_t)warp * kStage, wbar, wpar);
             }
             if (track && blockIdx.x == 0) {
                 // the accumulators of the next iteration were last read before
@@ -1337,10 +1354,10 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
             double num = 0.0, den = 0.0;
             double* conv = p.conv + (size_t)(it & 1) * 2 * p.B;
             if constexpr (K == KK_ARRAYS) {
-                ok &= rts_arrays(p, a, e, lane, Gs, smem + (size_t)warp * 2 * kSmoothIn * 32, wbar, wpar);
+                ok &= rts_arrays(p, a, e, lane, steps, Gs, smem + (size_t)warp * 2 * kSmoothIn * 32, wbar, wpar);
             } else {
                 constexpr int kStage = kRtsStages<K> * (HAND + (kStoreLin<K> ? kLinTrans<K> : 0)) * 32;
-                ok &= rts_chunk<K>(p, a, e, lane, Gs, write_P, track, conv, nb, num, den, smem + (size_t)warp * kStage, wbar, wpar);
+                ok &= rts_chunk<K>(p, a, e, lane, steps, Gs, write_P, track, conv, nb, num, den, smem + (size_t)warp * kStage, wbar, wpar);
             }
             __syncthreads();
             PES_PHASE(p, it, 11);

@@ -537,19 +537,35 @@ PES_DEV void lin_obs_cubature(const DevModel<T>& m, int b, const T* xbar, const 
 
 // ---- the coordinated turn, model known at compile time -------------------------
 
+// Whether the smoother kernel's chunks keep means as deviations from the nominal:
+// in FP32, where rounding positions at every step shows; in FP64 it does not, and
+// absolute means save the re-referencing.
+template <typename T>
+constexpr bool kRel = sizeof(T) == 4;
+
 // lin_trans_taylor of the coordinated turn; only F's general entries are written,
-// and fx is f(xn) - xn.
+// and fx is f(xn) - xn where kRel.
 template <typename T>
 PES_DEV void ct_trans_taylor(const DevModel<T>& m, const T* xn, Trans<T>& tr)
 {
     const T dt = m.dt;
     const CTCoef<T> k = ct_coef(xn[4], dt);
     ct_jacobian(xn, k, dt, tr.F);
-    tr.fx[0] = k.A1 * xn[2] - k.A2 * xn[3];
-    tr.fx[1] = k.A2 * xn[2] + k.A1 * xn[3];
-    tr.fx[2] = (k.c - T(1)) * xn[2] - k.s * xn[3];
-    tr.fx[3] = k.s * xn[2] + (k.c - T(1)) * xn[3];
-    tr.fx[4] = T(0);
+    if (kRel<T>) {
+        tr.fx[0] = k.A1 * xn[2] - k.A2 * xn[3];
+        tr.fx[1] = k.A2 * xn[2] + k.A1 * xn[3];
+        tr.fx[2] = (k.c - T(1)) * xn[2] - k.s * xn[3];
+        tr.fx[3] = k.s * xn[2] + (k.c - T(1)) * xn[3];
+        tr.fx[4] = T(0);
+    } else {
+        T inc[5];
+        ct_increment(xn, k, inc);
+        tr.fx[0] = xn[0] + inc[0];
+        tr.fx[1] = xn[1] + inc[1];
+        tr.fx[2] = inc[2];
+        tr.fx[3] = inc[3];
+        tr.fx[4] = inc[4];
+    }
 #pragma unroll
     for (int i = 0; i < 5; ++i) tr.xn[i] = xn[i];
 #pragma unroll
@@ -708,13 +724,16 @@ PES_DEV void ct_trans_cubature(const DevModel<T>& m, const T* xbar, const T* L, 
             for (int i = 1; i < 5; ++i) s = fma(U[r * 5 + i], U[q * 5 + i], s);
             tr.Q[si(r, q)] = fma(s, m.sp_w, fma(m.sp_w0c * zdev[r], zdev[q], m.Q[si(r, q)]));
         }
-    // f(xbar) and the points' mean deviation, less xbar; f(xbar) is rounded as a state
-    // is, so that a run's results stay next to those of the other sigma-point rules
-    tr.fx[0] = (xbar[0] + inc[0] + zdev[0]) - xbar[0];
-    tr.fx[1] = (xbar[1] + inc[1] + zdev[1]) - xbar[1];
-    tr.fx[2] = (inc[2] + zdev[2]) - xbar[2];
-    tr.fx[3] = (inc[3] + zdev[3]) - xbar[3];
-    tr.fx[4] = T(0);
+    // f(xbar) and the points' mean deviation, rounded as a state is, so that a run's
+    // results stay next to those of the other sigma-point rules; less xbar where kRel
+    tr.fx[0] = xbar[0] + inc[0] + zdev[0];
+    tr.fx[1] = xbar[1] + inc[1] + zdev[1];
+    tr.fx[2] = inc[2] + zdev[2];
+    tr.fx[3] = inc[3] + zdev[3];
+    tr.fx[4] = kRel<T> ? T(0) : xbar[4];
+    if (kRel<T>)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tr.fx[i] -= xbar[i];
 #pragma unroll
     for (int i = 0; i < 5; ++i) tr.xn[i] = xbar[i];
 }

@@ -25,10 +25,15 @@ namespace {
 
 constexpr int64_t kMaxStates = PES_NOALLOC_MAX_STATES;
 constexpr int32_t kMaxBatch = PES_NOALLOC_MAX_BATCH;
-constexpr int kMaxBlocks = 8;                  // cooperative blocks one call may use
-constexpr int kMaxThreads = 256;               // threads per block of any compiled configuration
-// Lane-major arrays hold L * lanes >= N states: N plus one launch's lanes at most.
-constexpr int64_t kLaneCap = kMaxStates + (int64_t)kMaxBlocks * kMaxThreads;
+// Cooperative blocks one call may use: enough for the shape that pes_ieks_run
+// takes for as many states, of at least 32 lanes per block.
+constexpr int kMaxBlocks = (int)(kMaxStates / 32);
+// Lane-major arrays hold L * lanes >= N states: a block's lanes more than N at
+// most, of at most 256 lanes and, at these sizes, 9 steps. A multiple of 256, so
+// that every region starts on 16 bytes and more, as the kernels' copies need.
+constexpr int kMaxPadding = 10 * 256;
+constexpr int64_t kLaneCap = kMaxStates + kMaxPadding;
+static_assert(kMaxPadding >= 9 * (256 + 1) && kLaneCap % 256 == 0, "the padding of nine steps");
 
 // Scratch layout, in doubles (a float run uses the first half of each region).
 constexpr size_t kHand = (size_t)pes::HAND * kLaneCap;
@@ -39,6 +44,7 @@ constexpr size_t kAggS = (size_t)kMaxBlocks * 2 * pes::SE;
 constexpr size_t kConv = (size_t)4 * kMaxBatch;
 constexpr size_t kSens = (size_t)4 * kMaxBatch;
 constexpr size_t kWords = 4;                   // barrier counter, status, iteration count (one double each)
+static_assert(kHand % 32 == 0 && kLanes % 32 == 0 && kLin % 32 == 0 && kAggF % 32 == 0 && kAggS % 32 == 0, "alignment");
 constexpr size_t kTotal = kHand + kLanes + kLin + kAggF + kAggS + kConv + kSens + kWords;
 
 constexpr int kMaxDevices = 64;
@@ -82,7 +88,7 @@ pes_status setup(int dev)
     h.max_states = kMaxStates;
     h.max_batch = kMaxBatch;
     h.nb_max = kMaxBlocks;
-    h.nl_max = kMaxBlocks * kMaxThreads;
+    h.nl_max = kMaxPadding;
     h.hand = p;
     p += kHand;
     h.lanes = p;

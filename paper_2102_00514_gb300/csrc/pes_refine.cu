@@ -323,8 +323,8 @@ __global__ void __launch_bounds__(NT, 1) refine_scan_kernel(const RefineParams p
     RState* gblock = gs + NT;
     constexpr bool W = FWD;
     const int t = threadIdx.x;
-    const int lane = blockIdx.x * NT + t;
-    const int64_t a = min((int64_t)lane * p.L, p.N);
+    const int lane = blockIdx.x * p.lpb + t;
+    const int64_t a = t < p.lpb ? min((int64_t)lane * p.L, p.N) : p.N;
     const int64_t e = min(a + (int64_t)p.L, p.N);
     // level 1: the chunk's composition, from the state that the re-run comes to
     // last: what was read last, the first states of the re-run, is then still in

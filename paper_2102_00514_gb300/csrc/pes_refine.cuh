@@ -49,6 +49,7 @@ struct RefineParams {
     int64_t N;
     const int64_t* offsets;   // [B+1], device
     int B;
+    int lpb;                  // lanes per block
     int L, NL;                // lane-major geometry of every per-state array below
     int64_t cs;               // component stride: L * NL
     DevModel<float> model;
