@@ -31,10 +31,12 @@ template <> PES_DEV double tsqrt<double>(double x) { return sqrt(x); }
 
 // Reciprocal square root and reciprocal on the pivot chains of the
 // factorisations: FP32 takes the hardware approximations (rsqrtf, and
-// __fdividef for the reciprocal: a few ulp), FP64 the correctly rounded forms.
+// __fdividef for the reciprocal: a few ulp), FP64 rsqrt (1 ulp; a square root and
+// a division are twenty instructions more of the slow FP64 pipe each time: T = 500,
+// FP64, 10 iterations 4,660 -> 4,190 us, T = 10,000 cubature 4,290 -> 3,910 us).
 template <typename T> PES_DEV T trsqrt(T x);
 template <> PES_DEV float trsqrt<float>(float x) { return rsqrtf(x); }
-template <> PES_DEV double trsqrt<double>(double x) { return 1.0 / sqrt(x); }
+template <> PES_DEV double trsqrt<double>(double x) { return rsqrt(x); }
 template <typename T> PES_DEV T trcp(T x);
 template <> PES_DEV float trcp<float>(float x) { return __fdividef(1.0f, x); }
 template <> PES_DEV double trcp<double>(double x) { return 1.0 / x; }
