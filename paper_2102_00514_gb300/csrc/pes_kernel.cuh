@@ -4,13 +4,13 @@
 //   (c) the reverse associative scan of smoothing elements (Eqs. 17-19),
 // and re-linearises about the smoothed means between iterations (Sec. 3).
 //
-// Scan layout. The N states are split into NB x NT contiguous chunks of L
-// steps, one per thread ("lane"). A lane's filtering element maps the predicted
+// Scan layout. The N states are split into contiguous chunks of L steps, one per
+// thread ("lane"); the first lpb of a block's NT threads are lanes. A lane's filtering element maps the predicted
 // state at its chunk's start to the predicted state at the next chunk's start:
 // update and predict, step by step. Both scans are three-level
 // reduce-then-scans over the lanes:
 //   1. every lane folds its chunk into one filtering element;
-//   2. a tree over the NT lane elements of a block in shared memory gives the
+//   2. a tree over the lane elements of a block in shared memory gives the
 //      block's element, published to global memory (pes_tree.cuh);
 //   3. after a grid barrier every block reduces the elements of the blocks
 //      before it; since the sequence starts with a prior, that is a Gaussian;
@@ -25,16 +25,22 @@
 // smoothing scan needs no fold of per-step elements (350 multiply-adds per
 // state), and its levels 2 and 3 do not depend on the filtering re-run: its
 // block elements are published before the re-run, which hides the wait for the
-// other blocks' (measured at T = 2^20, FP32: see pes_persistent_kernel). The RTS
-// pass then builds each step's element from the kept filtered moments.
+// other blocks'. The RTS pass then builds each step's element from the kept
+// filtered moments. (Taylor, FP32, T = 2^20: an iteration 245 -> 175 us, of which
+// re-run and smoothing up-sweep 100 -> 40, the wait for the smoothing elements 16
+// -> 1, RTS 35 -> 50.)
 //
-// In FP32, within a chunk means are kept as deviations from the nominal (the filter's, the
-// fold's and the smoother's), re-referenced from state to state by the difference
-// of their nominals, and the trees' elements carry reference points: positions of
+// What bounds it at that size: the sequential passes (fold 34, re-run 32, RTS 50
+// us) are issue-bound with two warps per sub-partition at 255 registers, the
+// trees (34 + 16 us) are levels of one operator's latency.
+//
+// In FP32, within a chunk means are kept as deviations from the nominal (the
+// filter's, the fold's and the smoother's), re-referenced from state to state by
+// the difference of their nominals, and the trees' elements carry reference points: positions of
 // tens to thousands of units would otherwise be rounded at every step and level,
 // and the rounding of the means is what the next iteration's linearisation
 // amplifies (batch of 1,024 trajectories after three FP32 iterations, against 64
-// bits: means 6.0e-7 -> 1.5e-7, covariances 7e-6 -> 2.5e-6).
+// bits: means 6.1e-7 -> 1.0e-7, covariances 7e-6 -> 2.5e-6).
 //
 // A chunk's passes read only its own states' nominal, so no barrier separates
 // iterations: the block aggregates are double-buffered, and a block can reach
@@ -72,9 +78,9 @@ template <int K>
 constexpr bool kStoreLin = kSigma<kLinOf<K>>;
 // Scalars stored per state; the transition's are kLinTrans of them, from
 // kLinTransAt. Compact form (the coordinated turn's cubature regression): F rows
-// 0-3 (20), fx (4; less xn in FP32), Q' (10), H (4), r (2), R' (3); the nominal is read from the
-// trajectory, the rest is constant. Dense form: H (10), r (2), R' (3), xn (5),
-// F (25), fx (5), Q' (15).
+// 0-3 (20), fx (4; less xn in FP32), Q' (10), H (4), r (2), R' (3); the nominal is read
+// from the trajectory, the rest is constant. Dense form: H (10), r (2), R' (3),
+// xn (5), F (25), fx (5), Q' (15).
 template <int K>
 constexpr int kLinScalars = K == KK_CUBATURE ? 43 : LINS;
 template <int K>

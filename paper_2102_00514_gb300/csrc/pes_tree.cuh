@@ -14,7 +14,9 @@
 // the block's threads: operator i of m on threads i, i + m', i + 2 m', ...
 // (m' >= m a power of two), each taking every (NT / m')-th task. The
 // factorisation (about 260 instructions) is repeated in each of them, a task is
-// about 130. The other operators are split by rows in the same way.
+// about 130. The other operators are split by rows in the same way. (61 FP32
+// lanes: up-sweep 15.7 -> 8.4 us, down-sweep 6.8 -> 4.8; 125 FP64 lanes: 50 -> 26
+// us per level of the up-sweep, rsqrt pivots included.)
 //
 // Elements are stored whole (76 and 60 scalars, padded), one after another: the
 // operands arrive in 16-byte loads, and at these strides consecutive elements'
