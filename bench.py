@@ -222,7 +222,7 @@ def peaks_file():
 
 
 KERNEL_HEADERS = ("pes_async.cuh", "pes_kernel.cuh", "pes_launch_impl.cuh", "pes_math.cuh", "pes_model.cuh",
-                  "pes_ops.cuh")
+                  "pes_ops.cuh", "pes_tree.cuh")
 
 
 def kernel_source_hash():
