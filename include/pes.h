@@ -343,7 +343,7 @@ pes_status pes_traj_iterations(pes_handle* h, int32_t* iters, int32_t B, void* s
  * latency-critical code that cannot afford an allocation, which may
  * synchronise the device. This entry point calls no cudaMalloc, cudaFree or
  * other allocating routine. Its scratch is one fixed array in the library's
- * device memory, about 11 MB, which every GPU that loads the library holds
+ * device memory, about 10 MB, which every GPU that loads the library holds
  * until the process exits.
  *
  * Arguments, layouts and results are those of pes_ieks_run (DEVICE pointers),
