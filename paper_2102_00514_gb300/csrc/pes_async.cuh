@@ -7,6 +7,13 @@
 // stage, the copies of the next steps land in the others. One lane issues the
 // copies; every lane reads its own column of the stage.
 //
+// Bulk copies read global memory through the asynchronous proxy, the lanes write
+// it through the generic one. A buffer that a kernel both writes and streams
+// needs, between the two: in every writing lane, after its last store of the
+// pass, stores_before_bulk_reads(); then a barrier (__syncwarp or __syncthreads)
+// that the writing lanes share with the lane that issues the copies. What an
+// earlier kernel wrote needs neither.
+//
 // Every wait is bounded: after about a second a wait gives up, sets
 // ST_TIMEOUT in the status word and returns, so the kernel always ends.
 #pragma once
@@ -27,6 +34,10 @@ PES_DEV void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.clust
 
 // Order earlier generic-proxy shared-memory accesses before later bulk copies.
 PES_DEV void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Order this thread's earlier stores to global memory before bulk copies that
+// read them, issued by any thread of the block after a barrier with it.
+PES_DEV void stores_before_bulk_reads() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 // The one arrival of a phase of `bar`, which completes with `bytes` copied.
 PES_DEV void bulk_expect(uint64_t* bar, uint32_t bytes)

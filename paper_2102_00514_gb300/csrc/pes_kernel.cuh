@@ -654,6 +654,7 @@ PES_DEV bool fold_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int la
         load_nominal(p, lane, acc.xr);
     }
     if (!prefetch) pf.wait_all();
+    if (store_lin) stores_before_bulk_reads();   // the re-run and the RTS pass stream them, after block barriers
     return ok;
 }
 
@@ -899,6 +900,7 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
         }
     }
     if (use_lin) wpar = ws.parity;
+    stores_before_bulk_reads();   // the RTS pass streams the filtered moments, after the grid barrier's block barrier
     return ok;
 }
 
