@@ -1297,7 +1297,9 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
     bool converged = false;
 #pragma unroll 1
     for (it = 0; it < p.iters; ++it) {
-        if (*(volatile int*)p.status & (ST_TIMEOUT | ST_BADARG)) break;
+        // another block may set the bit while this one reads it: one answer for all
+        // its threads, which meet at barriers from here on
+        if (__syncthreads_or(*(volatile int*)p.status & (ST_TIMEOUT | ST_BADARG))) break;
         const bool last = (it == p.iters - 1);
         T* aggF = p.aggF + (size_t)(it & 1) * p.agg_blocks * FE;
         T* aggS = p.aggS + (size_t)(it & 1) * p.agg_blocks * SE;

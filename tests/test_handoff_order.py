@@ -2,7 +2,8 @@
 the same launch reads by bulk copies: the copies go through another proxy than the
 stores, so every writing lane has to fence after its last store. A missing fence
 shows in no result on most runs, so the order is checked in the source here, and on
-the GPU by runs whose first copy is of the step written last."""
+the GPU by runs whose first copy is of the step written last. The same for the exit
+of the iterations' loop, which all of a block's threads have to take together."""
 import os
 import re
 
@@ -29,6 +30,15 @@ def test_stores_are_fenced_before_the_pass_returns(name, stores):
     code = body(name)
     last = max(code.rindex(s) for s in stores)
     assert FENCE in code[last:], f"{name}: stores that a later pass streams are not fenced"
+
+
+def test_blocks_leave_the_iterations_as_one():
+    """The status word can change while a block's warps read it; a loop exit taken
+    by some of them only would leave the others at barriers without them."""
+    src = open(KERNEL).read()
+    loop = src[src.index("for (it = 0; it < p.iters; ++it) {"):]
+    exit_line = next(l for l in loop.splitlines() if "p.status" in l and "break;" in l)
+    assert "__syncthreads_or(" in exit_line
 
 
 @pytest.mark.gpu
