@@ -15,7 +15,6 @@
 // (I + J_j C_i)^{-1} = I - J_j D.
 #pragma once
 
-#include "pes_ff.cuh"
 #include "pes_model.cuh"
 
 namespace pes {
@@ -577,55 +576,49 @@ PES_DEV void predict(const Trans<T>& tr, const T* m, const T* P, T* mp, T* FP, T
 }
 
 // Running log-likelihood of a trajectory's measurements: the sum over steps of
-// log N(v; 0, S) = -1/2 (v^T S^{-1} v + log det S) - log 2 pi, to FP64's accuracy
-// of the given S and v (1e-12 relative). The determinants are multiplied up with
-// the exponent kept apart, and one logarithm is taken at the end. FP32 runs form
-// the terms in float-float where the values allow it (neither near the ends of
-// the range nor a cancelling determinant): the FP64 pipe issues an instruction
-// per warp every 64 cycles, and with a logarithm and a quotient per step it was
-// more than half of the filter scan's re-run (41 us at N = 128,128).
+// log N(v; 0, S) = -1/2 (v^T S^{-1} v + log det S) - log 2 pi, every term in FP64.
+// Bound by the FP64 pipe, which issues one instruction per warp every 64 cycles: a
+// step takes about 18, of them 9 of the quotient. The determinants are multiplied
+// up, their binary exponents kept apart by integer instructions, and one logarithm
+// is taken at the end (a product is half an ulp of 1 off in a step, a logarithm per
+// step was up to an ulp of its value, and made the filter scan's re-run 41 us at N =
+// 128,128, FP32). A determinant that is negative or NaN makes the result NaN, as
+// its own logarithm would.
 template <typename T>
 struct LogLik {
-    double q = 0.0, det = 1.0;
-    ff qf = {0.0f, 0.0f}, df = {1.0f, 0.0f};
+    double q = 0.0, det = 1.0;   // det in [1, 2), or 0, infinite or NaN
     int exponent = 0, steps = 0;
+    // the exponent of a normal x out of it
+    PES_DEV void split(double& x)
+    {
+        const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+        if (e > 0 && e < 0x7ff) {
+            exponent += e - 1023;
+            x = __hiloint2double((hi & 0x800fffff) | 0x3ff00000, __double2loint(x));
+        }
+    }
     PES_DEV void add(T s00, T s01, T s11, T v0, T v1)
     {
         ++steps;
-        if constexpr (sizeof(T) == 4) {
-            const float a = s00, b = s11, top = fmaxf(fabsf(v0), fabsf(v1));
-            const ff p = two_prod(a, b), r = two_prod(s01, s01);
-            // both products exact; their difference to 2^-48 of them
-            const ff h = two_sum(p.hi, -r.hi);
-            const ff d = fast_two_sum(h.hi, __fadd_rn(h.lo, __fsub_rn(p.lo, r.lo)));
-            if (fminf(a, b) > 1e-7f && fmaxf(a, b) < 1e7f && top < 1e5f && d.hi > 1e-3f * p.hi) {
-                const ff n0 = ff_mul_f(two_prod(b, v0), v0), n1 = ff_mul_f(two_prod(a, v1), v1);
-                const ff n2 = ff_mul_f(two_prod(-2.0f * s01, v0), v1);
-                qf = ff_add(qf, ff_div(ff_add(ff_add(n0, n2), n1), d));
-                df = ff_mul(df, d);
-                const int e = (__float_as_int(df.hi) >> 23) - 127;   // df.hi > 0, normal
-                const float scale = __int_as_float((127 - e) << 23);
-                df.hi *= scale;
-                df.lo *= scale;
-                exponent += e;
-                return;
-            }
+        const double c00 = s00, c01 = s01, c11 = s11, c2 = T(-2) * s01, w0 = v0, w1 = v1;
+        double d = fma(-c01, c01, c00 * c11);
+        // v^T adj(S) v
+        q += fma(w0, fma(c2, w1, c11 * w0), w1 * (c00 * w1)) / d;
+        const int hi = __double2hiint(d);
+        if (hi < 0 && d != 0.0) {   // not positive definite
+            d = __longlong_as_double(0x7ff8000000000000LL);
+        } else if ((hi & 0x7ff00000) == 0) {   // subnormal or zero
+            d *= 18014398509481984.0;          // 2^54
+            exponent -= 54;
         }
-        const double c00 = s00, c01 = s01, c11 = s11, w0 = v0, w1 = v1;
-        const double d = c00 * c11 - c01 * c01;
-        q += (c11 * w0 * w0 - 2.0 * c01 * w0 * w1 + c00 * w1 * w1) / d;
+        split(d);
         det *= d;
-        const int hi = __double2hiint(det), e = (hi >> 20) & 0x7ff;
-        if (e > 0 && e < 0x7ff) {   // to [1, 2); zeros, subnormals, infinities and NaN stay
-            exponent += e - 1023;
-            det = __hiloint2double((hi & 0x800fffff) | 0x3ff00000, __double2loint(det));
-        }
+        split(det);
     }
     PES_DEV double value() const
     {
         const double ln2 = 0.69314718055994530942, log_2pi = 1.8378770664093454836;
-        const double quad = q + ((double)qf.hi + (double)qf.lo);
-        return -0.5 * (quad + (log(det * ((double)df.hi + (double)df.lo)) + exponent * ln2)) - steps * log_2pi;
+        return -0.5 * (q + (log(det) + exponent * ln2)) - steps * log_2pi;
     }
 };
 
