@@ -295,7 +295,8 @@ pes_status pes_ieks_run_sequential(pes_handle* h, const pes_model* model, pes_me
  * lowers the trajectory's MAP objective
  *   J = 1/2 |x_0 - m0|^2_{P0^-1} + 1/2 sum_k |x_k - f(x_{k-1})|^2_{Q^-1}
  *       + 1/2 sum_k |y_k - h(x_k)|^2_{R^-1}
- * (bearing residuals on the branch nearest zero; evaluated in FP64), and then
+ * (bearing residuals on the branch nearest zero; the step's change of J is
+ * evaluated in FP64, as a change, so that it is told from rounding), and then
  * lambda_b <- lambda_b / nu; otherwise the trajectory's nominal and
  * covariances stay and lambda_b <- lambda_b * nu. Every trajectory starts at
  * lambda0 (> 0), nu > 1. The objective needs a positive definite Q and R

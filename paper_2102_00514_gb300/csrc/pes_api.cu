@@ -746,7 +746,7 @@ static bool inv_spd_packed(const double* S, int n, double* Si)
 // The IEKS with Levenberg-Marquardt steps and adaptive per-trajectory damping
 // (host loop; kernels in pes_lm.cu). Every iteration: keep the nominal, run
 // one damped iteration of the smoother kernel with each trajectory's damping,
-// evaluate the MAP objective, keep or undo each trajectory's step.
+// evaluate what the step changes the MAP objective by, keep or undo it.
 template <typename T>
 static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_precision prec, const void* y,
                                 const int64_t* offsets, int32_t B, int64_t N, const void* m0, const void* P0,
@@ -765,7 +765,7 @@ static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_preci
     if (r != PES_OK) return r;
     if ((r = ensure_refine_workspace(h)) != PES_OK) return r;
     if (!h->lmw) {
-        const size_t per = 5 * sizeof(double) + 3 * sizeof(int);
+        const size_t per = 4 * sizeof(double) + 3 * sizeof(int);
         PES_CUDA(h, cudaMalloc(&h->lmw, per * (size_t)h->max_batch + 16));
     }
     const int NL = s.nb * s.lpb;
@@ -777,12 +777,11 @@ static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_preci
     T* Pold = xold + 5 * cs;
     const size_t Bm = (size_t)h->max_batch;
     double* dw = static_cast<double*>(h->lmw);
-    lp.cost = dw;
-    lp.cost_new = dw + Bm;
-    lp.num = dw + 2 * Bm;
-    lp.den = dw + 3 * Bm;
-    T* lam = reinterpret_cast<T*>(dw + 4 * Bm);
-    int* iw = reinterpret_cast<int*>(dw + 5 * Bm);
+    lp.change = dw;
+    lp.num = dw + Bm;
+    lp.den = dw + 2 * Bm;
+    T* lam = reinterpret_cast<T*>(dw + 3 * Bm);
+    int* iw = reinterpret_cast<int*>(dw + 4 * Bm);
     lp.reject = iw;
     lp.accepted = iw + Bm;
     lp.conv_iter = iw + 2 * Bm;
@@ -803,8 +802,6 @@ static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_preci
                                              x_init ? nullptr : lx, lP, st));
     PES_CUDA(h, cudaMemsetAsync(lp.accepted, 0, 2 * Bm * sizeof(int), st));
     PES_CUDA(h, launch_lm_fill<T>(lam, B, lambda0, st));
-    PES_CUDA(h, cudaMemsetAsync(lp.cost, 0, B * sizeof(double), st));
-    PES_CUDA(h, launch_lm_cost<T>(lp, lp.cost, lx, nullptr, ly, (const T*)m0, (const T*)P0, st));
     KParams<T> p{};
     p.N = N; p.offsets = offsets; p.B = B; p.mode = MODE_RUN; p.iters = 1; p.tol = 0.0;
     if ((r = device_model<T>(h, *model, B, st, p.model, PES_IEKS)) != PES_OK) return r;
@@ -817,9 +814,9 @@ static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_preci
     for (it = 1; it <= max_iters; ++it) {
         PES_CUDA(h, cudaMemcpyAsync(xold, lx, sizeof(T) * 20 * cs, cudaMemcpyDeviceToDevice, st));
         if ((r = run_persistent_shaped<T>(h, p, LIN_IEKS, s, st)) != PES_OK) return r;
-        PES_CUDA(h, cudaMemsetAsync(lp.cost_new, 0, 3 * Bm * sizeof(double), st));
+        PES_CUDA(h, cudaMemsetAsync(lp.change, 0, 3 * Bm * sizeof(double), st));
         PES_CUDA(h, cudaMemsetAsync(lp.unconv, 0, sizeof(int), st));
-        PES_CUDA(h, launch_lm_cost<T>(lp, lp.cost_new, lx, xold, ly, (const T*)m0, (const T*)P0, st));
+        PES_CUDA(h, launch_lm_change<T>(lp, lx, xold, ly, (const T*)m0, (const T*)P0, st));
         PES_CUDA(h, launch_lm_decide<T>(lp, lam, it, tol, nu, st));
         PES_CUDA(h, launch_lm_restore<T>(lp, lx, lP, xold, Pold, st));
         if (tol > 0.0) {

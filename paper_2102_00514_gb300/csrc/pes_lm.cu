@@ -1,9 +1,16 @@
 // Device side of the Levenberg-Marquardt iteration with adaptive damping
 // (Sec. 3 names the LM variant of the IEKS; the host loop is
-// pes_ieks_run_lm in pes_api.cu): the MAP objective of every trajectory, the
-// per-trajectory accept/reject decision and damping update, and the restore
-// of a rejected trajectory's nominal. Objective arithmetic is in FP64 for
-// either precision, so that the decisions do not turn on rounding.
+// pes_ieks_run_lm in pes_api.cu): the change of every trajectory's MAP objective
+// by a step, the per-trajectory accept/reject decision and damping update, and
+// the restore of a rejected trajectory's nominal.
+//
+// The change is summed over the states as it is, in FP64 for either precision,
+// and not as the difference of two objectives: near convergence a step of relative
+// size 1e-8 changes the objective by 1e-16 of it, and whether two rounded sums
+// compare as smaller would hang on the order of their additions. With a residual e
+// and its change D, a term's change is 1/2 D^T W (2 e + D); D is formed from the
+// state's change without cancellation (f_change, obs_change). Steps of relative
+// size 1e-9 (a change of 1e-19 of the objective) are then still told apart.
 #include "pes_internal.h"
 #include "pes_lm.cuh"
 
@@ -22,55 +29,96 @@ PES_DEV int traj_of_k(const int64_t* off, int B, int64_t k)
     return lo;
 }
 
-// f(x) of the model in FP64
-PES_DEV void f_model(const LMParams& p, const double* x, double* out)
+// x - f(xp) and its change by the steps d of x and dp of xp, in FP64
+PES_DEV void f_change(const LMParams& p, const double* x, const double* d, const double* xp, const double* dp, double* e,
+                      double* de)
 {
     if (p.kind == MODEL_LINEAR) {
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-            double s = p.c[i];
+            double s = p.c[i], t = 0.0;
 #pragma unroll
-            for (int l = 0; l < 5; ++l) s = fma(p.F[i * 5 + l], x[l], s);
-            out[i] = s;
+            for (int l = 0; l < 5; ++l) {
+                s = fma(p.F[i * 5 + l], xp[l], s);
+                t = fma(p.F[i * 5 + l], dp[l], t);
+            }
+            e[i] = x[i] - s;
+            de[i] = d[i] - t;
         }
         return;
     }
-    const CTCoef<double> k = ct_coef(x[4], p.dt);
+    const double dt = p.dt, w = xp[4], dw = dp[4], wn = w + dw;
+    const CTCoef<double> k = ct_coef(w, dt), n = ct_coef(wn, dt);
+    // changes of cos(w dt), sin(w dt), A1 = sin(w dt) / w and A2 = (1 - cos(w dt)) / w
+    const double a = w * dt, an = wn * dt, da = dw * dt;
+    double sh, ch, sm, cm;
+    sincos(0.5 * da, &sh, &ch);
+    sincos(a + 0.5 * da, &sm, &cm);
+    const double dc = -2.0 * sm * sh, ds = 2.0 * cm * sh;
+    double dA1, dA2;
+    if (fabs(a) < 0.01 && fabs(an) < 0.01) {   // ct_coef's series
+        const double s2 = a * a + an * an, m = a * an;
+        dA1 = dt * da * (a + an) * (s2 * (1.0 / 120.0) - 1.0 / 6.0);
+        dA2 = dt * da * (0.5 - (s2 + m) * (1.0 / 24.0) + (s2 * s2 - m * m + m * s2) * (1.0 / 720.0));
+    } else if (fabs(da) <= 0.5 * fabs(a)) {
+        dA1 = (ds - k.A1 * dw) / wn;
+        dA2 = (-dc - k.A2 * dw) / wn;
+    } else {
+        dA1 = n.A1 - k.A1;
+        dA2 = n.A2 - k.A2;
+    }
     double inc[5];
-    ct_increment(x, k, inc);
-    out[0] = x[0] + inc[0];
-    out[1] = x[1] + inc[1];
-    out[2] = inc[2];
-    out[3] = inc[3];
-    out[4] = inc[4];
+    ct_increment(xp, k, inc);
+    e[0] = (x[0] - xp[0]) - inc[0];
+    e[1] = (x[1] - xp[1]) - inc[1];
+#pragma unroll
+    for (int i = 2; i < 5; ++i) e[i] = x[i] - inc[i];
+    de[0] = (d[0] - dp[0]) - (n.A1 * dp[2] - n.A2 * dp[3] + dA1 * xp[2] - dA2 * xp[3]);
+    de[1] = (d[1] - dp[1]) - (n.A2 * dp[2] + n.A1 * dp[3] + dA2 * xp[2] + dA1 * xp[3]);
+    de[2] = d[2] - (n.c * dp[2] - n.s * dp[3] + dc * xp[2] - ds * xp[3]);
+    de[3] = d[3] - (n.s * dp[2] + n.c * dp[3] + ds * xp[2] + dc * xp[3]);
+    de[4] = d[4] - dp[4];
 }
 
-// the measurement residual y - h(x), bearings on the branch nearest zero
-PES_DEV void resid_model(const LMParams& p, int b, const double* x, const double* y, double* r)
+// y - h(x) (bearings on the branch nearest zero) and its change by the step d of x
+PES_DEV void obs_change(const LMParams& p, int b, const double* x, const double* d, const double* y, double* r,
+                            double* dr)
 {
     if (p.kind == MODEL_LINEAR) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            double s = p.d[i];
+            double s = p.d[i], t = 0.0;
 #pragma unroll
-            for (int l = 0; l < 5; ++l) s = fma(p.H[i * 5 + l], x[l], s);
+            for (int l = 0; l < 5; ++l) {
+                s = fma(p.H[i * 5 + l], x[l], s);
+                t = fma(p.H[i * 5 + l], d[l], t);
+            }
             r[i] = y[i] - s;
+            dr[i] = -t;
         }
         return;
     }
     const double* s = p.sensors + (p.sensors_per_traj ? 4 * b : 0);
 #pragma unroll
-    for (int i = 0; i < 2; ++i) r[i] = wrap_angle(y[i] - atan2(x[1] - s[2 * i + 1], x[0] - s[2 * i]));
+    for (int i = 0; i < 2; ++i) {
+        const double rx = x[0] - s[2 * i], ry = x[1] - s[2 * i + 1];
+        r[i] = wrap_angle(y[i] - atan2(ry, rx));
+        // the angle between the old and the new line of sight
+        const double turn = atan2(rx * d[1] - ry * d[0], rx * (rx + d[0]) + ry * (ry + d[1]));
+        const double rn = wrap_angle(r[i] - turn);
+        dr[i] = rn == r[i] - turn ? -turn : rn - r[i];   // else it crosses to another branch
+    }
 }
 
-PES_DEV double quad_sym(const double* S, const double* e, int n)
+// 1/2 de^T S (2 e + de), S symmetric packed
+PES_DEV double quad_change(const double* S, const double* e, const double* de, int n)
 {
     double q = 0.0;
     for (int i = 0; i < n; ++i)
         for (int j = 0; j < n; ++j) {
             const int a = i < j ? i : j, c = i < j ? j : i;
             const int ix = n == 5 ? si(a, c) : si2(a, c);
-            q = fma(e[i] * S[ix], e[j], q);
+            q = fma(de[i] * S[ix], fma(0.5, de[j], e[j]), q);
         }
     return q;
 }
@@ -93,12 +141,11 @@ PES_DEV void warp_segment_add(double v, int b, double* acc)
 
 }  // namespace
 
-// The MAP objective of every trajectory at the nominal x (PES_* layout of the
-// smoother kernel: lane-major slots), added into p.cost; with p.xold, also the
-// squared step ||x - xold||^2 into p.num and ||x||^2 into p.den.
+// What the step from xold to x (both in the smoother kernel's lane-major slots)
+// changes every trajectory's MAP objective by, added into p.change; also the
+// squared step into p.num and ||x||^2 into p.den.
 template <typename T>
-__global__ void lm_cost_kernel(const LMParams p, double* cost_out, const T* x, const T* xold, const T* y,
-                               const T* m0, const T* P0)
+__global__ void lm_change_kernel(const LMParams p, const T* x, const T* xold, const T* y, const T* m0, const T* P0)
 {
     const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool valid = ix < p.cs;
@@ -112,66 +159,58 @@ __global__ void lm_cost_kernel(const LMParams p, double* cost_out, const T* x, c
     }
     // every lane stays to the warp's reductions; one without a state adds nothing
     const int b = valid ? traj_of_k(p.offsets, p.B, k) : -1;
-    double xk[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    double J = 0.0;
+    double dJ = 0.0, num = 0.0, den = 0.0;
     if (valid) {
+        double xo[5], d[5];
 #pragma unroll
-    for (int c = 0; c < 5; ++c) xk[c] = (double)x[c * p.cs + ix];
-    if (k == __ldg(p.offsets + b)) {
-        // prior: 1/2 (x_0 - m0)^T P0^{-1} (x_0 - m0), by a Cholesky solve
-        double P[15], e[5], Lc[25], rd[5];
-#pragma unroll
-        for (int c = 0; c < 15; ++c) P[c] = (double)P0[15 * b + c];
-#pragma unroll
-        for (int c = 0; c < 5; ++c) e[c] = xk[c] - (double)m0[5 * b + c];
-        chol_pd(P, Lc, rd);
-        double z[5];   // L z = e
-#pragma unroll
-        for (int i = 0; i < 5; ++i) {
-            double t = e[i];
-#pragma unroll
-            for (int l = 0; l < i; ++l) t = fma(-Lc[i * 5 + l], z[l], t);
-            z[i] = t * rd[i];
+        for (int c = 0; c < 5; ++c) {
+            const double xn = (double)x[c * p.cs + ix];
+            xo[c] = (double)xold[c * p.cs + ix];
+            d[c] = xn - xo[c];
+            num = fma(d[c], d[c], num);
+            den = fma(xn, xn, den);
         }
+        if (k == __ldg(p.offsets + b)) {
+            // prior: 1/2 |L^{-1} (x_0 - m0)|^2, P0 = L L^T
+            double P[15], Lc[25], rd[5], z[5], dz[5];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) J = fma(0.5 * z[i], z[i], J);
-    } else {
-        const int64_t ixp = s > 0 ? ix - p.NL : (int64_t)(p.L - 1) * p.NL + (lane - 1);
-        double xp[5], fx[5], e[5];
+            for (int c = 0; c < 15; ++c) P[c] = (double)P0[15 * b + c];
+            chol_pd(P, Lc, rd);
 #pragma unroll
-        for (int c = 0; c < 5; ++c) xp[c] = (double)x[c * p.cs + ixp];
-        f_model(p, xp, fx);
+            for (int i = 0; i < 5; ++i) {
+                double t = xo[i] - (double)m0[5 * b + i], u = d[i];
 #pragma unroll
-        for (int c = 0; c < 5; ++c) e[c] = xk[c] - fx[c];
-        J = 0.5 * quad_sym(p.Qi, e, 5);
-        double yk[2] = {(double)y[ix], (double)y[p.cs + ix]}, r[2];
-        resid_model(p, b, xk, yk, r);
-        J = fma(0.5, quad_sym(p.Ri, r, 2), J);
-    }
-    }
-    warp_segment_add(J, b, cost_out);
-    if (xold) {
-        double num = 0.0, den = 0.0;
-        if (valid) {
+                for (int l = 0; l < i; ++l) {
+                    t = fma(-Lc[i * 5 + l], z[l], t);
+                    u = fma(-Lc[i * 5 + l], dz[l], u);
+                }
+                z[i] = t * rd[i];
+                dz[i] = u * rd[i];
+                dJ = fma(dz[i], fma(0.5, dz[i], z[i]), dJ);
+            }
+        } else {
+            const int64_t ixp = s > 0 ? ix - p.NL : (int64_t)(p.L - 1) * p.NL + (lane - 1);
+            double xp[5], dp[5], e[5], de[5];
 #pragma unroll
             for (int c = 0; c < 5; ++c) {
-                const double dv = xk[c] - (double)xold[c * p.cs + ix];
-                num = fma(dv, dv, num);
-                den = fma(xk[c], xk[c], den);
+                xp[c] = (double)xold[c * p.cs + ixp];
+                dp[c] = (double)x[c * p.cs + ixp] - xp[c];
             }
+            f_change(p, xo, d, xp, dp, e, de);
+            dJ = quad_change(p.Qi, e, de, 5);
+            double yk[2] = {(double)y[ix], (double)y[p.cs + ix]}, r[2], dr[2];
+            obs_change(p, b, xo, d, yk, r, dr);
+            dJ += quad_change(p.Ri, r, dr, 2);
         }
-        warp_segment_add(num, b, p.num);
-        warp_segment_add(den, b, p.den);
     }
+    warp_segment_add(dJ, b, p.change);
+    warp_segment_add(num, b, p.num);
+    warp_segment_add(den, b, p.den);
 }
 
 // Per trajectory: keep the step if it lowered the objective (damping / nu),
 // else keep the nominal (damping * nu); record convergence (the step's
-// relative size <= tol) and count the trajectories still unconverged. A step
-// within the tolerance, or of a relative size up to 1e-7, changes the objective by
-// about 1e-14 of it or less, which the rounding of its evaluation hides: such a
-// step is also kept when the objective does not tell the two apart, so that the
-// result and the iterations it takes do not hang on that rounding.
+// relative size <= tol) and count the trajectories still unconverged.
 template <typename T>
 __global__ void lm_decide_kernel(const LMParams p, T* lam, int it, double tol, double nu)
 {
@@ -179,10 +218,7 @@ __global__ void lm_decide_kernel(const LMParams p, T* lam, int it, double tol, d
     if (b >= p.B) return;
     const double num = p.num[b], den = p.den[b];
     const double rel = den > 0.0 ? sqrt(num / den) : sqrt(num);
-    const double tie = (tol > 0.0 && rel <= fmax(tol, 1e-7)) ? 1e-13 * fabs(p.cost[b]) : 0.0;
-    const bool acc = p.cost_new[b] < p.cost[b] + tie;
-    if (acc) {
-        p.cost[b] = p.cost_new[b];
+    if (p.change[b] < 0.0) {
         lam[b] = (T)((double)lam[b] / nu);
         p.accepted[b] += 1;
         p.reject[b] = 0;
@@ -221,11 +257,11 @@ __global__ void lm_fill_kernel(T* lam, int B, double v)
 }
 
 template <typename T>
-cudaError_t launch_lm_cost(const LMParams& p, double* cost_out, const T* x, const T* xold, const T* y, const T* m0,
-                           const T* P0, cudaStream_t st)
+cudaError_t launch_lm_change(const LMParams& p, const T* x, const T* xold, const T* y, const T* m0, const T* P0,
+                             cudaStream_t st)
 {
     const unsigned blocks = (unsigned)((p.cs + 255) / 256);
-    lm_cost_kernel<T><<<blocks, 256, 0, st>>>(p, cost_out, x, xold, y, m0, P0);
+    lm_change_kernel<T><<<blocks, 256, 0, st>>>(p, x, xold, y, m0, P0);
     return cudaGetLastError();
 }
 
@@ -252,8 +288,8 @@ cudaError_t launch_lm_fill(T* lam, int B, double v, cudaStream_t st)
 }
 
 #define PES_LM_INSTANTIATE(T)                                                                                     \
-    template cudaError_t launch_lm_cost<T>(const LMParams&, double*, const T*, const T*, const T*, const T*,      \
-                                           const T*, cudaStream_t);                                               \
+    template cudaError_t launch_lm_change<T>(const LMParams&, const T*, const T*, const T*, const T*, const T*,   \
+                                             cudaStream_t);                                                       \
     template cudaError_t launch_lm_decide<T>(const LMParams&, T*, int, double, double, cudaStream_t);           \
     template cudaError_t launch_lm_restore<T>(const LMParams&, T*, T*, const T*, const T*, cudaStream_t);       \
     template cudaError_t launch_lm_fill<T>(T*, int, double, cudaStream_t);

@@ -1,5 +1,5 @@
 // Parameters of the Levenberg-Marquardt kernels (pes_lm.cu): the model in
-// FP64 (the objective is evaluated in FP64 for either precision), the
+// FP64 (the objective's change is evaluated in FP64 for either precision), the
 // lane-major geometry of the smoother kernel, and per-trajectory accumulators.
 #pragma once
 
@@ -19,21 +19,20 @@ struct LMParams {
     const double* sensors;   // device [1 or B][4]
     double F[25], c[5], H[10], d[2];   // linear model
     double Qi[15], Ri[3];              // inverses of Q and R (packed)
-    double* cost;       // [B] objective at the nominal
-    double* cost_new;   // [B] objective at the step
+    double* change;     // [B] what the step changes the objective by
     double* num;        // [B] squared step
-    double* den;        // [B] squared nominal
+    double* den;        // [B] squared norm after it
     int* reject;        // [B]
     int* accepted;      // [B] steps accepted so far
     int* conv_iter;     // [B] first converged iteration (0: none)
     int* unconv;        // trajectories not yet converged
 };
 
-// The objective of every trajectory at x, added into cost_out [B]; with xold
-// also the squared step and squared nominal into p.num, p.den.
+// What the step from xold to x changes every trajectory's objective by, the
+// squared step and the squared norm after it, added into p.change, p.num, p.den.
 template <typename T>
-cudaError_t launch_lm_cost(const LMParams& p, double* cost_out, const T* x, const T* xold, const T* y, const T* m0,
-                           const T* P0, cudaStream_t st);
+cudaError_t launch_lm_change(const LMParams& p, const T* x, const T* xold, const T* y, const T* m0, const T* P0,
+                             cudaStream_t st);
 template <typename T>
 cudaError_t launch_lm_decide(const LMParams& p, T* lam, int it, double tol, double nu, cudaStream_t st);
 template <typename T>
