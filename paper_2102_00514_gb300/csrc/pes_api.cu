@@ -175,8 +175,9 @@ pes_status check_model(pes_handle* h, const pes_model* m)
 // choice, for tuning.
 // Threads per block and minimum steps per lane: the autotuned values of the
 // handle if pes_autotune set them, else the defaults (256 threads for FP32,
-// the 128 that the FP64 kernel is compiled for). Up to kMinStepsPerThread, the
-// steps per lane of a run are make_shape's choice.
+// the 128 that the FP64 kernel is compiled for). kMinStepsPerThread is the
+// defaults' own value: with it, lanes per block and steps per lane are make_shape's
+// choice; any other fixes them.
 static_assert(std::extent<decltype(pes_handle::tune)>::value > LIN_GH, "one tuning slot per linearisation");
 
 int choose_nt(const pes_handle* h, int lin, pes_precision prec)
@@ -230,8 +231,8 @@ pes_status make_shape(pes_handle* h, int lin, pes_precision prec, int64_t N, Sha
     }
     if (cap == 0) return fail(h, PES_ERR_CUDA, "the smoother kernel cannot be made co-resident on this device");
     const int64_t blocks = std::min(cap, h->nb_max);
-    if (lin == LIN_ARRAYS || min_steps > kMinStepsPerThread || N >= blocks * s.nt * kMinStepsPerThread) {
-        // A tuned shape; sizes at which all lanes have steps enough; and the scans
+    if (lin == LIN_ARRAYS || min_steps != kMinStepsPerThread || N >= blocks * s.nt * kMinStepsPerThread) {
+        // A fixed shape; sizes at which all lanes have steps enough; and the scans
         // over given arrays, which keep one partition for a size, and with it the
         // rounding that their FP64 log-likelihoods of FP32 filters show.
         const int64_t want = (N + (int64_t)s.nt * min_steps - 1) / ((int64_t)s.nt * min_steps);

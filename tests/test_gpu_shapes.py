@@ -119,3 +119,31 @@ def test_workspace_of_exactly_as_many_states():
             x, P = linear_run(s, w, pes.CUBATURE, prec)
             assert rel_err(x, ref["x"], w["off"]) < tol, N
         s.close()
+
+
+@pytest.mark.parametrize("prec,threads,tol", [(pes.FP64, 128, TOL_FP64), (pes.FP32, 256, TOL_FP32),
+                                              (pes.FP32, 128, TOL_FP32)])
+def test_a_minimum_of_steps_is_followed(prec, threads, tol):
+    """Any minimum but the defaults' own (8) gives full blocks of lanes with at least so
+    many steps, few as they may be; 8 with the default threads is the default."""
+    s = pes.Smoother(1 << 15, 4)
+    try:
+        for T in (60, 700, 20011):
+            N = T + 1
+            w = linear_case(T)
+            ref = oracle.iterated_smoother(w["om"], oracle.IEKS, w["off"], w["y"], w["m0"], w["P0"], iters=1)
+            default = s.launch_shape(pes.IEKS, prec, N)
+            for steps in (1, 2, 4, 7, 9, 32):
+                s.set_launch_shape(pes.IEKS, prec, threads, steps)
+                nb, nt, L = s.launch_shape(pes.IEKS, prec, N)
+                want = -(-N // (threads * steps))
+                assert nt == threads and nb <= want and L == -(-N // (nb * nt))
+                assert nb == want or nb >= 152, (steps, nb, want)
+                x, P = linear_run(s, w, pes.IEKS, prec)
+                assert rel_err(x, ref["x"], w["off"]) < tol, (T, steps)
+                assert rel_err(P, ref["P"], w["off"]) < tol, (T, steps)
+            s.set_launch_shape(pes.IEKS, prec, 128 if prec == pes.FP64 else 256, 8)
+            assert s.launch_shape(pes.IEKS, prec, N) == default
+            s.set_launch_shape(pes.IEKS, prec, 0, 0)
+    finally:
+        s.close()
