@@ -13,7 +13,9 @@ The metric counts only at oracle tolerance. Both FP32 and PES_REFINED (FP32
 iterations, the final one refined by a Newton step with float-float
 residuals) are timed; `value` is the rate of the fastest precision whose
 final iteration meets 1e-4 against the oracle in this run's parity check
-(`config.precision` names it), and the other rates are reported beside it.
+(`config.precision` names it), and the other rates are reported beside it. stdout
+gets one compact JSON line; the full record (per method, parity figures, length
+sweep, batched workload) goes to stderr as one line that starts with "detail".
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl pes|reference]
 Under torchrun (N > 1) every rank smooths its own replica of the workload
@@ -401,6 +403,42 @@ def choose_headline(result):
     else:
         result["at_oracle_tol"] = None
         result["config"]["precision"] = "fp32 (no precision met the tolerance in this run)"
+
+
+def compact_line(result):
+    """The line printed on stdout: the headline with its configuration, and one rate
+    per precision and workload, short enough to be read whole from the end of a log
+    that keeps a few thousand characters. The full record goes to stderr."""
+    def pick(d, *keys):
+        return {k: d[k] for k in keys if d.get(k) is not None} if d else None
+
+    def rounded(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            return {k: rounded(x) for k, x in v.items()}
+        return [rounded(x) for x in v] if isinstance(v, list) else v
+
+    rate = ("value", "ms_per_step")
+    cfg = result["config"]
+    out = pick(result, "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling")
+    out["vs_baseline"] = result["vs_baseline"]
+    out.update(pick(result, "dtype", "data", "gpu_launches", "at_oracle_tol", "iters_saved"))
+    out["config"] = pick(cfg, "workload", "T", "B", "N_states", "iterations", "methods", "precision", "l2")
+    out["config"]["launch"] = {k: list(v.values()) for k, v in cfg["launch"].items() if k != "autotuned"}
+    out["e2e"] = pick(result.get("e2e"), "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step",
+                      "precision")
+    out["clocks"] = pick(result.get("clocks"), "sm_mhz", "sm_max_mhz", "reasons")
+    out["roofline"] = pick(result["roofline"], "bound", "achieved", "peak", "unit", "frac", "kernel")
+    out["cpu_baseline"] = pick(result.get("cpu_baseline"), "value", "unit", "cores", "kind", "sample")
+    for key in ("fp32", "refined", "mixed", "fp64", "graph"):
+        out[key] = pick(result.get(key), *rate)
+    if "batched" in result:
+        b = result["batched"]
+        out["batched"] = dict(pick(b, "N_states", "B"), **{k: pick(b.get(k), *rate) for k in ("fp32", "refined")})
+    if "parity" in result:
+        out["within_tol"] = result["parity"]["within_tol"]
+    return rounded({k: v for k, v in out.items() if v is not None or k == "vs_baseline"})
 
 
 def executed_for(method: str):
@@ -1172,7 +1210,8 @@ def main():
                 result["length_sweep"] = length_sweep_key(args, flush)
             if not args.no_batched:
                 result["batched"] = batched_key(args, roofline["peak"], flush)
-        print(json.dumps(result), flush=True)
+        print("detail " + json.dumps(result), file=sys.stderr, flush=True)
+        print(json.dumps(compact_line(result)), flush=True)
     sm.close()
     if dist is not None:
         dist.barrier()

@@ -73,3 +73,49 @@ def test_per_state_errors_are_relative_to_each_state():
     e = bench.per_state_errors(a, b)
     assert np.allclose(e, [0.1, 0.0, 0.1])
     assert bench.per_state_max(a, b) == e.max()
+
+
+def full_record():
+    """A record with every block that a default run fills, long ones as long as there."""
+    r = line(False, True, True)
+    long_block = {f"key_{i}": {"value": 1.0 / 3.0, "per_method": {"ieks": [0.1] * 40}} for i in range(40)}
+    r.update({"metric": bench.METRIC, "unit": bench.UNIT, "n_gpus": 1, "warmup": 5, "higher_is_better": True,
+              "scaling": "weak", "vs_baseline": None,
+              "data": "synthetic coordinated-turn / bearings (seeded, seed 20210204), inputs resident in HBM",
+              "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": [], "nvidia_smi": long_block},
+              "roofline": {"bound": "alu", "achieved": 100.0 / 3.0, "peak": 80.5, "unit": "TFLOP/s", "frac": 1.0 / 3.0,
+                           "kernel": "pes_persistent_kernel<float, cubature>", "executed": long_block},
+              "fp64": {"value": 1.0e8 / 3.0, "ms_per_step": 635.0 / 3.0}, "graph": {"value": 3.1e9, "ms_per_step": 6.6},
+              "iters_saved": 1.46, "learned_init": long_block, "length_sweep": long_block,
+              "batched": dict(long_block, N_states=41900000, B=4096, fp32={"value": 5.8e9, "ms_per_step": 144.0},
+                              refined={"value": 3.8e9, "ms_per_step": 219.0}),
+              "cpu_baseline": {"value": 6.3e5, "unit": bench.UNIT, "cores": 1, "kind": "oracle",
+                               "sample": "first 131072 of 1048577 states (1 trajectories), IEKS + cubature, 10 "
+                                         "iterations, sequential FP64 oracle"}})
+    r["parity"]["rel_frobenius"] = long_block
+    r["config"].update({"workload": "single trajectory T=1048576, IEKS + cubature IPLS, 10 iterations each, FP32, "
+                                    "prior initialisation", "T": 1 << 20, "B": 1, "N_states": (1 << 20) + 1,
+                        "iterations": 10, "methods": ["ieks", "cubature"], "l2": "flushed before every step",
+                        "launch": {"ieks": {"blocks": 152, "threads": 256, "steps_per_thread": 27},
+                                   "cubature": {"blocks": 304, "threads": 128, "steps_per_thread": 27},
+                                   "autotuned": long_block}})
+    for e in (r["e2e"], *r["e2e_by_precision"].values()):
+        e.update({"unit": bench.UNIT, "h2d_bytes_per_step": 16777632, "d2h_bytes_per_step": 167772320,
+                  "ms_per_step": 7.0, "serial": long_block})
+    return r
+
+
+def test_printed_line_is_complete_and_short():
+    """stdout's line keeps the contract's keys and fits the last 2,800 characters of a log."""
+    import json
+    r = full_record()
+    bench.choose_headline(r)
+    c = bench.compact_line(r)
+    assert len(json.dumps(c)) < 2800
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline"):
+        assert k in c, k
+    assert c["value"] == r["value"] == 2.4e9 and c["config"]["precision"] == "refined"
+    assert c["e2e"]["value"] == 2.1e9 and {"h2d_bytes_per_step", "d2h_bytes_per_step"} <= set(c["e2e"])
+    assert {"sm_mhz", "sm_max_mhz", "reasons"} == set(c["clocks"])
+    assert c["batched"]["refined"] == {"value": 3.8e9, "ms_per_step": 219.0}
