@@ -383,8 +383,9 @@ def set_headline(result, key, value, ms):
     e2e = result.get("e2e_by_precision", {}).get(key)
     if e2e is not None:
         result["e2e"] = e2e
-    launches = {"fp32": 7, "refined": 12, "mixed": 12}
-    result["gpu_launches"] = launches.get(key, 7) * 2 * result["steps"]
+    # kernels of one run (a line without counts of its own has one layout launch per output array)
+    launches = result.get("launches_per_run", {"fp32": 7, "refined": 12, "mixed": 12})
+    result["gpu_launches"] = launches[key] * 2 * result["steps"]
 
 
 def choose_headline(result):
@@ -843,12 +844,15 @@ def main():
         total_ms = max_over_ranks(sum(step_ms[key]), dist, "cuda")
         rates[key] = {"value": whole_job_rate(world, work_per_step, args.steps, total_ms * 1e-3),
                       "ms_per_step": total_ms / args.steps}
-    # kernels of one run: FP32 = offsets validation, sensor conversion, y to the
-    # lane layout, nominal initialisation, persistent smoother, x and P back to
-    # the caller layout; PES_REFINED adds the final iteration's own persistent
-    # launch and the refinement's four kernels (forward residuals, forward
-    # correction scan, RTS residuals, RTS correction scan)
-    launches_per_run = {"fp32": 7, "refined": 12}
+    # kernels of one run from the prior: FP32 = offsets validation, sensor
+    # conversion, y to the lane layout, nominal initialisation, persistent
+    # smoother, x and P back to the caller layout in one launch; PES_REFINED adds
+    # the final iteration's own persistent launch and the refinement's four
+    # kernels (forward residuals, forward correction scan, RTS residuals, RTS
+    # correction scan); PES_MIXED adds conversions of the inputs, the nominal and
+    # the results, and the FP64 iteration's own sensor conversion, layout
+    # launches and persistent launch
+    launches_per_run = {"fp32": 6, "refined": 11, "mixed": 17}
     value = rates["fp32"]["value"]
     ms_per_step = rates["fp32"]["ms_per_step"]
 
@@ -908,6 +912,7 @@ def main():
                   "refined": dict(rates["refined"], per_method=per_prec["refined"],
                                   schedule=f"{iters - 1} FP32 iterations, then 1 FP32 iteration refined by a Newton "
                                            "step (float-float residuals, FP32 correction scans)"),
+                  "launches_per_run": launches_per_run,
                   "gpu_launches": launches_per_run["fp32"] * len(methods) * args.steps, "clocks": clk}
 
     # FP64 on the same GPU (the metric compares FP32 with FP64)

@@ -82,6 +82,7 @@ def full_record():
     r.update({"metric": bench.METRIC, "unit": bench.UNIT, "n_gpus": 1, "warmup": 5, "higher_is_better": True,
               "scaling": "weak", "vs_baseline": None,
               "data": "synthetic coordinated-turn / bearings (seeded, seed 20210204), inputs resident in HBM",
+              "launches_per_run": {"fp32": 6, "refined": 11, "mixed": 17},
               "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": [], "nvidia_smi": long_block},
               "roofline": {"bound": "alu", "achieved": 100.0 / 3.0, "peak": 80.5, "unit": "TFLOP/s", "frac": 1.0 / 3.0,
                            "kernel": "pes_persistent_kernel<float, cubature>", "executed": long_block},
@@ -119,3 +120,9 @@ def test_printed_line_is_complete_and_short():
     assert c["e2e"]["value"] == 2.1e9 and {"h2d_bytes_per_step", "d2h_bytes_per_step"} <= set(c["e2e"])
     assert {"sm_mhz", "sm_max_mhz", "reasons"} == set(c["clocks"])
     assert c["batched"]["refined"] == {"value": 3.8e9, "ms_per_step": 219.0}
+
+
+def test_launch_counts_of_the_line_are_used():
+    r = full_record()
+    bench.choose_headline(r)
+    assert r["gpu_launches"] == 11 * 2 * 20
