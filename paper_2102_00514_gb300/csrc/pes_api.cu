@@ -243,12 +243,17 @@ pes_status make_shape(pes_handle* h, int lin, pes_precision prec, int64_t N, Sha
     }
     // A run: few steps per lane and few lanes per block, which the device's other
     // multiprocessors make up for, against the levels of the grid's trees. A block of
-    // 32 lanes spares the first levels, whose operators have few threads each. With
-    // all the threads as lanes and at least 8 steps each: T = 500, FP64, 10
-    // iterations, 1 x 128 x 4: 7,570 us; 16 x 32 x 1: 4,750 us; T = 10,000 cubature,
-    // FP64, 5 iterations, 10 x 128 x 8: 7,250 us; 79 x 64 x 2: 4,250 us; 64
-    // trajectories of 1 to 400 states, cubature, FP32, 3 iterations, 6 x 256 x 8:
-    // 371 us; 117 x 96 x 1: 245 us. Full-size runs take all lanes either way.
+    // 32 lanes spares the first levels, whose operators have few threads each. Against
+    // all the threads as lanes with at least 9 steps each: T = 500, FP64, 10
+    // iterations, 1 x 128 lanes x 4 steps: 6,770 us; 16 x 32 x 1: 4,180 us; T = 10,000
+    // cubature, FP64, 5 iterations, 9 x 128 x 9: 7,230 us; 53 x 64 x 3: 3,940 us; 64
+    // trajectories, 13,100 states, cubature, FP32, 3 iterations, 6 x 256 x 9: 354 us;
+    // 103 x 64 x 2: 191 us. Full-size runs take all lanes either way.
+    //
+    // FP32 has two steps per lane at least: with one, every state goes through the
+    // trees' operators, and their rounding shows for little time (8 trajectories of 607,
+    // cubature: worst covariance error 6.9e-6 with two steps, 1.6e-5 with one; three
+    // iterations 176 and 169 us).
     const ShapeCost& c = sizeof(T) == 8 ? kCost64 : kCost32;
     const int top_nodes = sizeof(T) == 4 && s.nt == 256 ? 152 : c.top_nodes;
     double best = 1e300;

@@ -38,7 +38,7 @@ struct pes_handle {
     double* hsens = nullptr;
     void* sensT = nullptr;   // sensors converted to the kernel precision
     void* lanes = nullptr;   // x, P, y in the kernel's lane-major layout
-    void* lin = nullptr;     // cubature linearisation handed from the fold to the re-run
+    void* lin = nullptr;     // sigma-point linearisation handed from the fold to the later passes; the scans' inputs
     void* mix = nullptr;     // FP64 copies for PES_MIXED (allocated by its first call)
     void* refw = nullptr;    // PES_REFINED workspace (allocated by its first call)
     void* lmw = nullptr;     // per-trajectory state of pes_ieks_run_lm (allocated by its first call)

@@ -248,11 +248,10 @@ PES_DEV void load_prior(const KParams<T>& p, int b, T* m0, T* P0)
     for (int i = 0; i < 15; ++i) P0[i] = __ldg(p.P0 + 15 * b + i);
 }
 
-// The nominal trajectory is rewritten by every iteration. Reads of it (and of
-// other data written earlier in the same launch) are plain L1-cached loads:
-// every such read follows a grid barrier, whose gpu-scope acquire and fence
-// make the other blocks' writes visible, and consecutive steps of a lane share
-// cache sectors.
+// The nominal trajectory is rewritten by every iteration. A lane reads only its own
+// states' nominal, which it wrote itself in the iteration before (the first one finds
+// an earlier kernel's), so plain loads need no barrier between iterations; they are
+// L1-cached, and consecutive steps of a warp's lanes share cache sectors.
 template <typename T>
 PES_DEV void load_nominal(const KParams<T>& p, int64_t ix, T* x)
 {

@@ -217,14 +217,7 @@ PES_DEV void cub_trans_slope_ff(const DevModel<float>& m, const float* xbar, con
 // instructions per state and 1,500 of the RTS step's 7,700 (Taylor slope). The
 // loops over rows stay rolled (below).
 
-// a += x for a value that needs no product: float or float-float
-PES_DEV void acc_plus(ffacc& a, float x)
-{
-    const ff t = two_sum(a.s, x);
-    a.s = t.hi;
-    a.c = __fadd_rn(a.c, t.lo);
-}
-PES_DEV void acc_plus(ffacc& a, ff x) { acc_add(a, x); }
+// a float or a float-float as a float-float
 PES_DEV ff ff_of(float x) { return ff_make(x); }
 PES_DEV ff ff_of(ff x) { return x; }
 
