@@ -1079,7 +1079,9 @@ pes_status pes_autotune(pes_handle* h, const pes_model* model, pes_method method
     const int nts32[] = {128, 256}, nts64[] = {128};
     const int* nts = prec == PES_FP64 ? nts64 : nts32;
     const int n_nt = prec == PES_FP64 ? 1 : 2;
-    const int steps[] = {4, 8, 16, 32, 64, 128};
+    // the library's choice of steps first: of candidates that give the same launch, the
+    // first is kept, and with it the choice for other sizes
+    const int steps[] = {kMinStepsPerThread, 4, 16, 32, 64, 128};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     PES_CUDA(h, cudaEventCreate(&e0));
     PES_CUDA(h, cudaEventCreate(&e1));

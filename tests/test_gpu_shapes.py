@@ -255,3 +255,18 @@ def test_full_process_noise_through_the_stored_regression(sm, method):
             x, P = one_iteration(sm, wl, method, prec, x0, P0)
             assert rel_err(x, ref["x"], wl["offsets"]) < tol, (T, prec)
             assert rel_err(P, ref["P"], wl["offsets"]) < tol, (T, prec)
+
+
+def test_a_tuning_at_a_large_size_keeps_the_choice_for_small_ones():
+    """At sizes at which every lane has steps enough, small minima give one launch: the
+    tuning then records the library's own choice, which other sizes go by."""
+    T = (1 << 18) + 300000
+    s = pes.Smoother(T + 1, 1)
+    try:
+        w = linear_case(T)
+        small = s.launch_shape(pes.IEKS, pes.FP64, 501)
+        d = [to_dev(w["y"]), to_dev(w["off"], torch.int64), to_dev(w["m0"]), to_dev(w["P0"])]
+        assert s.autotune(w["gm"], pes.IEKS, pes.FP64, *d, iters=1)[1] == 8
+        assert s.launch_shape(pes.IEKS, pes.FP64, 501) == small
+    finally:
+        s.close()
