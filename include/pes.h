@@ -379,7 +379,7 @@ pes_status pes_ieks_run_noalloc(const pes_model* model, pes_method method, pes_p
 /*
  * A pes_ieks_run of fixed arguments (fixed iterations: no tolerance, no
  * iteration count read back) captured once into a CUDA graph: offsets
- * validation, sensor conversion, the layout transposes, the nominal
+ * validation, sensor conversion, the layout copies, the nominal
  * initialisation and the persistent launch that runs every iteration. The
  * graph keeps the pointers; replay it with pes_graph_launch after changing the
  * arrays' contents (not their addresses or sizes). Replays use the handle's
