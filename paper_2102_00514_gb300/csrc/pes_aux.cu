@@ -81,17 +81,19 @@ template cudaError_t launch_convert<double>(const double*, double*, int, cudaStr
 // state k = lane * L + s sits at s * NL + lane, for several arrays in one
 // launch (their components consecutive on the lane-major side).
 //
-// Bound by memory latency: what counts is bytes in flight. A block takes G lanes
-// of a few components: with L <= W steps a component's states are one
-// contiguous run of the caller's array, so both sides are read and written in
-// full lines whatever L is; longer chunks are cut into pieces of W steps, a warp
-// reading a lane's piece. Everything a block reads is in flight at once, copied
-// into the tile by cp.async, and its stores do not wait. The tile's rows are
-// steps, an odd number of words apart: no bank conflicts on either side. (32 x
-// 32 tiles of (lane, step) leave columns empty and start every row off a line's
-// boundary: the 20 components of 2^20 states, L = 27, took 62 us, here 40; the 7
-// components in 28, here 21.)
-constexpr int MV_W = 63, MV_THREADS = 256;
+// Bound by memory latency and by instructions: what counts is bytes in flight and
+// how few instructions a value takes. A block takes G lanes of some components: with L
+// <= W steps a component's states are one contiguous run of the caller's array, so
+// both sides are read and written in full lines whatever L is, and a place's index
+// serves all the block's components; longer chunks are cut into pieces of W steps, a
+// warp reading a lane's piece. Everything a block reads is in flight at once, copied
+// into the tile by cp.async, and its stores do not wait. The tile's rows are steps,
+// as far apart as keeps the banks free of conflicts on both sides (mv_row). (32 x 32
+// tiles of (lane, step) leave columns empty and start every row off a line's boundary:
+// the 20 components of 2^20 states, L = 27, took 62 us, one component's index at a
+// time 40, here 31; 62 components of 262,144 states, L = 8, 41 -> 23, 20 back 16 ->
+// 11; 20 of 5.2 million, L = 134, 211 -> 188.)
+constexpr int MV_W = 63, MV_THREADS = 256, MV_NC = 65, MV_BYTES = 47 * 1024;
 template <typename T>
 constexpr int MV_G = sizeof(T) == 4 ? 128 : 64;
 
@@ -101,16 +103,26 @@ PES_DEV void copy_async(T* dst, const T* src)
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(sizeof(T)) : "memory");
 }
 
-template <typename T, bool TO_LANES, bool BLOCKED>
-__global__ void __launch_bounds__(MV_THREADS) lanes_move_kernel(const LaneArrays<T> a, T* lanes, int64_t N, int L,
-                                                                int NL, int nc, int per_block)
+// Words from a row of the tile to the next. The caller's side goes through the tile
+// by consecutive states, so that a warp (doubles: half a warp) touches several rows
+// of several lanes if a lane has fewer steps than that: rows are as many banks apart.
+template <typename T>
+__host__ __device__ constexpr int mv_row(int w)
 {
-    constexpr int G = MV_G<T>, RS = G + 1;
+    constexpr int n = 128 / sizeof(T);   // words that the banks hold
+    return MV_G<T> + (w < n ? (n + w - 1) / w : 1);
+}
+
+template <typename T, bool TO_LANES, bool BLOCKED>
+__global__ void __launch_bounds__(MV_THREADS) lanes_move_kernel(const __grid_constant__ LaneArrays<T> a, T* lanes,
+                                                                int64_t N, int L, int NL, int nc, int per_block)
+{
+    constexpr int G = MV_G<T>;
     extern __shared__ __align__(16) unsigned char mv_raw[];
     T* tiles = reinterpret_cast<T*>(mv_raw);
     const int64_t cs = (int64_t)L * NL;
     const int l0 = blockIdx.x * G, s0 = blockIdx.y * MV_W;
-    const int w = min(MV_W, L - s0), g = min(G, NL - l0);
+    const int w = min(MV_W, L - s0), g = min(G, NL - l0), RS = mv_row<T>(w);
     const int64_t k0 = (int64_t)l0 * L + s0;
     const int64_t left = N - k0;   // states from k0 on
     const int t = threadIdx.x;
@@ -120,12 +132,13 @@ __global__ void __launch_bounds__(MV_THREADS) lanes_move_kernel(const LaneArrays
         if (w == L) {
             const int n = (int)min((int64_t)g * w, left);
             const int dl = MV_THREADS / w, dr = MV_THREADS - dl * w;
-            int l = t / w, r = t - l * w;
+            const int di = dr * RS + dl, wrap = 1 - w * RS;
+            int r = t % w, i = r * RS + t / w;
             for (int q = t; q < n; q += MV_THREADS) {
-                f(r * RS + l, (int64_t)q);
-                l += dl;
+                f(i, q);
                 r += dr;
-                if (r >= w) r -= w, ++l;
+                i += di;
+                if (r >= w) r -= w, i += wrap;
             }
         } else {
             for (int l = t >> 5; l < g; l += MV_THREADS / 32)
@@ -139,39 +152,42 @@ __global__ void __launch_bounds__(MV_THREADS) lanes_move_kernel(const LaneArrays
         const int64_t most = left - (int64_t)l * L;   // steps from s0 on that the lane has
         const int64_t row = BLOCKED ? nc * 32 : NL;
         const int64_t at = BLOCKED ? (int64_t)(l >> 5) * L * row + (l & 31) : l;
-        if (l < g)
-            for (int r = t / G; r < w && r < most; r += MV_THREADS / G) f(r * RS + l, r * row + at);
-    };
-    auto lane_major = [&](int c) {
-        return lanes + (BLOCKED ? ((int64_t)(l0 >> 5) * L + s0) * (nc * 32) + c * 32 : c * cs + (int64_t)s0 * NL + l0);
-    };
-    auto caller_of = [&](int c) {
-        int arr = 0;
-        while (c >= a.nc[arr]) c -= a.nc[arr++];
-        return a.ptr[arr] + (int64_t)c * N + k0;
-    };
-    for (int c = c0; c < c1; ++c) {
-        T* tile = tiles + (c - c0) * w * RS;
-        if (TO_LANES) {
-            const T* src = caller_of(c);
-            caller_side([&](int i, int64_t k) { copy_async(tile + i, src + k); });
-        } else {
-            const T* src = lane_major(c);
-            lane_side([&](int i, int64_t ix) { copy_async(tile + i, src + ix); });
+        if (l < g) {
+            const int n = (int)min((int64_t)w, most);
+            int64_t ix = t / G * row + at;
+            int i = t / G * RS + l;
+            for (int r = t / G; r < n; r += MV_THREADS / G, ix += MV_THREADS / G * row, i += MV_THREADS / G * RS) f(i, ix);
         }
+    };
+    const int nb = c1 - c0, tile = w * RS;
+    __shared__ T* s_caller[MV_NC];
+    if (t < nb) {
+        int arr = 0, c = c0 + t;
+        while (c >= a.nc[arr]) c -= a.nc[arr++];
+        s_caller[t] = a.ptr[arr] + (int64_t)c * N + k0;
     }
+    const int64_t cstep = BLOCKED ? 32 : cs;
+    T* const lane_major = lanes + (BLOCKED ? ((int64_t)(l0 >> 5) * L + s0) * (nc * 32) : (int64_t)s0 * NL + l0) + c0 * cstep;
+    __syncthreads();
+    // f(component of the block, word, place) for all of a side: whole chunks take a
+    // place's index for all components, pieces, of one component mostly, are quicker
+    // component by component
+    auto each = [&](auto side, auto f) {
+        if (w == L) {
+            side([&](int i, int64_t k) {
+#pragma unroll 4
+                for (int c = 0; c < nb; ++c) f(c, i, k);
+            });
+        } else {
+            for (int c = 0; c < nb; ++c) side([&](int i, int64_t k) { f(c, i, k); });
+        }
+    };
+    if (TO_LANES) each(caller_side, [&](int c, int i, int64_t k) { copy_async(tiles + c * tile + i, s_caller[c] + k); });
+    else each(lane_side, [&](int c, int i, int64_t ix) { copy_async(tiles + c * tile + i, lane_major + c * cstep + ix); });
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    for (int c = c0; c < c1; ++c) {
-        const T* tile = tiles + (c - c0) * w * RS;
-        if (TO_LANES) {
-            T* dst = lane_major(c);
-            lane_side([&](int i, int64_t ix) { dst[ix] = tile[i]; });
-        } else {
-            T* dst = caller_of(c);
-            caller_side([&](int i, int64_t k) { dst[k] = tile[i]; });
-        }
-    }
+    if (TO_LANES) each(lane_side, [&](int c, int i, int64_t ix) { lane_major[c * cstep + ix] = tiles[c * tile + i]; });
+    else each(caller_side, [&](int c, int i, int64_t k) { s_caller[c][k] = tiles[c * tile + i]; });
 }
 
 template <typename T>
@@ -180,12 +196,14 @@ cudaError_t launch_lanes_move(const LaneArrays<T>& a, T* lanes, int64_t N, int L
     constexpr int G = MV_G<T>;
     int nc = 0;
     for (int i = 0; i < a.n; ++i) nc += a.nc[i];
-    // up to about 32 steps of components a block: 16 KB in flight, of which an
-    // SM holds eight; fewer where the grid would not fill the SMs
+    // as many components a block as its shared memory holds without asking for more
+    // (an SM holds four such blocks), fewer where the grid would not fill the SMs
     const int w = std::min(L, MV_W);
     const int64_t pieces = (int64_t)((NL + G - 1) / G) * ((L + MV_W - 1) / MV_W);
-    const int per_block = (int)std::max<int64_t>(1, std::min<int64_t>({nc, 32 / w, nc * pieces / 608}));
-    const size_t smem = sizeof(T) * per_block * w * (G + 1);   // at most 33 KB
+    const size_t tile = sizeof(T) * w * mv_row<T>(w);   // at most 33 KB
+    const int per_block = (int)std::max<int64_t>(1, std::min<int64_t>({nc, (int64_t)(MV_BYTES / tile), nc * pieces / 608}));
+    if (nc > MV_NC) return cudaErrorInvalidValue;
+    const size_t smem = tile * per_block;
     const dim3 grid((NL + G - 1) / G, (L + MV_W - 1) / MV_W, (nc + per_block - 1) / per_block);
     auto kern = how == MOVE_OUT  ? lanes_move_kernel<T, false, false>
                 : how == MOVE_IN ? lanes_move_kernel<T, true, false>
