@@ -1305,6 +1305,8 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
         PES_PHASE(p, it, 0);
         SElem<T> accS;
         Gauss<T> G;
+        using Ops = std::conditional_t<kKeepRounding<K, T>, FilterOps1<T>, FilterOps<T>>;
+        using SOps = std::conditional_t<kKeepRounding<K, T>, SmootherOps1<T>, SmootherOps<T>>;
         if (do_filter) {
             FElem<T> acc;
             // the fold's prefetch goes to memory beside the leaves
@@ -1313,14 +1315,14 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
             else
                 ok &= fold_filter_chunk<K>(p, a, e, lane, acc, Prefetch<T, kStateIn>{smem + FE * NT + t, NT, p.x, p.cs});
             PES_PHASE(p, it, 1);
-            publish_block<T, NT, FilterOps<T, kKeepRounding<K, T>>>(acc, nl, aggF + (size_t)blockIdx.x * FE);
+            publish_block<T, NT, Ops>(acc, nl, aggF + (size_t)blockIdx.x * FE);
             PES_PHASE(p, it, 2);
             grid_arrive(p, gen);
             grid_wait(p, gen);
             PES_PHASE(p, it, 3);
-            tree_top<T, NT, FilterOps<T, kKeepRounding<K, T>>>(aggF, 0, blockIdx.x);
+            tree_top<T, NT, Ops>(aggF, 0, blockIdx.x);
             PES_PHASE(p, it, 4);
-            tree_down<T, NT, FilterOps<T, kKeepRounding<K, T>>>(nl);
+            tree_down<T, NT, Ops>(nl);
             G = reinterpret_cast<const Gauss<T>*>(smem + M::kGauss)[min(t, nl - 1)];
             PES_PHASE(p, it, 5);
             if (do_smooth) ok &= chunk_selem(p, a, e, reinterpret_cast<const FElem<T>*>(smem)[tree_place(min(t, nl - 1), nl)], G, accS);
@@ -1330,7 +1332,7 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
         }
         __syncthreads();   // the smoother's tree and the stream stages overlap the filter's
         if (do_smooth) {
-            publish_block<T, NT, SmootherOps<T>>(accS, nl, aggS + (size_t)blockIdx.x * SE);
+            publish_block<T, NT, SOps>(accS, nl, aggS + (size_t)blockIdx.x * SE);
             grid_arrive(p, gen);
         }
         PES_PHASE(p, it, 6);
@@ -1352,9 +1354,9 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
         if (do_smooth) {
             grid_wait(p, gen);
             PES_PHASE(p, it, 8);
-            tree_top<T, NT, SmootherOps<T>>(aggS, blockIdx.x + 1, gridDim.x);
+            tree_top<T, NT, SOps>(aggS, blockIdx.x + 1, gridDim.x);
             PES_PHASE(p, it, 9);
-            tree_down<T, NT, SmootherOps<T>>(nl);
+            tree_down<T, NT, SOps>(nl);
             const Gauss<T> Gs = reinterpret_cast<const Gauss<T>*>(smem + M::kGauss)[min(t, nl - 1)];
             __syncthreads();   // the stream stages overlap the tree
             PES_PHASE(p, it, 10);

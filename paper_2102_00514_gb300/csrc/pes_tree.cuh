@@ -99,10 +99,7 @@ PES_DEV void st_vec(double* s, const double* r)
 
 // o = a (x) b, Eq. 15. The first task's operands are loaded before the
 // factorisation, which hides them; tasks differ only in addresses and selects.
-// KEEP evaluates J through J_j - J_j D J_j as combine_filter does, at 200
-// multiply-adds more: the results then equal combine_filter's to the bit (the
-// scan over given arrays, whose FP64 log-likelihoods show every rounding).
-template <typename T, bool KEEP>
+template <typename T>
 PES_DEV void coop_combine_filter(int a, int b, int o, int part, int parts)
 {
     if (part >= 11) return;
@@ -139,24 +136,6 @@ PES_DEV void coop_combine_filter(int a, int b, int o, int part, int parts)
     T Ai[28], Aj[32];   // Aj: A then b
     ld_vec<28>(pa + FA, Ai);
     ld_vec<32>(pb + FA, Aj);
-    T K2[KEEP ? 15 : 1];
-    if constexpr (KEEP) {
-        T Df[25], JD[25];
-#pragma unroll
-        for (int i = 0; i < 5; ++i)
-#pragma unroll
-            for (int j = 0; j < 5; ++j) Df[i * 5 + j] = D[si(i, j)];
-        s_m(J, Df, JD);
-#pragma unroll
-        for (int i = 0; i < 5; ++i)
-#pragma unroll
-            for (int j = i; j < 5; ++j) {
-                T v = J[si(i, j)];
-#pragma unroll
-                for (int l = 0; l < 5; ++l) v = fma(-JD[i * 5 + l], J[si(l, j)], v);
-                K2[si(i, j)] = v;
-            }
-    }
 #pragma unroll 1
     for (int task = part;;) {
         T t[5], p[5], w[5];
@@ -169,12 +148,6 @@ PES_DEV void coop_combine_filter(int a, int b, int o, int part, int parts)
         sv(J, p, w);
 #pragma unroll
         for (int i = 0; i < 5; ++i) w[i] = t[i] - w[i];
-        if constexpr (KEEP) {
-            T k[5];
-            sv(K2, z, k);
-#pragma unroll
-            for (int i = 0; i < 5; ++i) w[i] = (row || vec) ? w[i] : k[i];
-        }
         T o1[5], o2[5];
         if (row || vec) {
             // A_i^T w: row r of A, or eta; A_j p (+ C), or A_j (z + p) + b
@@ -418,21 +391,58 @@ PES_DEV void apply_smoother1(int g, int e, int o)
     st_vec<28>(s + o, out);
 }
 
+// The filtering operators by one thread each, for means that are absolute: all
+// reference points are zero, and the results' stay so.
+template <typename T>
+PES_DEV void combine_filter1(int a, int b, int o)
+{
+    T* s = smem_as<T>();
+    const FElem<T> ai = *reinterpret_cast<const FElem<T>*>(s + a), aj = *reinterpret_cast<const FElem<T>*>(s + b);
+    FElem<T> out = aj;
+    combine_filter(ai, aj, out);
+    *reinterpret_cast<FElem<T>*>(s + o) = out;
+}
+
+template <typename T>
+PES_DEV void apply_filter1(int g, int e, int o)
+{
+    T* s = smem_as<T>();
+    const FElem<T> el = *reinterpret_cast<const FElem<T>*>(s + e);
+    Gauss<T> out = *reinterpret_cast<const Gauss<T>*>(s + g);
+    apply_filter(out, el, out);
+    *reinterpret_cast<Gauss<T>*>(s + o) = out;
+}
+
 // The operators of the two scans, for the tree code below. `wide`: more than 32
 // operators; all threads of a warp then have the same part. (A form of Eq. 15
 // by two threads in registers was 20 % faster than its tasks at such levels in
 // isolation, and slower in the kernel, where its code is fetched afresh in every
 // iteration: up-sweep 19.7 against 15.8 us at 256 FP32 lanes.)
-template <typename T, bool KEEP = false>
+template <typename T>
 struct FilterOps {
     static constexpr int NC = FE, kMean = FB, kCov = FC;
     PES_DEV static int ref(int q) { return f_ref(q); }
     static constexpr bool kSuffix = false;   // the Gaussian enters at the left
-    PES_DEV static void combine(int a, int b, int o, int part, int parts, bool)
-    {
-        coop_combine_filter<T, KEEP>(a, b, o, part, parts);
-    }
+    PES_DEV static void combine(int a, int b, int o, int part, int parts, bool) { coop_combine_filter<T>(a, b, o, part, parts); }
     PES_DEV static void apply(int g, int e, int o, int part, int parts, bool) { coop_apply_filter<T>(g, e, o, part, parts); }
+};
+
+// Those of the FP32 scans over given arrays: combine_filter's rounding to the bit,
+// which the FP64 log-likelihoods beside their results show. One thread per operator:
+// the tasks above, with J through J_j - J_j D J_j as that function has it, were slower
+// (251 lanes: up-sweep 16.2 us, here 12.6, down-sweep 9.0, here 6.1; 61 lanes the same,
+// 8.5 and 4.6), and tasks for the upper levels with this for the lower ones slower
+// still, as each launch fetches the code of both anew (256 lanes: up-sweep 17 to 23 us).
+template <typename T>
+struct FilterOps1 : FilterOps<T> {
+    PES_DEV static void combine(int a, int b, int o, int part, int, bool)
+    {
+        if (part == 0) combine_filter1<T>(a, b, o);
+    }
+    PES_DEV static void apply(int g, int e, int o, int part, int, bool)
+    {
+        if (part == 0) apply_filter1<T>(g, e, o);
+    }
 };
 
 template <typename T>
@@ -449,6 +459,20 @@ struct SmootherOps {
     {
         if (!wide) coop_apply_smoother<T>(g, e, o, part, parts);
         else if (part == 0) apply_smoother1<T>(g, e, o);
+    }
+};
+
+// The same for the smoothing scan over given arrays (256 lanes: down-sweep 4.8 us with
+// tasks for the upper levels, here 3.5).
+template <typename T>
+struct SmootherOps1 : SmootherOps<T> {
+    PES_DEV static void combine(int a, int b, int o, int part, int, bool)
+    {
+        if (part == 0) combine_smoother1<T>(a, b, o);
+    }
+    PES_DEV static void apply(int g, int e, int o, int part, int, bool)
+    {
+        if (part == 0) apply_smoother1<T>(g, e, o);
     }
 };
 
