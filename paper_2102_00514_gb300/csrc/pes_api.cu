@@ -195,6 +195,7 @@ int choose_min_steps(const pes_handle* h, int lin, pes_precision prec)
 
 struct Shape {
     int nb, nt, lpb, L;   // blocks, their threads, and of these lanes; steps per lane
+    int nb_max;           // blocks that one launch can have
 };
 
 // Time of one iteration by its launch shape, in microseconds: a step of every
@@ -230,11 +231,11 @@ pes_status make_shape(pes_handle* h, int lin, pes_precision prec, int64_t N, Sha
                     cudaGetErrorString((cudaError_t)(-cap)));
     }
     if (cap == 0) return fail(h, PES_ERR_CUDA, "the smoother kernel cannot be made co-resident on this device");
-    const int64_t blocks = std::min(cap, h->nb_max);
+    const int64_t blocks = s.nb_max = std::min(cap, h->nb_max);
     if (lin == LIN_ARRAYS || min_steps != kMinStepsPerThread || N >= blocks * s.nt * kMinStepsPerThread) {
         // A fixed shape; sizes at which all lanes have steps enough; and the scans
-        // over given arrays, which keep one partition for a size, and with it the
-        // rounding that their FP64 log-likelihoods of FP32 filters show.
+        // over given arrays, whose filter keeps one partition for a size, and with it
+        // the rounding that the FP64 log-likelihoods of FP32 filters show.
         const int64_t want = (N + (int64_t)s.nt * min_steps - 1) / ((int64_t)s.nt * min_steps);
         s.nb = (int)std::max<int64_t>(1, std::min(blocks, want));
         s.lpb = s.nt;
@@ -295,7 +296,7 @@ void fill_workspace(pes_handle* h, KParams<T>& p, const Shape& s)
     p.L = s.L;
     p.lpb = s.lpb;
     p.NL = s.nb * s.lpb;
-    p.cs = (int64_t)s.L * p.NL;
+    p.cs = p.in_place ? p.N : (int64_t)s.L * p.NL;
     p.timeout_ns = h->timeout_ns;
     p.ptime = h->ptime;
     h->ptime_blocks = s.nb;
@@ -354,8 +355,56 @@ pes_status run_persistent_shaped(pes_handle* h, KParams<T>& p, int lin, const Sh
 
 // The scans over given arrays stream lane-major copies of them, in the memory of
 // the run's stored linearisation (62 and 65 components in) and of its trajectory
-// (20 out): read in place, a lane's strided values cost every step the sectors of
-// the whole chunk (N = 128,128, FP32: 128 and 100 us per scan).
+// (20 out), or read and write the caller's arrays in place, which spares the two
+// copies' launches and costs every step the memory sectors of the whole chunk.
+//
+// FP32 filters go in place as long as one block of lanes with up to four steps each
+// takes them (us in place / with copies: 62 states 29 / 36, 501 36 / 45, 1,024 47 / 47,
+// 1,500 71 / 53, 10,001 105 / 64). FP64 does not: its time is arithmetic (62 states 299 /
+// 307, 1,024 695 / 638).
+template <typename T>
+static bool filter_in_place(const Shape& s)
+{
+    return sizeof(T) == 4 && s.nt == 256 && s.nb == 1 && s.L <= 4;
+}
+
+// FP32 smoothers go in place with one step per lane, a coalesced read, as long as the
+// grid has a lane for every state (us in place / with copies: 62 states 26 / 34, 1,024
+// 25 / 40, 10,001 25 / 57, 20,000 25 / 58). Their partition is free: the errors against
+// FP64 smoothing are those of more steps per lane (worst of 10,000 states, 8 runs: 4.1e-5
+// / 4.3e-5 in the means, 3.5e-5 / 4.3e-5 in the covariances).
+template <typename T>
+static bool smooth_in_place(Shape& s, int64_t N)
+{
+    if (sizeof(T) != 4 || s.nt != 256 || N > (int64_t)s.nb_max * s.nt) return false;
+    s.nb = (int)((N + s.nt - 1) / s.nt);
+    s.L = 1;
+    return true;
+}
+
+// One launch over the arrays of `in` (those of KParams::arr), results to `out`, a
+// mean and a covariance; `where` gives the kernel their place.
+template <typename T, class Where>
+static pes_status run_scan(pes_handle* h, KParams<T>& p, const Shape& s, bool in_place, const LaneArrays<T>& in,
+                           const LaneArrays<T>& out, cudaStream_t st, Where where)
+{
+    const int NL = s.nb * s.lpb;
+    T* const copy_out = static_cast<T*>(h->lanes);
+    p.iters = 1;
+    if (in_place) {
+        p.in_place = 1;
+        for (int i = 0; i < in.n; ++i) p.arr[i] = in.ptr[i];
+        where(out.ptr[0], out.ptr[1]);
+        return run_persistent_shaped(h, p, LIN_ARRAYS, s, st);
+    }
+    PES_CUDA(h, launch_lanes_move(in, static_cast<T*>(h->lin), p.N, s.L, NL, MOVE_IN_BLOCKED, st));
+    where(copy_out, copy_out + (int64_t)out.nc[0] * s.L * NL);
+    const pes_status r = run_persistent_shaped(h, p, LIN_ARRAYS, s, st);
+    if (r != PES_OK) return r;
+    PES_CUDA(h, launch_lanes_move(out, copy_out, p.N, s.L, NL, MOVE_OUT, st));
+    return PES_OK;
+}
+
 template <typename T>
 static pes_status filter_scan_t(pes_handle* h, const void* F, const void* c, const void* Qp, const void* H,
                                 const void* d, const void* Rp, const void* y, const void* m0, const void* P0,
@@ -363,25 +412,17 @@ static pes_status filter_scan_t(pes_handle* h, const void* F, const void* c, con
                                 cudaStream_t st, double* loglik = nullptr)
 {
     Shape s;
-    pes_status r = make_shape<T>(h, LIN_ARRAYS, prec, N, s);
+    const pes_status r = make_shape<T>(h, LIN_ARRAYS, prec, N, s);
     if (r != PES_OK) return r;
-    const int NL = s.nb * s.lpb;
-    const int64_t cs = (int64_t)s.L * NL;
-    T* in = static_cast<T*>(h->lin);
-    T* out = static_cast<T*>(h->lanes);
-    LaneArrays<T> ai, ao;
-    ai.add(F, 25).add(c, 5).add(Qp, 15).add(H, 10).add(d, 2).add(Rp, 3).add(y, 2);
-    ao.add(xf, 5).add(Pf, 15);
-    PES_CUDA(h, launch_lanes_move(ai, in, N, s.L, NL, MOVE_IN_BLOCKED, st));
+    LaneArrays<T> in, out;
+    in.add(F, 25).add(c, 5).add(Qp, 15).add(H, 10).add(d, 2).add(Rp, 3).add(y, 2);
+    out.add(xf, 5).add(Pf, 15);
     KParams<T> p{};
-    p.N = N; p.offsets = offsets; p.B = B; p.mode = MODE_FILTER; p.iters = 1;
+    p.N = N; p.offsets = offsets; p.B = B; p.mode = MODE_FILTER;
     if (loglik) PES_CUDA(h, cudaMemsetAsync(loglik, 0, sizeof(double) * B, st));
     p.loglik = loglik;
     p.m0 = (const T*)m0; p.P0 = (const T*)P0;
-    p.xf = out; p.Pf = out + 5 * cs;
-    if ((r = run_persistent_shaped(h, p, LIN_ARRAYS, s, st)) != PES_OK) return r;
-    PES_CUDA(h, launch_lanes_move(ao, out, N, s.L, NL, MOVE_OUT, st));
-    return PES_OK;
+    return run_scan(h, p, s, filter_in_place<T>(s), in, out, st, [&](T* m, T* P) { p.xf = m; p.Pf = P; });
 }
 
 template <typename T>
@@ -390,22 +431,15 @@ static pes_status smooth_scan_t(pes_handle* h, const void* F, const void* c, con
                                 pes_precision prec, cudaStream_t st)
 {
     Shape s;
-    pes_status r = make_shape<T>(h, LIN_ARRAYS, prec, N, s);
+    const pes_status r = make_shape<T>(h, LIN_ARRAYS, prec, N, s);
     if (r != PES_OK) return r;
-    const int NL = s.nb * s.lpb;
-    const int64_t cs = (int64_t)s.L * NL;
-    T* in = static_cast<T*>(h->lin);
-    T* out = static_cast<T*>(h->lanes);
-    LaneArrays<T> ai, ao;
-    ai.add(F, 25).add(c, 5).add(Qp, 15).add(xf, 5).add(Pf, 15);
-    ao.add(xs, 5).add(Ps, 15);
-    PES_CUDA(h, launch_lanes_move(ai, in, N, s.L, NL, MOVE_IN_BLOCKED, st));
+    const bool in_place = smooth_in_place<T>(s, N);
+    LaneArrays<T> in, out;
+    in.add(F, 25).add(c, 5).add(Qp, 15).add(xf, 5).add(Pf, 15);
+    out.add(xs, 5).add(Ps, 15);
     KParams<T> p{};
-    p.N = N; p.offsets = offsets; p.B = B; p.mode = MODE_SMOOTH; p.iters = 1;
-    p.x = out; p.P = out + 5 * cs;
-    if ((r = run_persistent_shaped(h, p, LIN_ARRAYS, s, st)) != PES_OK) return r;
-    PES_CUDA(h, launch_lanes_move(ao, out, N, s.L, NL, MOVE_OUT, st));
-    return PES_OK;
+    p.N = N; p.offsets = offsets; p.B = B; p.mode = MODE_SMOOTH;
+    return run_scan(h, p, s, in_place, in, out, st, [&](T* m, T* P) { p.x = m; p.P = P; });
 }
 
 // A run's lane-major arrays in h->lanes, from lx on: the trajectory's means (5),

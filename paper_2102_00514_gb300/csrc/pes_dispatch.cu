@@ -1,5 +1,7 @@
 // Dispatch from run-time (precision, linearisation, block size) to the
 // compiled configurations of the persistent kernel.
+#include <algorithm>
+
 #include "pes_internal.h"
 
 namespace pes {
@@ -8,6 +10,9 @@ template <typename T, int NT>
 static cudaError_t launch_nt(const KParams<T>& p, int lin, int nb, cudaStream_t st)
 {
     const bool ct = p.model.kind == MODEL_CT_BEARINGS;
+    if constexpr (sizeof(T) == 4 && NT == 256)   // the one compiled form (filter_in_place, smooth_in_place)
+        if (lin == LIN_ARRAYS && p.in_place) return launch_cfg<T, KK_ARRAYS_IN_PLACE, NT>(p, nb, st);
+    if (p.in_place) return cudaErrorInvalidValue;
     if (lin == LIN_ARRAYS) return launch_cfg<T, KK_ARRAYS, NT>(p, nb, st);
     if (lin == LIN_IEKS) return ct ? launch_cfg<T, KK_IEKS, NT>(p, nb, st) : launch_cfg<T, KK_IEKS_ANY, NT>(p, nb, st);
     if (lin == LIN_GH) return launch_cfg<T, KK_GH, NT>(p, nb, st);
@@ -18,7 +23,11 @@ static cudaError_t launch_nt(const KParams<T>& p, int lin, int nb, cudaStream_t 
 template <typename T, int NT>
 static int capacity_nt(int lin, int device)
 {
-    if (lin == LIN_ARRAYS) return capacity_cfg<T, KK_ARRAYS, NT>(device);
+    if (lin == LIN_ARRAYS) {
+        const int n = capacity_cfg<T, KK_ARRAYS, NT>(device);
+        if constexpr (sizeof(T) == 4 && NT == 256) return std::min(n, capacity_cfg<T, KK_ARRAYS_IN_PLACE, NT>(device));
+        return n;
+    }
     if (lin == LIN_GH) return capacity_cfg<T, KK_GH, NT>(device);
     const int a = lin == LIN_IEKS ? capacity_cfg<T, KK_IEKS, NT>(device) : capacity_cfg<T, KK_CUBATURE, NT>(device);
     const int b = lin == LIN_IEKS ? capacity_cfg<T, KK_IEKS_ANY, NT>(device) : capacity_cfg<T, KK_CUBATURE_ANY, NT>(device);

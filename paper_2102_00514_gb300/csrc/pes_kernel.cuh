@@ -64,10 +64,15 @@ constexpr int LINS = 65;          // stored linearisation scalars per state, at 
 
 // The compiled forms of the smoother: the linearisation, and whether the model
 // is known to be the coordinated turn (the structure of its slopes, and no code
-// for the linear model in the loops) or is looked up (_ANY).
-enum { KK_ARRAYS = 0, KK_IEKS = 1, KK_CUBATURE = 2, KK_GH = 3, KK_IEKS_ANY = 4, KK_CUBATURE_ANY = 5 };
+// for the linear model in the loops) or is looked up (_ANY); the scans over given
+// arrays read lane-major copies of them or the arrays themselves (_IN_PLACE).
+enum { KK_ARRAYS = 0, KK_IEKS = 1, KK_CUBATURE = 2, KK_GH = 3, KK_IEKS_ANY = 4, KK_CUBATURE_ANY = 5, KK_ARRAYS_IN_PLACE = 6 };
 template <int K>
-constexpr int kLinOf = K == KK_IEKS_ANY ? LIN_IEKS : (K == KK_CUBATURE_ANY ? LIN_CUBATURE : K);
+constexpr int kLinOf = K == KK_IEKS_ANY ? LIN_IEKS
+                       : K == KK_CUBATURE_ANY ? LIN_CUBATURE
+                       : K == KK_ARRAYS_IN_PLACE ? LIN_ARRAYS : K;
+template <int K>
+constexpr bool kArrays = kLinOf<K> == LIN_ARRAYS;
 template <int K>
 constexpr int kFS = K == KK_IEKS ? FS_CT : (K == KK_CUBATURE ? FS_SLR : FS_DENSE);
 
@@ -96,7 +101,7 @@ constexpr int kRtsStages = (kStoreLin<K> && K != KK_CUBATURE) ? 3 : 4;
 constexpr int kMaxStages = 4;
 // Whether the trees keep combine_filter's rounding (fold_filter_arrays).
 template <int K, typename T>
-constexpr bool kKeepRounding = K == KK_ARRAYS && sizeof(T) == 4;
+constexpr bool kKeepRounding = kArrays<K> && sizeof(T) == 4;
 
 template <typename T>
 struct KParams {
@@ -123,8 +128,12 @@ struct KParams {
     // workspace
     T* hand;           // MODE_RUN: filtered moments, kept for the RTS pass: [warp][s][HAND][32 lanes]
     // MODE_RUN: the sigma-point linearisation, handed from the fold to the later
-    // passes; MODE_FILTER / MODE_SMOOTH: the given arrays: [warp][s][component][32]
+    // passes; MODE_FILTER / MODE_SMOOTH: the given arrays' copy: [warp][s][component][32]
     T* lin;
+    // MODE_FILTER / MODE_SMOOTH, in_place (KK_ARRAYS_IN_PLACE): the given arrays
+    // themselves, [component][N], results in the caller's arrays too (cs = N)
+    const T* arr[7];   // F, c, Q', H, d, R', y or F, c, Q', filtered mean and covariance
+    int in_place;
     T* aggF;           // [2][agg_blocks][FE]: the blocks' filtering elements, by iteration parity
     T* aggS;           // [2][agg_blocks][SE]: their smoothing elements
     int agg_blocks;    // blocks the aggregates have room for
@@ -491,6 +500,33 @@ PES_DEV const T* array_warp(const KParams<T>& p, int s, int lane)
     return p.lin + ((size_t)(lane >> 5) * p.L + s) * (NC * 32);
 }
 
+// The same components of state k from the caller's arrays, NC of them in all.
+template <typename T, int NC>
+struct ArrayState {
+    const KParams<T>& p;
+    int64_t k;
+    // (read-only loads: the results' arrays may be the filtered moments', but a lane
+    // reads a state before it writes it, and no other lane reads it)
+    PES_DEV T at(int arr, int c) const { return __ldg(p.arr[arr] + c * p.N + k); }
+    PES_DEV T get(int, int c) const
+    {
+        if (c < 25) return at(0, c);
+        if (c < 30) return at(1, c - 25);
+        if (c < 45) return at(2, c - 30);
+        if (NC == kSmoothIn) return c < 50 ? at(3, c - 45) : at(4, c - 50);
+        if (c < 55) return at(3, c - 45);
+        if (c < 57) return at(4, c - 55);
+        return c < 60 ? at(5, c - 57) : at(6, c - 60);
+    }
+};
+
+// Place of state k = a + s of a lane in the scans' outputs.
+template <bool IP, typename T>
+PES_DEV int64_t array_ix(const KParams<T>& p, int64_t k, int s, int lane)
+{
+    return IP ? k : lane_ix(p, s, lane);
+}
+
 template <typename T, class S>
 PES_DEV void array_trans(const S& q, int i, Trans<T>& tr)
 {
@@ -518,10 +554,14 @@ PES_DEV void array_obs(const S& q, int i, Obs<T>& ob)
     for (int c = 0; c < 5; ++c) ob.xn[c] = T(0);
 }
 
-// The transition out of the last state of the lane before `lane`.
-template <typename T>
-PES_DEV void load_array_trans(const KParams<T>& p, int lane, Trans<T>& tr)
+// The transition out of state a - 1, the last one of the lane before `lane`.
+template <bool IP, typename T>
+PES_DEV void load_array_trans(const KParams<T>& p, int64_t a, int lane, Trans<T>& tr)
 {
+    if constexpr (IP) {
+        array_trans(ArrayState<T, kFilterIn>{p, a - 1}, 0, tr);
+        return;
+    }
     const T* h = array_warp<kFilterIn>(p, p.L - 1, lane - 1) + ((lane - 1) & 31);
 #pragma unroll
     for (int i = 0; i < 25; ++i) tr.F[i] = __ldg(h + i * 32);
@@ -660,8 +700,9 @@ PES_DEV bool fold_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int la
 // The same over given arrays (the filter scan). Its chunks' boundaries are the
 // filtered states, each step predicting from the previous state and then
 // updating: its results keep the rounding that they always had, which the FP64
-// log-likelihoods of FP32 runs show.
-template <typename T>
+// log-likelihoods of FP32 runs show. IP: from the caller's arrays in place, without
+// a stream.
+template <bool IP, typename T>
 PES_DEV bool fold_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, int steps, FElem<T>& acc, T* wstage,
                                 uint64_t* wbar, uint32_t& wpar)
 {
@@ -672,13 +713,13 @@ PES_DEV bool fold_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int l
     ws.init(wstage, wbar, wpar);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-        if (i < steps) ws.issue(array_warp<kFilterIn>(p, i, lane), i);
+        if (!IP && i < steps) ws.issue(array_warp<kFilterIn>(p, i, lane), i);
     SegCursor cur;
     if (a < e) {
         cur.init(p.offsets, p.B, a);
         if (!cur.is_head(a)) {   // the transition out of the previous lane's last state
             Trans<T> tr;
-            load_array_trans(p, lane, tr);
+            load_array_trans<IP>(p, a, lane, tr);
             fold_predict(acc, tr);
         }
     }
@@ -686,7 +727,8 @@ PES_DEV bool fold_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int l
     for (int s = 0; s < steps; ++s) {
         const int64_t k = a + s;
         const int st = s & 1;
-        ws.wait(st, p.status);
+        const ArrayState<T, kFilterIn> own{p, k};
+        if (!IP) ws.wait(st, p.status);
         if (k < e) {
             cur.forward(k);
             if (cur.is_head(k)) {
@@ -695,19 +737,22 @@ PES_DEV bool fold_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int l
                 felem_apply_prior(acc, m0, P0);
             } else {
                 Obs<T> ob;
-                array_obs(ws, st, ob);
+                if constexpr (IP) array_obs(own, 0, ob);
+                else array_obs(ws, st, ob);
                 ok &= fold_update(acc, ob);
             }
             if (!cur.is_tail(k) && k + 1 < e) {
                 Trans<T> tr;
-                array_trans(ws, st, tr);
+                if constexpr (IP) array_trans(own, 0, tr);
+                else array_trans(ws, st, tr);
                 fold_predict(acc, tr);
             }
         }
+        if (IP) continue;
         __syncwarp();
         if (s + 2 < steps) ws.issue(array_warp<kFilterIn>(p, s + 2, lane), st);
     }
-    wpar = ws.parity;
+    if (!IP) wpar = ws.parity;
     return ok;
 }
 
@@ -904,7 +949,7 @@ PES_DEV bool rerun_filter_chunk(const KParams<T>& p, int64_t a, int64_t e, int l
 }
 
 // The same over given arrays, with the log-likelihoods if they are wanted.
-template <typename T>
+template <bool IP, typename T>
 PES_DEV bool rerun_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, int steps, const Gauss<T>& G, T* wstage,
                                  uint64_t* wbar, uint32_t& wpar)
 {
@@ -920,31 +965,32 @@ PES_DEV bool rerun_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int 
     for (int i = 0; i < 15; ++i) P[i] = G.P[i];
     FilterStream<T> ws;
     ws.init(wstage, wbar, wpar);
-    ws.issue(array_warp<kFilterIn>(p, 0, lane), 0);
-    if (steps > 1) ws.issue(array_warp<kFilterIn>(p, 1, lane), 1);
+    if (!IP) ws.issue(array_warp<kFilterIn>(p, 0, lane), 0);
+    if (!IP && steps > 1) ws.issue(array_warp<kFilterIn>(p, 1, lane), 1);
     int st = 0;
 #pragma unroll 1
     for (int s = 0; s < steps; ++s) {
         const int64_t k = a + s;
         const int other = st == 0 ? 2 : st - 1;   // the stage of steps s - 1 and s + 2
-        ws.wait(st, p.status);
+        if (!IP) ws.wait(st, p.status);
         const bool head = k < e && (cur.forward(k), cur.is_head(k));
         T mp[5], Pp[15];
         if (k < e && !head) {
             Trans<T> tr;
-            if (s > 0) array_trans(ws, other, tr);
-            else load_array_trans(p, lane, tr);
+            if (!IP && s > 0) array_trans(ws, other, tr);
+            else load_array_trans<IP>(p, k, lane, tr);
             T FP[25];
             predict(tr, m, P, mp, FP, Pp);
         }
-        __syncwarp();   // every lane is done with step s - 1
-        if (s + 2 < steps) ws.issue(array_warp<kFilterIn>(p, s + 2, lane), other);
+        if (!IP) __syncwarp();   // every lane is done with step s - 1
+        if (!IP && s + 2 < steps) ws.issue(array_warp<kFilterIn>(p, s + 2, lane), other);
         if (k < e) {
             if (head) {
                 load_prior(p, cur.b, m, P);
             } else {
                 Obs<T> ob;
-                array_obs(ws, st, ob);
+                if constexpr (IP) array_obs(ArrayState<T, kFilterIn>{p, k}, 0, ob);
+                else array_obs(ws, st, ob);
                 if (p.loglik) {
                     if (cur.b != llb) {
                         if (llb >= 0) atomicAdd(p.loglik + llb, ll.value());
@@ -956,12 +1002,14 @@ PES_DEV bool rerun_filter_arrays(const KParams<T>& p, int64_t a, int64_t e, int 
                     ok &= kf_update(ob, mp, Pp, m, P);
                 }
             }
-            store_filtered(p, lane_ix(p, s, lane), m, P);
+            store_filtered(p, array_ix<IP>(p, k, s, lane), m, P);
         }
         st = st == 2 ? 0 : st + 1;
     }
-    __syncwarp();
-    wpar = ws.parity;
+    if (!IP) {
+        __syncwarp();
+        wpar = ws.parity;
+    }
     if (llb >= 0) atomicAdd(p.loglik + llb, ll.value());
     return ok;
 }
@@ -1018,9 +1066,10 @@ PES_DEV bool chunk_selem(const KParams<T>& p, int64_t a, int64_t e, const FElem<
     return selem_from_prediction(md, D, AD, Pp, mp, el);
 }
 
-// The smoothing element of a state from stage i of the given arrays' stream.
-template <typename T>
-PES_DEV bool array_selem(const SmoothStream<T>& ws, int i, bool tail, SElem<T>& el)
+// The smoothing element of a state from stage i of the given arrays' stream (or from
+// the arrays in place).
+template <typename T, class S>
+PES_DEV bool array_selem(const S& ws, int i, bool tail, SElem<T>& el)
 {
     T m[5], P[15];
 #pragma unroll
@@ -1038,9 +1087,27 @@ PES_DEV bool array_selem(const SmoothStream<T>& ws, int i, bool tail, SElem<T>& 
     return selem_from_prediction(m, P, FP, Pp, mp, el);
 }
 
+// IP: the elements themselves are kept for the RTS pass, [step][component][lane], each
+// written and read by its own lane (50 scalars; forming one again costs more than
+// they do where the arrays are read in place).
+template <typename T, typename F>
+PES_DEV void each_selem_scalar(const KParams<T>& p, int s, int lane, SElem<T>& el, F f)
+{
+    static_assert(LINS >= 50, "the scratch holds an element per state");
+    T* q = p.lin + (size_t)s * 50 * p.NL + lane;
+#pragma unroll
+    for (int i = 0; i < 25; ++i) f(el.E[i], q[(size_t)i * p.NL]);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) f(el.g[i], q[(size_t)(25 + i) * p.NL]);
+#pragma unroll
+    for (int i = 0; i < 15; ++i) f(el.L[i], q[(size_t)(30 + i) * p.NL]);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) f(el.xr[i], q[(size_t)(45 + i) * p.NL]);
+}
+
 // Smoothing, level 1 in MODE_SMOOTH: fold the chunk's smoothing elements from
 // the given filtered moments and transitions.
-template <typename T>
+template <bool IP, typename T>
 PES_DEV bool fold_smoother_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, int steps, SElem<T>& accS, T* wstage,
                                   uint64_t* wbar, uint32_t& wpar)
 {
@@ -1052,25 +1119,31 @@ PES_DEV bool fold_smoother_arrays(const KParams<T>& p, int64_t a, int64_t e, int
     ws.init(wstage, wbar, wpar);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-        if (i < steps) ws.issue(array_warp<kSmoothIn>(p, i, lane), i);
+        if (!IP && i < steps) ws.issue(array_warp<kSmoothIn>(p, i, lane), i);
 #pragma unroll 1
     for (int s = 0; s < steps; ++s) {
-        ws.wait(s & 1, p.status);
+        if (!IP) ws.wait(s & 1, p.status);
         if (a + s < e) {
             cur.forward(a + s);
             SElem<T> el;
-            ok &= array_selem(ws, s & 1, cur.is_tail(a + s), el);
+            if constexpr (IP) {
+                ok &= array_selem(ArrayState<T, kSmoothIn>{p, a + s}, 0, cur.is_tail(a + s), el);
+                each_selem_scalar(p, s, lane, el, [](T v, T& kept) { kept = v; });
+            } else {
+                ok &= array_selem(ws, s & 1, cur.is_tail(a + s), el);
+            }
             combine_smoother(accS, el, accS);
         }
+        if (IP) continue;
         __syncwarp();
         if (s + 2 < steps) ws.issue(array_warp<kSmoothIn>(p, s + 2, lane), s & 1);
     }
-    wpar = ws.parity;
+    if (!IP) wpar = ws.parity;
     return ok;
 }
 
 // Smoothing, level 5 in MODE_SMOOTH.
-template <typename T>
+template <bool IP, typename T>
 PES_DEV bool rts_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, int steps, const Gauss<T>& G, T* wstage,
                         uint64_t* wbar, uint32_t& wpar)
 {
@@ -1084,17 +1157,18 @@ PES_DEV bool rts_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, int
     ws.init(wstage, wbar, wpar);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-        if (i < steps) ws.issue(array_warp<kSmoothIn>(p, steps - 1 - i, lane), i);
+        if (!IP && i < steps) ws.issue(array_warp<kSmoothIn>(p, steps - 1 - i, lane), i);
     int st = 0;
 #pragma unroll 1
     for (int sidx = steps - 1; sidx >= 0; --sidx, st ^= 1) {
         const int64_t k = a + sidx;
-        ws.wait(st, p.status);
+        if (!IP) ws.wait(st, p.status);
         if (k < e) {
             cur.backward(k);
-            const int64_t ix = lane_ix(p, sidx, lane);
+            const int64_t ix = array_ix<IP>(p, k, sidx, lane);
             SElem<T> el;
-            ok &= array_selem(ws, st, cur.is_tail(k), el);
+            if constexpr (IP) each_selem_scalar(p, sidx, lane, el, [](T& v, T kept) { v = kept; });
+            else ok &= array_selem(ws, st, cur.is_tail(k), el);
             apply_smoother(el, s, s);
             bool finite = true;
 #pragma unroll
@@ -1106,10 +1180,11 @@ PES_DEV bool rts_arrays(const KParams<T>& p, int64_t a, int64_t e, int lane, int
 #pragma unroll
             for (int i = 0; i < 15; ++i) p.P[i * p.cs + ix] = s.P[i];
         }
+        if (IP) continue;
         __syncwarp();
         if (sidx >= 2) ws.issue(array_warp<kSmoothIn>(p, sidx - 2, lane), st);
     }
-    wpar = ws.parity;
+    if (!IP) wpar = ws.parity;
     return ok;
 }
 
@@ -1251,7 +1326,7 @@ constexpr size_t smem_bytes_for()
 {
     using M = TreeMem<T, NT>;
     static_assert(M::kEnd - FE * NT >= NT * 3 * kStateIn, "the sigma-point folds' prefetch fits beside the leaves");
-    static_assert(K != KK_ARRAYS || (M::kEnd - FE * NT >= NT * 2 * kFilterIn && M::kEnd >= NT * 3 * kFilterIn &&
+    static_assert(!kArrays<K> || (M::kEnd - FE * NT >= NT * 2 * kFilterIn && M::kEnd >= NT * 3 * kFilterIn &&
                                      M::kEnd - SE * NT >= NT * 2 * kSmoothIn),
                   "the streams of the scans over given arrays fit");
     static_assert(M::kBlock - M::kAfterSmootherTree >= NT * kLinStages<K> * kLinScalars<K>, "the re-run's stages fit");
@@ -1310,8 +1385,8 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
         if (do_filter) {
             FElem<T> acc;
             // the fold's prefetch goes to memory beside the leaves
-            if constexpr (K == KK_ARRAYS)
-                ok &= fold_filter_arrays(p, a, e, lane, steps, acc, smem + FE * NT + (size_t)warp * 2 * kFilterIn * 32, wbar, wpar);
+            if constexpr (kArrays<K>)
+                ok &= fold_filter_arrays<K == KK_ARRAYS_IN_PLACE>(p, a, e, lane, steps, acc, smem + FE * NT + (size_t)warp * 2 * kFilterIn * 32, wbar, wpar);
             else
                 ok &= fold_filter_chunk<K>(p, a, e, lane, acc, Prefetch<T, kStateIn>{smem + FE * NT + t, NT, p.x, p.cs});
             PES_PHASE(p, it, 1);
@@ -1327,8 +1402,8 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
             PES_PHASE(p, it, 5);
             if (do_smooth) ok &= chunk_selem(p, a, e, reinterpret_cast<const FElem<T>*>(smem)[tree_place(min(t, nl - 1), nl)], G, accS);
         } else {
-            if constexpr (K == KK_ARRAYS)
-                ok &= fold_smoother_arrays(p, a, e, lane, steps, accS, smem + SE * NT + (size_t)warp * 2 * kSmoothIn * 32, wbar, wpar);
+            if constexpr (kArrays<K>)
+                ok &= fold_smoother_arrays<K == KK_ARRAYS_IN_PLACE>(p, a, e, lane, steps, accS, smem + SE * NT + (size_t)warp * 2 * kSmoothIn * 32, wbar, wpar);
         }
         __syncthreads();   // the smoother's tree and the stream stages overlap the filter's
         if (do_smooth) {
@@ -1337,8 +1412,8 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
         }
         PES_PHASE(p, it, 6);
         if (do_filter) {
-            if constexpr (K == KK_ARRAYS) {
-                ok &= rerun_filter_arrays(p, a, e, lane, steps, G, smem + (size_t)warp * 3 * kFilterIn * 32, wbar, wpar);
+            if constexpr (kArrays<K>) {
+                ok &= rerun_filter_arrays<K == KK_ARRAYS_IN_PLACE>(p, a, e, lane, steps, G, smem + (size_t)warp * 3 * kFilterIn * 32, wbar, wpar);
             } else {
                 constexpr int kStage = kLinStages<K> * kLinScalars<K> * 32;
                 ok &= rerun_filter_chunk<K>(p, a, e, lane, steps, G, smem + M::kAfterSmootherTree + (size_t)warp * kStage, wbar, wpar);
@@ -1364,8 +1439,8 @@ __global__ void __launch_bounds__(NT, 1) pes_persistent_kernel(const KParams<T> 
             int nb = -1;
             double num = 0.0, den = 0.0;
             double* conv = p.conv + (size_t)(it & 1) * 2 * p.B;
-            if constexpr (K == KK_ARRAYS) {
-                ok &= rts_arrays(p, a, e, lane, steps, Gs, smem + (size_t)warp * 2 * kSmoothIn * 32, wbar, wpar);
+            if constexpr (kArrays<K>) {
+                ok &= rts_arrays<K == KK_ARRAYS_IN_PLACE>(p, a, e, lane, steps, Gs, smem + (size_t)warp * 2 * kSmoothIn * 32, wbar, wpar);
             } else {
                 constexpr int kStage = kRtsStages<K> * (HAND + (kStoreLin<K> ? kLinTrans<K> : 0)) * 32;
                 ok &= rts_chunk<K>(p, a, e, lane, steps, Gs, write_P, track, conv, nb, num, den, smem + (size_t)warp * kStage, wbar, wpar);

@@ -100,3 +100,36 @@ def test_filter_loglik_matches_oracle(sm, name, T_list, prec, tol):
     # the filtered moments are those of pes_filter_scan
     assert rel_err(xf.double().cpu().numpy(), refx["xf"], off) < tol
     assert rel_err(Pf.double().cpu().numpy(), refx["Pf"], off) < tol
+
+
+# the first and last sizes of the in-place routes (FP32 filter: 1,024 states, one block
+# of four steps; FP32 smoother: one lane per state of the grid), and trajectory edges
+# inside and at the ends of lanes, warps and blocks
+ROUTES = [[1022], [1023], [1024], [1025], [0, 0, 1, 2, 252, 0, 255, 511 - 9], [255, 255, 255, 255], [38910], [38911],
+          [38912], [19000, 0, 19909], [19000, 0, 19910]]
+
+
+@pytest.mark.parametrize("T_list", ROUTES, ids=lambda t: f"N{sum(t) + len(t)}B{len(t)}")
+def test_routes_of_the_fp32_scans_match_oracle(sm, T_list):
+    got, ref, off = _run(sm, pes.FP32, T_list, seed=len(T_list) + T_list[0])
+    for k in ("xf", "Pf", "xs", "Ps"):
+        assert rel_err(got[k], ref[k], off) < TOL_FP32, k
+
+
+@pytest.mark.parametrize("prec,tol", [(pes.FP64, TOL_FP64), (pes.FP32, TOL_FP32)])
+@pytest.mark.parametrize("T", [37, 700, 20011, 60000])
+def test_smoothed_moments_may_replace_the_filtered_ones(sm, prec, tol, T):
+    """xs and Ps in the buffers of xf and Pf, on every route."""
+    import ctypes
+    lin, y, m0, P0, off = random_linear_workload([T, 5], T)
+    dt = torch.float64 if prec == pes.FP64 else torch.float32
+    dlin = {k: to_dev(v, dt) for k, v in lin.items()}
+    doff = to_dev(off, torch.int64)
+    xf, Pf = sm.filter_scan(prec, dlin, to_dev(y, dt), to_dev(m0, dt), to_dev(P0, dt), doff)
+    xs, Ps = sm.smooth_scan(prec, dlin, xf, Pf, doff)
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    st = sm.lib.pes_smooth_scan(sm.h, prec, p(dlin["F"]), p(dlin["c"]), p(dlin["Qp"]), p(xf), p(Pf), p(doff), 2,
+                                y.shape[1], p(xf), p(Pf), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == pes.OK
+    sm.sync()
+    assert torch.equal(xf, xs) and torch.equal(Pf, Ps)
