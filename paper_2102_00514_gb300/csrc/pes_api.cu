@@ -203,13 +203,13 @@ struct Shape {
 // level's, each with at least 8, 4 or 2 threads to an operator (both scans, up and
 // down). Measured at T = 500 to 262,147 with 32 to 256 lanes per block.
 struct ShapeCost {
-    double step[2];    // Taylor, sigma points
+    double step[3];    // Taylor, symmetric sigma points, Gauss-Hermite (243 points)
     double level[3];
     double top[3];
     int top_nodes;     // of a grid level at a time (TreeMem::TOPN)
 };
-constexpr ShapeCost kCost32{{4.2, 6.0}, {3.4, 6.9, 9.6}, {1.9, 4.9, 6.0}, 80};
-constexpr ShapeCost kCost64{{61.0, 100.0}, {54.0, 71.0, 100.0}, {28.0, 42.0, 60.0}, 76};
+constexpr ShapeCost kCost32{{4.2, 6.0, 130.0}, {3.4, 6.9, 9.6}, {1.9, 4.9, 6.0}, 80};
+constexpr ShapeCost kCost64{{61.0, 100.0, 2000.0}, {54.0, 71.0, 100.0}, {28.0, 42.0, 60.0}, 76};
 
 // The tree over n elements.
 double tree_cost(const double (&c)[3], int nt, int n)
@@ -254,16 +254,20 @@ pes_status make_shape(pes_handle* h, int lin, pes_precision prec, int64_t N, Sha
     // FP32 has two steps per lane at least: with one, every state goes through the
     // trees' operators, and their rounding shows for little time (8 trajectories of 607,
     // cubature: worst covariance error 6.9e-6 with two steps, 1.6e-5 with one; three
-    // iterations 176 and 169 us).
+    // iterations 176 and 169 us). Where a step is worth ten levels, Gauss-Hermite, a
+    // block's worth of states still has one each (62 states, two iterations: 584 us with
+    // two steps, 332 with one).
     const ShapeCost& c = sizeof(T) == 8 ? kCost64 : kCost32;
     const int top_nodes = sizeof(T) == 4 && s.nt == 256 ? 152 : c.top_nodes;
+    const double step = c.step[lin == LIN_IEKS ? 0 : (lin == LIN_GH ? 2 : 1)];
+    const int64_t least = sizeof(T) == 8 || (lin == LIN_GH && N <= s.nt) ? 1 : 2;
     double best = 1e300;
     for (int lpb = 32; lpb <= s.nt; lpb += 32) {
-        const int64_t L0 = std::max<int64_t>((N + blocks * lpb - 1) / (blocks * lpb), sizeof(T) == 4 ? 2 : 1);
+        const int64_t L0 = std::max((N + blocks * lpb - 1) / (blocks * lpb), least);
         for (int64_t L = L0; L < L0 + 8; ++L) {
             const int64_t lanes = (N + L - 1) / L, nb = (lanes + lpb - 1) / lpb;
             if (L > L0 && L * nb * lpb > N + h->nl_max) break;   // the workspace
-            double t = L * c.step[lin != LIN_IEKS];
+            double t = L * step;
             if (t >= best) break;
             t += tree_cost(c.level, s.nt, (int)std::min<int64_t>(lanes, lpb));
             for (int64_t left = nb; left > 1; left -= top_nodes - 1)
