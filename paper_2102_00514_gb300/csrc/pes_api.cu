@@ -819,8 +819,13 @@ static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_preci
     T* ly = lP + 15 * cs;
     T* xold = static_cast<T*>(h->refw);
     T* Pold = xold + 5 * cs;
+    // the residuals follow them: 24 doubles of the 540 bytes per slot
+    static_assert(24 * sizeof(double) <= sizeof(float) * (20 + RE + RT + RD), "the workspace holds them");
+    lp.resid = static_cast<double*>(h->refw) + 20 * cs;
+    lp.resid_step = lp.resid + 2 * cs;
     const size_t Bm = (size_t)h->max_batch;
     double* dw = static_cast<double*>(h->lmw);
+    lp.norms = tol > 0.0;
     lp.change = dw;
     lp.num = dw + Bm;
     lp.den = dw + 2 * Bm;
@@ -846,6 +851,7 @@ static pes_status ieks_run_lm_t(pes_handle* h, const pes_model* model, pes_preci
                                              x_init ? nullptr : lx, lP, st));
     PES_CUDA(h, cudaMemsetAsync(lp.accepted, 0, 2 * Bm * sizeof(int), st));
     PES_CUDA(h, launch_lm_fill<T>(lam, B, lambda0, st));
+    PES_CUDA(h, launch_lm_resid<T>(lp, lx, ly, st));
     KParams<T> p{};
     p.N = N; p.offsets = offsets; p.B = B; p.mode = MODE_RUN; p.iters = 1; p.tol = 0.0;
     if ((r = device_model<T>(h, *model, B, st, p.model, PES_IEKS)) != PES_OK) return r;

@@ -19,7 +19,10 @@ struct LMParams {
     const double* sensors;   // device [1 or B][4]
     double F[25], c[5], H[10], d[2];   // linear model
     double Qi[15], Ri[3];              // inverses of Q and R (packed)
+    double* resid;      // [2][cs] the bearings' residuals at the nominal
+    double* resid_step; // [2][cs] and after the step
     double* change;     // [B] what the step changes the objective by
+    int norms;          // whether the two that follow are wanted
     double* num;        // [B] squared step
     double* den;        // [B] squared norm after it
     int* reject;        // [B]
@@ -28,6 +31,9 @@ struct LMParams {
     int* unconv;        // trajectories not yet converged
 };
 
+// The bearings' residuals at the first nominal x into p.resid (a linear model needs none).
+template <typename T>
+cudaError_t launch_lm_resid(const LMParams& p, const T* x, const T* y, cudaStream_t st);
 // What the step from xold to x changes every trajectory's objective by, the
 // squared step and the squared norm after it, added into p.change, p.num, p.den.
 template <typename T>
