@@ -270,3 +270,22 @@ def test_a_tuning_at_a_large_size_keeps_the_choice_for_small_ones():
         assert s.launch_shape(pes.IEKS, pes.FP64, 501) == small
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("prec,threads,tol", [(pes.FP64, 128, TOL_FP64), (pes.FP32, 256, TOL_FP32)])
+def test_layout_copies_at_whole_chunks_and_pieces(prec, threads, tol):
+    """Steps per lane around the widths at which the copies' tiles change (banks' words,
+    the widest whole chunk of 63 steps), in a block whose last lane lacks a state."""
+    s = pes.Smoother(1 << 15, 1)
+    try:
+        for L in (1, 2, 3, 5, 8, 15, 16, 17, 31, 32, 33, 62, 63, 64, 65, 126, 127):
+            N = L * threads - (1 if L > 1 else 0)
+            w = linear_case(N - 1, seed=L)
+            s.set_launch_shape(pes.IEKS, prec, threads, L if L != 8 else 9)   # 8 leaves the steps to the library
+            assert L == 8 or s.launch_shape(pes.IEKS, prec, N) == (1, threads, L)
+            ref = oracle.iterated_smoother(w["om"], oracle.IEKS, w["off"], w["y"], w["m0"], w["P0"], iters=1)
+            x, P = linear_run(s, w, pes.IEKS, prec)
+            assert rel_err(x, ref["x"], w["off"]) < tol, L
+            assert rel_err(P, ref["P"], w["off"]) < tol, L
+    finally:
+        s.close()
